@@ -423,20 +423,22 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       }
     }
   } else if (warp == 9) {
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();   // the warp walks the loop together; one lane issues
       constexpr uint32_t idesc_qk = umma_idesc_bf16(QT, KT);
       constexpr uint32_t idesc_pv = umma_idesc_bf16(QT, HD);
       const uint32_t q_addr = smem_u32(q_s);
       // S_t = Q_t K^T for the key tile in stage s
       auto issue_qk = [&](int t, int s) {
-        const uint32_t k_addr = smem_u32(k_s + s * Cfg::kKBytes);
-        const uint32_t qa = q_addr + t * Cfg::kQBytes;
+        const uint64_t kd = umma_desc_k_sw128(smem_u32(k_s + s * Cfg::kKBytes)), qd = umma_desc_k_sw128(q_addr + t * Cfg::kQBytes);
+        if (leader) {
 #pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * (QT * 128) + (kk & 3) * 32;
-          umma_bf16(tmem_base + t * KT, umma_desc_k_sw128(qa + off), umma_desc_k_sw128(k_addr + off), idesc_qk, kk != 0);
+          for (int kk = 0; kk < HD / 16; ++kk) {
+            const uint32_t off = ((kk >> 2) * (QT * 128) + (kk & 3) * 32) >> 4;
+            umma_bf16(tmem_base + t * KT, qd + off, kd + off, idesc_qk, kk != 0);
+          }
+          umma_commit(&s_full[t]);
         }
-        umma_commit(&s_full[t]);
       };
       uint32_t kt = 0;             // key tiles consumed so far (ring position)
       uint32_t pc[2] = {0, 0};     // probability tiles consumed per query tile (phase of p_full)
@@ -450,8 +452,10 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         if (!mbar_wait(q_full, seg & 1) || !mbar_wait(&k_full[kt % NS], (kt / NS) & 1)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
         tc_fence_after();
         for (int t = 0; t < sg.ntiles; ++t) issue_qk(t, kt % NS);
-        umma_commit(&k_empty[kt % NS]);
-        if (Tseg == 1) umma_commit(q_empty);
+        if (leader) {
+          umma_commit(&k_empty[kt % NS]);
+          if (Tseg == 1) umma_commit(q_empty);
+        }
         for (int jj = 0; ok && jj < Tseg; ++jj) {
           const uint32_t cur = kt + jj, nxt = cur + 1;
           const int s = cur % NS, sn = nxt % NS;
@@ -459,7 +463,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           if (!mbar_wait(&v_full[s], (cur / NS) & 1) || (more && !mbar_wait(&k_full[sn], (nxt / NS) & 1))) {
             report(p.status, DEV_TIMEOUT_MMA); ok = false; break;
           }
-          const uint32_t v_addr = smem_u32(v_s + s * Cfg::kVBytes);
+          const uint64_t vd = umma_desc_k_sw128(smem_u32(v_s + s * Cfg::kVBytes));
           for (int t = 0; t < sg.ntiles; ++t) {
             // the first P V of a segment overwrites O_t: the O of the last segment that used tile t must have been
             // read out (its softmax threads arrive once per segment in which the tile is used, so neither side can
@@ -470,18 +474,22 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             tc_fence_after();
             const uint32_t p_tmem = tmem_base + t * KT;              // P_t over the first 64 columns of S_t
             const uint32_t o_tmem = tmem_base + 256 + t * 128;
+            if (leader) {
 #pragma unroll
-            for (int kk = 0; kk < KT / 16; ++kk) {
-              const uint32_t b_off = (kk >> 2) * (HD * 128) + (kk & 3) * 32;
-              umma_bf16_ts(o_tmem, p_tmem + kk * 8, umma_desc_k_sw128(v_addr + b_off), idesc_pv, (jj | kk) != 0);
+              for (int kk = 0; kk < KT / 16; ++kk) {
+                const uint32_t b_off = ((kk >> 2) * (HD * 128) + (kk & 3) * 32) >> 4;
+                umma_bf16_ts(o_tmem, p_tmem + kk * 8, vd + b_off, idesc_pv, (jj | kk) != 0);
+              }
+              umma_commit(&o_done[t]);
             }
-            umma_commit(&o_done[t]);
             if (more) issue_qk(t, sn);
           }
           if (!ok) break;
-          umma_commit(&v_empty[s]);
-          if (more) umma_commit(&k_empty[sn]);
-          if (more && jj + 2 == Tseg) umma_commit(q_empty);   // the segment's last Q K^T have been issued
+          if (leader) {
+            umma_commit(&v_empty[s]);
+            if (more) umma_commit(&k_empty[sn]);
+            if (more && jj + 2 == Tseg) umma_commit(q_empty);   // the segment's last Q K^T have been issued
+          }
         }
         kt += Tseg;
         for (int t = 0; t < sg.ntiles; ++t) ++oc[t];
@@ -593,27 +601,29 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       }
     }
   } else if (warp == 9) {
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();   // the warp walks the loop together; one lane issues
       constexpr uint32_t idesc_qk = umma_idesc_bf16(QT, KT);
       constexpr uint32_t idesc_pv = umma_idesc_bf16(QT, HD);
       const uint32_t q_addr = smem_u32(q_s);
       // S_t = Q_t K^T for the key tile in stage s
       auto issue_qk = [&](int t, int s) {
-        const uint32_t k_addr = smem_u32(k_s + s * Cfg::kKBytes);
-        const uint32_t qa = q_addr + t * Cfg::kQBytes;
+        const uint64_t kd = umma_desc_k_sw128(smem_u32(k_s + s * Cfg::kKBytes)), qd = umma_desc_k_sw128(q_addr + t * Cfg::kQBytes);
+        if (leader) {
 #pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * (QT * 128) + (kk & 3) * 32;
-          umma_bf16(tmem_base + t * KT, umma_desc_k_sw128(qa + off), umma_desc_k_sw128(k_addr + off), idesc_qk, kk != 0);
+          for (int kk = 0; kk < HD / 16; ++kk) {
+            const uint32_t off = ((kk >> 2) * (QT * 128) + (kk & 3) * 32) >> 4;
+            umma_bf16(tmem_base + t * KT, qd + off, kd + off, idesc_qk, kk != 0);
+          }
+          umma_commit(&s_full[t]);
         }
-        umma_commit(&s_full[t]);
       };
       bool ok = mbar_wait(q_full, 0) && mbar_wait(&k_full[0], 0);
       if (!ok) report(p.status, DEV_TIMEOUT_MMA);
       if (ok) {
         tc_fence_after();
         for (int t = 0; t < ntiles; ++t) issue_qk(t, 0);
-        umma_commit(&k_empty[0]);
+        if (leader) umma_commit(&k_empty[0]);
       }
       for (int j = 0; ok && j < T; ++j) {
         const int s = j % NS, sn = (j + 1) % NS;
@@ -621,23 +631,27 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         if (!mbar_wait(&v_full[s], (j / NS) & 1) || (more && !mbar_wait(&k_full[sn], ((j + 1) / NS) & 1))) {
           report(p.status, DEV_TIMEOUT_MMA); ok = false; break;
         }
-        const uint32_t v_addr = smem_u32(v_s + s * Cfg::kVBytes);
+        const uint64_t vd = umma_desc_k_sw128(smem_u32(v_s + s * Cfg::kVBytes));
         for (int t = 0; t < ntiles; ++t) {
           if (!mbar_wait(&p_full[t], j & 1)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
           tc_fence_after();
           const uint32_t p_tmem = tmem_base + t * KT;              // P_t over the first 64 columns of S_t
           const uint32_t o_tmem = tmem_base + 256 + t * 128;
+          if (leader) {
 #pragma unroll
-          for (int kk = 0; kk < KT / 16; ++kk) {
-            const uint32_t b_off = (kk >> 2) * (HD * 128) + (kk & 3) * 32;
-            umma_bf16_ts(o_tmem, p_tmem + kk * 8, umma_desc_k_sw128(v_addr + b_off), idesc_pv, (j | kk) != 0);
+            for (int kk = 0; kk < KT / 16; ++kk) {
+              const uint32_t b_off = ((kk >> 2) * (HD * 128) + (kk & 3) * 32) >> 4;
+              umma_bf16_ts(o_tmem, p_tmem + kk * 8, vd + b_off, idesc_pv, (j | kk) != 0);
+            }
+            umma_commit(&o_done[t]);
           }
-          umma_commit(&o_done[t]);
           if (more) issue_qk(t, sn);
         }
         if (!ok) break;
-        umma_commit(&v_empty[s]);
-        if (more) umma_commit(&k_empty[sn]);
+        if (leader) {
+          umma_commit(&v_empty[s]);
+          if (more) umma_commit(&k_empty[sn]);
+        }
       }
     }
    }

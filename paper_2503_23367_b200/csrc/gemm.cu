@@ -38,10 +38,10 @@ constexpr int BK = 64;
 constexpr int kGemmThreads = 192;
 constexpr int kATileBytes = BM * BK * 2;  // 16 KB
 
-// kKps: k-blocks per pipeline stage.  The MMA-issuing thread pays a fixed price per stage (the wait on the full barrier
-// and the commit that frees the stage: about 0.2 us of dependent instructions), which for tiles of up to 128 columns
-// exceeds the time of the stage's MMAs; with two k-blocks behind one barrier it is paid half as often.  The wider
-// tiles keep one k-block per stage: their MMAs take that long anyway, and two k-blocks would leave two stages.
+// kKps: k-blocks per pipeline stage.  The producer and the MMA issuer both pay a fixed price per stage (a barrier's wait, a
+// commit or an expect), which for tiles of up to 128 columns exceeds the time of one k-block's MMAs: the producer alone takes
+// 394 clocks per k-block with one of them per stage and 282 with two.  The wider tiles keep one k-block per stage: their MMAs
+// take that long anyway, and two k-blocks would leave two stages (398 -> 537 clocks for 192-wide tiles).
 template <int BN> struct GemmCfg {
   static constexpr int kKps = (BN <= 128) ? 2 : 1;
   static constexpr int kBTileBytes = BN * BK * 2;
@@ -142,9 +142,10 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
   } else if (warp == 1) {
     pdl_wait();
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc = umma_idesc_bf16(BM, BN);
-      uint32_t it = 0, lt = 0;
+      const bool leader = elect_one();
+      uint32_t lt = 0, s = 0, ph = 0;   // tile count; ring stage and its phase
       bool ok = true;
       for (int item = blockIdx.x; ok && item < total_tiles; item += gridDim.x, ++lt) {
         const uint32_t buf = lt & 1;
@@ -153,23 +154,23 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const uint32_t d = tmem_base + buf * Cfg::kAccStride;
         const int slice = item % splits;
         const int kb0 = slice * p.kb_per_split, kb1 = min(num_kb, kb0 + p.kb_per_split);
-        for (int kb = kb0; kb < kb1; kb += KPS, ++it) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
+        for (int kb = kb0; kb < kb1; kb += KPS) {
           if (!mbar_wait(&full_bar[s], ph)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(smem + s * Cfg::kStageBytes);
+          const uint64_t desc = umma_desc_k_sw128(smem_u32(smem + s * Cfg::kStageBytes));
+          if (leader) {
 #pragma unroll
-          for (int u = 0; u < KPS; ++u) {
-            const uint64_t adesc = umma_desc_k_sw128(a_addr + u * Cfg::kSubBytes);
-            const uint64_t bdesc = umma_desc_k_sw128(a_addr + u * Cfg::kSubBytes + kATileBytes);
+            for (int u = 0; u < KPS; ++u) {
+              const uint64_t adesc = desc + u * (Cfg::kSubBytes >> 4), bdesc = adesc + (kATileBytes >> 4);
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-              umma_bf16(d, adesc + 2 * kk, bdesc + 2 * kk, idesc, (kb > kb0) || (u | kk) != 0);
+              for (int kk = 0; kk < BK / 16; ++kk)
+                umma_bf16(d, adesc + 2 * kk, bdesc + 2 * kk, idesc, (kb > kb0) || (u | kk) != 0);
+            }
+            umma_commit(&empty_bar[s]);
           }
-          umma_commit(&empty_bar[s]);
+          if (++s == STAGES) { s = 0; ph ^= 1; }
         }
-        if (ok) umma_commit(&acc_full[buf]);
+        if (ok && leader) umma_commit(&acc_full[buf]);
       }
     }
   } else {

@@ -134,27 +134,29 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
   } else if (warp == 1) {
     pdl_wait();
-    if (lane == 0) {
+    {
       constexpr uint32_t idesc = umma_idesc_bf16(BM, BN);
+      const bool leader = elect_one();
+      uint32_t s = 0, ph = 0;   // ring stage and its phase
       bool ok = true;
       const int nst = (kb1 - kb0 + KPS - 1) / KPS;
       for (int it = 0; it < nst; ++it) {
-        const int s = it % STAGES;
-        const uint32_t ph = (it / STAGES) & 1;
         if (!mbar_wait(&full_bar[s], ph)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
         tc_fence_after();
-        const uint32_t a_addr = smem_u32(smem + s * Cfg::kStageBytes);
+        const uint64_t desc = umma_desc_k_sw128(smem_u32(smem + s * Cfg::kStageBytes));
+        if (leader) {
 #pragma unroll
-        for (int u = 0; u < KPS; ++u) {
-          const uint64_t adesc = umma_desc_k_sw128(a_addr + u * Cfg::kSubBytes);
-          const uint64_t bdesc = umma_desc_k_sw128(a_addr + u * Cfg::kSubBytes + kATileBytes);
+          for (int u = 0; u < KPS; ++u) {
+            const uint64_t adesc = desc + u * (Cfg::kSubBytes >> 4), bdesc = adesc + (kATileBytes >> 4);
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
-            umma_bf16(tmem_base, adesc + 2 * kk, bdesc + 2 * kk, idesc, (it | u | kk) != 0);
+            for (int kk = 0; kk < BK / 16; ++kk)
+              umma_bf16(tmem_base, adesc + 2 * kk, bdesc + 2 * kk, idesc, (it | u | kk) != 0);
+          }
+          umma_commit(&empty_bar[s]);
         }
-        umma_commit(&empty_bar[s]);
+        if (++s == STAGES) { s = 0; ph ^= 1; }
       }
-      if (ok && kb1 > kb0) umma_commit(acc_full);
+      if (ok && leader && kb1 > kb0) umma_commit(acc_full);
     }
   } else {
     // ---- accumulator readers: thread = one accumulator row; its partial goes to the CTA that owns the row ----

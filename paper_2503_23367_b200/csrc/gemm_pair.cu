@@ -124,32 +124,33 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     }
   } else if (warp == 1) {
     pdl_wait();
-    if (rank == 0 && lane == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc = umma_idesc_bf16(2 * BM, BN);
-      uint32_t it = 0, lt = 0;
+      const bool leader = elect_one();
+      uint32_t lt = 0, s = 0, ph = 0;   // tile count; ring stage and its phase
       bool ok = true;
       for (int tile = pair; ok && tile < total_tiles; tile += npairs, ++lt) {
         const uint32_t buf = lt & 1;
         if (!mbar_wait(&acc_empty[buf], ((lt >> 1) & 1) ^ 1)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
         tc_fence_after();
         const uint32_t d = tmem_base + buf * Cfg::kAccStride;
-        for (int kb = 0; kb < num_kb; kb += KPS, ++it) {
-          const int s = it % STAGES;
-          const uint32_t ph = (it / STAGES) & 1;
+        for (int kb = 0; kb < num_kb; kb += KPS) {
           if (!mbar_wait(&full_bar[s], ph)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
           tc_fence_after();
-          const uint32_t a_addr = smem_u32(smem + s * Cfg::kStageBytes);
+          const uint64_t desc = umma_desc_k_sw128(smem_u32(smem + s * Cfg::kStageBytes));
+          if (leader) {
 #pragma unroll
-          for (int u = 0; u < KPS; ++u) {
-            const uint64_t adesc = umma_desc_k_sw128(a_addr + u * Cfg::kSubBytes);
-            const uint64_t bdesc = umma_desc_k_sw128(a_addr + u * Cfg::kSubBytes + kATileBytes);
+            for (int u = 0; u < KPS; ++u) {
+              const uint64_t adesc = desc + u * (Cfg::kSubBytes >> 4), bdesc = adesc + (kATileBytes >> 4);
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-              umma_bf16_pair(d, adesc + 2 * kk, bdesc + 2 * kk, idesc, (kb | u | kk) != 0);
+              for (int kk = 0; kk < BK / 16; ++kk)
+                umma_bf16_pair(d, adesc + 2 * kk, bdesc + 2 * kk, idesc, (kb | u | kk) != 0);
+            }
+            umma_commit_pair(&empty_bar[s]);
           }
-          umma_commit_pair(&empty_bar[s]);
+          if (++s == STAGES) { s = 0; ph ^= 1; }
         }
-        if (ok) umma_commit_pair(&acc_full[buf]);
+        if (ok && leader) umma_commit_pair(&acc_full[buf]);
       }
     }
   } else {

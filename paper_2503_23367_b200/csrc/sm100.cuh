@@ -95,6 +95,17 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// One lane of a converged warp, always the same one.  A loop that issues tcgen05.mma is walked by the WHOLE warp with only
+// the issue itself under this predicate: tcgen05 instructions take their descriptors from uniform registers, and inside
+// a one-lane branch the compiler cannot know its values uniform and moves each of them over lane by lane.  Measured per
+// k-block of 64 (1024 x 2048 x 8192, operands in L2): 362 -> 313 clocks for 128-wide tiles (259 is the tensor core's own
+// time), 510 -> 398 for 192-wide ones; launches: 43.6 -> 37.1 us at M 1280 N 2048 K 8192, 91.2 -> 81.9 at M 3277.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate; issued by ONE thread.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
