@@ -520,11 +520,10 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
   p.rope_idx = qk_extras ? g.rope_idx : nullptr;
   p.head_dim = g.head_dim;
   // Few tiles against a long K (every GEMM of the small scale steps): split K over the CTAs of a cluster, the
-  // partials reduced through distributed shared memory.  Measured back to back on B200 (us, against the best
-  // of the other paths): N 2048 K 2048: 6.6 / 7.4 / 8.0 / 12.0 / 12.4 at M = 2 / 32 / 128 / 288 / 512 (9.7 /
-  // 9.7 / 12.7 / 13.7 / 14.0); N 2048 K 8192: 14.9 / 15.0 / 15.9 / 26.9 / 27.5 (14.9 / 15.9 / 20.8 / 29.5 /
-  // 35.6); N 6144 K 2048 at M <= 128: 13.2 / 11.4 / 13.8 (14.4 / 14.1 / 14.3); N 8192: 13.6 / 12.0 / 14.3
-  // (17.7 / 14.6 / 15.1).  Which of the three shapes wins follows the tile counts:
+  // partials reduced through distributed shared memory.  Which shape wins follows the tile counts.  Up to 32 rows two CTAs
+  // share an SM and 64-wide tiles are the best everywhere: 4 slices while the CTAs stay near one per SM, else 2 (us at M 8, weights
+  // from HBM, 64 x 4 / 64 x 2 / 128 x 4 / 128 x 2: N 2048 K 2048 4.8 / 5.3 / 5.8 / 7.4; N 6144 10.1 / 8.3 / 8.2 / 9.5;
+  // N 8192 12.0 / 9.1 / 8.9 / 10.5; N 2048 K 8192 10.1 / 14.1 / 14.7 / 23.3; 1024-wide models N 3072 4.1 / 4.2 / 4.7 / 4.9).
   int cluster_slices = 0, cluster_bn = 0;
   if (g_force_path == 0 && !qk_extras) {
     const int num_kb = (g.K + BK - 1) / BK;
@@ -532,8 +531,9 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
     // (re-measured GPU-bound after the narrow tiles took two k-blocks per pipeline stage: with more than 32 rows the
     // 128-wide x 2 cluster, whose ring has no room for that, only wins on a long K; 64-wide x 2 wins on a short one)
     if (num_kb >= 8) {
-      if (g.M > 16 && t64 * 4 <= g_num_sms) { cluster_bn = 64; cluster_slices = 4; }
-      else if (g.M > 16 && t64 * 2 <= g_num_sms && num_kb < 64) { cluster_bn = 64; cluster_slices = 2; }
+      if (g.M <= 32 && t64 <= g_num_sms) { cluster_bn = 64; cluster_slices = t64 * 3 <= g_num_sms ? 4 : 2; }
+      else if (t64 * 4 <= g_num_sms) { cluster_bn = 64; cluster_slices = 4; }
+      else if (t64 * 2 <= g_num_sms && num_kb < 64) { cluster_bn = 64; cluster_slices = 2; }
       else if (t128 * 4 <= g_num_sms) { cluster_bn = 128; cluster_slices = 4; }
       else if (t128 * 2 <= g_num_sms && (g.M <= 32 || num_kb >= 64)) { cluster_bn = 128; cluster_slices = 2; }
     }

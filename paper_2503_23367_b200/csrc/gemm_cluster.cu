@@ -30,24 +30,25 @@ constexpr int kThreads = 192;
 // MMA always reads a 128-row A tile from shared memory; with AROWS = 32 the rows beyond the 4 KB that were
 // loaded are whatever follows in shared memory (the stage's own W tile, the next stage, the buffers behind the
 // ring -- all inside the allocation).  They only feed accumulator rows >= 32, which belong to no row of the
-// output and are neither reduced nor stored.  The 12 KB saved per k-block buy a deeper ring.
+// output and are neither reduced nor stored.
+// The small-row builds stay under 113 KB of shared memory, ring and reduce buffer together, so that TWO CTAs share an SM:
+// the CTAs of the next GEMM of the step start (programmatic launch) beside those of this one and fetch their first
+// 64 KB of weights while this one computes, and outputs of up to 8192 columns fit the GPU as 64-wide tiles.  Launches of a chain
+// (M 8, weights from HBM): N 2048 K 2048 5.4 -> 4.8 us, N 6144 8.7 -> 8.3, N 8192 9.6 -> 9.1, N 2048 K 8192 11.5 -> 10.1.
 //
-// kKps: k-blocks per pipeline stage.  The thread that issues the MMAs is a chain of dependent instructions: per stage
-// it spends about 0.16 us between its commit and seeing the next full barrier, 0.06 us on the commit and 0.03 us per
-// MMA, so with one k-block per stage a k-block costs 0.34 us whatever its bytes (measured with device timestamps: no
-// change without the A loads, with one MMA of four, with the weights resident in L2, with another weight pitch).
-// Two k-blocks behind one barrier halve the per-stage part: 0.24 us per k-block.  Where the ring would shrink to two
-// stages (128 rows of A against 128-wide tiles) one k-block per stage stays.
+// kKps: k-blocks per pipeline stage.  Producer and MMA issuer pay a fixed price per stage (a barrier's wait, a commit or an
+// expect) that exceeds the time of one k-block's MMAs: with two k-blocks behind one barrier it is paid half as often.
+// Where the ring would shrink to two stages (128 rows of A against 128-wide tiles) one k-block per stage stays.
 template <int BN, int AROWS> struct ClusterCfg {
   static constexpr int kKps = (AROWS == 128 && BN == 128) ? 1 : 2;
   static constexpr int kATile = AROWS * BK * 2;
   static constexpr int kBTileBytes = BN * BK * 2;
   static constexpr int kSubBytes = kATile + kBTileBytes;       // one k-block: A tile, then W tile
   static constexpr int kStageBytes = kKps * kSubBytes;
-  static constexpr int kStages = AROWS == 32 ? ((BN == 128) ? 3 : 5) : ((BN == 128) ? 4 : 3);
+  static constexpr int kStages = AROWS == 32 ? ((BN == 128) ? 2 : 4) : ((BN == 128) ? 4 : 3);
   static constexpr int kTmemCols = BN;                      // one accumulator (64 or 128: powers of two)
   static constexpr int kRedPitch = BN + 4;                  // floats per row of the reduce buffer (bank spread)
-  static constexpr int kRedBytes = BM * kRedPitch * 4;      // [S sources][128/S rows][pitch] = 128 rows in all
+  static constexpr int kRedBytes = AROWS * kRedPitch * 4;   // [S sources][AROWS/S rows][pitch] = AROWS rows in all
   // operand stages | per-warp bias slices | barriers | reduce buffer
   static constexpr int kSmemBytes = kStages * kStageBytes + kBiasSmemBytes + 256 + kRedBytes + 1024 /*alignment slack*/;
 };
@@ -68,7 +69,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   constexpr int kATileBytes = Cfg::kATile;
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;
-  constexpr int ROWS_PER = BM / S;        // rows of the tile each CTA finishes
+  constexpr int ROWS_PER = AROWS / S;     // rows of the tile each CTA finishes
   constexpr int CHUNKS = BN / 32;         // 32-column chunks per row
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -163,7 +164,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     pdl_wait();
     const int quarter = warp & 3;
     const int trow = quarter * 32 + lane;                 // row inside the tile
-    const uint32_t owner = (uint32_t)(trow / ROWS_PER);
+    const uint32_t owner = (uint32_t)min(trow / ROWS_PER, S - 1);   // (rows past AROWS belong to no row of the output)
     const int lrow = trow - (int)owner * ROWS_PER;
     stage_bias(p, bias_s + quarter * 32, lane, n0, BN);
     bool have = kb1 > kb0;
@@ -174,7 +175,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const uint32_t dst = map_to_cta(red + ((size_t)rank * ROWS_PER + lrow) * Cfg::kRedPitch, owner);
     const uint32_t t0 = tmem_base + (uint32_t(quarter * 32) << 16);
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 32) {
+    for (int c0 = 0; c0 < (AROWS == 128 || quarter == 0 ? BN : 0); c0 += 32) {
       uint32_t r[32];
       if (have) {            // uniform over the warp
         tmem_ld32(t0 + c0, r);

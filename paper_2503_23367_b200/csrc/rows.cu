@@ -32,16 +32,16 @@ __global__ void __launch_bounds__(256) gather_ln_kernel(const XT* __restrict__ x
   const int b = blockIdx.y, j = blockIdx.x * 8 + warp;
   const bool live = j < k;
   pdl_trigger();
+  if (sigma) {   // modulation vectors are never written by a kernel of the step: on their way while the kernel before this one ends
+    const float4* sg = reinterpret_cast<const float4*>(sigma + (size_t)b * mod_stride);
+    const float4* bt = reinterpret_cast<const float4*>(beta + (size_t)b * mod_stride);
+    for (int i = threadIdx.x; i < C4; i += 256) { s_mod[i] = __ldg(sg + i); s_mod[C4 + i] = __ldg(bt + i); }
+  }
   pdl_wait();
   int t = live ? (idx ? __ldg(idx + (size_t)b * k + j) : j) : 0;
   if (t < 0 || t >= n) {   // a caller's index outside the map: stay inside it and say so
     if (status && lane == 0) atomicCAS(status, 0, DEV_BAD_ROW_INDEX);
     t = min(max(t, 0), n - 1);
-  }
-  if (sigma) {
-    const float4* sg = reinterpret_cast<const float4*>(sigma + (size_t)b * mod_stride);
-    const float4* bt = reinterpret_cast<const float4*>(beta + (size_t)b * mod_stride);
-    for (int i = threadIdx.x; i < C4; i += 256) { s_mod[i] = __ldg(sg + i); s_mod[C4 + i] = __ldg(bt + i); }
   }
   const XT* row = x + ((size_t)b * n + t) * C4 * 4;
   float4 v[kMaxVec];
