@@ -348,7 +348,8 @@ fv_status fv_attention(const void *q_dev, const void *k_dev, const void *vt_dev,
                        void *stream);
 /* Test / profiling hook (process-wide): number of CTAs of a fv_attention launch that is given a workspace
  * (0 = one per SM where that pays, the default; n > 0 = always n pieces, capped at 160 and at what the work
- * allows; -1 = never cut the work, as if no workspace were given). */
+ * allows; -1 = never cut the work, as if no workspace were given; -2 / -3 = nor choose between whole items of
+ * 256 / of 128 queries). */
 fv_status fv_attention_force_ctas(int32_t ctas);
 
 /* ------------------------------------------------------------------------------------------------

@@ -3,29 +3,29 @@
 // the attention map, so a fused kernel applies).  Within a scale step there is no mask: a query sees
 // every cached key of the earlier scales and all keys appended by its own step.
 //
-// Work item = 256 queries (two tiles of 128) of one head of one image; keys are consumed in tiles of 128.
-// The kept-row counts of the pruned steps give item counts that fit the GPU badly (64, 80, 128 or 208 items
-// on 148 SMs, the last item of a head often a single, part-filled tile), so the (item, key tile) units are
-// laid out on one line (a weight per item kind; both kinds cost the same per key tile as measured) and the line
-// is cut into equal pieces, one per CTA (one CTA per SM), when that beats one whole item per CTA.  A CTA walks its piece as segments: a range of key tiles of
-// one item.  A segment that covers all key tiles of its item writes the output itself; otherwise it leaves
-// its unnormalised partial (O, running maximum, row sum) in scratch, and the last part of an item to arrive
-// (arrival counter) merges the parts IN KEY ORDER, so the result does not depend on arrival order.
-// Without scratch the kernel runs one whole item per CTA.
+// Two kernels.  attention_whole_kernel runs one work item per CTA: 256 queries (two tiles of 128), or 128, of one head of one
+// image.  attention_kernel, taken where whole items fit the SMs badly and the key range is long, lays the (256-query item, key
+// tile) units on one line and cuts it into equal pieces, one per CTA: a CTA walks its piece as segments (key tiles of one item); a
+// segment that covers its whole item writes the output, otherwise it leaves its unnormalised partial (O, running maximum, row
+// sum) in scratch, and the last part of an item to arrive (arrival counter) merges the parts IN KEY ORDER, so the
+// result does not depend on arrival order.  launch_hd chooses by cost.
 //
-// The two query tiles of a segment take turns on the tensor core: while the softmax warps of one tile work
-// on its scores, the MMAs of the other tile run.
-//   warp 8   : TMA producer (both Q tiles per segment; K tiles [128 keys x hd]; V^T tiles [hd x 128 keys]).
-//   warp 9   : one lane issues tcgen05.mma.  Per key tile j and query tile t:  O_t += P_t V_j  with P_t
-//              read from TENSOR MEMORY (it overwrites the first 64 columns of S_t), then
-//              S_t = Q_t K_{j+1}^T.  MMAs of one thread execute in issue order, which is what makes
-//              the P_t / S_t aliasing safe.
-//   warps 0-3, 4-7: online softmax of tile 0 / tile 1, thread = query row: the 128 scores of the row come
-//              out of TMEM in one go (four loads, one wait; the register file is re-divided between the
-//              warpgroups with setmaxnreg so that a thread can hold them), row maximum, base-2
-//              exponentials, row sum, and the bf16 probabilities go back to TMEM.  The running maximum is only raised when
-//              it would grow by more than 2^8, so the O accumulator (TMEM) is rescaled in place only
-//              on the rare tiles where that happens; the final O / l is written as bf16.
+// Whole-item kernel: two streams of key tiles, each with its own 128 columns of scores and its own O in tensor memory.
+//   warp 8 / 10 : TMA producers of Q and K tiles [128 keys x hd] / of V^T tiles [hd x 128 keys].
+//   warp 9 / 11 : issue the tcgen05.mma of stream 0 / stream 1.  Per half tile of 64 keys: O += P V with P read from TENSOR MEMORY
+//                 (it overwrites the first 32 columns of its score slot), then the scores of the half after next into the same
+//                 slot.  MMAs of one thread execute in issue order, which is what makes the aliasing safe.
+//   warps 0-3, 4-7: online softmax of stream 0 / 1, thread = query row: 64 scores out of TMEM, row maximum, base-2
+//                 exponentials, row sum, bf16 probabilities back.  The running maximum is only raised when it would grow by
+//                 more than 2^8, so O (TMEM) is rescaled in place only on the rare halves where that happens.
+// What bounds it (device timestamps, hd 128): the two slots keep the next half's scores ready, so the softmax warps (1000 clocks per
+// half) no longer wait for the tensor core; the MMAs of a half take 620 clocks per stream (64-wide score MMAs read 128 rows of Q per 64 keys
+// and run at 2/3 of the rate), 1240 for both, of 1500 measured.  Every wait or commit of an issuing warp takes 100 ... 300 clocks
+// because it queues behind the softmax warps' exponentials; with one issuing warp per stream those of one run under
+// the MMAs of the other (2.04 -> 1.95 us per 128 keys), and only the commits somebody waits for are made (-> 1.88).
+//
+// Piece kernel: one issuing warp, scores of a whole key tile at a time (the half-tile slots measured slower there: 88 -> 93 us at
+// 1280 queries, 7245 keys).  Its softmax threads hold 128 scores each (setmaxnreg re-divides the register file).
 // V is read transposed ([channel, key], keys contiguous), which makes it a K-major B operand.
 // Every wait is bounded (status word + normal unwind on expiry); a thread whose wait expired skips the
 // rest of its work but still takes part in every CTA-level barrier.
@@ -41,15 +41,18 @@ namespace {
 
 constexpr int QT = 128;   // queries per tile (two tiles per CTA)
 constexpr int KT = 128;   // keys per tile
-constexpr int kAttnThreads = 384;   // warps 0-3 / 4-7: softmax of query tile 0 / 1; warp 8: TMA; warp 9: MMA; 10-11: idle
+constexpr int kAttnThreads = 384;   // warps 0-3 / 4-7: softmax of stream 0 / 1; 8-11: TMA and MMA
 constexpr float kRescaleThreshold = 8.f;  // log2 units
 
-template <int HD> struct AttnCfg {
-  static constexpr int kStages = (HD == 128) ? 2 : 4;
+constexpr int HT = 64;    // keys per score slot of the whole-item kernel: a key tile is consumed in two halves
+
+// ONE_TILE: the build for one query tile per CTA (half the query storage, a deeper ring for 128-wide heads).
+template <int HD, bool ONE_TILE = false> struct AttnCfg {
+  static constexpr int kStages = (HD == 128) ? (ONE_TILE ? 3 : 2) : 4;
   static constexpr int kQBytes = QT * HD * 2;   // one query tile
   static constexpr int kKBytes = KT * HD * 2;
   static constexpr int kVBytes = HD * KT * 2;
-  static constexpr int kSmemBytes = 2 * kQBytes + kStages * (kKBytes + kVBytes) + 1024 + 256;
+  static constexpr int kSmemBytes = (ONE_TILE ? 1 : 2) * kQBytes + kStages * (kKBytes + kVBytes) + 1024 + 256;
   static constexpr int kTmemCols = 512;  // S0 [0,128) S1 [128,256) O0 [256,256+HD) O1 [384,384+HD)
   // one partial of a segment in scratch: (maximum, row sum) [2 tiles][128 rows], then O [2 tiles][HD/4][128 rows] float4
   static constexpr size_t kPartMlBytes = 2 * QT * sizeof(float2);
@@ -525,9 +528,120 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
   }
 }
 
-// ---- One whole work item per CTA: grid (query blocks, heads, images).  The launcher takes this kernel whenever it does
-// not cut the work into pieces: it is the kernel above without the segment bookkeeping, and its leaner loops hand
-// the tiles between the softmax warpgroups and the MMA thread measurably faster (15 % per key tile).
+// Two fp32 operations per instruction (the pairs are independent; the results are those of the scalar forms).
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+  uint64_t v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+  return v;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
+// Halves (of 64 keys) a stream of key tiles ja, ja + dj, ... (n of them) really has: the last one may end in its first half.
+__device__ __forceinline__ int stream_halves(int kv_len, int ja, int dj, int n) {
+  if (n <= 0) return 0;
+  return 2 * n - ((kv_len - (ja + (n - 1) * dj) * KT <= HT) ? 1 : 0);
+}
+
+// Online softmax of one query row over a stream of key tiles ja, ja + dj, ...: half tiles of 64 scores out of TMEM,
+// probabilities back into the first half of the same slot.  The stream has two slots (half 0 / half 1 of a tile), so the scores of
+// the next half are there while this one is worked on.  s_full / p_full: the barriers of the two slots; o_prev / o_last: the
+// P V of the stream's last half but one / last half has completed.  Returns false if a wait expired.
+template <int HD>
+__device__ __forceinline__ bool softmax_stream(int kv_len, float scale_log2, int32_t* status, int ja, int dj, int halves, uint32_t s_addr, uint32_t o_addr,
+                                               uint64_t* s_full, uint64_t* p_full, uint64_t* o_prev, uint64_t* o_last, float& m_out, float& l_out) {
+  float m_run = -INFINITY, l_run = 0.f;
+  const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
+#pragma unroll 1
+  for (int i = 0; i < halves; ++i) {
+    const int h = i & 1, jj = i >> 1;
+    if (!mbar_wait(&s_full[h], jj & 1)) { report(status, DEV_TIMEOUT_SOFTMAX); return false; }
+    tc_fence_after();
+    const int valid = kv_len - (ja + jj * dj) * KT - h * HT;  // >= 1
+    uint32_t a[32], b[32];
+    tmem_ld32(s_addr + h * HT, a);
+    tmem_ld32(s_addr + h * HT + 32, b);
+    tmem_wait_ld();
+    if (valid < HT) {
+#pragma unroll
+      for (int e = 0; e < 32; ++e) {
+        if (e >= valid) a[e] = 0xFF800000u;        // -inf
+        if (32 + e >= valid) b[e] = 0xFF800000u;
+      }
+    }
+    float mx0 = __uint_as_float(a[0]), mx1 = __uint_as_float(a[1]), mx2 = __uint_as_float(b[0]), mx3 = __uint_as_float(b[1]);
+#pragma unroll
+    for (int e = 2; e < 32; e += 2) {
+      mx0 = fmaxf(mx0, __uint_as_float(a[e])); mx1 = fmaxf(mx1, __uint_as_float(a[e + 1]));
+      mx2 = fmaxf(mx2, __uint_as_float(b[e])); mx3 = fmaxf(mx3, __uint_as_float(b[e + 1]));
+    }
+    const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * scale_log2;
+    // Raise the running maximum only when it would grow by more than the threshold: probabilities
+    // may then exceed 1 (by at most 2^threshold), which fp32 sums and bf16 P hold without loss.
+    float alpha = 1.f;
+    if (mx > m_run + kRescaleThreshold) {
+      alpha = fast_exp2(m_run - mx);  // 0 on the first half (m_run = -inf)
+      m_run = mx;
+    }
+    if (i > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
+      // O is at rest once the P V of the half before has completed.  The next half's scores were issued behind it; the last
+      // half has none behind it, so that one P V has a barrier of its own.
+      const bool still = i + 1 < halves ? mbar_wait(&s_full[h ^ 1], ((i + 1) >> 1) & 1) : mbar_wait(o_prev, 0);
+      if (!still) { report(status, DEV_TIMEOUT_SOFTMAX); return false; }
+      tc_fence_after();
+#pragma unroll 1
+      for (int c = 0; c < HD / 16; ++c) {
+        uint32_t o[16];
+        tmem_ld16(o_addr + c * 16, o);
+        tmem_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+        tmem_st16(o_addr + c * 16, o);
+      }
+    }
+    const uint64_t neg_m2 = pack_f32x2(-m_run, -m_run);
+    uint64_t rs = 0ull;        // row sums of the UNROUNDED probabilities, even and odd keys
+    uint32_t pk[32];
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+      const uint64_t x = e < 16 ? pack_f32x2(__uint_as_float(a[2 * e]), __uint_as_float(a[2 * e + 1]))
+                                : pack_f32x2(__uint_as_float(b[2 * e - 32]), __uint_as_float(b[2 * e - 31]));
+      float y0, y1;
+      unpack_f32x2(fma_f32x2(x, scale2, neg_m2), y0, y1);
+      const float p0 = fast_exp2(y0), p1 = fast_exp2(y1);
+      rs = add_f32x2(rs, pack_f32x2(p0, p1));
+      pk[e] = pack_bf16x2(p0, p1);
+    }
+    tmem_st32(s_addr + h * HT, pk);
+    float r0, r1;
+    unpack_f32x2(rs, r0, r1);
+    l_run = fmaf(l_run, alpha, r0 + r1);
+    tmem_wait_st();
+    tc_fence_before();
+    mbar_arrive(&p_full[h]);
+  }
+  m_out = m_run; l_out = l_run;
+  if (halves > 0) {
+    if (!mbar_wait(o_last, 0)) { report(status, DEV_TIMEOUT_SOFTMAX); return false; }
+    tc_fence_after();
+  }
+  return true;
+}
+
+// ---- One whole work item per CTA: grid (query blocks, heads, images), without the segment bookkeeping.
+// ONE_TILE false: 256 queries, one stream of key tiles per query tile.  ONE_TILE true: 128 queries; both streams work on the
+// same query tile, stream t on the key tiles t, t + 2, ..., each with its own maximum, row sum and O, and the two are merged
+// (stream 0, then stream 1) on the way out.  The same work per CTA and key, in items half as large: where the 256-query items
+// leave SMs idle or end in part-filled tiles, twice the CTAs are each done in half the time.
 struct WholeDev {
   __nv_bfloat16* out;
   int rows, C, kv_len, kv_capacity;
@@ -535,16 +649,17 @@ struct WholeDev {
   int32_t* status;
 };
 
-template <int HD>
+template <int HD, bool ONE_TILE>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, const WholeDev p) {
-  using Cfg = AttnCfg<HD>;
+  using Cfg = AttnCfg<HD, ONE_TILE>;
   constexpr int NS = Cfg::kStages;
+  constexpr int QB = ONE_TILE ? QT : 2 * QT;    // queries per CTA
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* q_s = smem;                          // two query tiles
-  uint8_t* k_s = q_s + 2 * Cfg::kQBytes;
+  uint8_t* q_s = smem;
+  uint8_t* k_s = q_s + (ONE_TILE ? 1 : 2) * Cfg::kQBytes;
   uint8_t* v_s = k_s + NS * Cfg::kKBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(v_s + NS * Cfg::kVBytes);
   uint64_t* q_full = bars;
@@ -552,21 +667,25 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   uint64_t* k_empty = k_full + NS;
   uint64_t* v_full = k_empty + NS;
   uint64_t* v_empty = v_full + NS;
-  uint64_t* s_full = v_empty + NS;   // [2] scores of query tile t are in TMEM
-  uint64_t* p_full = s_full + 2;     // [2] probabilities of query tile t are in TMEM (128 arrivals)
-  uint64_t* o_done = p_full + 2;     // [2] the latest P V of query tile t has completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_done + 2);
+  uint64_t* s_full = v_empty + NS;   // [2 t + half] scores of stream t are in TMEM
+  uint64_t* p_full = s_full + 4;     // [2 t + half] probabilities of stream t are in TMEM (128 arrivals)
+  uint64_t* o_prev = p_full + 4;     // [2] the P V of stream t's last half but one has completed
+  uint64_t* o_last = o_prev + 2;     // [2] ... of its last half
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_last + 2);
 
   pdl_trigger();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int q0 = blockIdx.x * (2 * QT), head = blockIdx.y, img = blockIdx.z;
+  const int q0 = blockIdx.x * QB, head = blockIdx.y, img = blockIdx.z;
   const int T = (p.kv_len + KT - 1) / KT;
-  const int ntiles = (p.rows - q0 > QT) ? 2 : 1;
+  const int ntiles = (!ONE_TILE && p.rows - q0 > QT) ? 2 : 1;                      // query tiles
+  const int n0 = ONE_TILE ? (T + 1) / 2 : T, n1 = ONE_TILE ? T / 2 : (ntiles == 2 ? T : 0);   // key tiles of either stream
+  const int nh0 = stream_halves(p.kv_len, 0, ONE_TILE ? 2 : 1, n0), nh1 = stream_halves(p.kv_len, ONE_TILE ? 1 : 0, ONE_TILE ? 2 : 1, n1);
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
-    for (int s = 0; s < NS; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], 1); mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1); }
-    for (int t = 0; t < 2; ++t) { mbar_init(&s_full[t], 1); mbar_init(&p_full[t], QT); mbar_init(&o_done[t], 1); }
+    for (int s = 0; s < NS; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], ONE_TILE ? 1 : ntiles); mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], ONE_TILE ? 1 : ntiles); }
+    for (int t = 0; t < 4; ++t) { mbar_init(&s_full[t], 1); mbar_init(&p_full[t], QT); }
+    for (int t = 0; t < 2; ++t) { mbar_init(&o_prev[t], 1); mbar_init(&o_last[t], 1); }
     mbar_fence_init();
     tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
   }
@@ -577,11 +696,7 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();  // set-up above overlaps the previous kernel; Q / K / V and the output are touched only from here
 
-  // A softmax thread holds a whole score row (128 fp32) in registers, so the register file is re-divided
-  // between the warpgroups: 2 x 128 x 216 + 128 x 40 <= 64 K registers.
-  if (warp >= 8) {
-   asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-   if (warp == 8) {
+  if (warp == 8) {          // queries and keys
     if (lane == 0) {
       mbar_expect_tx(q_full, ntiles * Cfg::kQBytes);
       for (int t = 0; t < ntiles; ++t)
@@ -589,143 +704,145 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           tma_load_2d(q_s + t * Cfg::kQBytes + a * (QT * 128), &tmQ, head * HD + a * 64, img * p.rows + q0 + t * QT, q_full);
       for (int j = 0; j < T; ++j) {
         const int s = j % NS;
-        const uint32_t ph = (j / NS) & 1;
-        if (!mbar_wait(&k_empty[s], ph ^ 1)) { report(p.status, DEV_TIMEOUT_TMA); break; }
+        if (!mbar_wait(&k_empty[s], ((j / NS) & 1) ^ 1)) { report(p.status, DEV_TIMEOUT_TMA); break; }
         mbar_expect_tx(&k_full[s], Cfg::kKBytes);
         for (int a = 0; a < HD / 64; ++a)
           tma_load_2d(k_s + s * Cfg::kKBytes + a * (KT * 128), &tmK, head * HD + a * 64, img * p.kv_capacity + j * KT, &k_full[s]);
-        if (!mbar_wait(&v_empty[s], ph ^ 1)) { report(p.status, DEV_TIMEOUT_TMA); break; }
+      }
+    }
+  } else if (warp == 10) {  // values: a warp of their own, so that a key tile never waits behind a value tile's stage
+    if (lane == 0) {
+      for (int j = 0; j < T; ++j) {
+        const int s = j % NS;
+        if (!mbar_wait(&v_empty[s], ((j / NS) & 1) ^ 1)) { report(p.status, DEV_TIMEOUT_TMA); break; }
         mbar_expect_tx(&v_full[s], Cfg::kVBytes);
         for (int a = 0; a < KT / 64; ++a)
           tma_load_2d(v_s + s * Cfg::kVBytes + a * (HD * 128), &tmV, j * KT + a * 64, img * p.C + head * HD, &v_full[s]);
       }
     }
-  } else if (warp == 9) {
-    {
-      const bool leader = elect_one();   // the warp walks the loop together; one lane issues
-      constexpr uint32_t idesc_qk = umma_idesc_bf16(QT, KT);
-      constexpr uint32_t idesc_pv = umma_idesc_bf16(QT, HD);
-      const uint32_t q_addr = smem_u32(q_s);
-      // S_t = Q_t K^T for the key tile in stage s
-      auto issue_qk = [&](int t, int s) {
-        const uint64_t kd = umma_desc_k_sw128(smem_u32(k_s + s * Cfg::kKBytes)), qd = umma_desc_k_sw128(q_addr + t * Cfg::kQBytes);
-        if (leader) {
+  } else if (warp == 9 || warp == 11) {   // one issuing warp per stream: the waits and commits of one run under the MMAs of the other
+    const int t = warp == 9 ? 0 : 1;
+    const int nh = t == 0 ? nh0 : nh1;
+    const bool leader = elect_one();   // the warp walks the loop together; one lane issues
+    constexpr uint32_t idesc_qk = umma_idesc_bf16(QT, HT);
+    constexpr uint32_t idesc_pv = umma_idesc_bf16(QT, HD);
+    const uint64_t qd = umma_desc_k_sw128(smem_u32(q_s) + (ONE_TILE ? 0 : t * Cfg::kQBytes));
+    const uint64_t kd0 = umma_desc_k_sw128(smem_u32(k_s)), vd0 = umma_desc_k_sw128(smem_u32(v_s));
+    const uint32_t s_tmem = tmem_base + t * KT, o_tmem = tmem_base + 256 + t * 128;
+    constexpr int DJ = ONE_TILE ? 2 : 1;
+    // scores of the stream against half h of the key tile in stage st
+    auto issue_qk = [&](int st, int h) {
+      const uint64_t kd = kd0 + ((st * Cfg::kKBytes + h * (HT * 128)) >> 4);
+      if (leader) {
 #pragma unroll
-          for (int kk = 0; kk < HD / 16; ++kk) {
-            const uint32_t off = ((kk >> 2) * (QT * 128) + (kk & 3) * 32) >> 4;
-            umma_bf16(tmem_base + t * KT, qd + off, kd + off, idesc_qk, kk != 0);
-          }
-          umma_commit(&s_full[t]);
+        for (int kk = 0; kk < HD / 16; ++kk) {
+          const uint32_t off = ((kk >> 2) * (QT * 128) + (kk & 3) * 32) >> 4;
+          umma_bf16(s_tmem + h * HT, qd + off, kd + off, idesc_qk, kk != 0);
         }
-      };
-      bool ok = mbar_wait(q_full, 0) && mbar_wait(&k_full[0], 0);
+        umma_commit(&s_full[2 * t + h]);
+      }
+    };
+    if (nh > 0) {
+      int j = ONE_TILE ? t : 0;
+      bool ok = mbar_wait(q_full, 0) && mbar_wait(&k_full[j % NS], (j / NS) & 1);
       if (!ok) report(p.status, DEV_TIMEOUT_MMA);
       if (ok) {
         tc_fence_after();
-        for (int t = 0; t < ntiles; ++t) issue_qk(t, 0);
-        if (leader) umma_commit(&k_empty[0]);
+        issue_qk(j % NS, 0);
+        if (nh > 1) issue_qk(j % NS, 1);
+        if (leader) umma_commit(&k_empty[j % NS]);
       }
-      for (int j = 0; ok && j < T; ++j) {
-        const int s = j % NS, sn = (j + 1) % NS;
-        const bool more = j + 1 < T;
-        if (!mbar_wait(&v_full[s], (j / NS) & 1) || (more && !mbar_wait(&k_full[sn], ((j + 1) / NS) & 1))) {
+      for (int i = 0; ok && i < nh; ++i) {
+        const int h = i & 1, jj = i >> 1;
+        j = ONE_TILE ? 2 * jj + t : jj;
+        const int jn = j + DJ;
+        const bool more = i + 2 < nh;
+        if (h == 0 && (!mbar_wait(&v_full[j % NS], (j / NS) & 1) || (more && !mbar_wait(&k_full[jn % NS], (jn / NS) & 1)))) {
           report(p.status, DEV_TIMEOUT_MMA); ok = false; break;
         }
-        const uint64_t vd = umma_desc_k_sw128(smem_u32(v_s + s * Cfg::kVBytes));
-        for (int t = 0; t < ntiles; ++t) {
-          if (!mbar_wait(&p_full[t], j & 1)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
-          tc_fence_after();
-          const uint32_t p_tmem = tmem_base + t * KT;              // P_t over the first 64 columns of S_t
-          const uint32_t o_tmem = tmem_base + 256 + t * 128;
-          if (leader) {
+        if (!mbar_wait(&p_full[2 * t + h], jj & 1)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
+        tc_fence_after();
+        const uint64_t vd = vd0 + (((j % NS) * Cfg::kVBytes + h * (HD * 128)) >> 4);
+        if (leader) {   // P over the first 32 columns of its slot
 #pragma unroll
-            for (int kk = 0; kk < KT / 16; ++kk) {
-              const uint32_t b_off = ((kk >> 2) * (HD * 128) + (kk & 3) * 32) >> 4;
-              umma_bf16_ts(o_tmem, p_tmem + kk * 8, vd + b_off, idesc_pv, (j | kk) != 0);
-            }
-            umma_commit(&o_done[t]);
-          }
-          if (more) issue_qk(t, sn);
+          for (int kk = 0; kk < HT / 16; ++kk) umma_bf16_ts(o_tmem, s_tmem + h * HT + kk * 8, vd + 2 * kk, idesc_pv, (i | kk) != 0);
+          if (i + 2 == nh) umma_commit(&o_prev[t]);
+          if (i + 1 == nh) umma_commit(&o_last[t]);
         }
-        if (!ok) break;
+        if (more) issue_qk(jn % NS, h);
         if (leader) {
-          umma_commit(&v_empty[s]);
-          if (more) umma_commit(&k_empty[sn]);
+          if (h == 1 || i == nh - 1) umma_commit(&v_empty[j % NS]);
+          if (more && (h == 1 || i + 2 == nh - 1)) umma_commit(&k_empty[jn % NS]);
         }
       }
     }
-   }
-  } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
-    // ---- softmax + output: thread = one query row of tile t ----
+  } else if (warp < 8) {
+    // ---- softmax + output: thread = one query row, warps 0-3 stream 0, warps 4-7 stream 1 ----
     const int t = warp >> 2;
     const int quarter = warp & 3;                 // the TMEM lanes this warp may touch
     const int r = quarter * 32 + lane;
     const uint32_t lane_off = uint32_t(quarter * 32) << 16;
     const uint32_t s_addr = tmem_base + lane_off + t * KT;
-    const uint32_t o_addr = tmem_base + lane_off + 256 + t * 128;
-    if (t < ntiles) {
-      float m_run = -INFINITY, l_run = 0.f;
-      bool ok = true;
-      for (int j = 0; j < T; ++j) {
-        if (!mbar_wait(&s_full[t], j & 1)) { report(p.status, DEV_TIMEOUT_SOFTMAX); ok = false; break; }
-        tc_fence_after();
-        const int valid = p.kv_len - j * KT;  // >= 1
-        float sc[KT];
-        if (valid < KT) tile_load_scores<true>(s_addr, valid, sc);
-        else tile_load_scores<false>(s_addr, valid, sc);
-        float mx0 = sc[0], mx1 = sc[1], mx2 = sc[2], mx3 = sc[3];
-#pragma unroll
-        for (int i = 4; i < KT; i += 4) {
-          mx0 = fmaxf(mx0, sc[i]); mx1 = fmaxf(mx1, sc[i + 1]); mx2 = fmaxf(mx2, sc[i + 2]); mx3 = fmaxf(mx3, sc[i + 3]);
-        }
-        const float mx = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * p.scale_log2;
-        // Raise the running maximum only when it would grow by more than the threshold: probabilities
-        // may then exceed 1 (by at most 2^threshold), which fp32 sums and bf16 P hold without loss.
-        float alpha = 1.f;
-        if (mx > m_run + kRescaleThreshold) {
-          alpha = fast_exp2(m_run - mx);  // 0 on the first tile (m_run = -inf)
-          m_run = mx;
-        }
-        // S_t of tile j was issued after P V of tile j-1, so O_t is at rest here.
-        if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
-#pragma unroll
-          for (int c = 0; c < HD / 32; ++c) {
-            uint32_t o[32];
-            tmem_ld32(o_addr + c * 32, o);
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-            tmem_st32(o_addr + c * 32, o);
-          }
-        }
-        const float rs = tile_exp_store(sc, s_addr, p.scale_log2, m_run);
-        l_run = fmaf(l_run, alpha, rs);
-        tmem_wait_st();
-        tc_fence_before();
-        mbar_arrive(&p_full[t]);
-      }
-      if (ok && !mbar_wait(&o_done[t], (T - 1) & 1)) { report(p.status, DEV_TIMEOUT_SOFTMAX); ok = false; }
+    const uint32_t o_base = tmem_base + lane_off + 256;
+    const int nh = t == 0 ? nh0 : nh1;
+    float m_run = -INFINITY, l_run = 0.f;
+    const bool ok = softmax_stream<HD>(p.kv_len, p.scale_log2, p.status, ONE_TILE ? t : 0, ONE_TILE ? 2 : 1, nh, s_addr, o_base + t * 128,
+                                       s_full + 2 * t, p_full + 2 * t, &o_prev[t], &o_last[t], m_run, l_run);
+    if (ONE_TILE) {
+      // merge: either warpgroup writes half of the channels, stream 0's part plus stream 1's
+      tc_fence_before();
+      asm volatile("bar.sync 1, 256;" ::: "memory");   // either warpgroup has waited for the last P V of its stream:
       tc_fence_after();
+      float2* ml_s = reinterpret_cast<float2*>(k_s);   // ... the key ring is idle
+      ml_s[t * QT + r] = make_float2(m_run, l_run);
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      const float2 a = ml_s[r], b = ml_s[QT + r];
+      const float m_star = fmaxf(a.x, b.x);
+      const float f0 = fast_exp2(a.x - m_star), f1 = fast_exp2(b.x - m_star);     // an empty stream: 2^-inf = 0
+      const float inv_l = 1.f / fmaf(b.y, f1, a.y * f0);
+      const float w0 = f0 * inv_l, w1 = f1 * inv_l;
+      const int row = q0 + r;
       if (ok) {
-        const float inv_l = 1.f / l_run;
-        const int row = q0 + t * QT + r;
-        __nv_bfloat16* dst = p.out + ((size_t)img * p.rows + row) * p.C + head * HD;
-#pragma unroll
-        for (int c = 0; c < HD / 32; ++c) {
-          uint32_t o[32];
-          tmem_ld32(o_addr + c * 32, o);
+        __nv_bfloat16* dst = p.out + ((size_t)img * p.rows + row) * p.C + head * HD + t * (HD / 2);
+#pragma unroll 1
+        for (int c = 0; c < HD / 64; ++c) {
+          uint32_t x[32], y[32];
+          const uint32_t col = o_base + t * (HD / 2) + c * 32;
+          tmem_ld32(col, x);
+          if (n1 > 0) tmem_ld32(col + 128, y);
           tmem_wait_ld();
+          float v[32];
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            v[e] = __uint_as_float(x[e]) * w0;
+            if (n1 > 0) v[e] = fmaf(__uint_as_float(y[e]), w1, v[e]);
+          }
           if (row < p.rows) {
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              uint4 v;
-              v.x = pack_bf16x2(__uint_as_float(o[8 * g + 0]) * inv_l, __uint_as_float(o[8 * g + 1]) * inv_l);
-              v.y = pack_bf16x2(__uint_as_float(o[8 * g + 2]) * inv_l, __uint_as_float(o[8 * g + 3]) * inv_l);
-              v.z = pack_bf16x2(__uint_as_float(o[8 * g + 4]) * inv_l, __uint_as_float(o[8 * g + 5]) * inv_l);
-              v.w = pack_bf16x2(__uint_as_float(o[8 * g + 6]) * inv_l, __uint_as_float(o[8 * g + 7]) * inv_l);
-              reinterpret_cast<uint4*>(dst + c * 32)[g] = v;
-            }
+            for (int g = 0; g < 4; ++g)
+              reinterpret_cast<uint4*>(dst + c * 32)[g] = make_uint4(pack_bf16x2(v[8 * g], v[8 * g + 1]), pack_bf16x2(v[8 * g + 2], v[8 * g + 3]),
+                                                                     pack_bf16x2(v[8 * g + 4], v[8 * g + 5]), pack_bf16x2(v[8 * g + 6], v[8 * g + 7]));
+          }
+        }
+      }
+    } else if (t < ntiles && ok) {
+      const float inv_l = 1.f / l_run;
+      const int row = q0 + t * QT + r;
+      __nv_bfloat16* dst = p.out + ((size_t)img * p.rows + row) * p.C + head * HD;
+#pragma unroll
+      for (int c = 0; c < HD / 32; ++c) {
+        uint32_t o[32];
+        tmem_ld32(o_base + t * 128 + c * 32, o);
+        tmem_wait_ld();
+        if (row < p.rows) {
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            uint4 v;
+            v.x = pack_bf16x2(__uint_as_float(o[8 * g + 0]) * inv_l, __uint_as_float(o[8 * g + 1]) * inv_l);
+            v.y = pack_bf16x2(__uint_as_float(o[8 * g + 2]) * inv_l, __uint_as_float(o[8 * g + 3]) * inv_l);
+            v.z = pack_bf16x2(__uint_as_float(o[8 * g + 4]) * inv_l, __uint_as_float(o[8 * g + 5]) * inv_l);
+            v.w = pack_bf16x2(__uint_as_float(o[8 * g + 6]) * inv_l, __uint_as_float(o[8 * g + 7]) * inv_l);
+            reinterpret_cast<uint4*>(dst + c * 32)[g] = v;
           }
         }
       }
@@ -765,21 +882,28 @@ template <int HD> fv_status launch_hd(const AttnArgs& a, cudaStream_t st) {
   p.cost_full = kWeightPair * p.T * (p.P - p.single);
   p.cost_group = p.cost_full + kWeightSingle * p.T * p.single;
   p.total_cost = p.cost_group * a.H * a.B;
+  // Which build: costs in key tiles of a CTA that works on two streams (1.9 us at 128-wide heads).  Whole items of two query tiles
+  // take ceil(items / SMs) rounds of T of them; items of one query tile, whose two streams share its keys, are twice as many
+  // (short of part-filled ends) and take half as long each; either kind about 1.8 more to fill and to write out.  Measured (us, two /
+  // one / pieces): 820 queries, T 57 (16 heads): 109 / 58 / 76; 1024, T 19: 41 / 23 / 46; 576, T 11: 26 / 15 / 37; 1844, T 72: 138 / 146
+  // / 145; 3277, T 97: 368 / 298 / 340; 1280, T 67: 128 / 131 / 97; 4 x 256 queries, 30 heads of 64, T 12: 25.5 / 27.2 / 37.4.
+  const long long items1 = (long long)((a.rows + QT - 1) / QT) * a.H * a.B;
+  const auto rounds = [](long long n) { return (n + g_attn_sms - 1) / g_attn_sms; };
+  const double cost_two = rounds(items) * (p.T + 1.8), cost_one = rounds(items1) * ((p.T + 1) / 2 + 1.8);
+  bool one = cost_one < cost_two;
+  if (g_attn_force_ctas <= -2) one = g_attn_force_ctas == -3;
   long long ctas = items;
   p.split = 0;
   if (a.workspace && items <= kAttnMaxItems && g_attn_force_ctas >= 0) {
-    // One piece per SM when that beats whole items: a launch of whole items takes ceil(items / SMs) rounds of T key
-    // tiles; the pieces take items * T / SMs key tiles plus what the cuts cost (query tiles loaded again, the
-    // partials written and merged: about kSplitOverheadTiles key tiles, measured; short key ranges lose).  A forced
-    // piece count always splits.
-    constexpr long long kSplitOverheadTiles = 10;
+    // One piece per SM: items * T / SMs key tiles plus what the cuts cost (query tiles loaded again, the partials written
+    // and merged: about kSplitOverheadTiles key tiles, measured; short key ranges lose), all of it about 15 % slower per key
+    // tile than the whole-item kernel.  A forced piece count always splits.
+    constexpr double kSplitOverheadTiles = 10.0;
     long long g = g_attn_force_ctas > 0 ? g_attn_force_ctas : g_attn_sms;
     if (g > kAttnMaxCtas) g = kAttnMaxCtas;
     const long long most = p.total_cost / (2 * kWeightPair);   // every piece at least two key tiles long
     if (g > most) g = most;
-    const long long rounds = (items + g_attn_sms - 1) / g_attn_sms;
-    // (the kernel that walks pieces also takes about 15 % longer per key tile than the one that runs whole items)
-    const bool pays = g >= 1 && p.T >= 16 && 115 * (items * p.T / g + kSplitOverheadTiles) < 100 * rounds * p.T;
+    const bool pays = g >= 1 && p.T >= 16 && 1.15 * ((double)items * p.T / g + kSplitOverheadTiles) < (one ? cost_one : cost_two);
     if (g >= 1 && (pays || g_attn_force_ctas > 0)) {
       p.split = 1;
       ctas = g;
@@ -792,9 +916,11 @@ template <int HD> fv_status launch_hd(const AttnArgs& a, cudaStream_t st) {
   if (!p.split) {
     WholeDev w;
     w.out = p.out; w.rows = p.rows; w.C = p.C; w.kv_len = p.kv_len; w.kv_capacity = p.kv_capacity; w.scale_log2 = p.scale_log2; w.status = p.status;
-    dim3 grid3((a.rows + 2 * QT - 1) / (2 * QT), a.H, a.B);
-    return launch_pdl(attention_whole_kernel<HD>, grid3, dim3(kAttnThreads), AttnCfg<HD>::kSmemBytes, st, tmQ, tmK, tmV, w) == cudaSuccess
-               ? FV_OK : FV_ERR_CUDA;
+    const int qb = one ? QT : 2 * QT;
+    dim3 grid3((a.rows + qb - 1) / qb, a.H, a.B);
+    const cudaError_t e = one ? launch_pdl(attention_whole_kernel<HD, true>, grid3, dim3(kAttnThreads), AttnCfg<HD, true>::kSmemBytes, st, tmQ, tmK, tmV, w)
+                              : launch_pdl(attention_whole_kernel<HD, false>, grid3, dim3(kAttnThreads), AttnCfg<HD>::kSmemBytes, st, tmQ, tmK, tmV, w);
+    return e == cudaSuccess ? FV_OK : FV_ERR_CUDA;
   }
   dim3 grid((unsigned)ctas);
   return launch_pdl(attention_kernel<HD>, grid, dim3(kAttnThreads), AttnCfg<HD>::kSmemBytes, st, tmQ, tmK, tmV, p) == cudaSuccess
@@ -813,8 +939,10 @@ cudaError_t attention_init() {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_attn_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(attention_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64>::kSmemBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_whole_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64>::kSmemBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_whole_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128>::kSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_whole_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64>::kSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_whole_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128>::kSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_whole_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<64, true>::kSmemBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_whole_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128, true>::kSmemBytes);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(attention_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnCfg<128>::kSmemBytes);
 }

@@ -603,6 +603,32 @@ def test_attention_split_into_any_number_of_pieces(B, rows, H, C, kv_len, cap, c
     _attention_reference_check(bf16_host(out), q, kk, vv, B, rows, H, C, kv_len)
 
 
+@pytest.mark.parametrize("build", [-2, -3])
+@pytest.mark.parametrize("B,rows,C,kv_len", [(1, 1, 256, 1), (2, 5, 256, 64), (2, 128, 128, 65), (1, 129, 256, 128), (1, 256, 256, 129), (1, 257, 128, 192),
+                                             (2, 300, 256, 193), (1, 100, 128, 320), (1, 60, 256, 385), (1, 200, 256, 1000)])
+@pytest.mark.parametrize("growing", [False, True])
+def test_attention_whole_items_of_either_size(build, B, rows, C, kv_len, growing):
+    """Both whole-item builds (256 queries; 128 queries with two streams of key tiles merged at the end) around the edges of
+    the half tiles of 64 keys: one half, a last tile of one half, an empty second stream.  growing: scores that rise along the
+    keys, so that the running maximum moves and O is rescaled again and again, up to the last half."""
+    cap = (kv_len + 7) // 8 * 8
+    q = I.normal_bf16(290, (B * rows, C)); kk = I.normal_bf16(291, (B, cap, C)); vv = I.normal_bf16(292, (B, cap, C))
+    if growing:
+        ramp = np.linspace(0.1, 12.0, cap)[None, :, None]
+        kk = I.to_bf16_bits((I.bf16_bits_to_f32(kk) * ramp).astype(np.float32))
+    vt = np.ascontiguousarray(vv.transpose(0, 2, 1))
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    for H in (C // 128, C // 64):
+        assert fv.lib().fv_attention_force_ctas(build) == 0
+        try:
+            out = fv.fv_attention(bf16_dev(q), bf16_dev(kk), bf16_dev(vt), B, rows, H, kv_len, status=status)
+            torch.cuda.synchronize()
+        finally:
+            fv.lib().fv_attention_force_ctas(0)
+        assert int(status.item()) == 0
+        _attention_reference_check(bf16_host(out), q, kk, vv, B, rows, H, C, kv_len)
+
+
 def test_attention_refuses_small_scratch():
     q = torch.zeros((8, 256), dtype=torch.bfloat16, device=DEV); k = torch.zeros((1, 8, 256), dtype=torch.bfloat16, device=DEV)
     with pytest.raises(fv.FvError) as e:
