@@ -99,7 +99,7 @@ fv_status fv_prune_select_static(const float *x_dev, int32_t B, int32_t h, int32
  *   pivots_dev     [B, k, C] bf16     : the forwarded rows.
  *   idx_dev        [B, k] int32       : their token indices (any order, no duplicates, in [0,h*w)).
  *   out_dev        [B, h*w, C] bf16.   C % 8 == 0.
- *   inv_scratch_dev[B, h*w] int32 scratch (overwritten).
+ *   inv_scratch_dev: unused, may be NULL (earlier versions built an inverse map in it).
  *   interp_mode    0: nearest, as above (the default reading of the paper's mode-less interpolate).
  *                  1: bilinear with half-pixel centres (source coordinate (dst+0.5)*in/out - 0.5 per axis,
  *                     clamped): an unkept token is the fp32 blend of four cached rows, rounded to bf16 once.

@@ -216,8 +216,7 @@ def fv_restore(cache_prev: torch.Tensor, hc: int, wc: int, pivots: torch.Tensor,
     B, k, Cw = pivots.shape
     if out is None:
         out = torch.empty((B, h * w, Cw), dtype=torch.bfloat16, device=pivots.device)
-    inv = torch.empty((B, h * w), dtype=torch.int32, device=pivots.device)
-    _check(lib().fv_restore(_ptr(cache_prev), hc, wc, _ptr(pivots), _ptr(idx), B, k, h, w, Cw, _ptr(out), _ptr(inv),
+    _check(lib().fv_restore(_ptr(cache_prev), hc, wc, _ptr(pivots), _ptr(idx), B, k, h, w, Cw, _ptr(out), None,
                             int(interp_mode), _stream()), "fv_restore")
     return out
 

@@ -242,22 +242,6 @@ __global__ void __launch_bounds__(256, RF == 2 ? 4 : 3) restore_residual_kernel(
     fold_group_partials(b, chunk, nchunks, group, ngroups, C8 * 2, chunk_partial, group_partial, tickets);
 }
 
-__global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* __restrict__ cache, int hc, int wc,
-                                                           const uint4* __restrict__ pivots, const int32_t* __restrict__ inv,
-                                                           int n, int k, int h, int w, int C8, uint4* __restrict__ out,
-                                                           int total_rows) {
-  pdl_trigger();
-  pdl_wait();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= total_rows) return;
-  const int b = warp / n, t = warp - b * n;
-  const int j = inv[warp];
-  const uint4* src = (j >= 0) ? pivots + ((size_t)b * k + j) * C8
-                              : cache + ((size_t)b * hc * wc + nearest_src(t, h, w, hc, wc)) * C8;
-  uint4* dst = out + (size_t)warp * C8;
-  for (int c8 = lane; c8 < C8; c8 += 32) dst[c8] = __ldg(src + c8);
-}
-
 // Per-step granularity: compact copy of the kept rows of the fp32 token map (Algorithm 1's gather).
 // grid (ceil(k / 8), B): one warp per kept row.
 __global__ void __launch_bounds__(256) gather_rows_kernel(const float4* __restrict__ x, const int32_t* __restrict__ idx, int n,
@@ -483,39 +467,66 @@ __global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* __r
     fold_group_partials(b, chunk, nchunks, group, ngroups, C8 * 2, chunk_partial, group_partial, tickets);
 }
 
-// Plain restoration (no residual) with bilinear / bicubic interpolation, one warp per output row; bf16 rows
-// (8 per uint4, blended in fp32 and rounded once) or fp32 rows.
-template <int TAPS>
-__global__ void __launch_bounds__(256) restore_bf16_interp_kernel(const uint4* __restrict__ cache, int hc, int wc,
-                                                                    const uint4* __restrict__ pivots, const int32_t* __restrict__ inv,
-                                                                    int n, int k, int h, int w, int C8, uint4* __restrict__ out,
-                                                                    int total_rows) {
+// Plain restoration (no residual) of a bf16 map: TAPS 0 copies the nearest source, 4 / 16 blend bilinearly / bicubically in fp32 and
+// round once.  CTA = RT consecutive tokens.  It finds their slots in the kept set itself, by reading the image's whole index list
+// (a few KB out of L2, all of it requested at once): an inverse map built by two launches before this one cost more than that
+// (2 x 64 x 64 tokens, k 820, C 2048: 2.2 + 2.3 + 8.5 us and two more launches of the host).  A warp takes a row at a time, up to eight
+// 16-byte loads per lane in flight.
+template <int TAPS, int RT>
+__global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* __restrict__ cache, int hc, int wc, const uint4* __restrict__ pivots,
+                                                           const int32_t* __restrict__ idx, int n, int k, int h, int w, int C8, uint4* __restrict__ out) {
+  __shared__ int s_slot[RT];
+  const int b = blockIdx.y, t0 = blockIdx.x * RT;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_trigger();
+  if (threadIdx.x < RT) s_slot[threadIdx.x] = -1;
+  __syncthreads();
   pdl_wait();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= total_rows) return;
-  const int b = warp / n, t = warp - b * n;
-  const int j = inv[warp];
-  uint4* dst = out + (size_t)warp * C8;
-  if (j >= 0) {
-    const uint4* src = pivots + ((size_t)b * k + j) * C8;
-    for (int c8 = lane; c8 < C8; c8 += 32) dst[c8] = __ldg(src + c8);
-    return;
+  const int32_t* ib = idx + (size_t)b * k;
+  for (int i0 = threadIdx.x; i0 < k; i0 += 256 * 8) {
+    int v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = i0 + 256 * u < k ? __ldg(ib + i0 + 256 * u) - t0 : -1;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (v[u] >= 0 && v[u] < RT) s_slot[v[u]] = i0 + 256 * u;
   }
-  const InterpTaps<TAPS> bt = interp_taps<TAPS>(t, h, w, hc, wc);
-  const uint4* base = cache + (size_t)b * hc * wc * C8;
-  for (int c8 = lane; c8 < C8; c8 += 32) {
-    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  __syncthreads();
+  for (int r = warp; r < RT; r += 8) {
+    const int t = t0 + r;
+    if (t >= n) break;
+    const int j = s_slot[r];
+    uint4* dst = out + ((size_t)b * n + t) * C8;
+    if (TAPS == 0 || j >= 0) {
+      const uint4* src = j >= 0 ? pivots + ((size_t)b * k + j) * C8 : cache + ((size_t)b * hc * wc + nearest_src(t, h, w, hc, wc)) * C8;
+      for (int c0 = lane; c0 < C8; c0 += 256) {
+        uint4 v[8];
 #pragma unroll
-    for (int q = 0; q < TAPS; ++q) {
-      float fq[8];
-      bf16x8_to_float(__ldg(base + (size_t)bt.src[q] * C8 + c8), fq);
+        for (int u = 0; u < 8; ++u)
+          if (c0 + 32 * u < C8) v[u] = __ldg(src + c0 + 32 * u);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) f[e] = fmaf(bt.wt[q], fq[e], f[e]);
+        for (int u = 0; u < 8; ++u)
+          if (c0 + 32 * u < C8) dst[c0 + 32 * u] = v[u];
+      }
+      continue;
     }
-    __nv_bfloat162 o[4] = {__floats2bfloat162_rn(f[0], f[1]), __floats2bfloat162_rn(f[2], f[3]), __floats2bfloat162_rn(f[4], f[5]),
-                           __floats2bfloat162_rn(f[6], f[7])};
-    dst[c8] = *reinterpret_cast<uint4*>(o);
+    if constexpr (TAPS != 0) {
+      const InterpTaps<TAPS> bt = interp_taps<TAPS>(t, h, w, hc, wc);
+      const uint4* base = cache + (size_t)b * hc * wc * C8;
+      for (int c8 = lane; c8 < C8; c8 += 32) {
+        float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int q = 0; q < TAPS; ++q) {
+          float fq[8];
+          bf16x8_to_float(__ldg(base + (size_t)bt.src[q] * C8 + c8), fq);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) f[e] = fmaf(bt.wt[q], fq[e], f[e]);
+        }
+        __nv_bfloat162 o[4] = {__floats2bfloat162_rn(f[0], f[1]), __floats2bfloat162_rn(f[2], f[3]), __floats2bfloat162_rn(f[4], f[5]),
+                               __floats2bfloat162_rn(f[6], f[7])};
+        dst[c8] = *reinterpret_cast<uint4*>(o);
+      }
+    }
   }
 }
 
@@ -656,13 +667,21 @@ cudaError_t launch_restore_residual(void* x, const void* y, const void* cache, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_restore_bf16(const void* cache, int hc, int wc, const void* pivots, const int32_t* inv, int B, int k,
+cudaError_t launch_restore_bf16(const void* cache, int hc, int wc, const void* pivots, const int32_t* idx, int B, int k,
                                 int h, int w, int C, void* out, int interp_mode, cudaStream_t st) {
-  const int rows = B * h * w;
+  const int n = h * w;
   const double rb_bytes = (double)B * C * (2.0 * h * w + 2.0 * k + 2.0 * hc * wc);
   LaunchScope scope(KC_RESTORE, 1, rb_bytes, rb_bytes, st);
-  return launch_pdl(interp_mode == 0 ? restore_bf16_kernel : (interp_mode == 1 ? restore_bf16_interp_kernel<4> : restore_bf16_interp_kernel<16>), dim3((rows + 7) / 8), dim3(256), 0, st, reinterpret_cast<const uint4*>(cache), hc, wc,
-                    reinterpret_cast<const uint4*>(pivots), inv, h * w, k, h, w, C / 8, reinterpret_cast<uint4*>(out), rows);
+  // 16 tokens per CTA (two rows per warp); 8 while that leaves SMs without a CTA
+  const bool small = (long)((n + 15) / 16) * B < g_rows_sms;
+  auto go = [&](auto* k16, auto* k8) {
+    const int rt = small ? 8 : 16;
+    return launch_pdl(small ? k8 : k16, dim3((n + rt - 1) / rt, B), dim3(256), 0, st, static_cast<const uint4*>(cache), hc, wc,
+                      static_cast<const uint4*>(pivots), idx, n, k, h, w, C / 8, static_cast<uint4*>(out));
+  };
+  if (interp_mode == 0) return go(restore_bf16_kernel<0, 16>, restore_bf16_kernel<0, 8>);
+  if (interp_mode == 1) return go(restore_bf16_kernel<4, 16>, restore_bf16_kernel<4, 8>);
+  return go(restore_bf16_kernel<16, 16>, restore_bf16_kernel<16, 8>);
 }
 
 cudaError_t launch_gather_rows(const float* x, const int32_t* idx, int B, int n, int k, int C, float* out, int32_t* status, cudaStream_t st) {
