@@ -91,59 +91,166 @@ __global__ void __launch_bounds__(256) residual_accumulate_kernel(const int32_t*
   }
 }
 
-// ---- x[b,t,:] = r[b, src(t), :] * W_in^T + b_in + pos[t,:];  CTA = 32 tokens x all channels ----
-constexpr int kNextTokens = 32;
+// ---- x[b,t,:] = r[b, src(t), :] * W_in^T + b_in + pos[t,:] ----
+// CTA = 64 tokens of the map r x 256 channels, thread = 8 tokens x 8 channels (two groups of four: a warp stores 512 contiguous bytes
+// at a time).  The product belongs to the SOURCE token, of which the next map has several copies (nearest interpolation), so it
+// is computed once and written, with each copy's own embedding, to all of them.  Up to 32 code channels at a time lie in
+// shared memory, W_in as [j][channel] and the tokens' vectors as [j][token]; the shared-memory port hands a warp one word per
+// lane and clock, a broadcast word included, so a thread tile of T x C costs T + C of its clocks for T C / 4 of an SM's multiply-adds: 8 x 8
+// balances the two.  The copies' embedding rows are fetched into L2 under the multiply-adds; a warp then walks the copies of its own
+// tokens, the products read back from shared memory, four embedding rows in flight.  Measured for 2 x 48 x 48 -> 64 x 64 tokens,
+// C 2048, d 32 (map written + embedding read: 16 us): 81 us with a product per target token and one channel per thread, 59 us
+// with a product per target token in 8 x 8 tiles, 51 us like this (two rounds of CTAs, each a chain of loads, products and
+// stores).  The additions keep their order (j ascending, bias, embedding).
+constexpr int kNextTokens = 64;
+constexpr int kNextChannels = 256;      // one per thread while W_in is staged
+// (r is written by the kernel before this one: without __restrict__ its loads stay behind the dependency wait)
 template <int D>
-__global__ void __launch_bounds__(256) next_input_kernel(const float* __restrict__ r, int h, int w, int h2, int w2, const float* __restrict__ w_in,
-                                                         const float* __restrict__ b_in, const float* __restrict__ pos, int C, int B,
-                                                         float* __restrict__ x_out) {
-  __shared__ __align__(16) float r_s[kNextTokens][D];
-  __shared__ int s_t2[kNextTokens];      // token index inside the next map (row of pos), per staged token
+__global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int h, int w, int h2, int w2, const float* __restrict__ w_in,
+                                                            const float* __restrict__ b_in, const float* __restrict__ pos, int C, int B, int vec,
+                                                            float* __restrict__ x_out) {
+  constexpr int DC = D < 32 ? D : 32;
+  __shared__ __align__(16) float w_s[DC][kNextChannels];
+  __shared__ __align__(16) float r_s[DC][kNextTokens];
+  __shared__ int s_first[kNextTokens], s_nx[kNextTokens], s_cnt[kNextTokens];   // a token's copies: first one, copies per row of the next map, all
+  __shared__ long s_img[kNextTokens];    // first row of its image in x_out
   pdl_trigger();
   const int n = h * w, n2 = h2 * w2;
-  const long rows = (long)B * n2;
-  const long row0 = (long)blockIdx.x * kNextTokens;
-  pdl_wait();
-  for (int i = threadIdx.x; i < kNextTokens * D; i += blockDim.x) {
-    const int t = i / D, j = i - t * D;
-    const long row = row0 + t;
-    float v = 0.f;
+  const long rows = (long)B * n;
+  const long row0 = (long)blockIdx.y * kNextTokens;
+  const int c0 = blockIdx.x * kNextChannels;
+  const int tid = threadIdx.x;
+  if (tid < kNextTokens) {   // token (y, x) is the source of the targets y2 with floor(y2 h / h2) = y, and x2 likewise
+    const long row = row0 + tid;
+    int first = 0, nx = 0, ny = 0;
     if (row < rows) {
-      const int b = (int)(row / n2), t2 = (int)(row - (long)b * n2);
-      const int y = t2 / w2, x = t2 - y * w2;
-      const int src = (int)(((long)y * h) / h2) * w + (int)(((long)x * w) / w2);
-      v = r[((size_t)b * n + src) * D + j];
-      if (j == 0) s_t2[t] = t2;
+      const int b = (int)row / n, t = (int)row - b * n, y = t / w, x = t - y * w;   // (32 bits: the launcher checks)
+      const int y0 = (y * h2 + h - 1) / h, x0 = (x * w2 + w - 1) / w;
+      ny = ((y + 1) * h2 + h - 1) / h - y0;
+      nx = ((x + 1) * w2 + w - 1) / w - x0;
+      first = y0 * w2 + x0;
+      s_img[tid] = (long)b * n2;
     }
-    r_s[t][j] = v;
+    s_first[tid] = first; s_nx[tid] = nx; s_cnt[tid] = nx * ny;
   }
+  float acc[8][8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t)
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[t][e] = 0.f;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int tl = warp * 8;               // this thread's tokens inside the tile; its channels are 4 lane .. and 128 + 4 lane ..
+  // target token d of the copies of staged token t, inside its image
+  auto target = [&](int t, int d) { const int yy = d / s_nx[t]; return s_first[t] + yy * w2 + (d - yy * s_nx[t]); };
   __syncthreads();
-  const int t_valid = (int)min((long)kNextTokens, rows - row0);
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    float wr[D];
+  if (pos) {   // a quarter warp per row: 8 lines of 128 bytes
+    const int t = tid >> 2;
+    for (int d = 0; d < s_cnt[t]; ++d) {
+      const float* q = pos + (size_t)target(t, d) * C;
 #pragma unroll
-    for (int j = 0; j < D; j += 4) {
-      const float4 q = __ldg(reinterpret_cast<const float4*>(w_in + (size_t)c * D + j));
-      wr[j] = q.x; wr[j + 1] = q.y; wr[j + 2] = q.z; wr[j + 3] = q.w;
+      for (int u = 0; u < 2; ++u) {
+        const int c = c0 + ((tid & 3) + 4 * u) * 32;
+        if (c < C) asm volatile("prefetch.global.L2 [%0];" ::"l"(q + c));
+      }
     }
-    const float bias = b_in ? __ldg(b_in + c) : 0.f;
-    float* out = x_out + (size_t)row0 * C + c;
-    for (int t0 = 0; t0 < t_valid; t0 += 8) {   // eight tokens at a time: their position-embedding loads go out together
-      float pe[8];
+  }
+  for (int d0 = 0; d0 < D; d0 += DC) {
+    if (d0) __syncthreads();             // the chunk before has been used
+    {   // all of a thread's loads are requested before the first is stored: one round trip each for W_in and r
+      float4 q[DC / 4];                  // channel c0 + tid
 #pragma unroll
-      for (int u = 0; u < 8; ++u) pe[u] = (pos && t0 + u < t_valid) ? __ldg(pos + (size_t)s_t2[t0 + u] * C + c) : 0.f;
+      for (int i = 0; i < DC / 4; ++i) {
+        q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c0 + tid < C) q[i] = __ldg(reinterpret_cast<const float4*>(w_in + (size_t)(c0 + tid) * D + d0 + 4 * i));
+      }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        if (t0 + u < t_valid) {
-          float acc = 0.f;
+      for (int i = 0; i < DC / 4; ++i) { w_s[4 * i][tid] = q[i].x; w_s[4 * i + 1][tid] = q[i].y; w_s[4 * i + 2][tid] = q[i].z; w_s[4 * i + 3][tid] = q[i].w; }
+    }
+    if (d0 == 0) pdl_wait();             // (weights and embeddings are never written by a kernel of the loop)
+    {
+      constexpr int JP = DC / 4;         // four threads per token
+      const int t = tid >> 2, j0 = (tid & 3) * JP;
+      const long src = row0 + t;
+      float v[JP];
 #pragma unroll
-          for (int j = 0; j < D; j += 4) {      // the token's vector is read as float4 broadcasts
-            const float4 q = *reinterpret_cast<const float4*>(&r_s[t0 + u][j]);
-            acc = fmaf(q.x, wr[j], acc); acc = fmaf(q.y, wr[j + 1], acc); acc = fmaf(q.z, wr[j + 2], acc); acc = fmaf(q.w, wr[j + 3], acc);
+      for (int u = 0; u < JP; ++u) v[u] = src < rows ? r[src * D + d0 + j0 + u] : 0.f;
+#pragma unroll
+      for (int u = 0; u < JP; ++u) r_s[j0 + u][t] = v[u];
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int j = 0; j < DC; ++j) {
+      const float4 wa = *reinterpret_cast<const float4*>(&w_s[j][4 * lane]), wb = *reinterpret_cast<const float4*>(&w_s[j][128 + 4 * lane]);
+      const float4 ra = *reinterpret_cast<const float4*>(&r_s[j][tl]), rb = *reinterpret_cast<const float4*>(&r_s[j][tl + 4]);
+      const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w}, rv[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+#pragma unroll
+      for (int t = 0; t < 8; ++t)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[t][e] = fmaf(rv[t], wv[e], acc[t][e]);
+    }
+  }
+  // The warp's products go to its own 4 KB of shared memory (over W_in, 128 channels at a time), and the warp walks the copies of its
+  // tokens: lane l knows copy l's token and place, four embedding rows in flight.
+  __syncthreads();
+  float4* mine = reinterpret_cast<float4*>(&w_s[0][0]) + warp * (DC * kNextChannels / 4 / 8);
+  constexpr int kRowsFit = DC * kNextChannels / 128 / 8;   // token rows of 128 channels in the warp's share: 8 for 32 code channels
+  int before[9];
+  before[0] = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) before[t + 1] = before[t] + s_cnt[tl + t];
+#pragma unroll 1
+  for (int g = 0; g < 2; ++g) {
+    const int c = c0 + 128 * g + 4 * lane;
+    const bool col_ok = c < C;
+    float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (b_in && col_ok) bias = make_float4(__ldg(b_in + c), __ldg(b_in + c + 1), __ldg(b_in + c + 2), __ldg(b_in + c + 3));
+#pragma unroll
+    for (int r0 = 0; r0 < 8; r0 += kRowsFit) {
+      __syncwarp();
+#pragma unroll
+      for (int t = r0; t < r0 + kRowsFit; ++t) {
+        const float4 v = g ? make_float4(acc[t][4], acc[t][5], acc[t][6], acc[t][7]) : make_float4(acc[t][0], acc[t][1], acc[t][2], acc[t][3]);
+        mine[(t - r0) * 32 + lane] = make_float4(v.x + bias.x, v.y + bias.y, v.z + bias.z, v.w + bias.w);
+      }
+      __syncwarp();
+      const int lo = before[r0], hi = before[r0 + kRowsFit];
+      for (int e0 = lo; e0 < hi; e0 += 32) {
+        int t = r0;
+#pragma unroll
+        for (int u = r0 + 1; u < r0 + kRowsFit; ++u) t += e0 + lane >= before[u];
+        int d = e0 + lane;
+#pragma unroll
+        for (int u = r0; u < r0 + kRowsFit; ++u)
+          if (t == u) d -= before[u];
+        const int nx = max(s_nx[tl + t], 1), yy = d / nx, t2 = s_first[tl + t] + yy * w2 + (d - yy * nx);
+        const long img = s_img[tl + t];
+        const int cnt = min(32, hi - e0);
+#pragma unroll 1
+        for (int k0 = 0; k0 < cnt; k0 += 4) {
+          float4 pe[4];
+          int tt[4];
+          long row[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int src = min(k0 + u, cnt - 1);
+            tt[u] = __shfl_sync(0xffffffffu, t, src);
+            const int k2 = __shfl_sync(0xffffffffu, t2, src);
+            row[u] = __shfl_sync(0xffffffffu, img, src) + k2;
+            pe[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (pos && col_ok) {
+              const float* q = pos + (size_t)k2 * C + c;
+              pe[u] = vec ? __ldg(reinterpret_cast<const float4*>(q)) : make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3));
+            }
           }
-          acc += bias;
-          acc += pe[u];
-          out[(size_t)(t0 + u) * C] = acc;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (k0 + u >= cnt || !col_ok) break;
+            const float4 a = mine[(tt[u] - r0) * 32 + lane];
+            const float4 o = make_float4(a.x + pe[u].x, a.y + pe[u].y, a.z + pe[u].z, a.w + pe[u].w);
+            float* dst = x_out + (size_t)row[u] * C + c;
+            if (vec) *reinterpret_cast<float4*>(dst) = o;
+            else { dst[0] = o.x; dst[1] = o.y; dst[2] = o.z; dst[3] = o.w; }
+          }
         }
       }
     }
@@ -186,12 +293,16 @@ cudaError_t launch_next_input(const float* r, int B, int h, int w, int d, int h2
   const long rows = (long)B * h2 * w2;
   const double bytes = (double)rows * C * (pos ? 8.0 : 4.0) + (double)rows * d * 4.0;
   LaunchScope scope(KC_RESTORE, 1, bytes, bytes, st);
-  const dim3 grid((unsigned)((rows + kNextTokens - 1) / kNextTokens));
+  // (tokens along y: up to 65535 x 64 of them, far past the largest token map)
+  const dim3 grid((unsigned)((C + kNextChannels - 1) / kNextChannels), (unsigned)(((long)B * h * w + kNextTokens - 1) / kNextTokens));
+  // (32-bit index arithmetic: maps of up to some 40000 tokens a side)
+  if (grid.y > 65535u || (long)(h + 1) * h2 + h > INT_MAX || (long)(w + 1) * w2 + w > INT_MAX || (long)B * h * w > INT_MAX) return cudaErrorInvalidValue;
+  const int vec = ((reinterpret_cast<uintptr_t>(x_out) | reinterpret_cast<uintptr_t>(pos)) & 15u) == 0;   // C is a multiple of 4
   switch (d) {
-    case 8: return launch_pdl(next_input_kernel<8>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, x_out);
-    case 16: return launch_pdl(next_input_kernel<16>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, x_out);
-    case 32: return launch_pdl(next_input_kernel<32>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, x_out);
-    case 64: return launch_pdl(next_input_kernel<64>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, x_out);
+    case 8: return launch_pdl(next_input_kernel<8>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, x_out);
+    case 16: return launch_pdl(next_input_kernel<16>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, x_out);
+    case 32: return launch_pdl(next_input_kernel<32>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, x_out);
+    case 64: return launch_pdl(next_input_kernel<64>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, x_out);
     default: return cudaErrorInvalidValue;
   }
 }

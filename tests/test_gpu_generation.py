@@ -114,6 +114,26 @@ def test_head_tokens_matches_oracle(B, n, C, V):
         np.testing.assert_array_equal(ids[~own_flag], own[~own_flag])
 
 
+@pytest.mark.parametrize("d,C,h,w,h2,w2,B", [(8, 260, 12, 11, 20, 31, 1), (32, 128, 1, 1, 9, 7, 3), (64, 516, 9, 8, 9, 8, 1), (16, 2048, 33, 31, 16, 50, 2),
+                                              (32, 4, 1, 70, 1, 200, 2)])
+def test_next_scale_input_copies_of_a_source_token(d, C, h, w, h2, w2, B):
+    """Source tokens with one, none and many copies (more than a warp holds at a time), ragged tiles of 64 tokens and of 256 channels, an
+    output and an embedding that are not 16-byte aligned: the same products and the same order of additions give the same bits."""
+    r = I.normal(141, (B, h * w, d), 2.0)
+    w_in, b_in, pos = I.normal(142, (C, d), 1 / np.sqrt(d)), I.normal(143, (C,), 0.1), I.normal(144, (h2 * w2, C), 0.5)
+    ref = G.next_scale_input(r, h, w, h2, w2, w_in, b_in, pos)
+    got = fv.fv_next_scale_input(T(r), h, w, h2, w2, T(w_in), T(b_in), T(pos))
+    np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=1e-5, atol=2e-5)      # fp32 dot products of d terms
+    big = torch.zeros(B * h2 * w2 * C + 1, dtype=torch.float32, device=DEV)
+    pos1 = torch.zeros(h2 * w2 * C + 1, dtype=torch.float32, device=DEV)
+    pos1[1:] = T(pos).reshape(-1)
+    rd, wd, bd = T(r), T(w_in), T(b_in)
+    rc = fv.lib().fv_next_scale_input(rd.data_ptr(), B, h, w, d, h2, w2, wd.data_ptr(), bd.data_ptr(), pos1.data_ptr() + 4, C, big.data_ptr() + 4,
+                                      torch.cuda.current_stream().cuda_stream)
+    assert rc == 0
+    assert torch.equal(big[1:].view(B, h2 * w2, C), got)
+
+
 def _gen_setup(keep, sides=(1, 2, 3, 4, 6, 8), L=2, C=128, H=2, B=2, V=256, d=16, cross_len=0):
     wl = I.Workload("gen", L=L, C=C, H=H, B=B, sides=tuple(sides), keep=tuple(keep), cross_len=cross_len, seed=31)
     mt = I.model_tensors(wl)
