@@ -388,29 +388,36 @@ cudaError_t gemm_init() {
   return cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
 }
 
-// Kernel and tile width for a shape.  Measured on B200 (launches replayed from a CUDA graph, so that the host does
-// not pace them), one launch costs about
+// Kernel and tile for a shape.  Measured on B200 (launches replayed from a CUDA graph, so that the host does not pace
+// them, weights rotating through HBM), one launch costs about
 //     fixed + rounds x (per_round + k-blocks x per_kblock)
-// where rounds = ceil(tiles / resident CTAs or pairs).  A k-block of a 128-wide tile is paced by the thread that
-// issues its MMAs (two k-blocks per pipeline stage there), the wider tiles by the MMAs themselves and the operand
-// loads; wider tiles and CTA pairs win by needing fewer rounds and less L2 traffic per flop.
-struct TileChoice { int bn; bool pair; };
+// where rounds = ceil(CTAs / SMs), or pairs / half the SMs.  A k-block of a 128-wide tile is paced by the operand loads (an SM takes
+// in about 110 bytes per clock, whatever the tile), the wider tiles by the MMAs themselves; wider tiles and CTA pairs win by needing
+// fewer rounds and less L2 traffic per flop.  Where tiles leave SMs idle, the CTAs of a cluster share a tile's K (2 or 4 slices,
+// gemm_cluster.cu); those only compete while all their CTAs run at once.
+struct TileChoice { int bn; bool pair; int slices; };   // slices 1: no cluster
 static TileChoice pick_tile(int M, int N, int K, int sms) {
   const int num_kb = (K + BK - 1) / BK;
-  struct Cand { int bn; bool pair; double fixed_us, round_us, kb_us; };
-  // least-squares fit over M 256 ... 3277 x the four projection shapes of a 2048-wide block, every candidate forced
-  const Cand cand[5] = {{128, false, 2.23, 0.98, 0.235}, {192, false, 2.16, 2.19, 0.292}, {256, false, 1.17, 3.01, 0.349},
-                        {256, true, 3.99, 2.30, 0.316}, {64, false, 2.9, 0.5, 0.21}};
-  TileChoice best{128, false};
+  struct Cand { int bn; bool pair; int slices; double fixed_us, round_us, kb_us; };
+  // Least-squares fits over M 36 ... 3277 x the four projection shapes of 1024-, 1920- and 2048-wide blocks, every candidate forced.  On
+  // that sweep the choice costs 0.3 % over the best candidate on average (10 % at worst, 0.5 us); e.g. (us) N 2048 K 8192: M 400 64-wide
+  // 23.0, 128 x 2 24.5; M 820 pair of 128 27.7, 128-wide 31.7, 192-wide 35.5; N 1024 K 4096: M 400 64 x 2 9.9, 128 x 4 11.4; M 816 64-wide
+  // 12.8, 128 x 2 14.5; N 2048 K 2048 M 3277 192-wide 24.6, 128-wide 30.4.
+  const Cand cand[10] = {{128, false, 1, 3.63, 0.81, 0.214}, {192, false, 1, 3.53, 1.79, 0.251}, {256, false, 1, 2.87, 2.28, 0.343},
+                         {256, true, 1, 6.47, 1.55, 0.292}, {128, true, 1, 5.09, 1.11, 0.168}, {64, false, 1, 3.17, 0.42, 0.151},
+                         {64, false, 4, 3.79, 0.0, 0.228}, {64, false, 2, 3.48, 0.0, 0.196},
+                         {128, false, 4, 5.75, 0.0, 0.304}, {128, false, 2, 5.38, 0.0, 0.295}};
+  TileChoice best{128, false, 1};
   double best_cost = 1e30;
   for (const Cand& c : cand) {
     if (c.pair && M <= 256) continue;
     const int rows = c.pair ? 256 : 128;
     const int slots = c.pair ? sms / 2 : sms;
-    const long tiles = (long)((M + rows - 1) / rows) * ((N + c.bn - 1) / c.bn);
-    const long rounds = (tiles + slots - 1) / slots;
-    const double cost = c.fixed_us + (double)rounds * (c.round_us + num_kb * c.kb_us);
-    if (cost < best_cost - 1e-9) { best_cost = cost; best = TileChoice{c.bn, c.pair}; }
+    const long ctas = (long)((M + rows - 1) / rows) * ((N + c.bn - 1) / c.bn) * c.slices;
+    if (c.slices > 1 && (ctas > slots || num_kb < 8)) continue;
+    const long rounds = (ctas + slots - 1) / slots;
+    const double cost = c.fixed_us + (double)rounds * (c.round_us + (num_kb + c.slices - 1) / c.slices * c.kb_us);
+    if (cost < best_cost - 1e-9) { best_cost = cost; best = TileChoice{c.bn, c.pair, c.slices}; }
   }
   return best;
 }
@@ -475,20 +482,17 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
   if (g.epilogue == EPI_QKV_SPLIT && (g.C % 128 || g.q_cols % 128)) return FV_ERR_UNSUPPORTED;
   const int tiles_m = (g.M + BM - 1) / BM;
   TileChoice tc = pick_tile(g.M, g.N, g.K, g_num_sms);
-  // Few rows against a narrow output (the out-projections and the second MLP GEMM of the small scale steps):
-  // 64-wide tiles double the CTAs that stream the weight matrix.  Measured (M <= 128, N = 2048): 9.7 us instead
-  // of 11.4 at M = 32, K = 2048; 20.6 instead of 30.1 at M = 128, K = 8192; wider outputs and more rows lose.
-  if (g.M <= 128 && g.N <= 2048 && g.N > 64) tc = TileChoice{64, false};
-  if (g_force_path == 1 && tc.pair) tc = TileChoice{256, false};
-  if (g_force_path == 2) tc = TileChoice{256, true};
-  if (g_force_path == 3) tc = TileChoice{128, true};
-  if (g_force_path >= 4 && g_force_path <= 6) tc = TileChoice{128 + 64 * (g_force_path - 4), false};
-  if (g_force_path == 7) tc = TileChoice{64, false};
+  const TileChoice picked = tc;
+  if (g_force_path == 1 && tc.pair) tc = TileChoice{256, false, 1};
+  if (g_force_path == 2) tc = TileChoice{256, true, 1};
+  if (g_force_path == 3) tc = TileChoice{128, true, 1};
+  if (g_force_path >= 4 && g_force_path <= 6) tc = TileChoice{128 + 64 * (g_force_path - 4), false, 1};
+  if (g_force_path == 7) tc = TileChoice{64, false, 1};
   // Q / K extras (cosine attention, rotary positions): one-CTA tiles that hold whole heads, no K split
   const bool qk_extras = g.epilogue == EPI_QKV_SPLIT && (g.qk_scale || g.rope_table);
   if (qk_extras) {
     if (g.head_dim != 64 && g.head_dim != 128) return FV_ERR_UNSUPPORTED;
-    if (tc.pair) tc = TileChoice{256, false};
+    if (tc.pair) tc = TileChoice{256, false, 1};
     if (tc.bn < 128) tc.bn = 128;            // the extras exist for tiles of at least 128 columns
     if (tc.bn % g.head_dim) tc.bn = 256;
   }
@@ -519,24 +523,15 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
   p.rope_table = qk_extras ? reinterpret_cast<const float2*>(g.rope_table) : nullptr;
   p.rope_idx = qk_extras ? g.rope_idx : nullptr;
   p.head_dim = g.head_dim;
-  // Few tiles against a long K (every GEMM of the small scale steps): split K over the CTAs of a cluster, the
-  // partials reduced through distributed shared memory.  Which shape wins follows the tile counts.  Up to 32 rows two CTAs
+  // K split over the CTAs of a cluster, the partials reduced through distributed shared memory.  Up to 32 rows two CTAs
   // share an SM and 64-wide tiles are the best everywhere: 4 slices while the CTAs stay near one per SM, else 2 (us at M 8, weights
   // from HBM, 64 x 4 / 64 x 2 / 128 x 4 / 128 x 2: N 2048 K 2048 4.8 / 5.3 / 5.8 / 7.4; N 6144 10.1 / 8.3 / 8.2 / 9.5;
   // N 8192 12.0 / 9.1 / 8.9 / 10.5; N 2048 K 8192 10.1 / 14.1 / 14.7 / 23.3; 1024-wide models N 3072 4.1 / 4.2 / 4.7 / 4.9).
   int cluster_slices = 0, cluster_bn = 0;
   if (g_force_path == 0 && !qk_extras) {
-    const int num_kb = (g.K + BK - 1) / BK;
-    const long t128 = (long)tiles_m * ((g.N + 127) / 128), t64 = (long)tiles_m * ((g.N + 63) / 64);
-    // (re-measured GPU-bound after the narrow tiles took two k-blocks per pipeline stage: with more than 32 rows the
-    // 128-wide x 2 cluster, whose ring has no room for that, only wins on a long K; 64-wide x 2 wins on a short one)
-    if (num_kb >= 8) {
-      if (g.M <= 32 && t64 <= g_num_sms) { cluster_bn = 64; cluster_slices = t64 * 3 <= g_num_sms ? 4 : 2; }
-      else if (t64 * 4 <= g_num_sms) { cluster_bn = 64; cluster_slices = 4; }
-      else if (t64 * 2 <= g_num_sms && num_kb < 64) { cluster_bn = 64; cluster_slices = 2; }
-      else if (t128 * 4 <= g_num_sms) { cluster_bn = 128; cluster_slices = 4; }
-      else if (t128 * 2 <= g_num_sms && (g.M <= 32 || num_kb >= 64)) { cluster_bn = 128; cluster_slices = 2; }
-    }
+    const long t64 = (g.N + 63) / 64;
+    if (g.M <= 32 && g.K > 7 * BK && t64 <= g_num_sms) { cluster_bn = 64; cluster_slices = t64 * 3 <= g_num_sms ? 4 : 2; }
+    else if (picked.slices > 1) { cluster_bn = picked.bn; cluster_slices = picked.slices; }
   }
   if (g_force_path >= 8 && g_force_path <= 11 && !qk_extras) {   // 8: 128 wide x 4 slices, 9: 128 x 2, 10: 64 x 4, 11: 64 x 2
     cluster_bn = g_force_path <= 9 ? 128 : 64;
