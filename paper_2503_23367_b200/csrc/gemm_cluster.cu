@@ -70,7 +70,13 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;
   constexpr int ROWS_PER = AROWS / S;     // rows of the tile each CTA finishes
-  constexpr int CHUNKS = BN / 32;         // 32-column chunks per row
+  // The CTA finishes ROWS_PER x BN values, four consecutive columns per epilogue thread and turn: lanes along the columns, so that a
+  // warp stores whole lines; along the rows where the columns are V's (its cache is transposed: a key's neighbours are rows).
+  // What a residual stream or gate contributes does not depend on the product and is fetched before the barriers, up to PRE turns
+  // of it: read after the reduction it cost two dependent trips to L2, 1.7 us of a 6.4 us launch.
+  constexpr int QUADS = BN / 4;
+  constexpr int TURNS = ROWS_PER * QUADS / 128;
+  constexpr int PRE = TURNS < 8 ? TURNS : 8;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint4* bias_s = reinterpret_cast<uint4*>(smem + STAGES * Cfg::kStageBytes);
@@ -104,6 +110,31 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   // first half of the "every CTA of the cluster has started" barrier; the second half precedes the first
   // store into another CTA's shared memory (a rank with an empty K slice gets there almost at once)
   cluster_arrive_relaxed();
+
+  const bool v_tile = p.epilogue == EPI_QKV_SPLIT && n0 >= p.q_cols + p.C;
+  const bool x_f32 = p.epilogue == EPI_RESIDUAL, x_b16 = p.epilogue == EPI_RESIDUAL_XBF16;
+  const int et = (int)threadIdx.x - 64;                   // 0..127 among the epilogue threads
+  auto place = [&](int i, int& lrow, int& quad) {
+    const int f = et + 128 * i;
+    lrow = v_tile ? f % ROWS_PER : f / QUADS;
+    quad = v_tile ? f / ROWS_PER : f % QUADS;
+  };
+  float4 xv[PRE], gv[PRE];
+  auto fetch = [&](int i, int slot) {   // stream and gate of turn i
+    int lrow, quad;
+    place(i, lrow, quad);
+    const int row = m0 + (int)rank * ROWS_PER + lrow, col = n0 + 4 * quad;
+    gv[slot] = make_float4(1.f, 1.f, 1.f, 1.f);
+    if (row >= p.M || col >= p.N) return;
+    const size_t at = (size_t)row * p.N + col;
+    if (x_f32) {
+      xv[slot] = *reinterpret_cast<const float4*>(static_cast<const float*>(p.out) + at);
+    } else {
+      const uint2 u = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(p.out) + at);
+      xv[slot] = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
+    }
+    if (p.gamma) gv[slot] = *reinterpret_cast<const float4*>(p.gamma + (size_t)(row / p.rows_per_image) * p.mod_stride + col);
+  };
 
   if (warp == 0) {
     if (lane == 0) {
@@ -161,12 +192,16 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
   } else {
     // ---- accumulator readers: thread = one accumulator row; its partial goes to the CTA that owns the row ----
+    stage_bias(p, bias_s + (warp & 3) * 32, lane, n0, BN);
     pdl_wait();
+    if (x_f32 || x_b16) {
+#pragma unroll
+      for (int i = 0; i < PRE; ++i) fetch(i, i);
+    }
     const int quarter = warp & 3;
     const int trow = quarter * 32 + lane;                 // row inside the tile
     const uint32_t owner = (uint32_t)min(trow / ROWS_PER, S - 1);   // (rows past AROWS belong to no row of the output)
     const int lrow = trow - (int)owner * ROWS_PER;
-    stage_bias(p, bias_s + quarter * 32, lane, n0, BN);
     bool have = kb1 > kb0;
     if (have && !mbar_wait(acc_full, 0)) { report(p.status, DEV_TIMEOUT_EPI); have = false; }
     have = __all_sync(0xffffffffu, have);   // the TMEM loads below are warp-wide
@@ -197,34 +232,83 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   if (warp < 2) cluster_wait();             // completes these warps' half of the start-up barrier
   cluster_sync_all();
   if (warp >= 2) {
-    const int e = threadIdx.x - 64;                        // 0..127
-    const uint4* bias_w = bias_s + (warp & 3) * 32;
-    for (int ci = e; ci < ROWS_PER * CHUNKS; ci += 128) {
-      const int lrow = ci / CHUNKS, ch = ci - lrow * CHUNKS;
-      const int row = m0 + (int)rank * ROWS_PER + lrow;
-      const int col = n0 + 32 * ch;
-      if (row >= p.M || col >= p.N) continue;
-      float acc[32];
-      const float* src = red + (size_t)lrow * Cfg::kRedPitch + 32 * ch;
+    const uint2* bias_w = reinterpret_cast<const uint2*>(bias_s + (warp & 3) * 32);
+#pragma unroll 1
+    for (int i0 = 0; i0 < TURNS; i0 += PRE) {
+      if (i0 > 0 && (x_f32 || x_b16)) {
 #pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        const float4 v = *reinterpret_cast<const float4*>(src + 4 * g);
-        acc[4 * g] = v.x; acc[4 * g + 1] = v.y; acc[4 * g + 2] = v.z; acc[4 * g + 3] = v.w;
+        for (int u = 0; u < PRE; ++u) fetch(i0 + u, u);
       }
+      float4 v[PRE];                       // the sums of all turns first: their shared-memory reads do not wait for one another
 #pragma unroll
-      for (int s = 1; s < S; ++s) {                        // rank order: the sum does not depend on timing
-        const float* ss = src + (size_t)s * ROWS_PER * Cfg::kRedPitch;
+      for (int u = 0; u < PRE; ++u) {
+        int lrow, quad;
+        place(i0 + u, lrow, quad);
+        const float* src = red + (size_t)lrow * Cfg::kRedPitch + 4 * quad;
+        v[u] = *reinterpret_cast<const float4*>(src);
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-          const float4 v = *reinterpret_cast<const float4*>(ss + 4 * g);
-          acc[4 * g] += v.x; acc[4 * g + 1] += v.y; acc[4 * g + 2] += v.z; acc[4 * g + 3] += v.w;
+        for (int s = 1; s < S; ++s) {      // rank order: the sum does not depend on timing
+          const float4 w = *reinterpret_cast<const float4*>(src + (size_t)s * ROWS_PER * Cfg::kRedPitch);
+          v[u].x += w.x; v[u].y += w.y; v[u].z += w.z; v[u].w += w.w;
+        }
+        if (p.bias) {
+          const uint2 bb = bias_w[quad];
+          v[u].x += __uint_as_float(bb.x << 16); v[u].y += __uint_as_float(bb.x & 0xFFFF0000u);
+          v[u].z += __uint_as_float(bb.y << 16); v[u].w += __uint_as_float(bb.y & 0xFFFF0000u);
         }
       }
-      uint32_t r[32];
+      if (x_f32 || x_b16) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(acc[i]);
-      const int img = row / p.rows_per_image;
-      epilogue_chunk(p, r, row, img, row - img * p.rows_per_image, col, bias_w + 4 * ch);
+        for (int u = 0; u < PRE; ++u) {
+          int lrow, quad;
+          place(i0 + u, lrow, quad);
+          const int row = m0 + (int)rank * ROWS_PER + lrow, col = n0 + 4 * quad;
+          if (row >= p.M || col >= p.N) continue;
+          const size_t at = (size_t)row * p.N + col;
+          const float4 g = gv[u];
+          float4 x = xv[u];
+          x.x = fmaf(g.x, v[u].x, x.x); x.y = fmaf(g.y, v[u].y, x.y); x.z = fmaf(g.z, v[u].z, x.z); x.w = fmaf(g.w, v[u].w, x.w);
+          if (x_f32) *reinterpret_cast<float4*>(static_cast<float*>(p.out) + at) = x;
+          else *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.out) + at) = make_uint2(pack_bf16x2(x.x, x.y), pack_bf16x2(x.z, x.w));
+          if (p.aux) *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(p.aux) + at) = make_uint2(pack_bf16x2(v[u].x, v[u].y), pack_bf16x2(v[u].z, v[u].w));
+        }
+      } else if (v_tile) {
+#pragma unroll
+        for (int u = 0; u < PRE; ++u) {
+          int lrow, quad;
+          place(i0 + u, lrow, quad);
+          const int row = m0 + (int)rank * ROWS_PER + lrow, col = n0 + 4 * quad;
+          if (row >= p.M || col >= p.N) continue;
+          const int img = row / p.rows_per_image, jrow = row - img * p.rows_per_image;
+          __nv_bfloat16* dst = p.vt_cache + ((size_t)img * p.C + (col - p.q_cols - p.C)) * p.kv_capacity + p.kv_offset + jrow;
+          dst[0] = __float2bfloat16_rn(v[u].x);
+          dst[p.kv_capacity] = __float2bfloat16_rn(v[u].y);
+          dst[2 * (size_t)p.kv_capacity] = __float2bfloat16_rn(v[u].z);
+          dst[3 * (size_t)p.kv_capacity] = __float2bfloat16_rn(v[u].w);
+        }
+      } else {
+        // rows of bf16 (or fp32) values; the K columns of a QKV projection belong to the cache
+        const bool k_tile = p.epilogue == EPI_QKV_SPLIT && n0 >= p.q_cols, f32 = p.epilogue == EPI_F32, gelu = p.epilogue == EPI_GELU_BF16;
+        const int ld = p.epilogue == EPI_QKV_SPLIT ? p.q_cols : p.N;
+#pragma unroll
+        for (int u = 0; u < PRE; ++u) {
+          int lrow, quad;
+          place(i0 + u, lrow, quad);
+          const int row = m0 + (int)rank * ROWS_PER + lrow, col = n0 + 4 * quad;
+          if (row >= p.M || col >= p.N) continue;
+          if (gelu) { v[u].x = gelu_tanh_fast(v[u].x); v[u].y = gelu_tanh_fast(v[u].y); v[u].z = gelu_tanh_fast(v[u].z); v[u].w = gelu_tanh_fast(v[u].w); }
+          if (f32) {
+            *reinterpret_cast<float4*>(static_cast<float*>(p.out) + (size_t)row * ld + col) = v[u];
+            continue;
+          }
+          __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.out) + (size_t)row * ld + col;
+          if (k_tile) {
+            const int img = row / p.rows_per_image, jrow = row - img * p.rows_per_image;
+            dst = p.k_cache + ((size_t)img * p.kv_capacity + p.kv_offset + jrow) * p.C + (col - p.q_cols);
+          }
+          *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(v[u].x, v[u].y), pack_bf16x2(v[u].z, v[u].w));
+        }
+      }
     }
   }
   __syncthreads();
