@@ -68,6 +68,7 @@ cudaError_t g_init_err = cudaSuccess;
 cudaError_t ensure_init() {
   std::call_once(g_init_once, [] {
     g_init_err = select_init();
+    if (g_init_err == cudaSuccess) g_init_err = select_small_init();
     if (g_init_err == cudaSuccess) g_init_err = rows_init();
     if (g_init_err == cudaSuccess) g_init_err = gemm_init();
     if (g_init_err == cudaSuccess) g_init_err = attention_init();
@@ -589,14 +590,17 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
   // kernel of the sublayer before it; only the first sublayer of a step has to sum the map itself.
   bool have_partials = false;
   const bool selecting = sub_pruned && !forced_idx_dev;
-  if (selecting && cudaMemsetAsync(ctx->sel_ws, 0, select_ticket_bytes(B), st) != cudaSuccess) return FV_ERR_CUDA;
   // Optional (fv_step_fused_selection): free-running selections take one launch each -- the previous sublayer's
   // kept-row restoration, the selection and the gather + LayerNorm of the newly kept rows (select_fused_kernel).  The
   // kept rows of a sublayer are then restored by the NEXT sublayer's launch; only the last sublayer of the step
   // restores its own.
   const bool fused = selecting && g_step_fused && !xb && select_fused_supported(B, n, C);
-  bool pending = false;                 // a kept-row restoration waits for the next fused selection
+  // Small maps: one launch between two branches (select_small.cu); the last sublayer's restoration is a launch of its own.
+  const bool small = selecting && !fused && c.interp_mode == 0 && select_small_supported(B, n, C, xb);
+  if (selecting && !small && cudaMemsetAsync(ctx->sel_ws, 0, select_ticket_bytes(B), st) != cudaSuccess) return FV_ERR_CUDA;
+  bool pending = false;                 // a restoration waits for the next selection's launch (fused: of the kept rows)
   const float* pending_gamma = nullptr;
+  const char* pending_cache = nullptr;
   int flip = 0;
 
   // A failed launch between the fork to the side stream and the join must not leave the side stream's part of the
@@ -620,12 +624,12 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
         if (forced_idx_dev) {
           idx = forced_idx_dev + trace_off;
           e = launch_inv_from_idx(idx, B, k, n, ctx->inv, st);
-        } else if (!fused) {
+        } else if (!fused && !small) {
           idx = ctx->idx;
           e = launch_select(x, B, n, C, k, ctx->idx, ctx->inv, nullptr, nullptr, ctx->sel_ws, have_partials, st, xb);
         }
         if (e != cudaSuccess) { s = FV_ERR_CUDA; break; }
-        if (!fused && idx_trace_dev && cudaMemcpyAsync(idx_trace_dev + trace_off, idx, (size_t)B * k * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+        if (!fused && !small && idx_trace_dev && cudaMemcpyAsync(idx_trace_dev + trace_off, idx, (size_t)B * k * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
           s = FV_ERR_CUDA; break;
         }
       }
@@ -659,7 +663,21 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
           s = FV_ERR_CUDA; break;
         }
       }
-      if (sub_pruned) {
+      if (small) {
+        SmallSelect f{};
+        int32_t* idx_cur = flip ? ctx->idx2 : ctx->idx;
+        inv_cur = flip ? ctx->inv2 : ctx->inv;
+        f.x = x; f.x_bf16 = xb; f.B = B; f.n = n; f.C = C; f.k = k; f.h = h; f.w = w; f.hc = hc; f.wc = wc; f.mod_stride = mod_stride;
+        if (pending) { f.y = ctx->y_buf; f.cache = pending_cache; f.inv_prev = flip ? ctx->inv : ctx->inv2; f.gamma_prev = pending_gamma; }
+        f.idx = idx_cur; f.inv = inv_cur; f.sigma = sigma; f.beta = beta; f.a_out = ctx->a_buf;
+        if (launch_select_small(f, st) != cudaSuccess) { s = FV_ERR_CUDA; break; }
+        pending = false;
+        idx = idx_cur;
+        flip ^= 1;
+        if (idx_trace_dev && cudaMemcpyAsync(idx_trace_dev + trace_off, idx, (size_t)B * k * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
+          s = FV_ERR_CUDA; break;
+        }
+      } else if (sub_pruned) {
         // Cached Token Restoration of the rows that were NOT kept needs only the selection and the cache:
         // it runs on the side stream while the gather and the branch below work on the kept rows (the two
         // touch disjoint rows of x).
@@ -670,7 +688,7 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
         forked = e_join == cudaSuccess;
         if (e != cudaSuccess || e_join != cudaSuccess) { s = FV_ERR_CUDA; break; }
       }
-      if (!fused) {
+      if (!fused && !small) {
         e = launch_gather_ln(xr, idx, B, nr, k, C, sigma, beta, mod_stride, ctx->a_buf, ctx->status, st, xb);
         if (e != cudaSuccess) { s = FV_ERR_CUDA; break; }
       }
@@ -720,9 +738,15 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
         o.epilogue = EPI_BF16; o.out = ctx->y_buf;
         s = launch_gemm(o, st);
         if (s != FV_OK) break;
-        if (fused && more) {     // the next sublayer's launch restores these kept rows
+        if ((fused || small) && more) {     // the next sublayer's launch restores these kept rows (small: all rows)
           pending = true;
           pending_gamma = gamma;
+          pending_cache = cache_sub;
+          continue;
+        }
+        if (small) {
+          if (launch_restore_residual(x, ctx->y_buf, cache_sub, inv_cur, gamma, mod_stride, B, k, h, w, hc, wc, C, nullptr, 0, c.interp_mode, st, xb) != cudaSuccess)
+            s = FV_ERR_CUDA;
           continue;
         }
         if (cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess) { s = FV_ERR_CUDA; break; }

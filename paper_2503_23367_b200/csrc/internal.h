@@ -125,6 +125,17 @@ cudaError_t launch_inv_from_idx(const int32_t* idx, int B, int k, int n, int32_t
 cudaError_t launch_inv_fill(int B, int n, int32_t* inv, cudaStream_t st);  // every token unkept (-1)
 cudaError_t select_init();  // one-time function attributes
 
+// ---- select_small.cu : restoration of the previous sublayer + selection + gather and LayerNorm, small maps, nearest interpolation
+struct SmallSelect {
+  void* x; bool x_bf16; int B, n, C, k, h, w, hc, wc, mod_stride;
+  const void* y; const void* cache; const int32_t* inv_prev; const float* gamma_prev;   // the previous sublayer's; y null: nothing to restore
+  int32_t* idx; int32_t* inv;                                                           // written (inv is not inv_prev)
+  const float* sigma; const float* beta; void* a_out;
+};
+cudaError_t select_small_init();
+bool select_small_supported(int B, int n, int C, bool x_bf16);
+cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st);
+
 // ---- rows.cu : gather + LayerNorm + modulate, restore (+ gate and residual) ----------------------
 // status (all gathers): device status word that receives DEV_BAD_ROW_INDEX when an index lies outside [0, n) (the
 // index is clamped, so the read stays inside the map), or null.

@@ -259,6 +259,44 @@ def test_every_selection_of_a_step_on_bit_identical_input(h, w, hc, wc, C, H, B,
     ctx.close()
 
 
+# Maps small enough for the one-launch form (a cluster of CTAs per image): one row per CTA, CTAs without a row, ragged last CTA, clusters
+# of 16 and (eight images) of 8, one and two chunks of rows per thread, channel groups that are not whole warps.
+SMALL_MAPS = [(1, 3, 1, 1, 128, 2, 2, 2, 0.5, "iid"), (5, 7, 3, 3, 256, 4, 3, 4, 0.3, "iid"), (16, 16, 10, 10, 1024, 16, 1, 1, 0.5, "structured"),
+              (13, 13, 10, 10, 1024, 16, 8, 8, 0.6, "structured"), (18, 18, 13, 13, 1920, 30, 2, 3, 0.75, "structured"), (24, 24, 9, 13, 256, 4, 2, 2, 0.15, "iid"),
+              (12, 12, 8, 8, 2048, 16, 2, 2, 0.6, "structured"), (20, 28, 13, 13, 384, 6, 1, 1, 0.9, "iid")]
+
+
+@pytest.mark.parametrize("h,w,hc,wc,C,H,B,B_max,keep,kind", SMALL_MAPS)
+def test_every_selection_on_small_maps(h, w, hc, wc, C, H, B, B_max, keep, kind):
+    test_every_selection_of_a_step_on_bit_identical_input(h, w, hc, wc, C, H, B, B_max, keep, kind, False, 0)
+
+
+@pytest.mark.parametrize("resid_dtype", [0, 1])
+@pytest.mark.parametrize("h,w,hc,wc,C,H,B,B_max,keep,kind", SMALL_MAPS)
+def test_small_map_step_equals_the_separate_kernels(h, w, hc, wc, C, H, B, B_max, keep, kind, resid_dtype):
+    """A free-running pruned step on a small map against the same step with its own kept sets forced, which runs the separate
+    inverse-map, gather and restoration kernels: the arithmetic on every element is the same, so the maps are, bit for bit."""
+    wl = I.Workload("small", L=2, C=C, H=H, B=B_max, sides=(hc, h), keep=(1.0, keep), cross_len=64, mlp_ratio=2, seed=812)
+    mt = I.model_tensors(wl)
+    k = O.kept_count(keep, h, w)
+    ctx = fv.FvContext(wl.L, C, H, [(hc, wc), (h, w)], 0, B_max, k, mt, cross_len=64, mlp_ratio=2, device=DEV, resid_dtype=resid_dtype)
+    for l in range(wl.L):
+        for si in range(3):
+            c = ctx.cache_view(l, si)
+            c.copy_(_bf16_t(I.normal_bf16(820 + 3 * l + si, tuple(c.shape))))
+    ctx.prepare_text(B)
+    x = torch.from_numpy(I.token_map(830, B, h, w, C, kind)).to(DEV).to(ctx.x_dtype)
+    trace = torch.full((wl.L, 3, B, k), -1, dtype=torch.int32, device=DEV)
+    outs = []
+    for forced in (None, None, trace):
+        ctx.set_state(1, 0)
+        outs.append(ctx.var_step(x, 1, keep, forced_idx=forced, idx_trace=trace if forced is None else None).clone())
+    assert ctx.device_status() == 0
+    assert torch.equal(outs[0], outs[1])
+    assert torch.equal(outs[0], outs[2])
+    ctx.close()
+
+
 def test_free_running_selection_matches_oracle_on_identical_input():
     wl = I.WORKLOADS["tiny"]
     mt = I.model_tensors(wl)
