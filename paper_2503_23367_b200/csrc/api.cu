@@ -68,7 +68,6 @@ cudaError_t g_init_err = cudaSuccess;
 cudaError_t ensure_init() {
   std::call_once(g_init_once, [] {
     g_init_err = select_init();
-    if (g_init_err == cudaSuccess) g_init_err = select_small_init();
     if (g_init_err == cudaSuccess) g_init_err = rows_init();
     if (g_init_err == cudaSuccess) g_init_err = gemm_init();
     if (g_init_err == cudaSuccess) g_init_err = attention_init();
@@ -175,8 +174,6 @@ fv_status fv_prune_select(const float* x_dev, int32_t B, int32_t h, int32_t w, i
   const int k = fv_k_for(keep_ratio, h, w);
   if (k_out_host) *k_out_host = k;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // the arrival counters at the head of the workspace must start at zero
-  if (cudaMemsetAsync(workspace_dev, 0, select_ticket_bytes(B), st) != cudaSuccess) return FV_ERR_CUDA;
   return cuda_status(launch_select(x_dev, B, (int)n, C, k, idx_out_dev, inv_out_dev, score_out_dev, near_tie_dev,
                                    workspace_dev, false, st));
 }
@@ -576,7 +573,6 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
       e = launch_inv_from_idx(forced_idx_dev, B, k, n, ctx->inv, st);
     } else {
       idx = ctx->idx;
-      if (cudaMemsetAsync(ctx->sel_ws, 0, select_ticket_bytes(B), st) != cudaSuccess) return FV_ERR_CUDA;
       e = launch_select(tokens_dev, B, n, C, k, ctx->idx, ctx->inv, nullptr, nullptr, ctx->sel_ws, false, st);
     }
     if (e != cudaSuccess) return FV_ERR_CUDA;

@@ -19,12 +19,16 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 }  // namespace fv
 #include <cuda_bf16.h>
 namespace fv {
-// Four / eight consecutive elements of the residual stream, fp32 or bf16, as floats.  NC: read-only path, else through L2.
-template <bool NC> __device__ __forceinline__ float4 x_load4(const float* p) {
-  return NC ? __ldg(reinterpret_cast<const float4*>(p)) : __ldcg(reinterpret_cast<const float4*>(p));
+// Four / eight consecutive elements of the residual stream, fp32 or bf16, as floats.  x_load4 reads through L2 and stays where it
+// is written: a plain read-only load may be moved up across the dependency wait by the compiler when its address allows it.
+__device__ __forceinline__ float4 x_load4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.cg.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+  return v;
 }
-template <bool NC> __device__ __forceinline__ float4 x_load4(const __nv_bfloat16* p) {
-  const uint2 u = NC ? __ldg(reinterpret_cast<const uint2*>(p)) : __ldcg(reinterpret_cast<const uint2*>(p));
+__device__ __forceinline__ float4 x_load4(const __nv_bfloat16* p) {
+  uint2 u;
+  asm volatile("ld.global.cg.v2.u32 {%0,%1}, [%2];" : "=r"(u.x), "=r"(u.y) : "l"(p) : "memory");
   return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
 }
 __device__ __forceinline__ void x_load8(const float* p, float (&f)[8]) {
@@ -95,7 +99,7 @@ struct SelectWs {
   int nchunks, group, ngroups;
 };
 size_t select_workspace_bytes(int B, int n, int C);
-size_t select_ticket_bytes(int B);  // leading bytes of the workspace that must be zero before first use
+size_t select_ticket_bytes(int B);  // leading bytes of the workspace: must be zero before a restoration folds its sums there, or a selection with have_partials
 SelectWs select_ws_carve(void* workspace, int B, int n, int C);
 // Scores [B,n] (fp32), then exact per-image top-k -> idx [B,k] ascending, inv [B,n].  have_partials:
 // the group partials in the workspace already hold the column sums of x (left there by
@@ -129,8 +133,8 @@ cudaError_t select_init();  // one-time function attributes
 struct SmallSelect {
   void* x; bool x_bf16; int B, n, C, k, h, w, hc, wc, mod_stride;
   const void* y; const void* cache; const int32_t* inv_prev; const float* gamma_prev;   // the previous sublayer's; y null: nothing to restore
-  int32_t* idx; int32_t* inv;                                                           // written (inv is not inv_prev)
-  const float* sigma; const float* beta; void* a_out;
+  int32_t* idx; int32_t* inv; float* score;                                             // written (inv is not inv_prev; inv, score may be null)
+  const float* sigma; const float* beta; void* a_out;                                   // a_out null: no gather
 };
 cudaError_t select_small_init();
 bool select_small_supported(int B, int n, int C, bool x_bf16);

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) gather_ln_kernel(const XT* __restrict__ x
 #pragma unroll
     for (int i = 0; i < kMaxVec; ++i) {
       const int c4 = lane + 32 * i;
-      if (c4 < C4) v[i] = x_load4<true>(row + (size_t)c4 * 4);
+      if (c4 < C4) v[i] = x_load4(row + (size_t)c4 * 4);
     }
 #pragma unroll
     for (int i = 0; i < kMaxVec; ++i) {

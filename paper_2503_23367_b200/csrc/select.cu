@@ -1,8 +1,8 @@
 // Pivotal Token Selection (Sec. 3.3, Eq. 4-5, Algorithm 1 first routine) on sm_100a.
 //
-//   colsum_chunk_kernel : Eq. 4's sum over tokens, one partial per chunk of 32 tokens, folded into at most
-//                         16 group partials per image by the last CTA of each group (fixed order).  Skipped
-//                         when the previous restore kernel has already left the partials of its output.
+//   colsum_chunk_kernel : Eq. 4's sum over tokens, one partial per chunk of 32 tokens; colsum_fold_kernel folds them into at most
+//                         16 group partials per image (fixed order).  Both are skipped when the previous restore kernel
+//                         has already left the partials of its output.
 //   score_topk_kernel   : s[b,t] = sum_c (x[b,t,c] - mean[b,c])^2, one warp per token, the mean token
 //                         rebuilt from the group partials in shared memory; the last CTA of each image to
 //                         finish then runs the exact top-k of that image: radix select on the fp32 bit
@@ -27,33 +27,58 @@ constexpr int kTopkThreads = 512;      // the fused kernel of a scale step (a th
 constexpr int kTopkWarps = kTopkThreads / 32;
 constexpr size_t kTopkMaxSmem = (size_t)kTopkMaxTokens * 4;   // one key per token (consecutive lanes on consecutive tokens)
 
+// grid (chunks, B, ceil(C4 / 256)): a thread sums four channels over the 32 rows of a chunk, 16 rows in flight.
 template <typename XT>
-__global__ void __launch_bounds__(256) colsum_chunk_kernel(const XT* __restrict__ x, int n, int C4, int nchunks, int group,
-                                                           int ngroups, float4* __restrict__ chunk_partial,
-                                                           float4* __restrict__ group_partial, unsigned int* tickets) {
+__global__ void __launch_bounds__(256) colsum_chunk_kernel(const XT* __restrict__ x, int n, int C4, int nchunks, float4* __restrict__ chunk_partial) {
   pdl_trigger();
   pdl_wait();
-  const int b = blockIdx.y, chunk = blockIdx.x;
+  const int b = blockIdx.y, chunk = blockIdx.x, c4 = blockIdx.z * 256 + threadIdx.x;
+  if (c4 >= C4) return;
   const int r0 = chunk * kColsumRows;
   const int r1 = min(n, r0 + kColsumRows);
-  const XT* base = x + (size_t)b * n * C4 * 4;
-  for (int c4 = threadIdx.x; c4 < C4; c4 += blockDim.x) {
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    int r = r0;
-    for (; r + 8 <= r1; r += 8) {
-      float4 v[8];
+  const XT* base = x + ((size_t)b * n * C4 + c4) * 4;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  int r = r0;
+  for (; r + 16 <= r1; r += 16) {
+    float4 v[16];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = x_load4<true>(base + ((size_t)(r + i) * C4 + c4) * 4);
+    for (int i = 0; i < 16; ++i) v[i] = x_load4(base + (size_t)(r + i) * C4 * 4);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) { acc.x += v[i].x; acc.y += v[i].y; acc.z += v[i].z; acc.w += v[i].w; }
-    }
-    for (; r < r1; ++r) {
-      const float4 v = x_load4<true>(base + ((size_t)r * C4 + c4) * 4);
-      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-    }
-    chunk_partial[((size_t)b * nchunks + chunk) * C4 + c4] = acc;
+    for (int i = 0; i < 16; ++i) { acc.x += v[i].x; acc.y += v[i].y; acc.z += v[i].z; acc.w += v[i].w; }
   }
-  fold_group_partials(b, chunk, nchunks, group, ngroups, C4, chunk_partial, group_partial, tickets);
+  for (; r < r1; ++r) {
+    const float4 v = x_load4(base + (size_t)r * C4 * 4);
+    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+  }
+  chunk_partial[((size_t)b * nchunks + chunk) * C4 + c4] = acc;
+}
+
+// Chunk partials -> group partials, in chunk order: grid (groups, B, ceil(C4 / 64)), four threads per four channels taking the
+// chunks in turn would change the order of the additions, so one thread adds them all, 16 loads in flight.  A launch of its own
+// behind the streaming kernel: folding by the last CTA of a group to arrive needs zeroed counters (a memset before
+// every stand-alone selection) and puts a fence, an atomic and a reload at the end of every CTA.  It also zeroes the counters
+// and range words of the scoring kernel behind it.
+__global__ void __launch_bounds__(64) colsum_fold_kernel(const float4* chunk_partial, int C4, int nchunks, int group, int ngroups, float4* __restrict__ group_partial,
+                                                         unsigned int* tickets, int ticket_words) {
+  pdl_trigger();
+  pdl_wait();
+  const int g = blockIdx.x, b = blockIdx.y, c4 = blockIdx.z * 64 + threadIdx.x;
+  if (g == 0 && b == 0 && blockIdx.z == 0)
+    for (int i = threadIdx.x; i < ticket_words; i += 64) tickets[i] = 0u;
+  if (c4 >= C4) return;
+  const int first = g * group, last = min(nchunks, first + group);
+  const float4* src = chunk_partial + (size_t)b * nchunks * C4 + c4;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int c = first; c < last; c += 16) {
+    float4 v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (c + i < last) v[i] = src[(size_t)(c + i) * C4];
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (c + i < last) { acc.x += v[i].x; acc.y += v[i].y; acc.z += v[i].z; acc.w += v[i].w; }
+  }
+  group_partial[((size_t)b * ngroups + g) * C4 + c4] = acc;
 }
 
 // Exclusive prefix sum of one value per thread over the whole CTA (T threads, the template argument); returns the
@@ -148,24 +173,24 @@ __device__ __forceinline__ void mean_from_partials_halves(float4* s_mean, float4
 static_assert(kMaxGroups == 16, "mean_from_partials_halves splits the groups 8 + 8");
 
 // ---- Eq. 5 / Algorithm 1: squared deviation from the mean, one warp per token row; the warps of an image stride
-// over its rows.  NC: the map was not written by this kernel, so its rows may take the read-only path; the fused
-// kernel, whose other CTAs have just updated rows of it, reads them through L2.
+// over its rows.
 // BATCH: 16-byte loads a lane requests together (8 with 64 registers per thread, 16 with 128).
 // lo / hi: running smallest / largest score key (the bit pattern without its sign) of the rows this warp has scored.
 // inv (may be null): the inverse map of the image is set to "not kept" for every row scored here, so that the CTA
 // that ranks the image only has to write the entries of the kept rows (one SM stores slowly).
-template <int T, bool NC, int BATCH, typename XT>
+template <int T, int BATCH, typename XT>
 __device__ __forceinline__ void score_rows(const XT* x, const float4* s_mean, int b, int n, int C4, float* __restrict__ score,
                                            int32_t* __restrict__ inv, uint32_t& lo, uint32_t& hi) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int r = blockIdx.x * (T / 32) + warp; r < n; r += gridDim.x * (T / 32)) {
+  // from the last row to the first: the kernel before has walked the map upwards, its end is what L2 still holds
+  for (int r = n - 1 - ((int)blockIdx.x * (T / 32) + warp); r >= 0; r -= gridDim.x * (T / 32)) {
     const XT* row = x + ((size_t)b * n + r) * C4 * 4;
     float acc = 0.f;
     int c4 = lane;
     for (; c4 + 32 * (BATCH - 1) < C4; c4 += 32 * BATCH) {
       float4 v[BATCH];
 #pragma unroll
-      for (int i = 0; i < BATCH; ++i) v[i] = x_load4<NC>(row + (size_t)(c4 + 32 * i) * 4);
+      for (int i = 0; i < BATCH; ++i) v[i] = x_load4(row + (size_t)(c4 + 32 * i) * 4);
 #pragma unroll
       for (int i = 0; i < BATCH; ++i) {
         const float4 m = s_mean[c4 + 32 * i];
@@ -174,7 +199,7 @@ __device__ __forceinline__ void score_rows(const XT* x, const float4* s_mean, in
       }
     }
     for (; c4 < C4; c4 += 32) {
-      const float4 v = x_load4<NC>(row + (size_t)c4 * 4);
+      const float4 v = x_load4(row + (size_t)c4 * 4);
       const float4 m = s_mean[c4];
       const float dx = v.x - m.x, dy = v.y - m.y, dz = v.z - m.z, dw = v.w - m.w;
       acc += dx * dx; acc += dy * dy; acc += dz * dz; acc += dw * dw;
@@ -467,7 +492,7 @@ __global__ void __launch_bounds__(kSelectThreads, 1) score_topk_kernel(const XT*
   else mean_from_partials<kSelectThreads>(s_mean, group_partial + (size_t)b * ngroups * C4, ngroups, nullptr, 0, C4, n);   // very wide maps
   __syncthreads();
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-  score_rows<kSelectThreads, true, 8, XT>(x, s_mean, b, n, C4, score, inv, lo, hi);
+  score_rows<kSelectThreads, 8, XT>(x, s_mean, b, n, C4, score, inv, lo, hi);
   publish_range<kSelectThreads>(lo, hi, sh, img_range + 2 * b);
   __threadfence();  // this thread's scores (and range) are visible device-wide before the CTA takes its ticket
 
@@ -700,7 +725,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) select_fused_kernel(const Fus
                      a.y ? a.kept_group + (size_t)b * a.ngk * C4 : nullptr, a.y ? a.ngk : 0, C4, n);
   __syncthreads();
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-  score_rows<kTopkThreads, false, 16, float>(reinterpret_cast<const float*>(a.x), s_dyn, b, n, C4, a.score, a.inv, lo, hi);
+  score_rows<kTopkThreads, 16, float>(reinterpret_cast<const float*>(a.x), s_dyn, b, n, C4, a.score, a.inv, lo, hi);
   publish_range<kTopkThreads>(lo, hi, sh, a.img_range + 2 * b);
   __threadfence();
   __syncthreads();
@@ -810,6 +835,8 @@ cudaError_t select_init() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
+  e = select_small_init();
+  if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(score_topk_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTopkMaxSmem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(score_topk_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTopkMaxSmem);
   if (e != cudaSuccess) return e;
@@ -817,12 +844,21 @@ cudaError_t select_init() {
 }
 
 template <typename XT>
+static cudaError_t launch_colsum_t(const XT* x, int B, int n, int C, const SelectWs& w, cudaStream_t st) {
+  const int C4 = C / 4;
+  cudaError_t e = launch_pdl(colsum_chunk_kernel<XT>, dim3(w.nchunks, B, (C4 + 255) / 256), dim3(256), 0, st, x, n, C4, w.nchunks,
+                             reinterpret_cast<float4*>(w.chunk_partial));
+  if (e != cudaSuccess) return e;
+  return launch_pdl(colsum_fold_kernel, dim3(w.ngroups, B, (C4 + 63) / 64), dim3(64), 0, st, reinterpret_cast<const float4*>(w.chunk_partial), C4, w.nchunks,
+                    w.group, w.ngroups, reinterpret_cast<float4*>(w.group_partial), w.tickets, (int)(select_ticket_bytes(B) / sizeof(unsigned int)));
+}
+
+template <typename XT>
 static cudaError_t launch_select_t(const XT* x, int B, int n, int C, int k, int32_t* idx, int32_t* inv, float* sc, int32_t* near_tie,
                                    const SelectWs& w, bool have_partials, cudaStream_t st) {
   const int C4 = C / 4;
   if (!have_partials)
-    launch_pdl(colsum_chunk_kernel<XT>, dim3(w.nchunks, B), dim3(256), 0, st, x, n, C4, w.nchunks, w.group,
-               w.ngroups, reinterpret_cast<float4*>(w.chunk_partial), reinterpret_cast<float4*>(w.group_partial), w.tickets);
+    launch_colsum_t(x, B, n, C, w, st);
   const size_t keys_smem = ((size_t)n + 3) / 4 * 16;   // whole 16-byte words
   const int staged = (size_t)C * 4 * 9 <= kTopkMaxSmem;  // room for the mean token and eight staged partial sums
   const size_t mean_smem = (size_t)C * 4 * (staged ? 9 : 1);
@@ -842,12 +878,18 @@ static cudaError_t launch_select_t(const XT* x, int B, int n, int C, int k, int3
 
 cudaError_t launch_select(const void* x, int B, int n, int C, int k, int32_t* idx, int32_t* inv, float* score,
                           int32_t* near_tie, void* workspace, bool have_partials, cudaStream_t st, bool x_bf16) {
+  if (!have_partials && !near_tie && select_small_supported(B, n, C, x_bf16)) {   // one launch, no scratch
+    SmallSelect f{};
+    f.x = const_cast<void*>(x); f.x_bf16 = x_bf16; f.B = B; f.n = n; f.C = C; f.k = k; f.h = 1; f.w = n; f.hc = 1; f.wc = 1;
+    f.idx = idx; f.inv = inv; f.score = score;
+    return launch_select_small(f, st);
+  }
   const SelectWs w = select_ws_carve(workspace, B, n, C);
   float* sc = score ? score : w.score;
   const double es = x_bf16 ? 2.0 : 4.0;
   const double sel_bytes = (double)B * n * C * es + 4.0 * B * n + 4.0 * B * ((double)k + n);
   // the stand-alone column-sum pass reads the map a second time
-  LaunchScope scope(KC_SELECT, have_partials ? 1 : 2, sel_bytes, sel_bytes + (have_partials ? 0.0 : (double)B * n * C * es), st);
+  LaunchScope scope(KC_SELECT, have_partials ? 1 : 3, sel_bytes, sel_bytes + (have_partials ? 0.0 : (double)B * n * C * es), st);
   if (x_bf16) return launch_select_t(static_cast<const __nv_bfloat16*>(x), B, n, C, k, idx, inv, sc, near_tie, w, have_partials, st);
   return launch_select_t(static_cast<const float*>(x), B, n, C, k, idx, inv, sc, near_tie, w, have_partials, st);
 }
@@ -921,9 +963,8 @@ cudaError_t launch_select_fused(const FusedSelect& f, cudaStream_t st) {
 
 cudaError_t launch_colsum(const float* x, int B, int n, int C, void* workspace, cudaStream_t st) {
   const SelectWs w = select_ws_carve(workspace, B, n, C);
-  LaunchScope scope(KC_SELECT, 1, (double)B * n * C * 4.0, (double)B * n * C * 4.0, st);
-  return launch_pdl(colsum_chunk_kernel<float>, dim3(w.nchunks, B), dim3(256), 0, st, x, n, C / 4, w.nchunks, w.group,
-                    w.ngroups, reinterpret_cast<float4*>(w.chunk_partial), reinterpret_cast<float4*>(w.group_partial), w.tickets);
+  LaunchScope scope(KC_SELECT, 2, (double)B * n * C * 4.0, (double)B * n * C * 4.0, st);
+  return launch_colsum_t(x, B, n, C, w, st);
 }
 
 cudaError_t launch_inv_fill(int B, int n, int32_t* inv, cudaStream_t st) {

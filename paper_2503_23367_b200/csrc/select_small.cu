@@ -34,6 +34,7 @@ struct SmallArgs {
   const float* gamma_prev;
   int n, C, k, h, w, hc, wc, mod_stride;
   int32_t *idx, *inv;
+  float* score;                       // [B, n] or null
   const float *sigma, *beta;
   uint2* a_out;
   int rows_per_cta;                   // R
@@ -90,16 +91,6 @@ __device__ __forceinline__ void load_row8(const float* p, float (&f)[8]) {
   f[4] = __uint_as_float(b.x); f[5] = __uint_as_float(b.y); f[6] = __uint_as_float(b.z); f[7] = __uint_as_float(b.w);
 }
 __device__ __forceinline__ void load_row8(const __nv_bfloat16* p, float (&f)[8]) { unpack8(load16(p), f); }
-
-__device__ __forceinline__ float4 load_row4(const float* p) {
-  const uint4 a = load16(p);
-  return make_float4(__uint_as_float(a.x), __uint_as_float(a.y), __uint_as_float(a.z), __uint_as_float(a.w));
-}
-__device__ __forceinline__ float4 load_row4(const __nv_bfloat16* p) {
-  uint2 u;
-  asm volatile("ld.global.cg.v2.u32 {%0,%1}, [%2];" : "=r"(u.x), "=r"(u.y) : "l"(p) : "memory");
-  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
-}
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
@@ -269,6 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
       float sc = 0.f;
       for (int w = 0; w < WG; ++w) sc += red[tid * WG + w];
       s_score[q * chunk_rows + tid] = sc;
+      if (a.score) a.score[(size_t)b * n + r0 + q * chunk_rows + tid] = sc;
     }
     __syncthreads();
   }
@@ -310,10 +302,11 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
     if (lane == 0) {
       const int pos = flags[t] ? below : -1;
       s_pos[i] = pos;
-      a.inv[(size_t)b * n + t] = pos;
+      if (a.inv) a.inv[(size_t)b * n + t] = pos;
       if (pos >= 0) a.idx[(size_t)b * a.k + pos] = t;
     }
   }
+  if (!a.a_out) return;        // a selection alone
   __syncthreads();
 
   // ---- LayerNorm + modulation of the kept rows -> bf16 A operand; a warp per row, the arithmetic (and bits) of gather_ln_kernel
@@ -326,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
     float sum = 0.f;
 #pragma unroll
     for (int j = 0; j < kVec; ++j)
-      if (lane + 32 * j < C4) r[j] = load_row4(row + (size_t)(lane + 32 * j) * 4);
+      if (lane + 32 * j < C4) r[j] = x_load4(row + (size_t)(lane + 32 * j) * 4);
 #pragma unroll
     for (int j = 0; j < kVec; ++j)
       if (lane + 32 * j < C4) sum += (r[j].x + r[j].y) + (r[j].z + r[j].w);
@@ -367,7 +360,7 @@ template <typename XT> cudaError_t attr() {
 
 }  // namespace
 
-cudaError_t select_small_init() {
+static cudaError_t init_once() {
   cudaError_t e = attr<float>();
   if (e == cudaSuccess) e = attr<__nv_bfloat16>();
   if (e != cudaSuccess) return e;
@@ -381,6 +374,10 @@ cudaError_t select_small_init() {
   if (cudaOccupancyMaxActiveClusters(&clusters, select_small_kernel<float>, &cfg) == cudaSuccess) g_clusters16 = clusters;
   else (void)cudaGetLastError();
   return cudaSuccess;
+}
+cudaError_t select_small_init() {
+  static const cudaError_t e = init_once();
+  return e;
 }
 
 // CTAs per image, or 0: the map is not for this kernel.  16 while the GPU holds a cluster of them per image, else 8.  A CTA works
@@ -403,11 +400,11 @@ cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st) {
   SmallArgs a{};
   a.x = f.x; a.y = static_cast<const uint4*>(f.y); a.cache = static_cast<const uint4*>(f.cache); a.inv_prev = f.inv_prev; a.gamma_prev = f.gamma_prev;
   a.n = f.n; a.C = f.C; a.k = f.k; a.h = f.h; a.w = f.w; a.hc = f.hc; a.wc = f.wc; a.mod_stride = f.mod_stride;
-  a.idx = f.idx; a.inv = f.inv; a.sigma = f.sigma; a.beta = f.beta; a.a_out = static_cast<uint2*>(f.a_out);
+  a.idx = f.idx; a.inv = f.inv; a.score = f.score; a.sigma = f.sigma; a.beta = f.beta; a.a_out = static_cast<uint2*>(f.a_out);
   a.rows_per_cta = (f.n + cl - 1) / cl;
   // algorithmic bytes: the map read (and written where it is restored from y and the cache), indices, the kept rows' bf16 copy
   const double es = f.x_bf16 ? 2.0 : 4.0;
-  const double bytes = (double)f.B * f.C * (f.n * es * (f.y ? 2.0 : 1.0) + (f.y ? 2.0 * f.k + 2.0 * f.hc * f.wc : 0.0) + 2.0 * f.k) + 4.0 * f.B * ((double)f.k + f.n);
+  const double bytes = (double)f.B * f.C * (f.n * es * (f.y ? 2.0 : 1.0) + (f.y ? 2.0 * f.k + 2.0 * f.hc * f.wc : 0.0) + (f.a_out ? 2.0 * f.k : 0.0)) + 4.0 * f.B * ((double)f.k + f.n);
   LaunchScope scope(KC_SELECT, 1, bytes, bytes, st);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(cl, f.B); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = (size_t)small_smem(f.n, f.C, a.rows_per_cta).total * 4; cfg.stream = st;

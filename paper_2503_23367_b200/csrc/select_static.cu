@@ -63,11 +63,9 @@ fv_status fv_prune_select_static(const float* x_dev, int32_t B, int32_t h, int32
   if (scratch_address(&scratch) != cudaSuccess) return FV_ERR_CUDA;
   const int k = fv_k_for(keep_ratio, h, w);
   if (k_out_host) *k_out_host = k;
-  // Of the scratch only the arrival counters at its head have to start at zero; they are cleared here on
-  // every call (a memset node on the stream, no allocation).  Every other word the kernels read
-  // (partial sums, scores) is written earlier in the same call, so the previous call's leftovers are harmless.
+  // Every word of the scratch that the kernels read (partial sums, counters, scores) is written earlier in the same call, so the
+  // previous call's leftovers are harmless.
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(scratch, 0, fv::select_ticket_bytes(B), st) != cudaSuccess) return FV_ERR_CUDA;
   cudaError_t e = fv::launch_select(x_dev, B, (int)n, C, k, idx_out_dev, inv_out_dev, score_out_dev, near_tie_dev, scratch,
                                     false, st);
   return e == cudaSuccess ? FV_OK : FV_ERR_CUDA;

@@ -112,6 +112,24 @@ def test_prune_select_scores_crowded_at_the_threshold(crowd, levels, keep):
     assert np.array_equal(r["inv"].cpu().numpy().astype(np.int64), O.inverse_map(idx_g, n))
 
 
+@pytest.mark.parametrize("B,h,w,C,keep,kind", [(1, 1, 1, 128, 1.0, "iid"), (3, 13, 18, 1920, 0.6, "structured"), (8, 16, 16, 1024, 0.5, "iid"), (20, 8, 9, 256, 0.3, "iid"),
+                                               (2, 25, 25, 256, 0.1, "structured"), (1, 16, 15, 2048, 0.999, "iid")])
+def test_prune_select_small_maps_in_one_launch(B, h, w, C, keep, kind):
+    """Without a near-tie count small maps are ranked by a cluster of CTAs per image: exact given its own scores, ties (rows repeated
+    in bulk) to the lowest index, the inverse map complete; more images than clusters of 16 fit as well."""
+    x = I.token_map(177 + B + h, B, h, w, C, kind)
+    for repeat in (False, True):
+        if repeat:
+            x = x[:, (np.arange(h * w) * 7919) % max(1, h * w // 5)]
+        r = fv.fv_prune_select(dev(x), h, w, keep, want_inv=True, want_score=True)
+        torch.cuda.synchronize()
+        score_g = r["score"].cpu().numpy()
+        idx_g = r["idx"].cpu().numpy().astype(np.int64)
+        np.testing.assert_allclose(score_g, O.pts_score(x), rtol=2e-5, atol=1e-4)
+        assert np.array_equal(idx_g, O.pts_topk(score_g, r["k"]))
+        assert np.array_equal(r["inv"].cpu().numpy().astype(np.int64), O.inverse_map(idx_g, h * w))
+
+
 def test_prune_select_argument_errors():
     big = torch.zeros((1, 193 * 256, 8), device=DEV)                      # one row of tokens beyond the largest map
     with pytest.raises(fv.FvError) as e:
