@@ -523,20 +523,21 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
   p.rope_table = qk_extras ? reinterpret_cast<const float2*>(g.rope_table) : nullptr;
   p.rope_idx = qk_extras ? g.rope_idx : nullptr;
   p.head_dim = g.head_dim;
-  // K split over the CTAs of a cluster, the partials reduced through distributed shared memory.  Up to 32 rows two CTAs
-  // share an SM and 64-wide tiles are the best everywhere: 4 slices while the CTAs stay near one per SM, else 2 (us at M 8, weights
-  // from HBM, 64 x 4 / 64 x 2 / 128 x 4 / 128 x 2: N 2048 K 2048 4.8 / 5.3 / 5.8 / 7.4; N 6144 10.1 / 8.3 / 8.2 / 9.5;
-  // N 8192 12.0 / 9.1 / 8.9 / 10.5; N 2048 K 8192 10.1 / 14.1 / 14.7 / 23.3; 1024-wide models N 3072 4.1 / 4.2 / 4.7 / 4.9).
+  // K split over the CTAs of a cluster, the partials reduced through distributed shared memory.  Up to 48 rows two CTAs
+  // share an SM (gemm_cluster.cu): 8 slices while the CTAs stay within one per SM, else 4 within two, else 2 (us at M 8, weights from HBM,
+  // 8 / 4 / 2 slices: N 2048 K 2048 3.9 / 4.6 / 6.4; N 6144 9.1 / 6.7 / 8.0; N 8192 10.1 / 7.6 / 8.9; N 2048 K 8192 9.0 / 11.9 / 20;
+  // 1024-wide models N 3072 3.7 / 3.6 / 4.2; N 1024 K 4096 4.6 / 6.4 / 10.3).  From 64 rows on the other tiles are as fast or faster.
   int cluster_slices = 0, cluster_bn = 0;
   if (g_force_path == 0 && !qk_extras) {
-    const long t64 = (g.N + 63) / 64;
-    if (g.M <= 32 && g.K > 7 * BK && t64 <= g_num_sms) { cluster_bn = 64; cluster_slices = t64 * 3 <= g_num_sms ? 4 : 2; }
+    const long t128 = (g.N + 127) / 128;
+    if (g.M <= 48 && g.K > 7 * BK && t128 <= g_num_sms) { cluster_bn = 128; cluster_slices = t128 * 8 <= g_num_sms ? 8 : (t128 * 4 <= 2 * g_num_sms ? 4 : 2); }
     else if (picked.slices > 1) { cluster_bn = picked.bn; cluster_slices = picked.slices; }
   }
   if (g_force_path >= 8 && g_force_path <= 11 && !qk_extras) {   // 8: 128 wide x 4 slices, 9: 128 x 2, 10: 64 x 4, 11: 64 x 2
     cluster_bn = g_force_path <= 9 ? 128 : 64;
     cluster_slices = (g_force_path & 1) ? 2 : 4;
   }
+  if (g_force_path == 12 && !qk_extras && g.M <= 48) { cluster_bn = 128; cluster_slices = 8; }   // (few rows only)
   if (cluster_slices) {
     const int num_kb = (g.K + BK - 1) / BK;
     p.splits = 1; p.sk_partial = nullptr; p.sk_tickets = nullptr;

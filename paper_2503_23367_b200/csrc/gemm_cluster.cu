@@ -26,50 +26,61 @@ constexpr int BM = 128;
 constexpr int BK = 64;
 constexpr int kThreads = 192;
 
-// AROWS: rows of A that are actually loaded per k-block (32 when the GEMM has at most 32 rows, else 128).  The
-// MMA always reads a 128-row A tile from shared memory; with AROWS = 32 the rows beyond the 4 KB that were
-// loaded are whatever follows in shared memory (the stage's own W tile, the next stage, the buffers behind the
-// ring -- all inside the allocation).  They only feed accumulator rows >= 32, which belong to no row of the
-// output and are neither reduced nor stored.
-// The small-row builds stay under 113 KB of shared memory, ring and reduce buffer together, so that TWO CTAs share an SM:
+// Up to 48 rows (FLIP) the operands change places: 128 rows of W are the M side of the MMA and the ROWS rows of A its N side, so the
+// accumulator is the tile transposed.  An MMA reads its M operand whole, 128 rows of it, whatever the GEMM's own rows: with A there, 64-wide
+// tiles cost 64 clocks per 16 of K, most of them for rows that do not exist, and the MMAs of a slice were the longest part of a launch
+// (M 4, K 4096 in four slices: 4500 of 7000 clocks).  Us per launch of a chain, weights from HBM, before -> after: M 4 N 6144 K 2048
+// 8.3 -> 6.6 (the weights alone take 3.8), N 2048 K 2048 4.5 -> 3.8, N 8192 K 2048 9.0 -> 7.4, N 2048 K 8192 9.9 -> 9.0; M 32 7.8 -> 6.9,
+// 4.8 -> 4.5, 8.8 -> 7.8, 10.3 -> 9.7; 1024-wide models M 25 4.1 -> 3.9, 3.4 -> 3.4, 4.7 -> 4.4, 5.4 -> 4.9.  At 64 rows the two are even:
+// the transposed accumulator goes to its owners one word per lane and row.  (Reducing and finishing it four rows at a time,
+// in wide words, costs more in the epilogue than it saves there: M 32 N 6144 6.9 -> 7.3.)
+//
+// The builds for few rows stay under 113 KB of shared memory, ring and reduce buffer together, so that TWO CTAs share an SM:
 // the CTAs of the next GEMM of the step start (programmatic launch) beside those of this one and fetch their first
-// 64 KB of weights while this one computes, and outputs of up to 8192 columns fit the GPU as 64-wide tiles.  Launches of a chain
-// (M 8, weights from HBM): N 2048 K 2048 5.4 -> 4.8 us, N 6144 8.7 -> 8.3, N 8192 9.6 -> 9.1, N 2048 K 8192 11.5 -> 10.1.
+// weights while this one computes, and outputs of up to 8192 columns fit the GPU in four slices.
 //
 // kKps: k-blocks per pipeline stage.  Producer and MMA issuer pay a fixed price per stage (a barrier's wait, a commit or an
-// expect) that exceeds the time of one k-block's MMAs: with two k-blocks behind one barrier it is paid half as often.
-// Where the ring would shrink to two stages (128 rows of A against 128-wide tiles) one k-block per stage stays.
-template <int BN, int AROWS> struct ClusterCfg {
-  static constexpr int kKps = (AROWS == 128 && BN == 128) ? 1 : 2;
-  static constexpr int kATile = AROWS * BK * 2;
+// expect) that exceeds the time of one k-block's MMAs of a 64-wide tile: with two k-blocks behind one barrier it is paid half as
+// often.  128-wide tiles keep one (two cost a stage of ring: M 32 N 2048 K 8192 9.7 -> 10.3).
+constexpr int kFlipRows = 48;   // most rows of the builds with W on the M side
+template <int BN, int ROWS> struct ClusterCfg {
+  static constexpr bool kFlip = ROWS < 128;
+  static constexpr int kKps = BN == 128 ? 1 : 2;
+  static constexpr int kATile = ROWS * BK * 2;
   static constexpr int kBTileBytes = BN * BK * 2;
   static constexpr int kSubBytes = kATile + kBTileBytes;       // one k-block: A tile, then W tile
   static constexpr int kStageBytes = kKps * kSubBytes;
-  static constexpr int kStages = AROWS == 32 ? ((BN == 128) ? 2 : 4) : ((BN == 128) ? 4 : 3);
-  static constexpr int kTmemCols = BN;                      // one accumulator (64 or 128: powers of two)
+  static constexpr int kStages = kFlip ? (ROWS == 32 ? 4 : 3) : (BN == 128 ? 4 : 3);
+  static constexpr int kTmemCols = kFlip ? ROWS : BN;       // one accumulator (powers of two)
   static constexpr int kRedPitch = BN + 4;                  // floats per row of the reduce buffer (bank spread)
-  static constexpr int kRedBytes = AROWS * kRedPitch * 4;   // [S sources][AROWS/S rows][pitch] = AROWS rows in all
+  static constexpr int kRedBytes = ROWS * kRedPitch * 4;    // [S sources][ROWS/S rows][pitch] = ROWS rows in all
   // operand stages | per-warp bias slices | barriers | reduce buffer
   static constexpr int kSmemBytes = kStages * kStageBytes + kBiasSmemBytes + 256 + kRedBytes + 1024 /*alignment slack*/;
+  static_assert(!kFlip || (BN == 128 && kSmemBytes <= 113 * 1024), "two CTAs per SM");
 };
 
-__device__ __forceinline__ uint32_t map_to_cta(const void* p, uint32_t cta) {
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t local, uint32_t cta) {
   uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(p)), "r"(cta));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(cta));
   return remote;
 }
 __device__ __forceinline__ void st_cluster_f4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
-template <int BN, int S, int AROWS>
+__device__ __forceinline__ void st_cluster_f1(uint32_t addr, uint32_t a) {
+  asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(a) : "memory");
+}
+
+template <int BN, int S, int ROWS>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmDev p) {
-  using Cfg = ClusterCfg<BN, AROWS>;
+  using Cfg = ClusterCfg<BN, ROWS>;
+  constexpr bool FLIP = Cfg::kFlip;
   constexpr int kATileBytes = Cfg::kATile;
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;
-  constexpr int ROWS_PER = AROWS / S;     // rows of the tile each CTA finishes
+  constexpr int ROWS_PER = ROWS / S;      // rows of the tile each CTA finishes
   // The CTA finishes ROWS_PER x BN values, four consecutive columns per epilogue thread and turn: lanes along the columns, so that a
   // warp stores whole lines; along the rows where the columns are V's (its cache is transposed: a key's neighbours are rows).
   // What a residual stream or gate contributes does not depend on the product and is fetched before the barriers, up to PRE turns
@@ -167,7 +178,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   } else if (warp == 1) {
     pdl_wait();
     {
-      constexpr uint32_t idesc = umma_idesc_bf16(BM, BN);
+      constexpr uint32_t idesc = FLIP ? umma_idesc_bf16(BN, ROWS) : umma_idesc_bf16(BM, BN);
       const bool leader = elect_one();
       uint32_t s = 0, ph = 0;   // ring stage and its phase
       bool ok = true;
@@ -182,7 +193,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             const uint64_t adesc = desc + u * (Cfg::kSubBytes >> 4), bdesc = adesc + (kATileBytes >> 4);
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
-              umma_bf16(tmem_base, adesc + 2 * kk, bdesc + 2 * kk, idesc, (it | u | kk) != 0);
+              umma_bf16(tmem_base, (FLIP ? bdesc : adesc) + 2 * kk, (FLIP ? adesc : bdesc) + 2 * kk, idesc, (it | u | kk) != 0);
           }
           umma_commit(&empty_bar[s]);
         }
@@ -191,7 +202,7 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       if (ok && leader && kb1 > kb0) umma_commit(acc_full);
     }
   } else {
-    // ---- accumulator readers: thread = one accumulator row; its partial goes to the CTA that owns the row ----
+    // ---- accumulator readers: thread = one row of the tile (FLIP: one column); a row's partial goes to the CTA that owns the row ----
     stage_bias(p, bias_s + (warp & 3) * 32, lane, n0, BN);
     pdl_wait();
     if (x_f32 || x_b16) {
@@ -199,18 +210,15 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       for (int i = 0; i < PRE; ++i) fetch(i, i);
     }
     const int quarter = warp & 3;
-    const int trow = quarter * 32 + lane;                 // row inside the tile
-    const uint32_t owner = (uint32_t)min(trow / ROWS_PER, S - 1);   // (rows past AROWS belong to no row of the output)
-    const int lrow = trow - (int)owner * ROWS_PER;
     bool have = kb1 > kb0;
     if (have && !mbar_wait(acc_full, 0)) { report(p.status, DEV_TIMEOUT_EPI); have = false; }
     have = __all_sync(0xffffffffu, have);   // the TMEM loads below are warp-wide
     tc_fence_after();
     cluster_wait();                         // every CTA of the cluster is running: its shared memory may be written
-    const uint32_t dst = map_to_cta(red + ((size_t)rank * ROWS_PER + lrow) * Cfg::kRedPitch, owner);
     const uint32_t t0 = tmem_base + (uint32_t(quarter * 32) << 16);
+    const int t = quarter * 32 + lane;      // accumulator lane
 #pragma unroll 1
-    for (int c0 = 0; c0 < (AROWS == 128 || quarter == 0 ? BN : 0); c0 += 32) {
+    for (int c0 = 0; c0 < (FLIP ? min(ROWS, p.M) : BN); c0 += 32) {
       uint32_t r[32];
       if (have) {            // uniform over the warp
         tmem_ld32(t0 + c0, r);
@@ -219,9 +227,17 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
         for (int i = 0; i < 32; ++i) r[i] = 0u;   // a slice without k-blocks (or an expired wait) adds nothing
       }
-      if (m0 + trow < p.M) {
+      if constexpr (FLIP) {  // rows c0 .. c0 + 31 of column t: a warp stores 32 consecutive columns of a row at a time
+        const uint32_t local = smem_u32(red + (size_t)rank * ROWS_PER * Cfg::kRedPitch + t);
 #pragma unroll
-        for (int g = 0; g < 8; ++g) st_cluster_f4(dst + (c0 + 4 * g) * 4, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+        for (int i = 0; i < 32; ++i) {
+          const int row = c0 + i;
+          if (row < p.M) st_cluster_f1(map_to_cta(local + (row % ROWS_PER) * (Cfg::kRedPitch * 4), row / ROWS_PER), r[i]);
+        }
+      } else if (m0 + t < p.M) {
+        const uint32_t dst = map_to_cta(smem_u32(red + ((size_t)rank * ROWS_PER + t % ROWS_PER) * Cfg::kRedPitch + c0), t / ROWS_PER);
+#pragma unroll
+        for (int g = 0; g < 8; ++g) st_cluster_f4(dst + 16 * g, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
       }
     }
     tc_fence_before();
@@ -318,24 +334,24 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   }
 }
 
-template <int BN, int S, int AROWS> cudaError_t set_attr() {
-  return cudaFuncSetAttribute(gemm_cluster_kernel<BN, S, AROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClusterCfg<BN, AROWS>::kSmemBytes);
+template <int BN, int S, int ROWS> cudaError_t set_attr() {
+  return cudaFuncSetAttribute(gemm_cluster_kernel<BN, S, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClusterCfg<BN, ROWS>::kSmemBytes);
 }
 
-template <int BN, int S, int AROWS>
+template <int BN, int S, int ROWS>
 cudaError_t launch(const GemmArgs& g, const GemmDev& p, long tiles, cudaStream_t st) {
   alignas(64) CUtensorMap tmA, tmB;
-  if (!make_tmap_bf16_2d(&tmA, g.a, g.M, g.K, AROWS)) return cudaErrorInvalidValue;
+  if (!make_tmap_bf16_2d(&tmA, g.a, g.M, g.K, ROWS)) return cudaErrorInvalidValue;
   if (!make_tmap_bf16_2d(&tmB, g.w, g.N, g.K, BN)) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(tiles * S)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = ClusterCfg<BN, AROWS>::kSmemBytes; cfg.stream = st;
+  cfg.gridDim = dim3((unsigned)(tiles * S)); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = ClusterCfg<BN, ROWS>::kSmemBytes; cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = S; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, gemm_cluster_kernel<BN, S, AROWS>, tmA, tmB, p);
+  return cudaLaunchKernelEx(&cfg, gemm_cluster_kernel<BN, S, ROWS>, tmA, tmB, p);
 }
 
 }  // namespace
@@ -347,19 +363,21 @@ cudaError_t gemm_cluster_init() {
   if (e == cudaSuccess) e = set_attr<64, 4, 128>();
   if (e == cudaSuccess) e = set_attr<128, 2, 32>();
   if (e == cudaSuccess) e = set_attr<128, 4, 32>();
-  if (e == cudaSuccess) e = set_attr<64, 2, 32>();
-  if (e == cudaSuccess) e = set_attr<64, 4, 32>();
+  if (e == cudaSuccess) e = set_attr<128, 8, 32>();
+  if (e == cudaSuccess) e = set_attr<128, 2, 64>();
+  if (e == cudaSuccess) e = set_attr<128, 4, 64>();
+  if (e == cudaSuccess) e = set_attr<128, 8, 64>();
   return e;
 }
 
-// bn in {64, 128}, slices in {2, 4}; p.kb_per_split k-blocks per CTA.
+// bn in {64, 128}, slices in {2, 4} (few rows: bn 128, slices in {2, 4, 8}); p.kb_per_split k-blocks per CTA.
 cudaError_t launch_gemm_cluster(const GemmArgs& g, const GemmDev& p, int bn, int slices, cudaStream_t st) {
   const long tiles = (long)((g.M + BM - 1) / BM) * ((g.N + bn - 1) / bn);
-  if (g.M <= 32) {   // at most 32 rows: short A tiles, deeper ring
-    if (bn == 128 && slices == 2) return launch<128, 2, 32>(g, p, tiles, st);
-    if (bn == 128 && slices == 4) return launch<128, 4, 32>(g, p, tiles, st);
-    if (bn == 64 && slices == 2) return launch<64, 2, 32>(g, p, tiles, st);
-    if (bn == 64 && slices == 4) return launch<64, 4, 32>(g, p, tiles, st);
+  if (g.M <= kFlipRows && bn == 128) {
+    const bool few = g.M <= 32;
+    if (slices == 2) return few ? launch<128, 2, 32>(g, p, tiles, st) : launch<128, 2, 64>(g, p, tiles, st);
+    if (slices == 4) return few ? launch<128, 4, 32>(g, p, tiles, st) : launch<128, 4, 64>(g, p, tiles, st);
+    if (slices == 8) return few ? launch<128, 8, 32>(g, p, tiles, st) : launch<128, 8, 64>(g, p, tiles, st);
   }
   if (bn == 128 && slices == 2) return launch<128, 2, 128>(g, p, tiles, st);
   if (bn == 128 && slices == 4) return launch<128, 4, 128>(g, p, tiles, st);

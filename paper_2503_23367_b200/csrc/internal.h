@@ -195,7 +195,8 @@ struct GemmArgs {
 // either group at frequency base^(-j / (head_dim/4)).  table: [h*w][head_dim/2][2] fp32.
 cudaError_t launch_rope_table(float* table, int h, int w, int h_last, int w_last, int head_dim, float base, cudaStream_t st);
 cudaError_t gemm_init();
-// Test / profiling hook: 0 = choose per shape, 1 = one-CTA kernel, 2 = CTA-pair kernel 256x256, 3 = CTA-pair 256x128.
+// Test / profiling hook: 0 = choose per shape, 1 = one-CTA kernel, 2 = CTA-pair kernel 256x256, 3 = CTA-pair 256x128,
+// 4 ... 7 = one-CTA tiles 128, 192, 256, 64 wide, 8 ... 12 = clusters (128 wide x 4, x 2, 64 wide x 4, x 2, up to 48 rows 128 wide x 8).
 void gemm_force_path(int path);
 size_t gemm_splitk_ws_bytes();      // size of the K-split scratch
 size_t gemm_splitk_ticket_bytes();  // its leading bytes that must be zero before first use

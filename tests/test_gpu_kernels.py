@@ -491,6 +491,32 @@ def test_gemm_bf16_split_inside_a_cluster(M, N, K, epilogue, path):
     assert err <= MAX_ABS and cos >= MIN_COS, (err, cos)
 
 
+@pytest.mark.parametrize("path", [8, 9, 12])
+@pytest.mark.parametrize("M,N,K", [(1, 136, 72), (31, 1032, 1024), (32, 2048, 2048), (33, 384, 512), (48, 2048, 8192), (49, 256, 1024)])
+def test_gemm_few_rows_with_the_weights_on_the_m_side(M, N, K, path):
+    """Up to 48 rows of A as the N side of the MMA, 2, 4 or 8 slices of K: the edges of both builds (32 and 48 rows), ragged columns, fewer
+    k-blocks than CTAs, one row more than they take (path 12 then chooses by shape), and the residual epilogue on the same tiles."""
+    a = I.normal_bf16(96, (M, K), 1.0 if K <= 2048 else 0.5); w = I.normal_bf16(97, (N, K), 0.02); b = I.normal_bf16(98, (N,), 0.02)
+    x = I.normal(99, (M, N)); g = I.normal(100, (N,), 0.3)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    xd, gd, aux = dev(x), dev(g), torch.zeros((M, N), dtype=torch.bfloat16, device=DEV)
+    ad, wd, bd = bf16_dev(a), bf16_dev(w), bf16_dev(b)
+    assert fv.lib().fv_gemm_force_path(path) == 0
+    try:
+        out = fv.fv_gemm_bf16(ad, wd, bd, status=status)
+        out2 = fv.fv_gemm_bf16(ad, wd, bd, status=status)
+        fv.fv_gemm_bf16(ad, wd, bd, epilogue=2, out=xd, aux=aux, gamma=gd, mod_stride=0, rows_per_image=M, status=status)
+        torch.cuda.synchronize()
+    finally:
+        fv.lib().fv_gemm_force_path(0)
+    assert int(status.item()) == 0
+    assert torch.equal(out, out2) and torch.equal(out, aux)
+    y = O.linear(I.bf16_bits_to_f32(a), I.bf16_bits_to_f32(w), I.bf16_bits_to_f32(b))
+    err, cos = per_token_errors(bf16_host(out), y)
+    assert err <= MAX_ABS and cos >= MIN_COS, (err, cos)
+    assert np.abs(xd.cpu().numpy() - (x.astype(np.float64) + g.astype(np.float64) * y)).max() <= 2e-3
+
+
 def test_gemm_residual_epilogue_with_cache_copy():
     B, rows, N, K = 2, 100, 256, 512
     M = B * rows
