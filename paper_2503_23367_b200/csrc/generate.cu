@@ -97,11 +97,13 @@ __global__ void __launch_bounds__(256) residual_accumulate_kernel(const int32_t*
 // is computed once and written, with each copy's own embedding, to all of them.  Up to 32 code channels at a time lie in
 // shared memory, W_in as [j][channel] and the tokens' vectors as [j][token]; the shared-memory port hands a warp one word per
 // lane and clock, a broadcast word included, so a thread tile of T x C costs T + C of its clocks for T C / 4 of an SM's multiply-adds: 8 x 8
-// balances the two.  The copies' embedding rows are fetched into L2 under the multiply-adds; a warp then walks the copies of its own
-// tokens, the products read back from shared memory, four embedding rows in flight.  Measured for 2 x 48 x 48 -> 64 x 64 tokens,
-// C 2048, d 32 (map written + embedding read: 16 us): 81 us with a product per target token and one channel per thread, 59 us
-// with a product per target token in 8 x 8 tiles, 51 us like this (two rounds of CTAs, each a chain of loads, products and
-// stores).  The additions keep their order (j ascending, bias, embedding).
+// balances the two, and two channels go through one packed multiply-add.  A warp then walks the copies of its own tokens, whose
+// products its lanes hold in registers, the embedding rows of two copies in flight.  Measured for 2 x 48 x 48 -> 64 x 64 tokens, C 2048, d 32
+// (map written + embedding read: 16 us), back to back: 38 us; 45.5 with single multiply-adds, the products passed through shared
+// memory to be indexed by copy and the embedding rows prefetched into L2 (which gives nothing); a product per target token in 8 x 8 tiles 52,
+// and with one channel per thread 73.  Two rounds of CTAs, each a chain of loads (embedding rows 11 us in all), products (8) and
+// stores (6); CTAs of 32 or 16 tokens, four or eight to an SM, do not overlap them better (40, 52).  The additions keep their order (j
+// ascending, bias, embedding).
 constexpr int kNextTokens = 64;
 constexpr int kNextChannels = 256;      // one per thread while W_in is staged
 // (r is written by the kernel before this one: without __restrict__ its loads stay behind the dependency wait)
@@ -133,27 +135,14 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
     }
     s_first[tid] = first; s_nx[tid] = nx; s_cnt[tid] = nx * ny;
   }
-  float acc[8][8];
+  uint64_t acc2[8][4];   // channel pairs
 #pragma unroll
   for (int t = 0; t < 8; ++t)
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[t][e] = 0.f;
+    for (int e = 0; e < 4; ++e) acc2[t][e] = 0ull;
   const int lane = tid & 31, warp = tid >> 5;
   const int tl = warp * 8;               // this thread's tokens inside the tile; its channels are 4 lane .. and 128 + 4 lane ..
-  // target token d of the copies of staged token t, inside its image
-  auto target = [&](int t, int d) { const int yy = d / s_nx[t]; return s_first[t] + yy * w2 + (d - yy * s_nx[t]); };
   __syncthreads();
-  if (pos) {   // a quarter warp per row: 8 lines of 128 bytes
-    const int t = tid >> 2;
-    for (int d = 0; d < s_cnt[t]; ++d) {
-      const float* q = pos + (size_t)target(t, d) * C;
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int c = c0 + ((tid & 3) + 4 * u) * 32;
-        if (c < C) asm volatile("prefetch.global.L2 [%0];" ::"l"(q + c));
-      }
-    }
-  }
   for (int d0 = 0; d0 < D; d0 += DC) {
     if (d0) __syncthreads();             // the chunk before has been used
     {   // all of a thread's loads are requested before the first is stored: one round trip each for W_in and r
@@ -180,77 +169,64 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
     __syncthreads();
 #pragma unroll 2
     for (int j = 0; j < DC; ++j) {
-      const float4 wa = *reinterpret_cast<const float4*>(&w_s[j][4 * lane]), wb = *reinterpret_cast<const float4*>(&w_s[j][128 + 4 * lane]);
+      const ulonglong2 wa = *reinterpret_cast<const ulonglong2*>(&w_s[j][4 * lane]), wb = *reinterpret_cast<const ulonglong2*>(&w_s[j][128 + 4 * lane]);
       const float4 ra = *reinterpret_cast<const float4*>(&r_s[j][tl]), rb = *reinterpret_cast<const float4*>(&r_s[j][tl + 4]);
-      const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w}, rv[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+      const uint64_t wv[4] = {wa.x, wa.y, wb.x, wb.y};
+      const float rv[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
 #pragma unroll
-      for (int t = 0; t < 8; ++t)
+      for (int t = 0; t < 8; ++t) {
+        uint64_t rr;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(rr) : "f"(rv[t]));
 #pragma unroll
-        for (int e = 0; e < 8; ++e) acc[t][e] = fmaf(rv[t], wv[e], acc[t][e]);
+        for (int e = 0; e < 4; ++e) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc2[t][e]) : "l"(rr), "l"(wv[e]));
+      }
     }
   }
-  // The warp's products go to its own 4 KB of shared memory (over W_in, 128 channels at a time), and the warp walks the copies of its
-  // tokens: lane l knows copy l's token and place, four embedding rows in flight.
-  __syncthreads();
-  float4* mine = reinterpret_cast<float4*>(&w_s[0][0]) + warp * (DC * kNextChannels / 4 / 8);
-  constexpr int kRowsFit = DC * kNextChannels / 128 / 8;   // token rows of 128 channels in the warp's share: 8 for 32 code channels
-  int before[9];
-  before[0] = 0;
+  float acc[8][8];
 #pragma unroll
-  for (int t = 0; t < 8; ++t) before[t + 1] = before[t] + s_cnt[tl + t];
-#pragma unroll 1
+  for (int t = 0; t < 8; ++t)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[t][2 * e]), "=f"(acc[t][2 * e + 1]) : "l"(acc2[t][e]));
+  // the copies of the warp's tokens, two at a time
+  const int ca = c0 + 4 * lane, cb = ca + 128;
+  float4 bias[2];
+#pragma unroll
   for (int g = 0; g < 2; ++g) {
-    const int c = c0 + 128 * g + 4 * lane;
-    const bool col_ok = c < C;
-    float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (b_in && col_ok) bias = make_float4(__ldg(b_in + c), __ldg(b_in + c + 1), __ldg(b_in + c + 2), __ldg(b_in + c + 3));
+    const int c = g ? cb : ca;
+    bias[g] = b_in && c < C ? make_float4(__ldg(b_in + c), __ldg(b_in + c + 1), __ldg(b_in + c + 2), __ldg(b_in + c + 3)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
 #pragma unroll
-    for (int r0 = 0; r0 < 8; r0 += kRowsFit) {
-      __syncwarp();
+  for (int t = 0; t < 8; ++t) {
+    const int cnt = s_cnt[tl + t], nx = s_nx[tl + t], first = s_first[tl + t];
+    const float4 va = make_float4(acc[t][0] + bias[0].x, acc[t][1] + bias[0].y, acc[t][2] + bias[0].z, acc[t][3] + bias[0].w);
+    const float4 vb = make_float4(acc[t][4] + bias[1].x, acc[t][5] + bias[1].y, acc[t][6] + bias[1].z, acc[t][7] + bias[1].w);
+    float* img = x_out + (cnt ? s_img[tl + t] : 0) * C;
+    for (int k0 = 0; k0 < cnt; k0 += 2) {
+      float4 pa[2], pb[2];
+      int t2[2];
 #pragma unroll
-      for (int t = r0; t < r0 + kRowsFit; ++t) {
-        const float4 v = g ? make_float4(acc[t][4], acc[t][5], acc[t][6], acc[t][7]) : make_float4(acc[t][0], acc[t][1], acc[t][2], acc[t][3]);
-        mine[(t - r0) * 32 + lane] = make_float4(v.x + bias.x, v.y + bias.y, v.z + bias.z, v.w + bias.w);
+      for (int u = 0; u < 2; ++u) {
+        const int d = min(k0 + u, cnt - 1), yy = d / nx;
+        t2[u] = first + yy * w2 + (d - yy * nx);
+        pa[u] = pb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (pos && k0 + u < cnt) {
+          const float* q = pos + (size_t)t2[u] * C;
+          if (ca < C) pa[u] = vec ? __ldg(reinterpret_cast<const float4*>(q + ca)) : make_float4(__ldg(q + ca), __ldg(q + ca + 1), __ldg(q + ca + 2), __ldg(q + ca + 3));
+          if (cb < C) pb[u] = vec ? __ldg(reinterpret_cast<const float4*>(q + cb)) : make_float4(__ldg(q + cb), __ldg(q + cb + 1), __ldg(q + cb + 2), __ldg(q + cb + 3));
+        }
       }
-      __syncwarp();
-      const int lo = before[r0], hi = before[r0 + kRowsFit];
-      for (int e0 = lo; e0 < hi; e0 += 32) {
-        int t = r0;
 #pragma unroll
-        for (int u = r0 + 1; u < r0 + kRowsFit; ++u) t += e0 + lane >= before[u];
-        int d = e0 + lane;
-#pragma unroll
-        for (int u = r0; u < r0 + kRowsFit; ++u)
-          if (t == u) d -= before[u];
-        const int nx = max(s_nx[tl + t], 1), yy = d / nx, t2 = s_first[tl + t] + yy * w2 + (d - yy * nx);
-        const long img = s_img[tl + t];
-        const int cnt = min(32, hi - e0);
-#pragma unroll 1
-        for (int k0 = 0; k0 < cnt; k0 += 4) {
-          float4 pe[4];
-          int tt[4];
-          long row[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int src = min(k0 + u, cnt - 1);
-            tt[u] = __shfl_sync(0xffffffffu, t, src);
-            const int k2 = __shfl_sync(0xffffffffu, t2, src);
-            row[u] = __shfl_sync(0xffffffffu, img, src) + k2;
-            pe[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (pos && col_ok) {
-              const float* q = pos + (size_t)k2 * C + c;
-              pe[u] = vec ? __ldg(reinterpret_cast<const float4*>(q)) : make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3));
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if (k0 + u >= cnt || !col_ok) break;
-            const float4 a = mine[(tt[u] - r0) * 32 + lane];
-            const float4 o = make_float4(a.x + pe[u].x, a.y + pe[u].y, a.z + pe[u].z, a.w + pe[u].w);
-            float* dst = x_out + (size_t)row[u] * C + c;
-            if (vec) *reinterpret_cast<float4*>(dst) = o;
-            else { dst[0] = o.x; dst[1] = o.y; dst[2] = o.z; dst[3] = o.w; }
-          }
+      for (int u = 0; u < 2; ++u) {
+        if (k0 + u >= cnt) break;
+        float* dst = img + (size_t)t2[u] * C;
+        const float4 oa = make_float4(va.x + pa[u].x, va.y + pa[u].y, va.z + pa[u].z, va.w + pa[u].w);
+        const float4 ob = make_float4(vb.x + pb[u].x, vb.y + pb[u].y, vb.z + pb[u].z, vb.w + pb[u].w);
+        if (vec) {
+          if (ca < C) *reinterpret_cast<float4*>(dst + ca) = oa;
+          if (cb < C) *reinterpret_cast<float4*>(dst + cb) = ob;
+        } else {
+          if (ca < C) { dst[ca] = oa.x; dst[ca + 1] = oa.y; dst[ca + 2] = oa.z; dst[ca + 3] = oa.w; }
+          if (cb < C) { dst[cb] = ob.x; dst[cb + 1] = ob.y; dst[cb + 2] = ob.z; dst[cb + 3] = ob.w; }
         }
       }
     }
