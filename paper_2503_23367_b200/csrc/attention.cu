@@ -32,6 +32,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include "attention_ring.h"
 #include "internal.h"
 #include "sm100.cuh"
 
@@ -655,6 +656,9 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
                  const __grid_constant__ CUtensorMap tmV, const WholeDev p) {
   using Cfg = AttnCfg<HD, ONE_TILE>;
   constexpr int NS = Cfg::kStages;
+  using Ring = TileRing<NS, ONE_TILE ? 2 : 1>;   // of key tiles, and of value tiles
+  constexpr int NF = Ring::kFull;
+  static_assert((1 + 2 * (NF + NS) + 12) * 8 + 4 <= 256, "barriers and the TMEM slot lie in the last 256 bytes");
   constexpr int QB = ONE_TILE ? QT : 2 * QT;    // queries per CTA
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -663,10 +667,10 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   uint8_t* v_s = k_s + NS * Cfg::kKBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(v_s + NS * Cfg::kVBytes);
   uint64_t* q_full = bars;
-  uint64_t* k_full = bars + 1;
-  uint64_t* k_empty = k_full + NS;
+  uint64_t* k_full = bars + 1;       // [NF], the others [NS]
+  uint64_t* k_empty = k_full + NF;
   uint64_t* v_full = k_empty + NS;
-  uint64_t* v_empty = v_full + NS;
+  uint64_t* v_empty = v_full + NF;
   uint64_t* s_full = v_empty + NS;   // [2 t + half] scores of stream t are in TMEM
   uint64_t* p_full = s_full + 4;     // [2 t + half] probabilities of stream t are in TMEM (128 arrivals)
   uint64_t* o_prev = p_full + 4;     // [2] the P V of stream t's last half but one has completed
@@ -683,7 +687,8 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
 
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
-    for (int s = 0; s < NS; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_empty[s], ONE_TILE ? 1 : ntiles); mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], ONE_TILE ? 1 : ntiles); }
+    for (int s = 0; s < NF; ++s) { mbar_init(&k_full[s], 1); mbar_init(&v_full[s], 1); }
+    for (int s = 0; s < NS; ++s) { mbar_init(&k_empty[s], ONE_TILE ? 1 : ntiles); mbar_init(&v_empty[s], ONE_TILE ? 1 : ntiles); }
     for (int t = 0; t < 4; ++t) { mbar_init(&s_full[t], 1); mbar_init(&p_full[t], QT); }
     for (int t = 0; t < 2; ++t) { mbar_init(&o_prev[t], 1); mbar_init(&o_last[t], 1); }
     mbar_fence_init();
@@ -703,21 +708,21 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         for (int a = 0; a < HD / 64; ++a)
           tma_load_2d(q_s + t * Cfg::kQBytes + a * (QT * 128), &tmQ, head * HD + a * 64, img * p.rows + q0 + t * QT, q_full);
       for (int j = 0; j < T; ++j) {
-        const int s = j % NS;
-        if (!mbar_wait(&k_empty[s], ((j / NS) & 1) ^ 1)) { report(p.status, DEV_TIMEOUT_TMA); break; }
-        mbar_expect_tx(&k_full[s], Cfg::kKBytes);
+        const int s = Ring::stage(j), f = Ring::full(j);
+        if (!mbar_wait(&k_empty[s], Ring::empty_parity(j))) { report(p.status, DEV_TIMEOUT_TMA); break; }
+        mbar_expect_tx(&k_full[f], Cfg::kKBytes);
         for (int a = 0; a < HD / 64; ++a)
-          tma_load_2d(k_s + s * Cfg::kKBytes + a * (KT * 128), &tmK, head * HD + a * 64, img * p.kv_capacity + j * KT, &k_full[s]);
+          tma_load_2d(k_s + s * Cfg::kKBytes + a * (KT * 128), &tmK, head * HD + a * 64, img * p.kv_capacity + j * KT, &k_full[f]);
       }
     }
   } else if (warp == 10) {  // values: a warp of their own, so that a key tile never waits behind a value tile's stage
     if (lane == 0) {
       for (int j = 0; j < T; ++j) {
-        const int s = j % NS;
-        if (!mbar_wait(&v_empty[s], ((j / NS) & 1) ^ 1)) { report(p.status, DEV_TIMEOUT_TMA); break; }
-        mbar_expect_tx(&v_full[s], Cfg::kVBytes);
+        const int s = Ring::stage(j), f = Ring::full(j);
+        if (!mbar_wait(&v_empty[s], Ring::empty_parity(j))) { report(p.status, DEV_TIMEOUT_TMA); break; }
+        mbar_expect_tx(&v_full[f], Cfg::kVBytes);
         for (int a = 0; a < KT / 64; ++a)
-          tma_load_2d(v_s + s * Cfg::kVBytes + a * (HD * 128), &tmV, j * KT + a * 64, img * p.C + head * HD, &v_full[s]);
+          tma_load_2d(v_s + s * Cfg::kVBytes + a * (HD * 128), &tmV, j * KT + a * 64, img * p.C + head * HD, &v_full[f]);
       }
     }
   } else if (warp == 9 || warp == 11) {   // one issuing warp per stream: the waits and commits of one run under the MMAs of the other
@@ -744,35 +749,35 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     };
     if (nh > 0) {
       int j = ONE_TILE ? t : 0;
-      bool ok = mbar_wait(q_full, 0) && mbar_wait(&k_full[j % NS], (j / NS) & 1);
+      bool ok = mbar_wait(q_full, 0) && mbar_wait(&k_full[Ring::full(j)], Ring::full_parity(j));
       if (!ok) report(p.status, DEV_TIMEOUT_MMA);
       if (ok) {
         tc_fence_after();
-        issue_qk(j % NS, 0);
-        if (nh > 1) issue_qk(j % NS, 1);
-        if (leader) umma_commit(&k_empty[j % NS]);
+        issue_qk(Ring::stage(j), 0);
+        if (nh > 1) issue_qk(Ring::stage(j), 1);
+        if (leader) umma_commit(&k_empty[Ring::stage(j)]);
       }
       for (int i = 0; ok && i < nh; ++i) {
         const int h = i & 1, jj = i >> 1;
         j = ONE_TILE ? 2 * jj + t : jj;
         const int jn = j + DJ;
         const bool more = i + 2 < nh;
-        if (h == 0 && (!mbar_wait(&v_full[j % NS], (j / NS) & 1) || (more && !mbar_wait(&k_full[jn % NS], (jn / NS) & 1)))) {
+        if (h == 0 && (!mbar_wait(&v_full[Ring::full(j)], Ring::full_parity(j)) || (more && !mbar_wait(&k_full[Ring::full(jn)], Ring::full_parity(jn))))) {
           report(p.status, DEV_TIMEOUT_MMA); ok = false; break;
         }
         if (!mbar_wait(&p_full[2 * t + h], jj & 1)) { report(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
         tc_fence_after();
-        const uint64_t vd = vd0 + (((j % NS) * Cfg::kVBytes + h * (HD * 128)) >> 4);
+        const uint64_t vd = vd0 + ((Ring::stage(j) * Cfg::kVBytes + h * (HD * 128)) >> 4);
         if (leader) {   // P over the first 32 columns of its slot
 #pragma unroll
           for (int kk = 0; kk < HT / 16; ++kk) umma_bf16_ts(o_tmem, s_tmem + h * HT + kk * 8, vd + 2 * kk, idesc_pv, (i | kk) != 0);
           if (i + 2 == nh) umma_commit(&o_prev[t]);
           if (i + 1 == nh) umma_commit(&o_last[t]);
         }
-        if (more) issue_qk(jn % NS, h);
+        if (more) issue_qk(Ring::stage(jn), h);
         if (leader) {
-          if (h == 1 || i == nh - 1) umma_commit(&v_empty[j % NS]);
-          if (more && (h == 1 || i + 2 == nh - 1)) umma_commit(&k_empty[jn % NS]);
+          if (h == 1 || i == nh - 1) umma_commit(&v_empty[Ring::stage(j)]);
+          if (more && (h == 1 || i + 2 == nh - 1)) umma_commit(&k_empty[Ring::stage(jn)]);
         }
       }
     }
