@@ -203,12 +203,12 @@ gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     }
   } else {
     // ---- accumulator readers: thread = one row of the tile (FLIP: one column); a row's partial goes to the CTA that owns the row ----
-    stage_bias(p, bias_s + (warp & 3) * 32, lane, n0, BN);
-    pdl_wait();
+    pdl_wait();                             // (the bias may be a product of the kernel before, like A and the stream)
     if (x_f32 || x_b16) {
 #pragma unroll
       for (int i = 0; i < PRE; ++i) fetch(i, i);
     }
+    stage_bias(p, bias_s + (warp & 3) * 32, lane, n0, BN);
     const int quarter = warp & 3;
     bool have = kb1 > kb0;
     if (have && !mbar_wait(acc_full, 0)) { report(p.status, DEV_TIMEOUT_EPI); have = false; }
