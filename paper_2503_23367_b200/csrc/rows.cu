@@ -21,7 +21,7 @@ namespace {
 constexpr int kMaxVec = 16;  // float4 per lane -> C <= 2048
 
 // grid (ceil(k / 8), B): one warp per kept row; sigma / beta of the image staged in shared memory while
-// the row index and the row itself are in flight.
+// the row itself is in flight.
 template <typename XT>
 __global__ void __launch_bounds__(256) gather_ln_kernel(const XT* __restrict__ x, const int32_t* __restrict__ idx, int n,
                                                         int k, int C4, const float* __restrict__ sigma,
@@ -32,11 +32,6 @@ __global__ void __launch_bounds__(256) gather_ln_kernel(const XT* __restrict__ x
   const int b = blockIdx.y, j = blockIdx.x * 8 + warp;
   const bool live = j < k;
   pdl_trigger();
-  if (sigma) {   // modulation vectors are never written by a kernel of the step: on their way while the kernel before this one ends
-    const float4* sg = reinterpret_cast<const float4*>(sigma + (size_t)b * mod_stride);
-    const float4* bt = reinterpret_cast<const float4*>(beta + (size_t)b * mod_stride);
-    for (int i = threadIdx.x; i < C4; i += 256) { s_mod[i] = __ldg(sg + i); s_mod[C4 + i] = __ldg(bt + i); }
-  }
   pdl_wait();
   int t = live ? (idx ? __ldg(idx + (size_t)b * k + j) : j) : 0;
   if (t < 0 || t >= n) {   // a caller's index outside the map: stay inside it and say so
@@ -52,6 +47,13 @@ __global__ void __launch_bounds__(256) gather_ln_kernel(const XT* __restrict__ x
       const int c4 = lane + 32 * i;
       if (c4 < C4) v[i] = x_load4(row + (size_t)c4 * 4);
     }
+  }
+  if (sigma) {   // behind the wait (the kernel before may have produced them) and behind the row's loads, which they then travel beside
+    const float4* sg = reinterpret_cast<const float4*>(sigma + (size_t)b * mod_stride);
+    const float4* bt = reinterpret_cast<const float4*>(beta + (size_t)b * mod_stride);
+    for (int i = threadIdx.x; i < C4; i += 256) { s_mod[i] = __ldg(sg + i); s_mod[C4 + i] = __ldg(bt + i); }
+  }
+  if (live) {
 #pragma unroll
     for (int i = 0; i < kMaxVec; ++i) {
       const int c4 = lane + 32 * i;

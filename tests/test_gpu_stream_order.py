@@ -65,3 +65,12 @@ def test_gemm_bias_written_by_the_kernel_before(M, N, K):
     bias = _LongGemm(8, N, torch.bfloat16)
     a, w = _randn(3, M, K, dtype=torch.bfloat16), _randn(4, N, K, std=0.02, dtype=torch.bfloat16)
     _check_in_order(bias, lambda: fv.fv_gemm_bf16(a, w, bias.out[0]), bias.renew)
+
+
+@pytest.mark.parametrize("k,n,C", [(1, 1, 1024), (9, 256, 2048), (600, 1024, 512)])
+def test_layernorm_modulation_written_by_the_kernel_before(k, n, C):
+    mod = _LongGemm(2, 2 * C, torch.float32)               # two images: sigma, beta
+    x = _randn(5, 2, n, C)
+    idx = torch.stack([torch.randperm(n, generator=torch.Generator().manual_seed(b))[:k].sort().values for b in range(2)]).int().to(DEV)
+    flat = mod.out.view(-1)
+    _check_in_order(mod, lambda: fv.fv_gather_ln(x, idx, flat[:C], flat.data_ptr() + 4 * C, mod_stride=2 * C), mod.renew)
