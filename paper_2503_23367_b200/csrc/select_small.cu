@@ -25,6 +25,7 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kRows = 8;              // rows of a chunk per thread
 constexpr int kMaxCluster = 16;
+static_assert(2048 / 4 <= kThreads, "one thread per four channels");
 
 struct SmallArgs {
   void* x;
@@ -126,30 +127,29 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
   pdl_trigger();
   cluster_arrive_relaxed();
   for (int i = tid; i < (n + 15) / 16 * 4; i += kThreads) reinterpret_cast<uint32_t*>(flags)[i] = 0u;
-  // gate and modulation vectors are never written by a kernel of the step: on their way before the dependency wait
-  float gam[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) gam[e] = 1.f;
-  if (live && a.y && a.gamma_prev) {
-    const float4* gp = reinterpret_cast<const float4*>(a.gamma_prev + (size_t)b * a.mod_stride + ct * 8);
-    const float4 g0 = __ldg(gp), g1 = __ldg(gp + 1);
-    gam[0] = g0.x; gam[1] = g0.y; gam[2] = g0.z; gam[3] = g0.w; gam[4] = g1.x; gam[5] = g1.y; gam[6] = g1.z; gam[7] = g1.w;
-  }
-  if (a.sigma) {
-    const float4* sp = reinterpret_cast<const float4*>(a.sigma + (size_t)b * a.mod_stride);
-    const float4* bp = reinterpret_cast<const float4*>(a.beta + (size_t)b * a.mod_stride);
-    for (int c4 = tid; c4 < C / 4; c4 += kThreads) { mod[c4] = __ldg(sp + c4); mod[C / 4 + c4] = __ldg(bp + c4); }
-  }
   pdl_wait();
+  // (gate and modulation vectors too: the step may be in place and they the product of the kernel before it)
   float v[kRows][8];
 #pragma unroll
   for (int u = 0; u < 4; ++u)            // the first rows are fetched while the sources of all rows are looked up
     if (live && u * G + g < own) load_row8(xb + (size_t)(r0 + u * G + g) * C, v[u]);
-  if (a.y && tid < own) {
-    const int t = r0 + tid, j = load_index(a.inv_prev + (size_t)b * n + t);
-    const int yy = t / a.w, xx = t - yy * a.w;
+  const bool lookup = a.y && tid < own, modulate = a.sigma && tid < C / 4;   // (own <= R and C / 4 are at most kThreads)
+  int j = 0;
+  float4 sg = make_float4(0.f, 0.f, 0.f, 0.f), bt = sg;
+  if (lookup) j = load_index(a.inv_prev + (size_t)b * n + r0 + tid);
+  float gam[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) gam[e] = 1.f;
+  if (live && a.y && a.gamma_prev) load_row8(a.gamma_prev + (size_t)b * a.mod_stride + ct * 8, gam);
+  if (modulate) {
+    sg = x_load4(a.sigma + (size_t)b * a.mod_stride + tid * 4);
+    bt = x_load4(a.beta + (size_t)b * a.mod_stride + tid * 4);
+  }
+  if (lookup) {
+    const int t = r0 + tid, yy = t / a.w, xx = t - yy * a.w;
     s_src[tid] = j >= 0 ? j : ~((yy * a.hc) / a.h * a.wc + (xx * a.wc) / a.w);
   }
+  if (modulate) { mod[tid] = sg; mod[C / 4 + tid] = bt; }
   __syncthreads();
 
   // ---- restoration of the previous sublayer, column sums of the restored rows

@@ -7,7 +7,6 @@ import pytest
 import torch
 
 from paper_2503_23367_b200 import binding as fv
-from paper_2503_23367_b200 import inputs as I
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -37,10 +36,11 @@ class _LongGemm:
         fv.fv_gemm_bf16(self.a, self.w, None, 4 if self.out.dtype == torch.float32 else 0, out=self.out)
 
 
-def _check_in_order(produce, consume, renew, rounds=4):
-    """consume() -> a tensor or a list of them."""
+def _check_in_order(produce, consume, renew, rewind=lambda: None, rounds=4):
+    """consume() -> a tensor or a list of them; rewind() puts back what it works on in place."""
     as_list = lambda v: list(v) if isinstance(v, (list, tuple)) else [v]
     renew(0)
+    rewind()
     produce()
     consume()
     torch.cuda.synchronize()
@@ -50,10 +50,12 @@ def _check_in_order(produce, consume, renew, rounds=4):
         got = as_list(consume())
     for i in range(1, rounds + 1):
         renew(i)
+        rewind()
         torch.cuda.synchronize()
         g.replay()
         torch.cuda.synchronize()
         mine = [t.clone() for t in got]
+        rewind()
         want = as_list(consume())                  # the produced buffer at rest
         torch.cuda.synchronize()
         for a, b in zip(mine, want):
@@ -74,3 +76,39 @@ def test_layernorm_modulation_written_by_the_kernel_before(k, n, C):
     idx = torch.stack([torch.randperm(n, generator=torch.Generator().manual_seed(b))[:k].sort().values for b in range(2)]).int().to(DEV)
     flat = mod.out.view(-1)
     _check_in_order(mod, lambda: fv.fv_gather_ln(x, idx, flat[:C], flat.data_ptr() + 4 * C, mod_stride=2 * C), mod.renew)
+
+
+@pytest.mark.parametrize("step,keep,last", [(1, 1.0, 16), (2, 0.5, 16), (2, 0.3, 40)])
+def test_step_in_place_with_modulation_written_by_the_kernel_before(step, keep, last):
+    """No copy stands in front of the step's first kernel: gather + LayerNorm (unpruned), the one-launch selection of a small map,
+    the selection of a larger one."""
+    L, B, C, H = 2, 2, 256, 4
+    sides = [(2, 2), (8, 8), (last, last)]
+    g = torch.Generator(device=DEV)
+    g.manual_seed(3)
+
+    def w(*shape):
+        return [(torch.randn(*shape, generator=g, device=DEV) * 0.02).bfloat16() for _ in range(L)]
+
+    class Tensors:
+        w_qkv, b_qkv, w_o, b_o = w(3 * C, C), w(3 * C), w(C, C), w(C)
+        w_fc1, b_fc1, w_fc2, b_fc2 = w(4 * C, C), w(4 * C), w(C, 4 * C), w(C)
+        w_q_x = w_kv_x = w_o_x = text = None
+        mod = torch.randn(L, B, 6, C, generator=g, device=DEV) * 0.3
+
+    ctx = fv.FvContext(L, C, H, sides, 1, B, 4 + 64 + last * last, Tensors)
+    produce = _LongGemm(L * B, 6 * C, torch.float32)
+    produce.out = ctx.mod.view(L * B, 6 * C)
+    maps = [_randn(20 + i, B, a * b, C) for i, (a, b) in enumerate(sides)]
+    for i, m in enumerate(maps):                       # fills the caches and the keys of the steps before
+        ctx.var_step(m, i, keep if i == 2 else 1.0)
+    x = maps[step].clone()
+    kv = sum(a * b for a, b in sides[:step])
+
+    def consume():
+        ctx.set_state(step, kv)
+        return ctx.var_step(x, step, keep, out=x).clone()
+
+    _check_in_order(produce, consume, produce.renew, rewind=lambda: x.copy_(maps[step]))
+    assert ctx.device_status() == 0
+    ctx.close()
