@@ -143,9 +143,10 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
   const int lane = tid & 31, warp = tid >> 5;
   const int tl = warp * 8;               // this thread's tokens inside the tile; its channels are 4 lane .. and 128 + 4 lane ..
   __syncthreads();
+  pdl_wait();                            // W_in, b_in and pos are the caller's like r: any of them may come from the kernel before
   for (int d0 = 0; d0 < D; d0 += DC) {
     if (d0) __syncthreads();             // the chunk before has been used
-    {   // all of a thread's loads are requested before the first is stored: one round trip each for W_in and r
+    {   // all of a thread's loads are requested before the first is stored: one round trip for W_in, one for r
       float4 q[DC / 4];                  // channel c0 + tid
 #pragma unroll
       for (int i = 0; i < DC / 4; ++i) {
@@ -155,7 +156,6 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
 #pragma unroll
       for (int i = 0; i < DC / 4; ++i) { w_s[4 * i][tid] = q[i].x; w_s[4 * i + 1][tid] = q[i].y; w_s[4 * i + 2][tid] = q[i].z; w_s[4 * i + 3][tid] = q[i].w; }
     }
-    if (d0 == 0) pdl_wait();             // (weights and embeddings are never written by a kernel of the loop)
     {
       constexpr int JP = DC / 4;         // four threads per token
       const int t = tid >> 2, j0 = (tid & 3) * JP;

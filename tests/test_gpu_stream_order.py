@@ -112,3 +112,11 @@ def test_step_in_place_with_modulation_written_by_the_kernel_before(step, keep, 
     _check_in_order(produce, consume, produce.renew, rewind=lambda: x.copy_(maps[step]))
     assert ctx.device_status() == 0
     ctx.close()
+
+
+@pytest.mark.parametrize("d", [8, 32, 64])
+def test_next_token_map_with_w_in_written_by_the_kernel_before(d):
+    C = 512
+    w_in = _LongGemm(C, d, torch.float32)
+    r, b_in, pos = _randn(6, 2, 36, d), _randn(7, C), _randn(8, 64, C)
+    _check_in_order(w_in, lambda: fv.fv_next_scale_input(r, 6, 6, 8, 8, w_in.out, b_in, pos), w_in.renew)
