@@ -47,7 +47,7 @@ __device__ __forceinline__ void report(int32_t* status, int code) {
 // for its accumulator, so that no chunk stalls on a global load of 64 bytes of bias.
 constexpr int kBiasSmemBytes = 4 * 512;   // one slice per epilogue warp
 __device__ __forceinline__ void stage_bias(const GemmDev& p, uint4* bias_w, int lane, int n0, int bn) {
-  if (p.bias && lane * 8 < bn && n0 + lane * 8 < p.N) bias_w[lane] = __ldg(reinterpret_cast<const uint4*>(p.bias + n0) + lane);
+  if (p.bias && lane * 8 < bn && n0 + lane * 8 < p.N) bias_w[lane] = dep_load16(p.bias + n0 + lane * 8);
   __syncwarp();
 }
 
@@ -140,8 +140,8 @@ __device__ __forceinline__ void residual_chunk(const GemmDev& p, const ResidRows
   if (col + 4 * (lane & 7) < p.N) {
     float4 g0 = make_float4(1.f, 1.f, 1.f, 1.f), g1 = g0;
     if (rr.gam0) {
-      g0 = __ldg(reinterpret_cast<const float4*>(rr.gam0 + col));
-      if (rr.n_first < rr.n_rows) g1 = __ldg(reinterpret_cast<const float4*>(rr.gam1 + col));
+      g0 = dep_load4(rr.gam0 + col);
+      if (rr.n_first < rr.n_rows) g1 = dep_load4(rr.gam1 + col);
     }
     const float* trow = tile + (lane >> 3) * kResidTilePitch + 4 * (lane & 7);
 #pragma unroll
@@ -200,7 +200,7 @@ __device__ __forceinline__ void store_chunk(const GemmDev& p, const float (&v)[3
       if (col + 4 * g < p.N) {
         float4 xv = xr[g];
         if (gp) {
-          float4 gg = __ldg(gp + g);
+          float4 gg = dep_load4(gp + g);
           xv.x = fmaf(gg.x, v[4 * g + 0], xv.x); xv.y = fmaf(gg.y, v[4 * g + 1], xv.y);
           xv.z = fmaf(gg.z, v[4 * g + 2], xv.z); xv.w = fmaf(gg.w, v[4 * g + 3], xv.w);
         } else {
@@ -234,7 +234,7 @@ __device__ __forceinline__ void store_chunk(const GemmDev& p, const float (&v)[3
 #pragma unroll
         for (int i = 0; i < 4; ++i) { xv[2 * i] = __uint_as_float(u[i] << 16); xv[2 * i + 1] = __uint_as_float(u[i] & 0xFFFF0000u); }
         if (gp) {
-          const float4 ga = __ldg(gp + 2 * g), gb = __ldg(gp + 2 * g + 1);
+          const float4 ga = dep_load4(gp + 2 * g), gb = dep_load4(gp + 2 * g + 1);
           xv[0] = fmaf(ga.x, v[8 * g + 0], xv[0]); xv[1] = fmaf(ga.y, v[8 * g + 1], xv[1]); xv[2] = fmaf(ga.z, v[8 * g + 2], xv[2]); xv[3] = fmaf(ga.w, v[8 * g + 3], xv[3]);
           xv[4] = fmaf(gb.x, v[8 * g + 4], xv[4]); xv[5] = fmaf(gb.y, v[8 * g + 5], xv[5]); xv[6] = fmaf(gb.z, v[8 * g + 6], xv[6]); xv[7] = fmaf(gb.w, v[8 * g + 7], xv[7]);
         } else {
@@ -297,9 +297,9 @@ __device__ __forceinline__ void qk_head_epilogue(const GemmDev& p, uint32_t tadd
       for (int i = 0; i < 32; ++i) ss = fmaf(v[i], v[i], ss);
     }
     scale = 1.f / fmaxf(sqrtf(ss), 1e-12f);
-    if (is_query) scale *= __ldg(p.qk_scale + (col % p.C) / hd);
+    if (is_query) scale *= dep_load(p.qk_scale + (col % p.C) / hd);
   }
-  const int token = (p.rope_idx && row_ok) ? __ldg(p.rope_idx + (size_t)img * p.rows_per_image + jrow) : jrow;
+  const int token = (p.rope_idx && row_ok) ? dep_load(p.rope_idx + (size_t)img * p.rows_per_image + jrow) : jrow;
   const float4* tab = (p.rope_table && row_ok) ? reinterpret_cast<const float4*>(p.rope_table + (size_t)token * (hd / 2)) : nullptr;
   for (int c = 0; c < hd; c += 32) {
     uint32_t r[32];
@@ -314,7 +314,7 @@ __device__ __forceinline__ void qk_head_epilogue(const GemmDev& p, uint32_t tadd
     if (tab) {
 #pragma unroll
       for (int g = 0; g < 8; ++g) {   // two channel pairs per float4 of (cos, sin, cos, sin)
-        const float4 cs = __ldg(tab + c / 4 + g);
+        const float4 cs = dep_load4(tab + c / 4 + g);
         const float a0 = v[4 * g], b0 = v[4 * g + 1], a1 = v[4 * g + 2], b1 = v[4 * g + 3];
         v[4 * g] = a0 * cs.x - b0 * cs.y;
         v[4 * g + 1] = a0 * cs.y + b0 * cs.x;

@@ -16,7 +16,7 @@ namespace fv {
 namespace {
 
 // ---- ids[r] = argmax_v (logits[r, v] + tau * noise[r, v]), lowest v on ties; one warp per row ----
-__global__ void __launch_bounds__(256) argmax_rows_kernel(const float4* __restrict__ logits, const float4* __restrict__ noise, float tau,
+__global__ void __launch_bounds__(256) argmax_rows_kernel(const float4* logits, const float4* noise, float tau,
                                                           int rows, int V4, int32_t* __restrict__ ids) {
   pdl_trigger();
   const int lane = threadIdx.x & 31;
@@ -64,8 +64,8 @@ __global__ void __launch_bounds__(256) argmax_rows_kernel(const float4* __restri
 }
 
 // ---- Eq. 2: r_out[b,t,:] = (r_prev ? r_prev[b, src(t), :] : 0) + codebook[ids[b,t], :] ----
-__global__ void __launch_bounds__(256) residual_accumulate_kernel(const int32_t* __restrict__ ids, const float4* __restrict__ codebook,
-                                                                  const float4* __restrict__ r_prev, int hp, int wp, int B, int h,
+__global__ void __launch_bounds__(256) residual_accumulate_kernel(const int32_t* ids, const float4* codebook,
+                                                                  const float4* r_prev, int hp, int wp, int B, int h,
                                                                   int w, int d4, int V, float4* __restrict__ r_out, int32_t* status) {
   pdl_trigger();
   pdl_wait();
@@ -75,16 +75,16 @@ __global__ void __launch_bounds__(256) residual_accumulate_kernel(const int32_t*
     const int c = (int)(i % d4);
     const long tok = i / d4;
     const int t = (int)(tok % n), b = (int)(tok / n);
-    int id = ids[tok];
+    int id = dep_load(ids + tok);
     if (id < 0 || id >= V) {
       if (status) atomicCAS(status, 0, DEV_BAD_TOKEN_ID);
       id = id < 0 ? 0 : V - 1;
     }
-    float4 f = __ldg(codebook + (size_t)id * d4 + c);
+    float4 f = dep_load4(codebook + (size_t)id * d4 + c);
     if (r_prev) {
       const int y = t / w, x = t - y * w;
       const int src = (int)(((long)y * hp) / h) * wp + (int)(((long)x * wp) / w);
-      const float4 p = r_prev[((size_t)b * hp * wp + src) * d4 + c];
+      const float4 p = dep_load4(r_prev + ((size_t)b * hp * wp + src) * d4 + c);
       f.x += p.x; f.y += p.y; f.z += p.z; f.w += p.w;
     }
     r_out[i] = f;
@@ -106,10 +106,13 @@ __global__ void __launch_bounds__(256) residual_accumulate_kernel(const int32_t*
 // ascending, bias, embedding).
 constexpr int kNextTokens = 64;
 constexpr int kNextChannels = 256;      // one per thread while W_in is staged
-// (r is written by the kernel before this one: without __restrict__ its loads stay behind the dependency wait)
+// Four floats at an address that is 16-byte aligned (vec) or not.
+__device__ __forceinline__ float4 load4_any(const float* p, int vec) {
+  return vec ? dep_load4(p) : make_float4(dep_load(p), dep_load(p + 1), dep_load(p + 2), dep_load(p + 3));
+}
 template <int D>
-__global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int h, int w, int h2, int w2, const float* __restrict__ w_in,
-                                                            const float* __restrict__ b_in, const float* __restrict__ pos, int C, int B, int vec,
+__global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int h, int w, int h2, int w2, const float* w_in,
+                                                            const float* b_in, const float* pos, int C, int B, int vec,
                                                             float* __restrict__ x_out) {
   constexpr int DC = D < 32 ? D : 32;
   __shared__ __align__(16) float w_s[DC][kNextChannels];
@@ -151,7 +154,7 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
 #pragma unroll
       for (int i = 0; i < DC / 4; ++i) {
         q[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c0 + tid < C) q[i] = __ldg(reinterpret_cast<const float4*>(w_in + (size_t)(c0 + tid) * D + d0 + 4 * i));
+        if (c0 + tid < C) q[i] = dep_load4(w_in + (size_t)(c0 + tid) * D + d0 + 4 * i);
       }
 #pragma unroll
       for (int i = 0; i < DC / 4; ++i) { w_s[4 * i][tid] = q[i].x; w_s[4 * i + 1][tid] = q[i].y; w_s[4 * i + 2][tid] = q[i].z; w_s[4 * i + 3][tid] = q[i].w; }
@@ -162,7 +165,7 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
       const long src = row0 + t;
       float v[JP];
 #pragma unroll
-      for (int u = 0; u < JP; ++u) v[u] = src < rows ? r[src * D + d0 + j0 + u] : 0.f;
+      for (int u = 0; u < JP; ++u) v[u] = src < rows ? dep_load(r + src * D + d0 + j0 + u) : 0.f;
 #pragma unroll
       for (int u = 0; u < JP; ++u) r_s[j0 + u][t] = v[u];
     }
@@ -193,7 +196,7 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
     const int c = g ? cb : ca;
-    bias[g] = b_in && c < C ? make_float4(__ldg(b_in + c), __ldg(b_in + c + 1), __ldg(b_in + c + 2), __ldg(b_in + c + 3)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    bias[g] = b_in && c < C ? load4_any(b_in + c, 0) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
@@ -211,8 +214,8 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
         pa[u] = pb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (pos && k0 + u < cnt) {
           const float* q = pos + (size_t)t2[u] * C;
-          if (ca < C) pa[u] = vec ? __ldg(reinterpret_cast<const float4*>(q + ca)) : make_float4(__ldg(q + ca), __ldg(q + ca + 1), __ldg(q + ca + 2), __ldg(q + ca + 3));
-          if (cb < C) pb[u] = vec ? __ldg(reinterpret_cast<const float4*>(q + cb)) : make_float4(__ldg(q + cb), __ldg(q + cb + 1), __ldg(q + cb + 2), __ldg(q + cb + 3));
+          if (ca < C) pa[u] = load4_any(q + ca, vec);
+          if (cb < C) pb[u] = load4_any(q + cb, vec);
         }
       }
 #pragma unroll

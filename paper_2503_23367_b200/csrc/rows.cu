@@ -23,9 +23,9 @@ constexpr int kMaxVec = 16;  // float4 per lane -> C <= 2048
 // grid (ceil(k / 8), B): one warp per kept row; sigma / beta of the image staged in shared memory while
 // the row itself is in flight.
 template <typename XT>
-__global__ void __launch_bounds__(256) gather_ln_kernel(const XT* __restrict__ x, const int32_t* __restrict__ idx, int n,
-                                                        int k, int C4, const float* __restrict__ sigma,
-                                                        const float* __restrict__ beta, int mod_stride,
+__global__ void __launch_bounds__(256) gather_ln_kernel(const XT* x, const int32_t* idx, int n,
+                                                        int k, int C4, const float* sigma,
+                                                        const float* beta, int mod_stride,
                                                         uint2* __restrict__ a_out, int32_t* status) {
   extern __shared__ float4 s_mod[];  // sigma [C4] then beta [C4]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256) gather_ln_kernel(const XT* __restrict__ x
   const bool live = j < k;
   pdl_trigger();
   pdl_wait();
-  int t = live ? (idx ? __ldg(idx + (size_t)b * k + j) : j) : 0;
+  int t = live ? (idx ? dep_load(idx + (size_t)b * k + j) : j) : 0;
   if (t < 0 || t >= n) {   // a caller's index outside the map: stay inside it and say so
     if (status && lane == 0) atomicCAS(status, 0, DEV_BAD_ROW_INDEX);
     t = min(max(t, 0), n - 1);
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256) gather_ln_kernel(const XT* __restrict__ x
   if (sigma) {   // behind the wait (the kernel before may have produced them) and behind the row's loads, which they then travel beside
     const float4* sg = reinterpret_cast<const float4*>(sigma + (size_t)b * mod_stride);
     const float4* bt = reinterpret_cast<const float4*>(beta + (size_t)b * mod_stride);
-    for (int i = threadIdx.x; i < C4; i += 256) { s_mod[i] = __ldg(sg + i); s_mod[C4 + i] = __ldg(bt + i); }
+    for (int i = threadIdx.x; i < C4; i += 256) { s_mod[i] = dep_load4(sg + i); s_mod[C4 + i] = dep_load4(bt + i); }
   }
   if (live) {
 #pragma unroll
@@ -172,9 +172,9 @@ __device__ __forceinline__ void bf16x8_to_float(const uint4& p, float (&f)[8]) {
 //   summed, by the next selection's kernel).
 // RF: rows in flight per thread (4, or 2 in the build that fits four CTAs per SM: 64 registers).
 template <typename XT, int RF>
-__global__ void __launch_bounds__(256, RF == 2 ? 4 : 3) restore_residual_kernel(XT* __restrict__ x, const uint4* __restrict__ y,
-                                                               const uint4* __restrict__ cache, const int32_t* __restrict__ inv,
-                                                               const float* __restrict__ gamma, int mod_stride, int n, int k,
+__global__ void __launch_bounds__(256, RF == 2 ? 4 : 3) restore_residual_kernel(XT* x, const uint4* y,
+                                                               const uint4* cache, const int32_t* inv,
+                                                               const float* gamma, int mod_stride, int n, int k,
                                                                int h, int w, int hc, int wc, int C8, int nchunks, int group,
                                                                int ngroups, float4* __restrict__ chunk_partial,
                                                                float4* __restrict__ group_partial, unsigned int* tickets,
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(256, RF == 2 ? 4 : 3) restore_residual_kernel(
   const int rows = min(kColsumRows, n - t0);
   if (threadIdx.x < rows) {
     const int t = t0 + threadIdx.x;
-    const int j = __ldg(inv + (size_t)b * n + t);
+    const int j = dep_load(inv + (size_t)b * n + t);
     s_src[threadIdx.x] = (j >= 0) ? y + ((size_t)b * k + j) * C8
                                   : cache + ((size_t)b * hc * wc + nearest_src(t, h, w, hc, wc)) * C8;
     s_on[threadIdx.x] = part == 0 || (part == 1 || part == 3) == (j < 0);
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(256, RF == 2 ? 4 : 3) restore_residual_kernel(
     float4 g0 = make_float4(1.f, 1.f, 1.f, 1.f), g1 = g0;
     if (gamma) {
       const float4* g = reinterpret_cast<const float4*>(gamma + (size_t)b * mod_stride);
-      g0 = __ldg(g + 2 * c8); g1 = __ldg(g + 2 * c8 + 1);
+      g0 = dep_load4(g + 2 * c8); g1 = dep_load4(g + 2 * c8 + 1);
     }
     float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
     if (part == 2 && chunk_partial) {  // continue the sums of the rows updated by part 1
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(256, RF == 2 ? 4 : 3) restore_residual_kernel(
       for (int i = 0; i < RF; ++i) {
         if (r + i < rows && s_on[r + i]) {
           x_load8(xbase + ((size_t)(r + i) * C8 + c8) * 8, xv[i]);
-          p[i] = __ldg(s_src[r + i] + c8);
+          p[i] = dep_load16(s_src[r + i] + c8);
         }
       }
 #pragma unroll
@@ -244,29 +244,42 @@ __global__ void __launch_bounds__(256, RF == 2 ? 4 : 3) restore_residual_kernel(
     fold_group_partials(b, chunk, nchunks, group, ngroups, C8 * 2, chunk_partial, group_partial, tickets);
 }
 
+// One fp32 row by one warp, up to eight 16-byte loads per lane requested before the first store.
+__device__ __forceinline__ void copy_row_f32(float4* dst, const float4* src, int C4, int lane) {
+  for (int c0 = lane; c0 < C4; c0 += 256) {
+    float4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (c0 + 32 * u < C4) v[u] = dep_load4(src + c0 + 32 * u);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (c0 + 32 * u < C4) dst[c0 + 32 * u] = v[u];
+  }
+}
+
 // Per-step granularity: compact copy of the kept rows of the fp32 token map (Algorithm 1's gather).
 // grid (ceil(k / 8), B): one warp per kept row.
-__global__ void __launch_bounds__(256) gather_rows_kernel(const float4* __restrict__ x, const int32_t* __restrict__ idx, int n,
+__global__ void __launch_bounds__(256) gather_rows_kernel(const float4* x, const int32_t* idx, int n,
                                                           int k, int C4, float4* __restrict__ out, int32_t* status) {
   pdl_trigger();
   pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.y, j = blockIdx.x * 8 + warp;
   if (j >= k) return;
-  int t = __ldg(idx + (size_t)b * k + j);
+  int t = dep_load(idx + (size_t)b * k + j);
   if (t < 0 || t >= n) {
     if (status && lane == 0) atomicCAS(status, 0, DEV_BAD_ROW_INDEX);
     t = min(max(t, 0), n - 1);
   }
   const float4* src = x + ((size_t)b * n + t) * C4;
   float4* dst = out + ((size_t)b * k + j) * C4;
-  for (int c4 = lane; c4 < C4; c4 += 32) dst[c4] = __ldg(src + c4);
+  copy_row_f32(dst, src, C4, lane);
 }
 
 // Per-step granularity: Cached Token Restoration of the step's output map (Eq. 6), fp32, a copy:
 // out[b,t,:] = inv[b,t] >= 0 ? pivots[b, inv[b,t], :] : cache[b, src(t), :].
-__global__ void __launch_bounds__(256) restore_rows_f32_kernel(const float4* __restrict__ cache, int hc, int wc,
-                                                               const float4* __restrict__ pivots, const int32_t* __restrict__ inv,
+__global__ void __launch_bounds__(256) restore_rows_f32_kernel(const float4* cache, int hc, int wc,
+                                                               const float4* pivots, const int32_t* inv,
                                                                int n, int k, int h, int w, int C4, float4* __restrict__ out,
                                                                int total_rows) {
   pdl_trigger();
@@ -274,11 +287,11 @@ __global__ void __launch_bounds__(256) restore_rows_f32_kernel(const float4* __r
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= total_rows) return;
   const int b = warp / n, t = warp - b * n;
-  const int j = __ldg(inv + warp);
+  const int j = dep_load(inv + warp);
   const float4* src = (j >= 0) ? pivots + ((size_t)b * k + j) * C4
                                : cache + ((size_t)b * hc * wc + nearest_src(t, h, w, hc, wc)) * C4;
   float4* dst = out + (size_t)warp * C4;
-  for (int c4 = lane; c4 < C4; c4 += 32) dst[c4] = __ldg(src + c4);
+  copy_row_f32(dst, src, C4, lane);
 }
 
 
@@ -389,9 +402,9 @@ __global__ void __launch_bounds__(256) restore_kept_cluster_kernel(float4* __res
 // and column-sum handling; fewer rows in flight (two, or one with sixteen source rows).  part 2 (kept rows only) never interpolates and
 // runs the kernel above.
 template <int TAPS>
-__global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* __restrict__ xf, const uint4* __restrict__ y,
-                                                                        const uint4* __restrict__ cache, const int32_t* __restrict__ inv,
-                                                                        const float* __restrict__ gamma, int mod_stride, int n, int k,
+__global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* xf, const uint4* y,
+                                                                        const uint4* cache, const int32_t* inv,
+                                                                        const float* gamma, int mod_stride, int n, int k,
                                                                         int h, int w, int hc, int wc, int C8, int nchunks, int group,
                                                                         int ngroups, float4* __restrict__ chunk_partial,
                                                                         float4* __restrict__ group_partial, unsigned int* tickets,
@@ -408,7 +421,7 @@ __global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* __r
   const int rows = min(kColsumRows, n - t0);
   if (threadIdx.x < rows) {
     const int t = t0 + threadIdx.x;
-    const int j = __ldg(inv + (size_t)b * n + t);
+    const int j = dep_load(inv + (size_t)b * n + t);
     if (j >= 0) {
       for (int q = 0; q < TAPS; ++q) { s_src[threadIdx.x][q] = y + ((size_t)b * k + j) * C8; s_wt[threadIdx.x][q] = q == 0 ? 1.f : 0.f; }
     } else {
@@ -423,7 +436,7 @@ __global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* __r
     float4 g0 = make_float4(1.f, 1.f, 1.f, 1.f), g1 = g0;
     if (gamma) {
       const float4* g = reinterpret_cast<const float4*>(gamma + (size_t)b * mod_stride);
-      g0 = __ldg(g + 2 * c8); g1 = __ldg(g + 2 * c8 + 1);
+      g0 = dep_load4(g + 2 * c8); g1 = dep_load4(g + 2 * c8 + 1);
     }
     float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
     for (int r = 0; r < rows; r += ROWS) {
@@ -435,7 +448,7 @@ __global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* __r
           float4* xr = xbase + (size_t)(r + i) * C8 * 2 + 2 * c8;
           x0[i] = xr[0]; x1[i] = xr[1];
 #pragma unroll
-          for (int q = 0; q < TAPS; ++q) p[i][q] = __ldg(s_src[r + i][q] + c8);
+          for (int q = 0; q < TAPS; ++q) p[i][q] = dep_load16(s_src[r + i][q] + c8);
         }
       }
 #pragma unroll
@@ -475,8 +488,8 @@ __global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* __r
 // (2 x 64 x 64 tokens, k 820, C 2048: 2.2 + 2.3 + 8.5 us and two more launches of the host).  A warp takes a row at a time, up to eight
 // 16-byte loads per lane in flight.
 template <int TAPS, int RT>
-__global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* __restrict__ cache, int hc, int wc, const uint4* __restrict__ pivots,
-                                                           const int32_t* __restrict__ idx, int n, int k, int h, int w, int C8, uint4* __restrict__ out) {
+__global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* cache, int hc, int wc, const uint4* pivots,
+                                                           const int32_t* idx, int n, int k, int h, int w, int C8, uint4* __restrict__ out) {
   __shared__ int s_slot[RT];
   const int b = blockIdx.y, t0 = blockIdx.x * RT;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -488,7 +501,7 @@ __global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* __restri
   for (int i0 = threadIdx.x; i0 < k; i0 += 256 * 8) {
     int v[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = i0 + 256 * u < k ? __ldg(ib + i0 + 256 * u) - t0 : -1;
+    for (int u = 0; u < 8; ++u) v[u] = i0 + 256 * u < k ? dep_load(ib + i0 + 256 * u) - t0 : -1;
 #pragma unroll
     for (int u = 0; u < 8; ++u)
       if (v[u] >= 0 && v[u] < RT) s_slot[v[u]] = i0 + 256 * u;
@@ -505,7 +518,7 @@ __global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* __restri
         uint4 v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if (c0 + 32 * u < C8) v[u] = __ldg(src + c0 + 32 * u);
+          if (c0 + 32 * u < C8) v[u] = dep_load16(src + c0 + 32 * u);
 #pragma unroll
         for (int u = 0; u < 8; ++u)
           if (c0 + 32 * u < C8) dst[c0 + 32 * u] = v[u];
@@ -520,7 +533,7 @@ __global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* __restri
 #pragma unroll
         for (int q = 0; q < TAPS; ++q) {
           float fq[8];
-          bf16x8_to_float(__ldg(base + (size_t)bt.src[q] * C8 + c8), fq);
+          bf16x8_to_float(dep_load16(base + (size_t)bt.src[q] * C8 + c8), fq);
 #pragma unroll
           for (int e = 0; e < 8; ++e) f[e] = fmaf(bt.wt[q], fq[e], f[e]);
         }
@@ -533,8 +546,8 @@ __global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* __restri
 }
 
 template <int TAPS>
-__global__ void __launch_bounds__(256) restore_rows_f32_interp_kernel(const float4* __restrict__ cache, int hc, int wc,
-                                                                        const float4* __restrict__ pivots, const int32_t* __restrict__ inv,
+__global__ void __launch_bounds__(256) restore_rows_f32_interp_kernel(const float4* cache, int hc, int wc,
+                                                                        const float4* pivots, const int32_t* inv,
                                                                         int n, int k, int h, int w, int C4, float4* __restrict__ out,
                                                                         int total_rows) {
   pdl_trigger();
@@ -542,11 +555,11 @@ __global__ void __launch_bounds__(256) restore_rows_f32_interp_kernel(const floa
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= total_rows) return;
   const int b = warp / n, t = warp - b * n;
-  const int j = __ldg(inv + warp);
+  const int j = dep_load(inv + warp);
   float4* dst = out + (size_t)warp * C4;
   if (j >= 0) {
     const float4* src = pivots + ((size_t)b * k + j) * C4;
-    for (int c4 = lane; c4 < C4; c4 += 32) dst[c4] = __ldg(src + c4);
+    copy_row_f32(dst, src, C4, lane);
     return;
   }
   const InterpTaps<TAPS> bt = interp_taps<TAPS>(t, h, w, hc, wc);
@@ -555,7 +568,7 @@ __global__ void __launch_bounds__(256) restore_rows_f32_interp_kernel(const floa
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int q = 0; q < TAPS; ++q) {
-      const float4 v = __ldg(base + (size_t)bt.src[q] * C4 + c4);
+      const float4 v = dep_load4(base + (size_t)bt.src[q] * C4 + c4);
       acc.x = fmaf(bt.wt[q], v.x, acc.x); acc.y = fmaf(bt.wt[q], v.y, acc.y); acc.z = fmaf(bt.wt[q], v.z, acc.z); acc.w = fmaf(bt.wt[q], v.w, acc.w);
     }
     dst[c4] = acc;

@@ -44,7 +44,7 @@ __device__ __forceinline__ float4 x_load4_hint(const __nv_bfloat16* p, uint64_t 
   return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
 }
 template <typename XT>
-__global__ void __launch_bounds__(256) colsum_chunk_kernel(const XT* __restrict__ x, int n, int C4, int nchunks, float4* __restrict__ chunk_partial) {
+__global__ void __launch_bounds__(256) colsum_chunk_kernel(const XT* x, int n, int C4, int nchunks, float4* __restrict__ chunk_partial) {
   pdl_trigger();
   pdl_wait();
   const int b = blockIdx.y, chunk = blockIdx.x, c4 = blockIdx.z * 256 + threadIdx.x;
@@ -498,8 +498,8 @@ __device__ __forceinline__ void topk_image(const float* __restrict__ sc, int n, 
 // latencies of its sweeps with); the warps of an image stride over its token rows.  Dynamic shared memory
 // max(9 C, n) * 4 bytes (mean token and staged partial sums, then keys).
 template <typename XT>
-__global__ void __launch_bounds__(kSelectThreads, 1) score_topk_kernel(const XT* __restrict__ x,
-                                                                  const float4* __restrict__ group_partial, int ngroups, int n,
+__global__ void __launch_bounds__(kSelectThreads, 1) score_topk_kernel(const XT* x,
+                                                                  const float4* group_partial, int ngroups, int n,
                                                                   int C4, int k, int staged, float* __restrict__ score,
                                                                   unsigned int* img_tickets, unsigned int* img_range, int32_t* __restrict__ idx,
                                                                   int32_t* __restrict__ inv, int32_t* __restrict__ near_tie) {
@@ -667,7 +667,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) select_fused_kernel(const Fus
       float4 g0 = make_float4(1.f, 1.f, 1.f, 1.f), g1 = g0;
       if (a.gamma_prev) {
         const float4* g = reinterpret_cast<const float4*>(a.gamma_prev + (size_t)b * a.mod_stride);
-        g0 = __ldg(g + 2 * c8); g1 = __ldg(g + 2 * c8 + 1);
+        g0 = dep_load4(g + 2 * c8); g1 = dep_load4(g + 2 * c8 + 1);
       }
       const int stride = G * rows_par;
       const int32_t* ip = a.idx_prev + (size_t)b * a.k_prev;
@@ -676,15 +676,15 @@ __global__ void __launch_bounds__(kTopkThreads, 1) select_fused_kernel(const Fus
       for (int j = cta + G * rp; j < a.k_prev; j += 2 * stride) {     // two rows in flight
         const int j2 = j + stride;
         const bool two = j2 < a.k_prev;
-        const int t1 = min(max(__ldg(ip + j), 0), n - 1);
-        const int t2 = two ? min(max(__ldg(ip + j2), 0), n - 1) : t1;
+        const int t1 = min(max(dep_load(ip + j), 0), n - 1);
+        const int t2 = two ? min(max(dep_load(ip + j2), 0), n - 1) : t1;
         float4* xr1 = xb + (size_t)t1 * C4 + 2 * c8;
         float4* xr2 = xb + (size_t)t2 * C4 + 2 * c8;
         float4 u0 = xr1[0], u1 = xr1[1];
-        const uint4 p1 = __ldg(yb + (size_t)j * C8 + c8);
+        const uint4 p1 = dep_load16(yb + (size_t)j * C8 + c8);
         float4 w0 = u0, w1 = u1;
         uint4 p2 = p1;
-        if (two) { w0 = xr2[0]; w1 = xr2[1]; p2 = __ldg(yb + (size_t)j2 * C8 + c8); }
+        if (two) { w0 = xr2[0]; w1 = xr2[1]; p2 = dep_load16(yb + (size_t)j2 * C8 + c8); }
         float f[8];
         bf16x8_widen(p1, f);
         if (a.gamma_prev) {
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) select_fused_kernel(const Fus
     s_sigma = s_dyn; s_beta = s_dyn + C4;
     const float4* sg = reinterpret_cast<const float4*>(a.sigma + (size_t)b * a.mod_stride);
     const float4* bt = reinterpret_cast<const float4*>(a.beta + (size_t)b * a.mod_stride);
-    for (int i = tid; i < C4; i += kTopkThreads) { s_sigma[i] = __ldg(sg + i); s_beta[i] = __ldg(bt + i); }
+    for (int i = tid; i < C4; i += kTopkThreads) { s_sigma[i] = dep_load4(sg + i); s_beta[i] = dep_load4(bt + i); }
   }
   if (!last) {
     if (tid == 0) {
@@ -805,13 +805,13 @@ __global__ void inv_fill_kernel(int32_t* inv, size_t total) {
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < total) inv[i] = -1;
 }
-__global__ void inv_scatter_kernel(const int32_t* __restrict__ idx, int B, int k, int n, int32_t* __restrict__ inv) {
+__global__ void inv_scatter_kernel(const int32_t* idx, int B, int k, int n, int32_t* __restrict__ inv) {
   pdl_trigger();
   pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * k) return;
   int b = i / k, j = i - b * k;
-  int t = idx[i];
+  int t = dep_load(idx + i);
   if (t >= 0 && t < n) inv[(size_t)b * n + t] = j;
 }
 

@@ -120,3 +120,58 @@ def test_next_token_map_with_w_in_written_by_the_kernel_before(d):
     w_in = _LongGemm(C, d, torch.float32)
     r, b_in, pos = _randn(6, 2, 36, d), _randn(7, C), _randn(8, 64, C)
     _check_in_order(w_in, lambda: fv.fv_next_scale_input(r, 6, 6, 8, 8, w_in.out, b_in, pos), w_in.renew)
+
+
+class _Selection:
+    """The library's selection into the caller's buffers, on a map that changes from round to round."""
+
+    def __init__(self, B, h, w, C, keep):
+        self.B, self.h, self.w, self.C, self.keep = B, h, w, C, keep
+        self.k = fv.fv_k_for(keep, h, w)
+        self.x = torch.empty(B, h * w, C, device=DEV)
+        self.idx = torch.zeros(B, self.k, dtype=torch.int32, device=DEV)
+        self.ws = fv.fv_prune_select_workspace(B, h * w, C, DEV)
+
+    def renew(self, i):
+        self.x.copy_(_randn(40 + i, self.B, self.h * self.w, self.C))
+        self.idx.copy_(torch.arange(self.k, dtype=torch.int32, device=DEV).expand(self.B, -1))
+
+    def __call__(self):
+        rc = fv.lib().fv_prune_select(self.x.data_ptr(), self.B, self.h, self.w, self.C, self.keep, self.idx.data_ptr(), None, None, None, None,
+                                      self.ws.data_ptr(), self.ws.numel(), torch.cuda.current_stream().cuda_stream)
+        assert rc == 0
+
+
+@pytest.mark.parametrize("B,h,w,C,keep", [(2, 12, 12, 256, 0.4), (1, 64, 64, 2048, 0.2)])
+@pytest.mark.parametrize("interp", [0, 1, 2])
+def test_restoration_of_indices_written_by_the_kernel_before(B, h, w, C, keep, interp):
+    sel = _Selection(B, h, w, C, keep)
+    cache, pivots = _randn(50, B, (h // 2) * (w // 2), C, dtype=torch.bfloat16), _randn(51, B, sel.k, C, dtype=torch.bfloat16)
+    _check_in_order(sel, lambda: fv.fv_restore(cache, h // 2, w // 2, pivots, sel.idx, h, w, interp_mode=interp), sel.renew)
+
+
+def test_gather_of_indices_written_by_the_kernel_before():
+    sel = _Selection(2, 40, 40, 1024, 0.3)
+    _check_in_order(sel, lambda: fv.fv_gather_ln(sel.x, sel.idx, None, None), sel.renew)
+
+
+def test_restoration_of_rows_written_by_the_kernel_before():
+    B, h, w, C, k = 2, 12, 12, 512, 48
+    pivots = _LongGemm(B * k, C, torch.bfloat16)
+    cache = _randn(52, B, 36, C, dtype=torch.bfloat16)
+    idx = torch.arange(0, 3 * k, 3, dtype=torch.int32, device=DEV).expand(B, -1).contiguous()
+    _check_in_order(pivots, lambda: fv.fv_restore(cache, 6, 6, pivots.out.view(B, k, C), idx, h, w), pivots.renew)
+
+
+def test_residual_and_next_map_of_tokens_written_by_the_kernel_before():
+    """Head logits -> ids -> Eq. 2 -> next map, each kernel the producer of the next."""
+    B, h, w, V, d, C = 2, 16, 16, 1024, 32, 512
+    logits = _LongGemm(B * h * w, V, torch.float32, K=2048)
+    codebook, r_prev, w_in = _randn(60, V, d), _randn(61, B, 64, d), _randn(62, C, d)
+
+    def consume():
+        ids = fv.fv_argmax_rows(logits.out).view(B, h * w)
+        r = fv.fv_residual_accumulate(ids, h, w, codebook, r_prev, 8, 8)
+        return ids, r, fv.fv_next_scale_input(r, h, w, 20, 20, w_in, None, None)
+
+    _check_in_order(logits, consume, logits.renew)
