@@ -156,7 +156,7 @@ cudaError_t select_init();  // one-time function attributes
 struct SmallSelect {
   void* x; bool x_bf16; int B, n, C, k, h, w, hc, wc, mod_stride;
   const void* y; const void* cache; const int32_t* inv_prev; const float* gamma_prev;   // the previous sublayer's; y null: nothing to restore
-  int32_t* idx; int32_t* inv; float* score;                                             // written (inv is not inv_prev; inv, score may be null)
+  int32_t* idx; int32_t* inv; float* score; int32_t* near_tie;                          // written (inv is not inv_prev; all but idx may be null)
   const float* sigma; const float* beta; void* a_out;                                   // a_out null: no gather
 };
 cudaError_t select_small_init();

@@ -901,10 +901,10 @@ static cudaError_t launch_select_t(const XT* x, int B, int n, int C, int k, int3
 
 cudaError_t launch_select(const void* x, int B, int n, int C, int k, int32_t* idx, int32_t* inv, float* score,
                           int32_t* near_tie, void* workspace, bool have_partials, cudaStream_t st, bool x_bf16) {
-  if (!have_partials && !near_tie && select_small_supported(B, n, C, x_bf16)) {   // one launch, no scratch
+  if (!have_partials && select_small_supported(B, n, C, x_bf16)) {   // one launch, no scratch
     SmallSelect f{};
     f.x = const_cast<void*>(x); f.x_bf16 = x_bf16; f.B = B; f.n = n; f.C = C; f.k = k; f.h = 1; f.w = n; f.hc = 1; f.wc = 1;
-    f.idx = idx; f.inv = inv; f.score = score;
+    f.idx = idx; f.inv = inv; f.score = score; f.near_tie = near_tie;
     return launch_select_small(f, st);
   }
   const SelectWs w = select_ws_carve(workspace, B, n, C);

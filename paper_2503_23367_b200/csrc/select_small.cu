@@ -25,6 +25,7 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kRows = 8;              // rows of a chunk per thread
 constexpr int kMaxCluster = 16;
+static_assert(2 * kWarps <= kRows * kWarps, "the near-tie count reduces in the words of the partial scores");
 static_assert(2048 / 4 <= kThreads, "one thread per four channels");
 
 struct SmallArgs {
@@ -36,6 +37,7 @@ struct SmallArgs {
   int n, C, k, h, w, hc, wc, mod_stride;
   int32_t *idx, *inv;
   float* score;                       // [B, n] or null
+  int32_t* near_tie;                  // [B] or null
   const float *sigma, *beta;
   uint2* a_out;
   int rows_per_cta;                   // R
@@ -306,6 +308,26 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
       if (pos >= 0) a.idx[(size_t)b * a.k + pos] = t;
     }
   }
+  if (a.near_tie && rank == 0) {   // tokens within 1e-5 of the threshold, the smallest kept key (all keys and flags are here)
+    uint32_t* r = reinterpret_cast<uint32_t*>(red);
+    uint32_t tau = 0xFFFFFFFFu;
+    for (int j = tid; j < n; j += kThreads)
+      if (flags[j]) tau = min(tau, keys[j]);
+    tau = __reduce_min_sync(0xffffffffu, tau);
+    if (lane == 0) r[warp] = tau;
+    __syncthreads();
+    for (int w = 0; w < kWarps; ++w) tau = min(tau, r[w]);
+    const float tau_f = __uint_as_float(tau), band = 1e-5f * tau_f;
+    uint32_t near = 0;
+    for (int j = tid; j < n; j += kThreads) near += fabsf(__uint_as_float(keys[j]) - tau_f) <= band;
+    near = __reduce_add_sync(0xffffffffu, near);
+    if (lane == 0) r[kWarps + warp] = near;
+    __syncthreads();
+    if (tid == 0) {
+      for (int w = 1; w < kWarps; ++w) near += r[kWarps + w];
+      a.near_tie[b] = (int32_t)near;
+    }
+  }
   if (!a.a_out) return;        // a selection alone
   __syncthreads();
 
@@ -400,7 +422,7 @@ cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st) {
   SmallArgs a{};
   a.x = f.x; a.y = static_cast<const uint4*>(f.y); a.cache = static_cast<const uint4*>(f.cache); a.inv_prev = f.inv_prev; a.gamma_prev = f.gamma_prev;
   a.n = f.n; a.C = f.C; a.k = f.k; a.h = f.h; a.w = f.w; a.hc = f.hc; a.wc = f.wc; a.mod_stride = f.mod_stride;
-  a.idx = f.idx; a.inv = f.inv; a.score = f.score; a.sigma = f.sigma; a.beta = f.beta; a.a_out = static_cast<uint2*>(f.a_out);
+  a.idx = f.idx; a.inv = f.inv; a.score = f.score; a.near_tie = f.near_tie; a.sigma = f.sigma; a.beta = f.beta; a.a_out = static_cast<uint2*>(f.a_out);
   a.rows_per_cta = (f.n + cl - 1) / cl;
   // algorithmic bytes: the map read (and written where it is restored from y and the cache), indices, the kept rows' bf16 copy
   const double es = f.x_bf16 ? 2.0 : 4.0;

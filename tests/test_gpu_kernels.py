@@ -130,6 +130,25 @@ def test_prune_select_small_maps_in_one_launch(B, h, w, C, keep, kind):
         assert np.array_equal(r["inv"].cpu().numpy().astype(np.int64), O.inverse_map(idx_g, h * w))
 
 
+@pytest.mark.parametrize("B,h,w,C,keep", [(2, 12, 12, 256, 0.4), (3, 13, 18, 1920, 0.6), (20, 8, 9, 128, 0.3), (1, 16, 15, 2048, 1.0), (2, 64, 64, 256, 0.2)])
+def test_prune_select_near_tie_count_leaves_the_selection_alone(B, h, w, C, keep):
+    """Scores a few ulps apart around the threshold: asking for the count changes neither scores nor kept set, and it counts those very scores."""
+    n = h * w
+    x = np.repeat(I.normal(7, (1, 1, C)), n, axis=1) * np.where(np.arange(n) % 2, 1.0, -1.0)[None, :, None]
+    x = np.repeat(x * (1.0 + np.arange(n)[None, :, None] % 50 * 2.0 ** -21), B, axis=0).astype(np.float32)
+    x += I.normal(8, (B, n, C)).astype(np.float32) * 1e-6
+    plain = fv.fv_prune_select(dev(x), h, w, keep, want_inv=True, want_score=True)
+    counted = fv.fv_prune_select(dev(x), h, w, keep, want_inv=True, want_score=True, want_near_tie=True)
+    torch.cuda.synchronize()
+    for key in ("score", "idx", "inv"):
+        assert torch.equal(plain[key], counted[key]), key
+    s = plain["score"].cpu().numpy()
+    tau = np.sort(s, axis=1)[:, ::-1][:, plain["k"] - 1][:, None]
+    want = (np.abs(s - tau) <= np.float32(1e-5) * tau).sum(axis=1)
+    assert np.array_equal(counted["near_tie"].cpu().numpy(), want)
+    assert (want > 1).all()
+
+
 def test_prune_select_argument_errors():
     big = torch.zeros((1, 193 * 256, 8), device=DEV)                      # one row of tokens beyond the largest map
     with pytest.raises(fv.FvError) as e:
