@@ -5,6 +5,7 @@
 // the small d -> C map (d <= 64: a dot product per output element, no tensor-core shape).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <climits>
 #include <cstdint>
 #include <vector>
@@ -104,49 +105,74 @@ __global__ void __launch_bounds__(256) residual_accumulate_kernel(const int32_t*
 // and with one channel per thread 73.  Two rounds of CTAs, each a chain of loads (embedding rows 11 us in all), products (8) and
 // stores (6); CTAs of 32 or 16 tokens, four or eight to an SM, do not overlap them better (40, 52).  The additions keep their order (j
 // ascending, bias, embedding).
-constexpr int kNextTokens = 64;
+// TW: tokens per warp.  One instead of eight where tiles of 64 tokens leave the GPU to a few CTAs, each of which then takes its warps' tokens one
+// after the other: MEASURED
 constexpr int kNextChannels = 256;      // one per thread while W_in is staged
 // Four floats at an address that is 16-byte aligned (vec) or not.
 __device__ __forceinline__ float4 load4_any(const float* p, int vec) {
   return vec ? dep_load4(p) : make_float4(dep_load(p), dep_load(p + 1), dep_load(p + 2), dep_load(p + 3));
 }
-template <int D>
+template <int D, int TW>
 __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int h, int w, int h2, int w2, const float* w_in,
-                                                            const float* b_in, const float* pos, int C, int B, int vec,
+                                                            const float* b_in, const float* pos, int C, int B, int vec, int slice,
                                                             float* __restrict__ x_out) {
   constexpr int DC = D < 32 ? D : 32;
+  constexpr int kNextTokens = 8 * TW;
   __shared__ __align__(16) float w_s[DC][kNextChannels];
   __shared__ __align__(16) float r_s[DC][kNextTokens];
   __shared__ int s_first[kNextTokens], s_nx[kNextTokens], s_cnt[kNextTokens];   // a token's copies: first one, copies per row of the next map, all
-  __shared__ long s_img[kNextTokens];    // first row of its image in x_out
+  __shared__ long s_img[kNextTokens], s_row[kNextTokens];                       // first row of its image in x_out; its row of r, or -1
   pdl_trigger();
-  const int n = h * w, n2 = h2 * w2;
-  const long rows = (long)B * n;
-  const long row0 = (long)blockIdx.y * kNextTokens;
-  const int c0 = blockIdx.x * kNextChannels;
+  const int hu = min(h, h2), wu = min(w, w2), nu = hu * wu;   // along an axis that shrinks only the tokens that have a target take part
+  const long rows = (long)B * nu;
+  const int cblocks = (C + kNextChannels - 1) / kNextChannels;
+  const long row0 = (long)(blockIdx.x / cblocks) * kNextTokens;
+  const int c0 = (int)(blockIdx.x % cblocks) * kNextChannels;
   const int tid = threadIdx.x;
   if (tid < kNextTokens) {   // token (y, x) is the source of the targets y2 with floor(y2 h / h2) = y, and x2 likewise
     const long row = row0 + tid;
     int first = 0, nx = 0, ny = 0;
+    long src = -1;
     if (row < rows) {
-      const int b = (int)row / n, t = (int)row - b * n, y = t / w, x = t - y * w;   // (32 bits: the launcher checks)
-      const int y0 = (y * h2 + h - 1) / h, x0 = (x * w2 + w - 1) / w;
-      ny = ((y + 1) * h2 + h - 1) / h - y0;
-      nx = ((x + 1) * w2 + w - 1) / w - x0;
+      const int b = (int)(row / nu), t = (int)(row - (long)b * nu), i = t / wu, j = t - i * wu;
+      const int y0 = h2 <= h ? i : (int)(((long)i * h2 + h - 1) / h), x0 = w2 <= w ? j : (int)(((long)j * w2 + w - 1) / w);
+      ny = h2 <= h ? 1 : (int)(((long)(i + 1) * h2 + h - 1) / h) - y0;
+      nx = w2 <= w ? 1 : (int)(((long)(j + 1) * w2 + w - 1) / w) - x0;
       first = y0 * w2 + x0;
-      s_img[tid] = (long)b * n2;
+      src = (long)b * h * w + (h2 <= h ? (long)i * h / h2 : i) * w + (w2 <= w ? (long)j * w / w2 : j);
+      s_img[tid] = (long)b * h2 * w2;
     }
-    s_first[tid] = first; s_nx[tid] = nx; s_cnt[tid] = nx * ny;
+    s_first[tid] = first; s_nx[tid] = nx; s_cnt[tid] = nx * ny; s_row[tid] = src;
   }
-  uint64_t acc2[8][4];   // channel pairs
+  uint64_t acc2[TW][4];   // channel pairs
 #pragma unroll
-  for (int t = 0; t < 8; ++t)
+  for (int t = 0; t < TW; ++t)
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc2[t][e] = 0ull;
   const int lane = tid & 31, warp = tid >> 5;
-  const int tl = warp * 8;               // this thread's tokens inside the tile; its channels are 4 lane .. and 128 + 4 lane ..
+  const int tl = warp * TW;              // this thread's tokens inside the tile; its channels are 4 lane .. and 128 + 4 lane ..
+  const int ca = c0 + 4 * lane, cb = ca + 128;
   __syncthreads();
   pdl_wait();                            // W_in, b_in and pos are the caller's like r: any of them may come from the kernel before
+  // embedding rows of the copies k0 and k0 + 1 of a token
+  float4 pa[2], pb[2];
+  int t2[2];
+  auto fetch = [&](int k0, int cnt, int nx, int first) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int d = min(k0 + u, cnt - 1), yy = d / nx;
+      t2[u] = first + yy * w2 + (d - yy * nx);
+      pa[u] = pb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (pos && k0 + u < cnt) {
+        const float* q = pos + (size_t)t2[u] * C;
+        if (ca < C) pa[u] = load4_any(q + ca, vec);
+        if (cb < C) pb[u] = load4_any(q + cb, vec);
+      }
+    }
+  };
+  const int k_first = (int)blockIdx.y * slice;   // this slice's copies
+  auto k_end = [&](int t) { return (int)min((long)s_cnt[tl + t], ((long)blockIdx.y + 1) * slice); };
+  if (TW == 1 && k_first < k_end(0)) fetch(k_first, k_end(0), s_nx[tl], s_first[tl]);   // on their way beside W_in and r
   for (int d0 = 0; d0 < D; d0 += DC) {
     if (d0) __syncthreads();             // the chunk before has been used
     {   // all of a thread's loads are requested before the first is stored: one round trip for W_in, one for r
@@ -159,25 +185,33 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
 #pragma unroll
       for (int i = 0; i < DC / 4; ++i) { w_s[4 * i][tid] = q[i].x; w_s[4 * i + 1][tid] = q[i].y; w_s[4 * i + 2][tid] = q[i].z; w_s[4 * i + 3][tid] = q[i].w; }
     }
-    {
+    if constexpr (TW == 8) {
       constexpr int JP = DC / 4;         // four threads per token
       const int t = tid >> 2, j0 = (tid & 3) * JP;
-      const long src = row0 + t;
+      const long src = s_row[t];
       float v[JP];
 #pragma unroll
-      for (int u = 0; u < JP; ++u) v[u] = src < rows ? dep_load(r + src * D + d0 + j0 + u) : 0.f;
+      for (int u = 0; u < JP; ++u) v[u] = src >= 0 ? dep_load(r + src * D + d0 + j0 + u) : 0.f;
 #pragma unroll
       for (int u = 0; u < JP; ++u) r_s[j0 + u][t] = v[u];
+    } else if (tid < kNextTokens * DC) { // at most one word per thread
+      const int t = tid / DC, j = tid - t * DC;
+      r_s[j][t] = s_row[t] >= 0 ? dep_load(r + s_row[t] * D + d0 + j) : 0.f;
     }
     __syncthreads();
 #pragma unroll 2
     for (int j = 0; j < DC; ++j) {
       const ulonglong2 wa = *reinterpret_cast<const ulonglong2*>(&w_s[j][4 * lane]), wb = *reinterpret_cast<const ulonglong2*>(&w_s[j][128 + 4 * lane]);
-      const float4 ra = *reinterpret_cast<const float4*>(&r_s[j][tl]), rb = *reinterpret_cast<const float4*>(&r_s[j][tl + 4]);
       const uint64_t wv[4] = {wa.x, wa.y, wb.x, wb.y};
-      const float rv[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+      float rv[TW];
+      if constexpr (TW == 8) {
+        const float4 ra = *reinterpret_cast<const float4*>(&r_s[j][tl]), rb = *reinterpret_cast<const float4*>(&r_s[j][tl + 4]);
+        rv[0] = ra.x; rv[1] = ra.y; rv[2] = ra.z; rv[3] = ra.w; rv[4] = rb.x; rv[5] = rb.y; rv[6] = rb.z; rv[7] = rb.w;
+      } else {
+        rv[0] = r_s[j][tl];
+      }
 #pragma unroll
-      for (int t = 0; t < 8; ++t) {
+      for (int t = 0; t < TW; ++t) {
         uint64_t rr;
         asm("mov.b64 %0, {%1, %1};" : "=l"(rr) : "f"(rv[t]));
 #pragma unroll
@@ -185,13 +219,12 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
       }
     }
   }
-  float acc[8][8];
+  float acc[TW][8];
 #pragma unroll
-  for (int t = 0; t < 8; ++t)
+  for (int t = 0; t < TW; ++t)
 #pragma unroll
     for (int e = 0; e < 4; ++e) asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[t][2 * e]), "=f"(acc[t][2 * e + 1]) : "l"(acc2[t][e]));
   // the copies of the warp's tokens, two at a time
-  const int ca = c0 + 4 * lane, cb = ca + 128;
   float4 bias[2];
 #pragma unroll
   for (int g = 0; g < 2; ++g) {
@@ -199,25 +232,13 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
     bias[g] = b_in && c < C ? load4_any(b_in + c, 0) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 #pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    const int cnt = s_cnt[tl + t], nx = s_nx[tl + t], first = s_first[tl + t];
+  for (int t = 0; t < TW; ++t) {
+    const int cnt = k_end(t), nx = s_nx[tl + t], first = s_first[tl + t];
     const float4 va = make_float4(acc[t][0] + bias[0].x, acc[t][1] + bias[0].y, acc[t][2] + bias[0].z, acc[t][3] + bias[0].w);
     const float4 vb = make_float4(acc[t][4] + bias[1].x, acc[t][5] + bias[1].y, acc[t][6] + bias[1].z, acc[t][7] + bias[1].w);
     float* img = x_out + (cnt ? s_img[tl + t] : 0) * C;
-    for (int k0 = 0; k0 < cnt; k0 += 2) {
-      float4 pa[2], pb[2];
-      int t2[2];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int d = min(k0 + u, cnt - 1), yy = d / nx;
-        t2[u] = first + yy * w2 + (d - yy * nx);
-        pa[u] = pb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (pos && k0 + u < cnt) {
-          const float* q = pos + (size_t)t2[u] * C;
-          if (ca < C) pa[u] = load4_any(q + ca, vec);
-          if (cb < C) pb[u] = load4_any(q + cb, vec);
-        }
-      }
+    for (int k0 = k_first; k0 < cnt; k0 += 2) {
+      if (TW > 1 || k0 > k_first) fetch(k0, cnt, nx, first);
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         if (k0 + u >= cnt) break;
@@ -272,16 +293,25 @@ cudaError_t launch_next_input(const float* r, int B, int h, int w, int d, int h2
   const long rows = (long)B * h2 * w2;
   const double bytes = (double)rows * C * (pos ? 8.0 : 4.0) + (double)rows * d * 4.0;
   LaunchScope scope(KC_RESTORE, 1, bytes, bytes, st);
-  // (tokens along y: up to 65535 x 64 of them, far past the largest token map)
-  const dim3 grid((unsigned)((C + kNextChannels - 1) / kNextChannels), (unsigned)(((long)B * h * w + kNextTokens - 1) / kNextTokens));
-  // (32-bit index arithmetic: maps of up to some 40000 tokens a side)
-  if (grid.y > 65535u || (long)(h + 1) * h2 + h > INT_MAX || (long)(w + 1) * w2 + w > INT_MAX || (long)B * h * w > INT_MAX) return cudaErrorInvalidValue;
+  // Token tiles x channel blocks along x: eight tokens per warp, or one where eight would not give every SM a CTA of its own.  A warp writes a token's copies two at a time, so where
+  // the tiles still leave room on the GPU (two CTAs per SM) the copies of a token are cut into slices along y, each with the product computed again.
+  const long tokens = (long)B * std::min(h, h2) * std::min(w, w2), cblocks = (C + kNextChannels - 1) / kNextChannels;
+  const int tw = (tokens + 63) / 64 * cblocks < 148 ? 1 : 8;
+  const long ctas = (tokens + 8 * tw - 1) / (8 * tw) * cblocks;
+  const long copies = (long)(h2 > h ? (h2 + h - 1) / h : 1) * (w2 > w ? (w2 + w - 1) / w : 1);   // most copies of a token
+  const long slices = std::max(1L, std::min((copies + 1) / 2, 2L * 148 / ctas));
+  const int slice = (int)((copies + slices - 1) / slices);
+  if (ctas > INT_MAX) return cudaErrorInvalidValue;
+  const dim3 grid((unsigned)ctas, (unsigned)((copies + slice - 1) / slice));
   const int vec = ((reinterpret_cast<uintptr_t>(x_out) | reinterpret_cast<uintptr_t>(pos)) & 15u) == 0;   // C is a multiple of 4
+  auto go = [&](auto* one, auto* eight) {
+    return launch_pdl(tw == 1 ? one : eight, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, slice, x_out);
+  };
   switch (d) {
-    case 8: return launch_pdl(next_input_kernel<8>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, x_out);
-    case 16: return launch_pdl(next_input_kernel<16>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, x_out);
-    case 32: return launch_pdl(next_input_kernel<32>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, x_out);
-    case 64: return launch_pdl(next_input_kernel<64>, grid, dim3(256), 0, st, r, h, w, h2, w2, w_in, b_in, pos, C, B, vec, x_out);
+    case 8: return go(next_input_kernel<8, 1>, next_input_kernel<8, 8>);
+    case 16: return go(next_input_kernel<16, 1>, next_input_kernel<16, 8>);
+    case 32: return go(next_input_kernel<32, 1>, next_input_kernel<32, 8>);
+    case 64: return go(next_input_kernel<64, 1>, next_input_kernel<64, 8>);
     default: return cudaErrorInvalidValue;
   }
 }

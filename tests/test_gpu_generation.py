@@ -134,6 +134,18 @@ def test_next_scale_input_copies_of_a_source_token(d, C, h, w, h2, w2, B):
     assert torch.equal(big[1:].view(B, h2 * w2, C), got)
 
 
+@pytest.mark.parametrize("d,C,h,w,h2,w2,B", [(8, 64, 1, 1, 16, 16, 1), (16, 256, 2, 1, 40, 33, 2), (32, 128, 40, 30, 7, 9, 2), (64, 512, 8, 8, 10, 10, 1), (16, 300, 9, 30, 40, 5, 3),
+                                              (8, 4, 1, 50000, 1, 50001, 1), (8, 4, 1, 70000, 1, 300, 2), (8, 4, 2100, 2000, 2100, 2000, 1)])
+def test_next_scale_input_between_sizes_far_apart(d, C, h, w, h2, w2, B):
+    """Few tokens with many copies each (cut into slices), maps that shrink along one axis or both (only the tokens with a target
+    take part), sizes whose products pass 32 bits, more than four million tokens."""
+    r = I.normal(241, (B, h * w, d), 2.0)
+    w_in, b_in, pos = I.normal(242, (C, d), 1 / np.sqrt(d)), I.normal(243, (C,), 0.1), I.normal(244, (h2 * w2, C), 0.5)
+    ref = G.next_scale_input(r, h, w, h2, w2, w_in, b_in, pos)
+    got = fv.fv_next_scale_input(T(r), h, w, h2, w2, T(w_in), T(b_in), T(pos)).cpu().numpy()
+    np.testing.assert_allclose(got, ref, rtol=1e-5, atol=2e-5)      # fp32 dot products of d terms
+
+
 def _gen_setup(keep, sides=(1, 2, 3, 4, 6, 8), L=2, C=128, H=2, B=2, V=256, d=16, cross_len=0):
     wl = I.Workload("gen", L=L, C=C, H=H, B=B, sides=tuple(sides), keep=tuple(keep), cross_len=cross_len, seed=31)
     mt = I.model_tensors(wl)
