@@ -100,13 +100,13 @@ __global__ void __launch_bounds__(256) residual_accumulate_kernel(const int32_t*
 // lane and clock, a broadcast word included, so a thread tile of T x C costs T + C of its clocks for T C / 4 of an SM's multiply-adds: 8 x 8
 // balances the two, and two channels go through one packed multiply-add.  A warp then walks the copies of its own tokens, whose
 // products its lanes hold in registers, the embedding rows of two copies in flight.  Measured for 2 x 48 x 48 -> 64 x 64 tokens, C 2048, d 32
-// (map written + embedding read: 16 us), back to back: 38 us; 45.5 with single multiply-adds, the products passed through shared
+// (map written + embedding read: 16 us), back to back: 41 us (38 while W_in was read before the dependency wait); 45.5 with single multiply-adds, the products passed through shared
 // memory to be indexed by copy and the embedding rows prefetched into L2 (which gives nothing); a product per target token in 8 x 8 tiles 52,
 // and with one channel per thread 73.  Two rounds of CTAs, each a chain of loads (embedding rows 11 us in all), products (8) and
 // stores (6); CTAs of 32 or 16 tokens, four or eight to an SM, do not overlap them better (40, 52).  The additions keep their order (j
 // ascending, bias, embedding).
 // TW: tokens per warp.  One instead of eight where tiles of 64 tokens leave the GPU to a few CTAs, each of which then takes its warps' tokens one
-// after the other: MEASURED
+// after the other (launch_next_input draws the line).
 constexpr int kNextChannels = 256;      // one per thread while W_in is staged
 // Four floats at an address that is 16-byte aligned (vec) or not.
 __device__ __forceinline__ float4 load4_any(const float* p, int vec) {
@@ -293,10 +293,13 @@ cudaError_t launch_next_input(const float* r, int B, int h, int w, int d, int h2
   const long rows = (long)B * h2 * w2;
   const double bytes = (double)rows * C * (pos ? 8.0 : 4.0) + (double)rows * d * 4.0;
   LaunchScope scope(KC_RESTORE, 1, bytes, bytes, st);
-  // Token tiles x channel blocks along x: eight tokens per warp, or one where eight would not give every SM a CTA of its own.  A warp writes a token's copies two at a time, so where
-  // the tiles still leave room on the GPU (two CTAs per SM) the copies of a token are cut into slices along y, each with the product computed again.
+  // Token tiles x channel blocks along x.  A warp takes its tokens one after the other and writes the copies of each two at a time: eight tokens per warp
+  // use the GPU best, but where their tiles would not even give every second SM a CTA, one per warp is sooner done (us, eight -> one: 8 x 8 -> 10 x 10
+  // tokens, C 256 8.3 -> 3.4; 16 x 16 -> 20 x 20 twice, C 1024 11.4 -> 10.4; 20 x 20 -> 24 x 24, C 2048 14.0 -> 10.6; with 100 tiles 24.9 -> 34.1, with 128
+  // 16.4 -> 24.5).  Where a few tokens become many the copies of a token are cut into slices along y, as many as run at once at two CTAs per
+  // SM, each with the product computed again (8 x 8 -> 64 x 64, C 2048: 18 us in 37 slices, 24 in 16).
   const long tokens = (long)B * std::min(h, h2) * std::min(w, w2), cblocks = (C + kNextChannels - 1) / kNextChannels;
-  const int tw = (tokens + 63) / 64 * cblocks < 148 ? 1 : 8;
+  const int tw = 2 * ((tokens + 63) / 64 * cblocks) < 148 ? 1 : 8;
   const long ctas = (tokens + 8 * tw - 1) / (8 * tw) * cblocks;
   const long copies = (long)(h2 > h ? (h2 + h - 1) / h : 1) * (w2 > w ? (w2 + w - 1) / w : 1);   // most copies of a token
   const long slices = std::max(1L, std::min((copies + 1) / 2, 2L * 148 / ctas));
