@@ -99,7 +99,8 @@ fv_status fv_prune_select_static(const float *x_dev, int32_t B, int32_t h, int32
  *   pivots_dev     [B, k, C] bf16     : the forwarded rows.
  *   idx_dev        [B, k] int32       : their token indices (any order, no duplicates, in [0,h*w)).
  *   out_dev        [B, h*w, C] bf16.   C % 8 == 0.
- *   inv_scratch_dev: unused, may be NULL (earlier versions built an inverse map in it).
+ *   inv_scratch_dev[B, h*w] int32 scratch (may be overwritten), or NULL.  Large maps build an inverse map of idx in it;
+ *                  without it every 16 tokens read their image's whole index list, which grows with h*w*k.
  *   interp_mode    0: nearest, as above (the default reading of the paper's mode-less interpolate).
  *                  1: bilinear with half-pixel centres (source coordinate (dst+0.5)*in/out - 0.5 per axis,
  *                     clamped): an unkept token is the fp32 blend of four cached rows, rounded to bf16 once.

@@ -223,7 +223,8 @@ def fv_restore(cache_prev: torch.Tensor, hc: int, wc: int, pivots: torch.Tensor,
     B, k, Cw = pivots.shape
     if out is None:
         out = _empty((B, h * w, Cw), torch.bfloat16, pivots.device)
-    _check(lib().fv_restore(_ptr(cache_prev), hc, wc, _ptr(pivots), _ptr(idx), B, k, h, w, Cw, _ptr(out), None,
+    inv = _empty((B, h * w), torch.int32, pivots.device) if B * k * h * w > 1 << 25 else None   # (smaller maps never use it)
+    _check(lib().fv_restore(_ptr(cache_prev), hc, wc, _ptr(pivots), _ptr(idx), B, k, h, w, Cw, _ptr(out), _ptr(inv),
                             int(interp_mode), _stream()), "fv_restore")
     return out
 

@@ -181,14 +181,13 @@ fv_status fv_prune_select(const float* x_dev, int32_t B, int32_t h, int32_t w, i
 fv_status fv_restore(const void* cache_prev_dev, int32_t hc, int32_t wc, const void* pivots_dev, const int32_t* idx_dev,
                      int32_t B, int32_t k, int32_t h, int32_t w, int32_t C, void* out_dev, int32_t* inv_scratch_dev,
                      int32_t interp_mode, void* stream) {
-  (void)inv_scratch_dev;   // not needed any more: the kernel finds the tokens' slots itself
   if (!cache_prev_dev || !pivots_dev || !idx_dev || !out_dev) return FV_ERR_INVALID_ARG;
   if (interp_mode < 0 || interp_mode > 2) return FV_ERR_INVALID_ARG;
   if (B <= 0 || k <= 0 || h <= 0 || w <= 0 || hc <= 0 || wc <= 0 || C <= 0 || (C % 8) || k > h * w) return FV_ERR_INVALID_ARG;
   if (!aligned16(cache_prev_dev) || !aligned16(pivots_dev) || !aligned16(out_dev)) return FV_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (ensure_init() != cudaSuccess) return FV_ERR_CUDA;
-  return cuda_status(launch_restore_bf16(cache_prev_dev, hc, wc, pivots_dev, idx_dev, B, k, h, w, C, out_dev, interp_mode, st));
+  return cuda_status(launch_restore_bf16(cache_prev_dev, hc, wc, pivots_dev, idx_dev, inv_scratch_dev, B, k, h, w, C, out_dev, interp_mode, st));
 }
 
 fv_status fv_gather_ln(const float* x_dev, const int32_t* idx_dev, int32_t B, int32_t n_tokens, int32_t k, int32_t C,

@@ -183,7 +183,7 @@ void restore_force_fold(int mode);     // test hook: 0 by shape, 1 fold through 
 cudaError_t launch_gather_rows(const float* x, const int32_t* idx, int B, int n, int k, int C, float* out, int32_t* status, cudaStream_t st);
 cudaError_t launch_restore_rows_f32(const float* cache, int hc, int wc, const float* pivots, const int32_t* inv, int B, int k,
                                     int h, int w, int C, float* out, int interp_mode, cudaStream_t st);
-cudaError_t launch_restore_bf16(const void* cache, int hc, int wc, const void* pivots, const int32_t* idx, int B,
+cudaError_t launch_restore_bf16(const void* cache, int hc, int wc, const void* pivots, const int32_t* idx, int32_t* inv_scratch, int B,
                                 int k, int h, int w, int C, void* out, int interp_mode, cudaStream_t st);
 
 // ---- gemm.cu : tcgen05 GEMM with fused epilogues -----------------------------------------------

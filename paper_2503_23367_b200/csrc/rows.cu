@@ -483,22 +483,24 @@ __global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* xf,
 }
 
 // Plain restoration (no residual) of a bf16 map: TAPS 0 copies the nearest source, 4 / 16 blend bilinearly / bicubically in fp32 and
-// round once.  CTA = RT consecutive tokens.  It finds their slots in the kept set itself, by reading the image's whole index list
-// (a few KB out of L2, all of it requested at once): an inverse map built by two launches before this one cost more than that
-// (2 x 64 x 64 tokens, k 820, C 2048: 2.2 + 2.3 + 8.5 us and two more launches of the host).  A warp takes a row at a time, up to eight
+// round once.  CTA = RT consecutive tokens.  Without inv it finds their slots in the kept set itself, by reading the image's whole index
+// list, k words for every RT tokens: on small maps an inverse map built by two launches before this one costs more than that
+// (2 x 64 x 64 tokens, k 820, C 2048: 2.2 + 2.3 + 8.5 us and two more launches of the host); launch_restore_bf16 draws the line.  A warp takes a row at a time, up to eight
 // 16-byte loads per lane in flight.
 template <int TAPS, int RT>
 __global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* cache, int hc, int wc, const uint4* pivots,
-                                                           const int32_t* idx, int n, int k, int h, int w, int C8, uint4* __restrict__ out) {
+                                                           const int32_t* idx, const int32_t* inv, int n, int k, int h, int w, int C8, uint4* __restrict__ out) {
   __shared__ int s_slot[RT];
-  const int b = blockIdx.y, t0 = blockIdx.x * RT;
+  const int tiles = (n + RT - 1) / RT, b = blockIdx.x / tiles, t0 = (blockIdx.x - b * tiles) * RT;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_trigger();
   if (threadIdx.x < RT) s_slot[threadIdx.x] = -1;
   __syncthreads();
   pdl_wait();
   const int32_t* ib = idx + (size_t)b * k;
-  for (int i0 = threadIdx.x; i0 < k; i0 += 256 * 8) {
+  if (inv) {
+    if (threadIdx.x < min(RT, n - t0)) s_slot[threadIdx.x] = dep_load(inv + (size_t)b * n + t0 + threadIdx.x);
+  } else for (int i0 = threadIdx.x; i0 < k; i0 += 256 * 8) {
     int v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = i0 + 256 * u < k ? dep_load(ib + i0 + 256 * u) - t0 : -1;
@@ -682,17 +684,28 @@ cudaError_t launch_restore_residual(void* x, const void* y, const void* cache, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_restore_bf16(const void* cache, int hc, int wc, const void* pivots, const int32_t* idx, int B, int k,
+cudaError_t launch_restore_bf16(const void* cache, int hc, int wc, const void* pivots, const int32_t* idx, int32_t* inv_scratch, int B, int k,
                                 int h, int w, int C, void* out, int interp_mode, cudaStream_t st) {
   const int n = h * w;
   const double rb_bytes = (double)B * C * (2.0 * h * w + 2.0 * k + 2.0 * hc * wc);
+  // Where the slots come from: the index list, which every CTA reads whole, or an inverse map built by two launches before (1.4 us, and 8 bytes a token).
+  // The lists read, in all, have to stay below 16 MB and a tenth of the rows' own bytes, behind which they hide.  Us back to back, lists / map, keep
+  // 0.2 | 0.5 | 0.9: 64 x 64 tokens C 2048 5.9 / 7.7 | 6.1 / 7.8 | 6.6 / 7.9; 96 x 96 C 256 3.9 / 5.3 | 4.7 / 5.1 | 5.2 / 4.7; 128 x 128 C 256 6.5 / 6.9 | 7.7 / 6.7 |
+  // 10.1 / 6.3, C 2048 14.7 / 15.5 | 19.4 / 19.0 | 25.3 / 21.1; 512 x 512 C 256 279 / 71 | 643 / 71 | 1116 / 69; 8 images of 64 x 64 C 1024 15.8 / 16.3 | 19.5 / 19.2 |
+  // 24.1 / 21.3.  A caller without scratch gets the lists at every size.
+  const double lists = (double)B * ((n + 15) / 16) * k * 4.0;
+  const bool map = inv_scratch && lists > 16e6 + 0.1 * rb_bytes;
   LaunchScope scope(KC_RESTORE, 1, rb_bytes, rb_bytes, st);
+  if (map) {
+    const cudaError_t e = launch_inv_from_idx(idx, B, k, n, inv_scratch, st);
+    if (e != cudaSuccess) return e;
+  }
   // 16 tokens per CTA (two rows per warp); 8 while that leaves SMs without a CTA
   const bool small = (long)((n + 15) / 16) * B < g_rows_sms;
   auto go = [&](auto* k16, auto* k8) {
     const int rt = small ? 8 : 16;
-    return launch_pdl(small ? k8 : k16, dim3((n + rt - 1) / rt, B), dim3(256), 0, st, static_cast<const uint4*>(cache), hc, wc,
-                      static_cast<const uint4*>(pivots), idx, n, k, h, w, C / 8, static_cast<uint4*>(out));
+    return launch_pdl(small ? k8 : k16, dim3((unsigned)((n + rt - 1) / rt * (long)B)), dim3(256), 0, st, static_cast<const uint4*>(cache), hc, wc,
+                      static_cast<const uint4*>(pivots), idx, map ? inv_scratch : nullptr, n, k, h, w, C / 8, static_cast<uint4*>(out));
   };
   if (interp_mode == 0) return go(restore_bf16_kernel<0, 16>, restore_bf16_kernel<0, 8>);
   if (interp_mode == 1) return go(restore_bf16_kernel<4, 16>, restore_bf16_kernel<4, 8>);

@@ -204,6 +204,36 @@ def test_restore_is_bit_exact(B, hc, wc, h, w, C, k):
     assert torch.equal(out2, out)
 
 
+def test_restore_of_more_images_than_a_grid_has_rows():
+    B, C = 70000, 8
+    cache, piv = I.normal_bf16(23, (B, 1, C)), I.normal_bf16(24, (B, 1, C))
+    idx = (np.arange(B) % 4).astype(np.int32)[:, None]
+    out = fv.fv_restore(bf16_dev(cache), 1, 1, bf16_dev(piv), dev(idx), 2, 2)
+    got = out.view(torch.int16).cpu().numpy().view(np.uint16)
+    want = np.repeat(cache, 4, axis=1)
+    want[np.arange(B), idx[:, 0]] = piv[:, 0]
+    assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("h,w,k,launches", [(128, 128, 16384, 3), (192, 256, 20000, 3), (128, 128, 2000, 1), (40, 40, 1600, 1)])
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_restore_finds_the_slots_by_list_or_by_map(h, w, k, launches, mode):
+    """Large maps with many kept tokens go through an inverse map (two launches more) when the caller gives scratch for it, the others
+    read the index list; both give the same bits, in any order of the indices."""
+    C, hc, wc, n = 64, 32, 32, h * w
+    perm = np.argsort(I.uniform01(25, n), kind="stable")[:k].astype(np.int32)[None]
+    cache, piv = bf16_dev(I.normal_bf16(26, (1, hc * wc, C))), bf16_dev(I.normal_bf16(27, (1, k, C)))
+    before = fv.fv_kernel_launches()
+    out = fv.fv_restore(cache, hc, wc, piv, dev(perm), h, w, interp_mode=mode)
+    assert fv.fv_kernel_launches() - before == launches
+    lists = torch.empty_like(out)
+    idx = dev(perm)
+    assert fv.lib().fv_restore(cache.data_ptr(), hc, wc, piv.data_ptr(), idx.data_ptr(), 1, k, h, w, C, lists.data_ptr(), None, mode,
+                               torch.cuda.current_stream().cuda_stream) == 0
+    assert torch.equal(out.view(torch.int16), lists.view(torch.int16))
+    assert torch.equal(out[0, idx[0].long()], piv[0])
+
+
 @pytest.mark.parametrize("with_gamma", [True, False])
 def test_restore_residual(with_gamma):
     B, hc, wc, h, w, C, k = 2, 10, 10, 16, 16, 1024, 128
