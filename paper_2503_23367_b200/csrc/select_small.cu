@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
   }
 }
 
-int g_clusters16 = 0;     // clusters of 16 CTAs the GPU holds at once
+int g_clusters[2] = {0, 0};     // clusters of 8 / of 16 CTAs the GPU holds at once
 
 template <typename XT> cudaError_t attr() {
   cudaError_t e = cudaFuncSetAttribute(select_small_kernel<XT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -386,15 +386,18 @@ static cudaError_t init_once() {
   cudaError_t e = attr<float>();
   if (e == cudaSuccess) e = attr<__nv_bfloat16>();
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(kMaxCluster); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = 200 * 1024;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = kMaxCluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, select_small_kernel<float>, &cfg) == cudaSuccess) g_clusters16 = clusters;
-  else (void)cudaGetLastError();
+  for (int i = 0; i < 2; ++i) {
+    const int cl = kMaxCluster / 2 << i;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cl); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = 200 * 1024;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, select_small_kernel<float>, &cfg) == cudaSuccess) g_clusters[i] = clusters;
+    else (void)cudaGetLastError();
+  }
   return cudaSuccess;
 }
 cudaError_t select_small_init() {
@@ -402,14 +405,17 @@ cudaError_t select_small_init() {
   return e;
 }
 
-// CTAs per image, or 0: the map is not for this kernel.  16 while the GPU holds a cluster of them per image, else 8.  A CTA works
+// CTAs per image, or 0: the map is not for this kernel.  16 while the GPU holds a cluster of them per image, else 8 while it holds one of
+// those: images that wait for a second round of clusters pay the whole chain again (16 x 16 tokens, C 1024, us a selection alone, separate kernels ->
+// this one: 12 images 14.2 -> 10.3, 16 images 15.0 -> 19.0, 64 images 27.5 -> 47.6; us per block of a step 114 -> 107, 125 -> 149, 352 -> 434).  A CTA works
 // through its rows alone, so the gain over the separate kernels (some 9 ... 12 us per sublayer on the smallest maps) is used up
 // at about 50 rows, or 200 KB of them.  Measured, us per block of 2 sublayers (3 at C 2048), separate kernels -> this one: 16 rows C 1024
 // 91 -> 69, C 2048 161 -> 137; 32 rows (clusters of 8) C 1024 107 -> 94; 21 rows C 1920 179 -> 170; 25 rows C 2048 183 -> 190; 36 rows
 // C 256 74 -> 63, C 512 84 -> 80, C 1024 bf16 stream 119 -> 107; 64 rows C 256 76 -> 78, C 512 90 -> 98, C 1024 bf16 148 -> 155.
 static int small_cluster(int B, int n, int C, bool x_bf16) {
   if (C % 128 || C > 2048) return 0;
-  const int cl = g_clusters16 >= B ? 16 : 8;
+  const int cl = g_clusters[1] >= B ? 16 : (g_clusters[0] >= B ? 8 : 0);
+  if (cl == 0) return 0;
   const int R = (n + cl - 1) / cl;
   if (R > 40 || (size_t)R * C * (x_bf16 ? 2 : 4) > 176 * 1024 || (size_t)small_smem(n, C, R).total * 4 > 200 * 1024) return 0;
   return cl;

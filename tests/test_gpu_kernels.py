@@ -130,6 +130,20 @@ def test_prune_select_small_maps_in_one_launch(B, h, w, C, keep, kind):
         assert np.array_equal(r["inv"].cpu().numpy().astype(np.int64), O.inverse_map(idx_g, h * w))
 
 
+@pytest.mark.parametrize("B,launches", [(1, 1), (9, 1), (40, 3), (64, 3)])
+def test_prune_select_takes_one_launch_only_while_all_images_fit(B, launches):
+    """A cluster of at least eight CTAs, one per SM, works on an image: more images than the GPU holds clusters go to the kernels that stream."""
+    h = w = 10
+    x = I.token_map(277, B, h, w, 256, "structured")
+    before = fv.fv_kernel_launches()
+    r = fv.fv_prune_select(dev(x), h, w, 0.5, want_inv=True, want_score=True)
+    assert fv.fv_kernel_launches() - before == launches
+    score_g, idx_g = r["score"].cpu().numpy(), r["idx"].cpu().numpy().astype(np.int64)
+    np.testing.assert_allclose(score_g, O.pts_score(x), rtol=2e-5, atol=1e-4)
+    assert np.array_equal(idx_g, O.pts_topk(score_g, r["k"]))
+    assert np.array_equal(r["inv"].cpu().numpy().astype(np.int64), O.inverse_map(idx_g, h * w))
+
+
 @pytest.mark.parametrize("B,h,w,C,keep", [(2, 12, 12, 256, 0.4), (3, 13, 18, 1920, 0.6), (20, 8, 9, 128, 0.3), (1, 16, 15, 2048, 1.0), (2, 64, 64, 256, 0.2)])
 def test_prune_select_near_tie_count_leaves_the_selection_alone(B, h, w, C, keep):
     """Scores a few ulps apart around the threshold: asking for the count changes neither scores nor kept set, and it counts those very scores."""
