@@ -35,7 +35,8 @@ constexpr int kThreads = 192;
 // the transposed accumulator goes to its owners one word per lane and row.  (Reducing and finishing it four rows at a time,
 // in wide words, costs more in the epilogue than it saves there: M 32 N 6144 6.9 -> 7.3.)
 //
-// The builds for few rows stay under 113 KB of shared memory, ring and reduce buffer together, so that TWO CTAs share an SM:
+// The builds for few rows stay under 113 KB of shared memory, ring and reduce buffer together, and under 168 registers (the launch bounds say
+// so: two slices of 64 rows took 190 without, and one CTA per SM), so that TWO CTAs share an SM:
 // the CTAs of the next GEMM of the step start (programmatic launch) beside those of this one and fetch their first
 // weights while this one computes, and outputs of up to 8192 columns fit the GPU in four slices.
 //
@@ -73,7 +74,7 @@ __device__ __forceinline__ void st_cluster_f1(uint32_t addr, uint32_t a) {
 }
 
 template <int BN, int S, int ROWS>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, ClusterCfg<BN, ROWS>::kFlip ? 2 : 1)
 gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmDev p) {
   using Cfg = ClusterCfg<BN, ROWS>;
   constexpr bool FLIP = Cfg::kFlip;
