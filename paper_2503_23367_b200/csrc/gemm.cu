@@ -23,6 +23,7 @@
 
 #include <mutex>
 
+#include "gemm_choice.h"
 #include "gemm_epilogue.cuh"
 #include "internal.h"
 #include "sm100.cuh"
@@ -388,40 +389,6 @@ cudaError_t gemm_init() {
   return cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
 }
 
-// Kernel and tile for a shape.  Measured on B200 (launches replayed from a CUDA graph, so that the host does not pace
-// them, weights rotating through HBM), one launch costs about
-//     fixed + rounds x (per_round + k-blocks x per_kblock)
-// where rounds = ceil(CTAs / SMs), or pairs / half the SMs.  A k-block of a 128-wide tile is paced by the operand loads (an SM takes
-// in about 110 bytes per clock, whatever the tile), the wider tiles by the MMAs themselves; wider tiles and CTA pairs win by needing
-// fewer rounds and less L2 traffic per flop.  Where tiles leave SMs idle, the CTAs of a cluster share a tile's K (2 or 4 slices,
-// gemm_cluster.cu); those only compete while all their CTAs run at once.
-struct TileChoice { int bn; bool pair; int slices; };   // slices 1: no cluster
-static TileChoice pick_tile(int M, int N, int K, int sms) {
-  const int num_kb = (K + BK - 1) / BK;
-  struct Cand { int bn; bool pair; int slices; double fixed_us, round_us, kb_us; };
-  // Least-squares fits over M 36 ... 3277 x the four projection shapes of 1024-, 1920- and 2048-wide blocks, every candidate forced.  On
-  // that sweep the choice costs 0.3 % over the best candidate on average (10 % at worst, 0.5 us); e.g. (us) N 2048 K 8192: M 400 64-wide
-  // 23.0, 128 x 2 24.5; M 820 pair of 128 27.7, 128-wide 31.7, 192-wide 35.5; N 1024 K 4096: M 400 64 x 2 9.9, 128 x 4 11.4; M 816 64-wide
-  // 12.8, 128 x 2 14.5; N 2048 K 2048 M 3277 192-wide 24.6, 128-wide 30.4.
-  const Cand cand[10] = {{128, false, 1, 3.63, 0.81, 0.214}, {192, false, 1, 3.53, 1.79, 0.251}, {256, false, 1, 2.87, 2.28, 0.343},
-                         {256, true, 1, 6.47, 1.55, 0.292}, {128, true, 1, 5.09, 1.11, 0.168}, {64, false, 1, 3.17, 0.42, 0.151},
-                         {64, false, 4, 3.79, 0.0, 0.228}, {64, false, 2, 3.48, 0.0, 0.196},
-                         {128, false, 4, 5.75, 0.0, 0.304}, {128, false, 2, 5.38, 0.0, 0.295}};
-  TileChoice best{128, false, 1};
-  double best_cost = 1e30;
-  for (const Cand& c : cand) {
-    if (c.pair && M <= 256) continue;
-    const int rows = c.pair ? 256 : 128;
-    const int slots = c.pair ? sms / 2 : sms;
-    const long ctas = (long)((M + rows - 1) / rows) * ((N + c.bn - 1) / c.bn) * c.slices;
-    if (c.slices > 1 && (ctas > slots || num_kb < 8)) continue;
-    const long rounds = (ctas + slots - 1) / slots;
-    const double cost = c.fixed_us + (double)rounds * (c.round_us + (num_kb + c.slices - 1) / c.slices * c.kb_us);
-    if (cost < best_cost - 1e-9) { best_cost = cost; best = TileChoice{c.bn, c.pair, c.slices}; }
-  }
-  return best;
-}
-
 // K-split scratch: room for two work items per SM of the widest tile, after 4 KB of arrival counters.
 constexpr size_t kSplitTicketBytes = 4096;
 constexpr int kSplitMaxItems = 2 * 148;
@@ -481,17 +448,17 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
   if (g.rows_per_image <= 0) return FV_ERR_INVALID_ARG;
   if (g.epilogue == EPI_QKV_SPLIT && (g.C % 128 || g.q_cols % 128)) return FV_ERR_UNSUPPORTED;
   const int tiles_m = (g.M + BM - 1) / BM;
-  TileChoice tc = pick_tile(g.M, g.N, g.K, g_num_sms);
+  // Q / K extras (cosine attention, rotary positions): one-CTA tiles that hold whole heads, no K split
+  const bool qk_extras = g.epilogue == EPI_QKV_SPLIT && (g.qk_scale || g.rope_table);
+  if (qk_extras && g.head_dim != 64 && g.head_dim != 128) return FV_ERR_UNSUPPORTED;
+  TileChoice tc = pick_tile(g.M, g.N, g.K, g_num_sms, qk_extras ? g.head_dim : 0);
   const TileChoice picked = tc;
   if (g_force_path == 1 && tc.pair) tc = TileChoice{256, false, 1};
   if (g_force_path == 2) tc = TileChoice{256, true, 1};
   if (g_force_path == 3) tc = TileChoice{128, true, 1};
   if (g_force_path >= 4 && g_force_path <= 6) tc = TileChoice{128 + 64 * (g_force_path - 4), false, 1};
   if (g_force_path == 7) tc = TileChoice{64, false, 1};
-  // Q / K extras (cosine attention, rotary positions): one-CTA tiles that hold whole heads, no K split
-  const bool qk_extras = g.epilogue == EPI_QKV_SPLIT && (g.qk_scale || g.rope_table);
-  if (qk_extras) {
-    if (g.head_dim != 64 && g.head_dim != 128) return FV_ERR_UNSUPPORTED;
+  if (qk_extras) {   // (a forced tile is widened until it is allowed)
     if (tc.pair) tc = TileChoice{256, false, 1};
     if (tc.bn < 128) tc.bn = 128;            // the extras exist for tiles of at least 128 columns
     if (tc.bn % g.head_dim) tc.bn = 256;
