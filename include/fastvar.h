@@ -314,13 +314,11 @@ fv_status fv_restore_force_fold(int32_t mode);
  *   which (programmatic dependent launch) can be while the kernel enqueued just before it is still
  *   finishing -- do not produce W with that kernel.  A, bias and the outputs are touched only after it.
  *   status_dev: int32 device word that receives a non-zero code if a bounded wait expires (or NULL).
- *   splitk_ws_dev: NULL, or scratch of fv_gemm_splitk_workspace_bytes() bytes whose first 4096 bytes are
- *               zero (the kernel leaves them zero): shapes with too few output tiles to occupy the GPU
- *               (few rows against a large weight matrix) are then split along K, the slices' fp32
- *               partial sums added in slice order.  CAPACITY if splitk_ws_bytes is too small. */
+ *   splitk_ws_dev: not used any more (shapes with too few output tiles to occupy the GPU split K over the CTAs of a cluster, without
+ *               scratch); NULL, or a buffer of at least fv_gemm_splitk_workspace_bytes() bytes, CAPACITY if it is smaller. */
 size_t fv_gemm_splitk_workspace_bytes(void);
-/* Test / profiling hook (process-wide): which GEMM kernel fv_gemm_bf16 and the step use when no K split is
- * taken.  0 = chosen per shape (default); 1 = one CTA per 128-row tile, width chosen per shape; 2 = CTA
+/* Test / profiling hook (process-wide): which GEMM kernel fv_gemm_bf16 and the step use.
+ * 0 = chosen per shape (default); 1 = one CTA per 128-row tile, width chosen per shape; 2 = CTA
  * pairs sharing 256 x 256 tiles (tcgen05 cta_group::2); 3 = CTA pairs, 256 x 128 tiles; 4 / 5 / 6 = one CTA
  * per tile of width 128 / 192 / 256; 7 = one CTA per tile of width 64; 8 / 9 = K split over a cluster of 4 / 2
  * CTAs per 128-wide tile, 10 / 11 = the same with 64-wide tiles (partials reduced through distributed shared

@@ -285,7 +285,7 @@ def fv_gemm_bf16(a: torch.Tensor, w: torch.Tensor, bias: Optional[torch.Tensor],
                  out: Optional[torch.Tensor] = None, aux: Optional[torch.Tensor] = None,
                  gamma: Optional[torch.Tensor] = None, mod_stride: int = 0, rows_per_image: int = 0,
                  status: Optional[torch.Tensor] = None, splitk_ws: Optional[torch.Tensor] = None) -> torch.Tensor:
-    """splitk_ws: uint8 scratch of fv_gemm_splitk_workspace_bytes() bytes, first 4096 zero, or None (no K split)."""
+    """splitk_ws: not used any more; None, or at least fv_gemm_splitk_workspace_bytes() bytes."""
     M, K = a.shape
     N = w.shape[0]
     assert w.shape[1] == K and a.dtype == torch.bfloat16 and w.dtype == torch.bfloat16

@@ -33,7 +33,6 @@ struct fv_ctx {
   void* sel_ws = nullptr;
   void* fsel_ws = nullptr;                    // scratch of the fused selection (arrival counts, kept-row partial sums)
   unsigned int fsel_done = 0, fsel_epoch = 0; // what its grid-wide waits compare against (grow with every launch)
-  void* splitk_ws = nullptr;
   void* attn_ws = nullptr;
   cudaStream_t side = nullptr;           // the unkept rows of a restoration run here, beside the sublayer's branch
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -78,7 +77,7 @@ cudaError_t ensure_init() {
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 struct Layout {
-  size_t status, a, q, o, y, hbuf, idx, inv, idx2, inv2, sel, fsel, splitk, attn, xc, rope, total;
+  size_t status, a, q, o, y, hbuf, idx, inv, idx2, inv2, sel, fsel, attn, xc, rope, total;
 };
 
 int max_tokens(const fv_config* c) {
@@ -118,7 +117,6 @@ Layout workspace_layout(const fv_config* c) {
   l.inv2 = take(M * 4);
   l.sel = take(select_workspace_bytes(c->B_max, max_tokens(c), c->C));
   l.fsel = take(select_fused_ws_bytes(c->B_max, c->C));
-  l.splitk = take(gemm_splitk_ws_bytes());
   l.attn = take(attention_ws_bytes());
   l.xc = take(c->granularity == 1 ? M * C * 4 : 0);
   size_t rope_bytes = 0;
@@ -267,7 +265,6 @@ fv_status fv_gemm_bf16(const void* a_dev, const void* w_dev, const void* bias_de
   g.a = a_dev; g.w = w_dev; g.bias = bias_dev; g.M = M; g.N = N; g.K = K; g.epilogue = epilogue; g.out = out_dev;
   g.aux = aux_dev; g.gamma = gamma_dev; g.mod_stride = mod_stride; g.rows_per_image = rows_per_image > 0 ? rows_per_image : M;
   g.status = status_dev;
-  g.splitk_ws = splitk_ws_dev;
   return launch_gemm(g, static_cast<cudaStream_t>(stream));
 }
 
@@ -383,7 +380,6 @@ fv_status fv_create(const fv_config* cfg, const fv_weights* wts, void* kv_dev, v
   c->inv2 = reinterpret_cast<int32_t*>(c->ws + lay.inv2);
   c->sel_ws = c->ws + lay.sel;
   c->fsel_ws = c->ws + lay.fsel;
-  c->splitk_ws = c->ws + lay.splitk;
   c->attn_ws = c->ws + lay.attn;
   c->xc = reinterpret_cast<float*>(c->ws + lay.xc);
   c->qk_scale = wts->qk_scale_dev;
@@ -401,7 +397,6 @@ fv_status fv_create(const fv_config* cfg, const fv_weights* wts, void* kv_dev, v
   if (!rope_ok || cudaMemset(kv_dev, 0, fv_kv_bytes(cfg)) != cudaSuccess || cudaMemset(c->status, 0, 256) != cudaSuccess ||
       cudaMemset(c->sel_ws, 0, select_ticket_bytes(cfg->B_max)) != cudaSuccess ||
       cudaMemset(c->fsel_ws, 0, select_fused_sync_bytes(cfg->B_max)) != cudaSuccess ||
-      cudaMemset(c->splitk_ws, 0, gemm_splitk_ticket_bytes()) != cudaSuccess ||
       cudaMemset(c->attn_ws, 0, attention_ws_ticket_bytes()) != cudaSuccess ||
       cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -478,7 +473,7 @@ fv_status fv_prepare_text(fv_ctx* ctx, int32_t B, void* stream) {
     g.a = ctx->text; g.w = ctx->w_kv_x[l]; g.bias = nullptr; g.M = B * c.cross_len; g.N = 2 * c.C; g.K = c.C;
     g.epilogue = EPI_QKV_SPLIT; g.out = nullptr; g.q_cols = 0; g.C = c.C; g.rows_per_image = c.cross_len;
     g.k_cache = text_k(ctx, l); g.vt_cache = text_k(ctx, l) + ctx->text_k_bytes; g.kv_capacity = c.cross_len; g.kv_offset = 0;
-    g.status = ctx->status; g.splitk_ws = ctx->splitk_ws;
+    g.status = ctx->status;
     fv_status s = launch_gemm(g, static_cast<cudaStream_t>(stream));
     if (s != FV_OK) return s;
   }
@@ -498,7 +493,6 @@ fv_status fv_device_status(fv_ctx* ctx, int32_t* code_host, void* stream) {
     // a kernel that gave up may have left arrival counts half-way: every counter starts afresh
     cudaMemsetAsync(ctx->sel_ws, 0, select_ticket_bytes(ctx->cfg.B_max), st);
     cudaMemsetAsync(ctx->fsel_ws, 0, select_fused_sync_bytes(ctx->cfg.B_max), st);
-    cudaMemsetAsync(ctx->splitk_ws, 0, gemm_splitk_ticket_bytes(), st);
     cudaMemsetAsync(ctx->attn_ws, 0, attention_ws_ticket_bytes(), st);
     ctx->fsel_done = 0; ctx->fsel_epoch = 0;
     cudaStreamSynchronize(st);
@@ -689,7 +683,7 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
       }
       // ---- branch on the compact rows
       GemmArgs g{};
-      g.status = ctx->status; g.rows_per_image = k; g.mod_stride = mod_stride; g.splitk_ws = ctx->splitk_ws;
+      g.status = ctx->status; g.rows_per_image = k; g.mod_stride = mod_stride;
       const void* last_in = nullptr; const void* last_w = nullptr; const void* last_b = nullptr; int last_K = C;
       if (kind == 0) {
         g.a = ctx->a_buf; g.w = ctx->w_qkv[l]; g.bias = ctx->b_qkv[l]; g.M = M; g.N = 3 * C; g.K = C;
@@ -727,7 +721,7 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
       }
       // ---- last projection, then Cached Token Restoration + gate + residual
       GemmArgs o{};
-      o.status = ctx->status; o.rows_per_image = k; o.mod_stride = mod_stride; o.splitk_ws = ctx->splitk_ws;
+      o.status = ctx->status; o.rows_per_image = k; o.mod_stride = mod_stride;
       o.a = last_in; o.w = last_w; o.bias = last_b; o.M = M; o.N = C; o.K = last_K;
       if (sub_pruned) {
         o.epilogue = EPI_BF16; o.out = ctx->y_buf;

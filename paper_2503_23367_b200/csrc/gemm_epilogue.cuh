@@ -22,9 +22,7 @@ struct GemmDev {
   __nv_bfloat16* vt_cache;
   int kv_capacity, kv_offset;
   int32_t* status;
-  int splits, kb_per_split;   // K slices per tile (1 = no split) and 64-wide k-blocks per slice
-  float* sk_partial;          // [tile][slice][128][BN] fp32 partial accumulators
-  unsigned int* sk_tickets;   // [tile] arrival counters, zero between launches
+  int kb_per_split;           // 64-wide k-blocks per CTA of a cluster
   // EPI_QKV_SPLIT extras on the Q and K columns (the instantiation of their own, KIND 2):
   const float* qk_scale;      // [H] per-head query scale of cosine attention (q, k divided by their norm), or null
   const float2* rope_table;   // [tokens of the scale][head_dim / 2] (cos, sin), or null

@@ -257,13 +257,12 @@ __global__ void __launch_bounds__(256, 2) next_input_kernel(const float* r, int 
   }
 }
 
-struct HeadLayout { size_t a, logits, splitk, total; };
+struct HeadLayout { size_t a, logits, total; };
 HeadLayout head_layout(int rows, int C, int V, bool own_logits) {
   HeadLayout l{};
   size_t off = 0;
   l.a = off; off = align_up(off + (size_t)rows * C * 2, 256);
   l.logits = off; if (own_logits) off = align_up(off + (size_t)rows * V * 4, 256);
-  l.splitk = off; off = align_up(off + gemm_splitk_ws_bytes(), 256);
   l.total = off;
   return l;
 }
@@ -354,12 +353,9 @@ fv_status fv_head_tokens(const float* y_dev, int32_t B, int32_t n, int32_t C, co
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace_dev);
   float* logits = logits_out_dev ? logits_out_dev : reinterpret_cast<float*>(ws + l.logits);
-  // the K-split arrival counters must start at zero (the GEMM leaves them zero)
-  if (cudaMemsetAsync(ws + l.splitk, 0, gemm_splitk_ticket_bytes(), st) != cudaSuccess) return FV_ERR_CUDA;
   fv_status s = fv_gather_ln(y_dev, nullptr, B, n, n, C, mod_head_dev, mod_head_dev + C, 2 * C, ws + l.a, status_dev, stream);
   if (s != FV_OK) return s;
-  s = fv_gemm_bf16(ws + l.a, w_head_dev, b_head_dev, rows, V, C, EPI_F32, logits, nullptr, nullptr, 0, n, status_dev, ws + l.splitk,
-                   gemm_splitk_ws_bytes(), stream);
+  s = fv_gemm_bf16(ws + l.a, w_head_dev, b_head_dev, rows, V, C, EPI_F32, logits, nullptr, nullptr, 0, n, status_dev, nullptr, 0, stream);
   if (s != FV_OK) return s;
   return cu(launch_argmax_rows(logits, noise_dev, tau, rows, V, ids_out_dev, st));
 }

@@ -206,7 +206,6 @@ struct GemmArgs {
   void* vt_cache;      // [B, C, kv_capacity] bf16
   int kv_capacity, kv_offset;
   int32_t* status;     // device status word or null
-  void* splitk_ws;     // scratch for K-split partials (gemm_splitk_ws_bytes(), tickets at its head zero) or null
   // EPI_QKV_SPLIT extras on the Q and K columns (all null = none):
   const float* qk_scale;      // [H] fp32: cosine attention (q, k divided by their per-head norm, q times this)
   const float* rope_table;    // [tokens of the scale][head_dim/2][2] fp32 (cos, sin) of the rotary angles
@@ -221,8 +220,7 @@ cudaError_t gemm_init();
 // Test / profiling hook: 0 = choose per shape, 1 = one-CTA kernel, 2 = CTA-pair kernel 256x256, 3 = CTA-pair 256x128,
 // 4 ... 7 = one-CTA tiles 128, 192, 256, 64 wide, 8 ... 12 = clusters (128 wide x 4, x 2, 64 wide x 4, x 2, up to 48 rows 128 wide x 8).
 void gemm_force_path(int path);
-size_t gemm_splitk_ws_bytes();      // size of the K-split scratch
-size_t gemm_splitk_ticket_bytes();  // its leading bytes that must be zero before first use
+size_t gemm_splitk_ws_bytes();      // what fv_gemm_splitk_workspace_bytes reports
 fv_status launch_gemm(const GemmArgs& g, cudaStream_t st);
 
 // ---- attention.cu : flash-style attention over the KV cache ------------------------------------
