@@ -44,6 +44,9 @@ constexpr int QT = 128;   // queries per tile (two tiles per CTA)
 constexpr int KT = 128;   // keys per tile
 constexpr int kAttnThreads = 384;   // warps 0-3 / 4-7: softmax of stream 0 / 1; 8-11: TMA and MMA
 constexpr float kRescaleThreshold = 8.f;  // log2 units
+// The running maximum before the first key, below every finite score.  Not -inf: keys whose scores are all -inf (masked by an infinite
+// key channel) leave it there, and -inf - -inf would make their probabilities NaN where they are 0.
+constexpr float kNoMaximum = -3.402823466e38f;
 
 constexpr int HT = 64;    // keys per score slot of the whole-item kernel: a key tile is consumed in two halves
 
@@ -167,7 +170,7 @@ __device__ __noinline__ void item_parts(const AttnDev& p, int c, int nctas, int 
 template <int HD>
 __device__ __noinline__ bool softmax_key_tiles(const AttnDev& p, int ja, int jb, uint32_t s_addr, uint32_t o_addr, uint64_t* s_full_t,
                                                uint64_t* p_full_t, uint64_t* o_done_t, uint32_t& tiles, float& m_out, float& l_out) {
-  float m_run = -INFINITY, l_run = 0.f;
+  float m_run = kNoMaximum, l_run = 0.f;
   uint32_t sc_cnt = tiles;
   const float scale_log2 = p.scale_log2;
   for (int j = ja; j < jb; ++j, ++sc_cnt) {
@@ -187,7 +190,7 @@ __device__ __noinline__ bool softmax_key_tiles(const AttnDev& p, int ja, int jb,
     // may then exceed 1 (by at most 2^threshold), which fp32 sums and bf16 P hold without loss.
     float alpha = 1.f;
     if (mx > m_run + kRescaleThreshold) {
-      alpha = fast_exp2(m_run - mx);  // 0 on the first tile (m_run = -inf)
+      alpha = fast_exp2(m_run - mx);  // 0 on the first tile
       m_run = mx;
     }
     // S_t of tile j was issued after P V of tile j-1, so O_t is at rest here.
@@ -292,7 +295,7 @@ __device__ __noinline__ void finish_segment(const AttnDev& p, int u0, int u_hi, 
   __threadfence();
   // part q of the item was left by CTA c_first + q: the first in its slot 1, the others in slot 0
   auto part_slot = [&](int q) { return p.parts + ((size_t)(c_first + q) * 2 + (q == 0 ? 1 : 0)) * Cfg::kPartBytes; };
-  float m_star = -INFINITY;
+  float m_star = kNoMaximum;
   for (int q = 0; q < nparts; ++q) m_star = fmaxf(m_star, __ldcg(reinterpret_cast<const float2*>(part_slot(q)) + t * QT + r).x);
   float l_star = 0.f;
   for (int q = 0; q < nparts; ++q) {
@@ -516,7 +519,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
       const Seg sg = segment_at(u);
       u += sg.jb - sg.ja;
       const bool active = t < sg.ntiles;
-      float m_run = -INFINITY, l_run = 0.f;
+      float m_run = kNoMaximum, l_run = 0.f;
       if (active && ok) ok = softmax_key_tiles<HD>(p, sg.ja, sg.jb, s_addr, o_addr, &s_full[t], &p_full[t], &o_done[t], sc_cnt, m_run, l_run);
       finish_segment<HD>(p, u0, u_hi, t, r, o_addr, m_run, l_run, ok, &o_free[t], s_info);
     }
@@ -560,7 +563,7 @@ __device__ __forceinline__ int stream_halves(int kv_len, int ja, int dj, int n) 
 template <int HD>
 __device__ __forceinline__ bool softmax_stream(int kv_len, float scale_log2, int32_t* status, int ja, int dj, int halves, uint32_t s_addr, uint32_t o_addr,
                                                uint64_t* s_full, uint64_t* p_full, uint64_t* o_prev, uint64_t* o_last, float& m_out, float& l_out) {
-  float m_run = -INFINITY, l_run = 0.f;
+  float m_run = kNoMaximum, l_run = 0.f;
   const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
 #pragma unroll 1
   for (int i = 0; i < halves; ++i) {
@@ -590,7 +593,7 @@ __device__ __forceinline__ bool softmax_stream(int kv_len, float scale_log2, int
     // may then exceed 1 (by at most 2^threshold), which fp32 sums and bf16 P hold without loss.
     float alpha = 1.f;
     if (mx > m_run + kRescaleThreshold) {
-      alpha = fast_exp2(m_run - mx);  // 0 on the first half (m_run = -inf)
+      alpha = fast_exp2(m_run - mx);  // 0 on the first half
       m_run = mx;
     }
     if (i > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
@@ -790,7 +793,7 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     const uint32_t s_addr = tmem_base + lane_off + t * KT;
     const uint32_t o_base = tmem_base + lane_off + 256;
     const int nh = t == 0 ? nh0 : nh1;
-    float m_run = -INFINITY, l_run = 0.f;
+    float m_run = kNoMaximum, l_run = 0.f;
     const bool ok = softmax_stream<HD>(p.kv_len, p.scale_log2, p.status, ONE_TILE ? t : 0, ONE_TILE ? 2 : 1, nh, s_addr, o_base + t * 128,
                                        s_full + 2 * t, p_full + 2 * t, &o_prev[t], &o_last[t], m_run, l_run);
     if (ONE_TILE) {
@@ -803,7 +806,7 @@ attention_whole_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       asm volatile("bar.sync 1, 256;" ::: "memory");
       const float2 a = ml_s[r], b = ml_s[QT + r];
       const float m_star = fmaxf(a.x, b.x);
-      const float f0 = fast_exp2(a.x - m_star), f1 = fast_exp2(b.x - m_star);     // an empty stream: 2^-inf = 0
+      const float f0 = fast_exp2(a.x - m_star), f1 = fast_exp2(b.x - m_star);     // an empty stream: 0
       const float inv_l = 1.f / fmaf(b.y, f1, a.y * f0);
       const float w0 = f0 * inv_l, w1 = f1 * inv_l;
       const int row = q0 + r;

@@ -736,6 +736,32 @@ def test_attention_whole_items_of_either_size(build, B, rows, C, kv_len, growing
         _attention_reference_check(bf16_host(out), q, kk, vv, B, rows, H, C, kv_len)
 
 
+@pytest.mark.parametrize("masked", [range(0, 64), range(0, 128), range(64, 128), range(40, 700), [*range(128, 256), *range(384, 512), *range(640, 768)], range(700, 800)])
+@pytest.mark.parametrize("rows,H", [(100, 2), (300, 2), (300, 4)])
+def test_attention_over_masked_keys(rows, H, masked):
+    """Keys taken out by an infinite channel (their scores are all -inf): whole halves and tiles of them, a whole stream, wherever they
+    stand, in every build; what is left gives the softmax over the other keys."""
+    C, kv_len = 256, 800
+    q = I.to_bf16_bits(I.normal(390, (rows, C)).astype(np.float32)); kk = I.normal(391, (1, kv_len, C)).astype(np.float32); vv = I.normal_bf16(392, (1, kv_len, C))
+    qf = I.bf16_bits_to_f32(q).reshape(rows, C).copy()
+    qf[:, ::C // H] = 1.0
+    kept = np.setdiff1d(np.arange(kv_len), list(masked))
+    kk[0, list(masked), ::C // H] = -np.inf
+    q, kk = I.to_bf16_bits(qf), I.to_bf16_bits(kk)
+    vt = np.ascontiguousarray(vv.transpose(0, 2, 1))
+    ref = O.attention(qf.astype(np.float64), I.bf16_bits_to_f32(kk)[0, kept].astype(np.float64), I.bf16_bits_to_f32(vv)[0, kept].astype(np.float64), H)
+    ws = fv.fv_attention_workspace(DEV)
+    for build in (-2, -3, 0, 1, 3, 5):
+        assert fv.lib().fv_attention_force_ctas(build) == 0
+        try:
+            out = fv.fv_attention(bf16_dev(q), bf16_dev(kk), bf16_dev(vt), 1, rows, H, kv_len, workspace=ws)
+            torch.cuda.synchronize()
+        finally:
+            fv.lib().fv_attention_force_ctas(0)
+        err, cos = per_token_errors(bf16_host(out), ref)
+        assert err <= MAX_ABS and cos >= MIN_COS, (build, err, cos)
+
+
 def test_attention_refuses_small_scratch():
     q = torch.zeros((8, 256), dtype=torch.bfloat16, device=DEV); k = torch.zeros((1, 8, 256), dtype=torch.bfloat16, device=DEV)
     with pytest.raises(fv.FvError) as e:
