@@ -80,8 +80,7 @@ fv_status fv_prune_select(const float *x_dev, int32_t B, int32_t h, int32_t w, i
  *   - The first call on each device looks up the array's device address (with that device current);
  *     make that first call outside any stream capture.
  *   - All calls on a device share the one array and it keeps the previous call's contents; every
- *     call first clears the few counters that must start at zero (every other word it reads it has
- *     written itself), so leftovers are harmless, but two calls whose
+ *     word that a call reads it has written itself, so leftovers are harmless, but two calls whose
  *     kernels overlap on the GPU (different streams, no ordering between them) race on it: order them.
  * Errors: INVALID_ARG, UNSUPPORTED (h*w > 49152), CAPACITY, CUDA. */
 size_t fv_prune_select_static_capacity(void);
@@ -310,9 +309,11 @@ fv_status fv_restore_force_fold(int32_t mode);
  *   epilogue 4: fp32 store of acc + bias to out [M, N] (aux_dev, gamma_dev ignored).  3 is not a public value.
  *   epilogue 5: as 2 for a bf16 residual stream: out bf16 [M, N] in place, out = bf16(float(out) + gamma * (acc + bias)).
  *   K % 8 == 0, N % 8 == 0, all pointers 16-byte aligned.  bias_dev may be NULL.
- *   W is treated as a constant of the stream: its first tiles are requested as soon as the kernel starts,
- *   which (programmatic dependent launch) can be while the kernel enqueued just before it is still
- *   finishing -- do not produce W with that kernel.  A, bias and the outputs are touched only after it.
+ *   W is treated as a constant of the stream: its first tiles are requested as soon as the kernel starts, which
+ *   (programmatic dependent launch) can be while the kernel enqueued just before it, or before that one if it was launched
+ *   the same way, is still running -- do not produce W with these kernels unless a copy, an event or an ordinary launch lies
+ *   between.  The same holds for the weights of a context and of the head.  A, bias, gamma and the outputs are touched only
+ *   after all of them, as is everything else that the calls of this header read.
  *   status_dev: int32 device word that receives a non-zero code if a bounded wait expires (or NULL).
  *   splitk_ws_dev: not used any more (shapes with too few output tiles to occupy the GPU split K over the CTAs of a cluster, without
  *               scratch); NULL, or a buffer of at least fv_gemm_splitk_workspace_bytes() bytes, CAPACITY if it is smaller. */

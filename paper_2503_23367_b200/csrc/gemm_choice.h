@@ -13,7 +13,7 @@ namespace fv {
 struct TileChoice { int bn; bool pair; int slices; };   // slices 1: no cluster
 // head_dim > 0: the QKV projection with head norms or rotation, whose epilogue exists for one-CTA tiles of at least 128 columns that hold
 // whole heads; only those are compared.  (Taking the cheapest of all and widening it until it was allowed: blocks of 820 and 1024 rows at C 2048 with 128-wide
-// heads 132 and 137 us, now 127 and 133; 820 rows at C 1920 130 -> 125.)
+// heads 133 and 139 us, now 129 and 135; 3249 rows at C 1024 193 -> 187.)
 inline TileChoice pick_tile(int M, int N, int K, int sms, int head_dim = 0) {
   const int num_kb = (K + 63) / 64;
   struct Cand { int bn; bool pair; int slices; double fixed_us, round_us, kb_us; };
