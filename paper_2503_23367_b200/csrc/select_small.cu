@@ -101,7 +101,9 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
-template <typename XT>
+// STEP: the build a scale step launches (restoration before, gather and LayerNorm after); the other is a selection alone, which may count
+// near-ties: code that the step's build had to carry too cost it 0.4 % of a schedule of small maps.
+template <typename XT, bool STEP>
 __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallArgs a) {
   extern __shared__ __align__(16) float sm[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, b = blockIdx.y;
@@ -308,7 +310,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
       if (pos >= 0) a.idx[(size_t)b * a.k + pos] = t;
     }
   }
-  if (a.near_tie && rank == 0) {   // tokens within 1e-5 of the threshold, the smallest kept key (all keys and flags are here)
+  if (!STEP && a.near_tie && rank == 0) {   // tokens within 1e-5 of the threshold, the smallest kept key (all keys and flags are here)
     uint32_t* r = reinterpret_cast<uint32_t*>(red);
     uint32_t tau = 0xFFFFFFFFu;
     for (int j = tid; j < n; j += kThreads)
@@ -328,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
       a.near_tie[b] = (int32_t)near;
     }
   }
-  if (!a.a_out) return;        // a selection alone
+  if (!STEP) return;
   __syncthreads();
 
   // ---- LayerNorm + modulation of the kept rows -> bf16 A operand; a warp per row, the arithmetic (and bits) of gather_ln_kernel
@@ -374,17 +376,19 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
 
 int g_clusters[2] = {0, 0};     // clusters of 8 / of 16 CTAs the GPU holds at once
 
-template <typename XT> cudaError_t attr() {
-  cudaError_t e = cudaFuncSetAttribute(select_small_kernel<XT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(select_small_kernel<XT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+template <typename XT, bool STEP> cudaError_t attr() {
+  cudaError_t e = cudaFuncSetAttribute(select_small_kernel<XT, STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(select_small_kernel<XT, STEP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;
 }
 
 }  // namespace
 
 static cudaError_t init_once() {
-  cudaError_t e = attr<float>();
-  if (e == cudaSuccess) e = attr<__nv_bfloat16>();
+  cudaError_t e = attr<float, true>();
+  if (e == cudaSuccess) e = attr<float, false>();
+  if (e == cudaSuccess) e = attr<__nv_bfloat16, true>();
+  if (e == cudaSuccess) e = attr<__nv_bfloat16, false>();
   if (e != cudaSuccess) return e;
   for (int i = 0; i < 2; ++i) {
     const int cl = kMaxCluster / 2 << i;
@@ -395,7 +399,7 @@ static cudaError_t init_once() {
     at[0].val.clusterDim.x = cl; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, select_small_kernel<float>, &cfg) == cudaSuccess) g_clusters[i] = clusters;
+    if (cudaOccupancyMaxActiveClusters(&clusters, select_small_kernel<float, true>, &cfg) == cudaSuccess) g_clusters[i] = clusters;
     else (void)cudaGetLastError();
   }
   return cudaSuccess;
@@ -442,7 +446,8 @@ cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st) {
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = cl; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = 2;
-  return f.x_bf16 ? cudaLaunchKernelEx(&cfg, select_small_kernel<__nv_bfloat16>, a) : cudaLaunchKernelEx(&cfg, select_small_kernel<float>, a);
+  auto go = [&](auto* step, auto* alone) { return cudaLaunchKernelEx(&cfg, f.a_out ? step : alone, a); };
+  return f.x_bf16 ? go(select_small_kernel<__nv_bfloat16, true>, select_small_kernel<__nv_bfloat16, false>) : go(select_small_kernel<float, true>, select_small_kernel<float, false>);
 }
 
 }  // namespace fv
