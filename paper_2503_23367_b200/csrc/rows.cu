@@ -487,20 +487,19 @@ __global__ void __launch_bounds__(256) restore_residual_interp_kernel(float* xf,
 // list, k words for every RT tokens: on small maps an inverse map built by two launches before this one costs more than that
 // (2 x 64 x 64 tokens, k 820, C 2048: 2.2 + 2.3 + 8.5 us and two more launches of the host); launch_restore_bf16 draws the line.  A warp takes a row at a time, up to eight
 // 16-byte loads per lane in flight.
-template <int TAPS, int RT>
+template <int TAPS, int RT, bool MAP>
 __global__ void __launch_bounds__(256) restore_bf16_kernel(const uint4* cache, int hc, int wc, const uint4* pivots,
-                                                           const int32_t* idx, const int32_t* inv, int n, int k, int h, int w, int C8, uint4* __restrict__ out) {
+                                                           const int32_t* idx, const int32_t* inv, int b0, int n, int k, int h, int w, int C8, uint4* __restrict__ out) {
   __shared__ int s_slot[RT];
-  const int tiles = (n + RT - 1) / RT, b = blockIdx.x / tiles, t0 = (blockIdx.x - b * tiles) * RT;
+  const int b = b0 + blockIdx.y, t0 = blockIdx.x * RT;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_trigger();
   if (threadIdx.x < RT) s_slot[threadIdx.x] = -1;
   __syncthreads();
   pdl_wait();
   const int32_t* ib = idx + (size_t)b * k;
-  if (inv) {
-    if (threadIdx.x < min(RT, n - t0)) s_slot[threadIdx.x] = dep_load(inv + (size_t)b * n + t0 + threadIdx.x);
-  } else for (int i0 = threadIdx.x; i0 < k; i0 += 256 * 8) {
+  if (MAP && threadIdx.x < min(RT, n - t0)) s_slot[threadIdx.x] = dep_load(inv + (size_t)b * n + t0 + threadIdx.x);
+  for (int i0 = MAP ? k : threadIdx.x; i0 < k; i0 += 256 * 8) {
     int v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = i0 + 256 * u < k ? dep_load(ib + i0 + 256 * u) - t0 : -1;
@@ -704,12 +703,20 @@ cudaError_t launch_restore_bf16(const void* cache, int hc, int wc, const void* p
   const bool small = (long)((n + 15) / 16) * B < g_rows_sms;
   auto go = [&](auto* k16, auto* k8) {
     const int rt = small ? 8 : 16;
-    return launch_pdl(small ? k8 : k16, dim3((unsigned)((n + rt - 1) / rt * (long)B)), dim3(256), 0, st, static_cast<const uint4*>(cache), hc, wc,
-                      static_cast<const uint4*>(pivots), idx, map ? inv_scratch : nullptr, n, k, h, w, C / 8, static_cast<uint4*>(out));
+    cudaError_t e = cudaSuccess;
+    for (int b0 = 0; b0 < B && e == cudaSuccess; b0 += 65535)   // (images along y, of which a grid has 65535)
+      e = launch_pdl(small ? k8 : k16, dim3((n + rt - 1) / rt, B - b0 < 65535 ? B - b0 : 65535), dim3(256), 0, st, static_cast<const uint4*>(cache), hc, wc,
+                     static_cast<const uint4*>(pivots), idx, inv_scratch, b0, n, k, h, w, C / 8, static_cast<uint4*>(out));
+    return e;
   };
-  if (interp_mode == 0) return go(restore_bf16_kernel<0, 16>, restore_bf16_kernel<0, 8>);
-  if (interp_mode == 1) return go(restore_bf16_kernel<4, 16>, restore_bf16_kernel<4, 8>);
-  return go(restore_bf16_kernel<16, 16>, restore_bf16_kernel<16, 8>);
+  if (map) {
+    if (interp_mode == 0) return go(restore_bf16_kernel<0, 16, true>, restore_bf16_kernel<0, 8, true>);
+    if (interp_mode == 1) return go(restore_bf16_kernel<4, 16, true>, restore_bf16_kernel<4, 8, true>);
+    return go(restore_bf16_kernel<16, 16, true>, restore_bf16_kernel<16, 8, true>);
+  }
+  if (interp_mode == 0) return go(restore_bf16_kernel<0, 16, false>, restore_bf16_kernel<0, 8, false>);
+  if (interp_mode == 1) return go(restore_bf16_kernel<4, 16, false>, restore_bf16_kernel<4, 8, false>);
+  return go(restore_bf16_kernel<16, 16, false>, restore_bf16_kernel<16, 8, false>);
 }
 
 cudaError_t launch_gather_rows(const float* x, const int32_t* idx, int B, int n, int k, int C, float* out, int32_t* status, cudaStream_t st) {
