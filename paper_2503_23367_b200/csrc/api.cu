@@ -540,8 +540,10 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
   if (c.cross_len && scale_idx > 0 && !ctx->text_ready) return FV_ERR_BAD_STATE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   void* x = out_dev;
+  // The copy below waits for everything before it, so the step's kernels may read the modulation vectors as early as they start.
+  const bool copied = out_dev != tokens_dev && !(pruned && c.granularity == 1);
   // (per-step granularity, pruned step: the output map is written whole by the final restoration)
-  if (out_dev != tokens_dev && !(pruned && c.granularity == 1) &&
+  if (copied &&
       cudaMemcpyAsync(out_dev, tokens_dev, (size_t)B * n * C * xes, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return FV_ERR_CUDA;
   if (c.cross_len && scale_idx == 0) {
@@ -658,7 +660,7 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
         inv_cur = flip ? ctx->inv2 : ctx->inv;
         f.x = x; f.x_bf16 = xb; f.B = B; f.n = n; f.C = C; f.k = k; f.h = h; f.w = w; f.hc = hc; f.wc = wc; f.mod_stride = mod_stride;
         if (pending) { f.y = ctx->y_buf; f.cache = pending_cache; f.inv_prev = flip ? ctx->inv : ctx->inv2; f.gamma_prev = pending_gamma; }
-        f.idx = idx_cur; f.inv = inv_cur; f.sigma = sigma; f.beta = beta; f.a_out = ctx->a_buf;
+        f.idx = idx_cur; f.inv = inv_cur; f.sigma = sigma; f.beta = beta; f.a_out = ctx->a_buf; f.early = copied;
         if (launch_select_small(f, st) != cudaSuccess) { s = FV_ERR_CUDA; break; }
         pending = false;
         idx = idx_cur;
@@ -678,7 +680,7 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
         if (e != cudaSuccess || e_join != cudaSuccess) { s = FV_ERR_CUDA; break; }
       }
       if (!fused && !small) {
-        e = launch_gather_ln(xr, idx, B, nr, k, C, sigma, beta, mod_stride, ctx->a_buf, ctx->status, st, xb);
+        e = launch_gather_ln(xr, idx, B, nr, k, C, sigma, beta, mod_stride, ctx->a_buf, ctx->status, st, xb, copied);
         if (e != cudaSuccess) { s = FV_ERR_CUDA; break; }
       }
       // ---- branch on the compact rows

@@ -158,6 +158,7 @@ struct SmallSelect {
   const void* y; const void* cache; const int32_t* inv_prev; const float* gamma_prev;   // the previous sublayer's; y null: nothing to restore
   int32_t* idx; int32_t* inv; float* score; int32_t* near_tie;                          // written (inv is not inv_prev; all but idx may be null)
   const float* sigma; const float* beta; void* a_out;                                   // a_out null: no gather
+  bool early;                                                                           // as for launch_gather_ln, gate included
 };
 cudaError_t select_small_init();
 bool select_small_supported(int B, int n, int C, bool x_bf16);
@@ -167,7 +168,9 @@ cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st);
 // status (all gathers): device status word that receives DEV_BAD_ROW_INDEX when an index lies outside [0, n) (the
 // index is clamped, so the read stays inside the map), or null.
 cudaError_t launch_gather_ln(const void* x, const int32_t* idx, int B, int n, int k, int C, const float* sigma,
-                             const float* beta, int mod_stride, void* a_out, int32_t* status, cudaStream_t st, bool x_bf16 = false);
+                             const float* beta, int mod_stride, void* a_out, int32_t* status, cudaStream_t st, bool x_bf16 = false, bool early = false);
+// (early: sigma and beta may be read before the launches in front have finished.  Only for a caller that has put a copy, or another operation that is not
+// launched programmatically, between whatever writes them and its first kernel: fv_var_step out of place.)
 // A wait nobody ends: one warp waits on an mbarrier without arrivals for limit_ns, then writes DEV_TIMEOUT_SELFTEST.
 cudaError_t launch_expired_wait(int32_t* status, unsigned long long limit_ns, cudaStream_t st);
 // colsum_ws: null, or the selection workspace that receives the column sums of the updated x.

@@ -41,6 +41,7 @@ struct SmallArgs {
   const float *sigma, *beta;
   uint2* a_out;
   int rows_per_cta;                   // R
+  bool early;                         // gate and modulation may be read before the dependency wait
 };
 
 // shared memory of a CTA, in 4-byte words
@@ -131,24 +132,28 @@ __global__ void __launch_bounds__(kThreads, 1) select_small_kernel(const SmallAr
   pdl_trigger();
   cluster_arrive_relaxed();
   for (int i = tid; i < (n + 15) / 16 * 4; i += kThreads) reinterpret_cast<uint32_t*>(flags)[i] = 0u;
+  // gate and modulation vectors: behind the wait when the kernel before may have produced them (a step in place), else at once
+  const bool lookup = a.y && tid < own, modulate = a.sigma && tid < C / 4;   // (own <= R and C / 4 are at most kThreads)
+  float4 sg = make_float4(0.f, 0.f, 0.f, 0.f), bt = sg;
+  float gam[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) gam[e] = 1.f;
+  auto fetch_mod = [&] {
+    if (live && a.y && a.gamma_prev) load_row8(a.gamma_prev + (size_t)b * a.mod_stride + ct * 8, gam);
+    if (modulate) {
+      sg = x_load4(a.sigma + (size_t)b * a.mod_stride + tid * 4);
+      bt = x_load4(a.beta + (size_t)b * a.mod_stride + tid * 4);
+    }
+  };
+  if (STEP && a.early) fetch_mod();
   pdl_wait();
-  // (gate and modulation vectors too: the step may be in place and they the product of the kernel before it)
   float v[kRows][8];
 #pragma unroll
   for (int u = 0; u < 4; ++u)            // the first rows are fetched while the sources of all rows are looked up
     if (live && u * G + g < own) load_row8(xb + (size_t)(r0 + u * G + g) * C, v[u]);
-  const bool lookup = a.y && tid < own, modulate = a.sigma && tid < C / 4;   // (own <= R and C / 4 are at most kThreads)
   int j = 0;
-  float4 sg = make_float4(0.f, 0.f, 0.f, 0.f), bt = sg;
   if (lookup) j = load_index(a.inv_prev + (size_t)b * n + r0 + tid);
-  float gam[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) gam[e] = 1.f;
-  if (live && a.y && a.gamma_prev) load_row8(a.gamma_prev + (size_t)b * a.mod_stride + ct * 8, gam);
-  if (modulate) {
-    sg = x_load4(a.sigma + (size_t)b * a.mod_stride + tid * 4);
-    bt = x_load4(a.beta + (size_t)b * a.mod_stride + tid * 4);
-  }
+  if (STEP && !a.early) fetch_mod();
   if (lookup) {
     const int t = r0 + tid, yy = t / a.w, xx = t - yy * a.w;
     s_src[tid] = j >= 0 ? j : ~((yy * a.hc) / a.h * a.wc + (xx * a.wc) / a.w);
@@ -432,7 +437,7 @@ cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st) {
   SmallArgs a{};
   a.x = f.x; a.y = static_cast<const uint4*>(f.y); a.cache = static_cast<const uint4*>(f.cache); a.inv_prev = f.inv_prev; a.gamma_prev = f.gamma_prev;
   a.n = f.n; a.C = f.C; a.k = f.k; a.h = f.h; a.w = f.w; a.hc = f.hc; a.wc = f.wc; a.mod_stride = f.mod_stride;
-  a.idx = f.idx; a.inv = f.inv; a.score = f.score; a.near_tie = f.near_tie; a.sigma = f.sigma; a.beta = f.beta; a.a_out = static_cast<uint2*>(f.a_out);
+  a.idx = f.idx; a.inv = f.inv; a.score = f.score; a.near_tie = f.near_tie; a.early = f.early; a.sigma = f.sigma; a.beta = f.beta; a.a_out = static_cast<uint2*>(f.a_out);
   a.rows_per_cta = (f.n + cl - 1) / cl;
   // algorithmic bytes: the map read (and written where it is restored from y and the cache), indices, the kept rows' bf16 copy
   const double es = f.x_bf16 ? 2.0 : 4.0;

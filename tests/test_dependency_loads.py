@@ -43,6 +43,24 @@ def _kernels():
 KERNELS = _kernels()
 
 
+def _before_the_wait(body):
+    """The statements in front of the first wait.  Local functions are taken out (they count where they are called), and one that loads may
+    be called there under `early` alone, the launcher's word that nothing still running writes what it reads."""
+    head = body[:body.index("pdl_wait()")]
+    for m in reversed(list(re.finditer(r"auto (\w+) = \[&\][^{]*\{", head))):
+        k, depth = m.end(), 1
+        while depth:
+            depth += {"{": 1, "}": -1}.get(head[k], 0)
+            k += 1
+        loads = re.search(LOADS, head[m.end():k])
+        head = head[:m.start()] + head[k:]
+        if loads:
+            for call in re.finditer(r"\b" + m.group(1) + r"\(", head):
+                line = head[head.rfind("\n", 0, call.start()) + 1:call.start()]
+                assert re.search(r"&& (a\.)?early\)", line), f"{m.group(1)} is called before the dependency wait"
+    return head
+
+
 def test_the_kernels_are_found():
     names = {k[1] for k in KERNELS}
     assert {"gather_ln_kernel", "select_small_kernel", "next_input_kernel", "gemm_cluster_kernel", "restore_bf16_kernel", "score_topk_kernel"} <= names
@@ -58,12 +76,20 @@ def test_loads_of_a_programmatic_kernel(file, name, params, body):
         launches = _strip(open(os.path.join(CSRC, file)).read())
         assert not re.search(r"launch_pdl\(\s*" + name, launches)
         return
-    assert not re.search(LOADS, body[:body.index("pdl_wait()")]), "loaded before the dependency wait"
+    assert not re.search(LOADS, _before_the_wait(body)), "loaded before the dependency wait"
     for chunk in re.split(r"\belse\b", body):           # the GEMM kernels' warp roles wait for themselves
         if "stage_bias(" in chunk and "gemm" in file:
             assert "pdl_wait()" in chunk[:chunk.index("stage_bias(")], "bias staged before the dependency wait"
     assert "__ldg" not in body
     assert not re.search(r"\bconst\s+\w+\s*\*\s*__restrict__", params), "read-only parameters may be loaded non-coherently"
+
+
+def test_only_a_step_out_of_place_lets_a_launch_read_early():
+    api = _strip(open(os.path.join(CSRC, "api.cu")).read())
+    calls = re.findall(r"launch_gather_ln\((.*?)\);", api, flags=re.S)
+    assert [c.split(",")[-1].strip() == "copied" for c in calls].count(True) == 1
+    assert re.search(r"const bool copied = out_dev != tokens_dev && !\(pruned && c\.granularity == 1\);", api)
+    assert re.search(r"if \(copied &&\s*cudaMemcpyAsync\(out_dev, tokens_dev", api)
 
 
 def test_no_other_code_loads_non_coherently():

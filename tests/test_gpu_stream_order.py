@@ -79,9 +79,10 @@ def test_layernorm_modulation_written_by_the_kernel_before(k, n, C):
 
 
 @pytest.mark.parametrize("step,keep,last", [(1, 1.0, 16), (2, 0.5, 16), (2, 0.3, 40)])
-def test_step_in_place_with_modulation_written_by_the_kernel_before(step, keep, last):
-    """No copy stands in front of the step's first kernel: gather + LayerNorm (unpruned), the one-launch selection of a small map,
-    the selection of a larger one."""
+@pytest.mark.parametrize("in_place", [True, False])
+def test_step_with_modulation_written_by_the_kernel_before(step, keep, last, in_place):
+    """In place no copy stands in front of the step's first kernel: gather + LayerNorm (unpruned), the one-launch selection of a small map,
+    the selection of a larger one.  Out of place one does, and the kernels behind it may read the modulation before their own waits."""
     L, B, C, H = 2, 2, 256, 4
     sides = [(2, 2), (8, 8), (last, last)]
     g = torch.Generator(device=DEV)
@@ -107,7 +108,7 @@ def test_step_in_place_with_modulation_written_by_the_kernel_before(step, keep, 
 
     def consume():
         ctx.set_state(step, kv)
-        return ctx.var_step(x, step, keep, out=x).clone()
+        return ctx.var_step(x, step, keep, out=x if in_place else None).clone()
 
     _check_in_order(produce, consume, produce.renew, rewind=lambda: x.copy_(maps[step]))
     assert ctx.device_status() == 0
