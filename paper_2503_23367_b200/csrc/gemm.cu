@@ -11,7 +11,7 @@
 //   warps 2-5: epilogue -- tcgen05.ld the accumulator (thread = row, 32 columns at a time), fuse bias /
 //              GELU / gate+residual / the Q | K-cache | V^T-cache split, and store; the accumulator is
 //              handed back as soon as it is in registers, so the epilogue of tile i runs under the
-//              MMAs of tile i+1.
+//              MMAs of tile i+1.  (Residual epilogues: warps 2-9, gemm_epilogue.cuh.)
 // BN (128 / 192 / 256) is picked per shape on the host to minimise rounds x tile width on the SM count.
 // Shapes with too few tiles to occupy the GPU (the small scale steps, where the GEMM is a stream of weights) split K over the CTAs of a
 // cluster (gemm_cluster.cu).
@@ -34,7 +34,6 @@ namespace {
 
 constexpr int BM = 128;
 constexpr int BK = 64;
-constexpr int kGemmThreads = 192;
 constexpr int kATileBytes = BM * BK * 2;  // 16 KB
 
 // kKps: k-blocks per pipeline stage.  The producer and the MMA issuer both pay a fixed price per stage (a barrier's wait, a
@@ -51,25 +50,27 @@ template <int BN> struct GemmCfg {
   static constexpr int kAccStride = (BN <= 64) ? 64 : ((BN == 128) ? 128 : 256);  // column offset of the second accumulator
   // operand stages | per-warp bias slices | barriers | (residual-epilogue kernels only) one turning tile per warp
   static constexpr int smem_bytes(bool resid) {
-    return kStages * kStageBytes + kBiasSmemBytes + 256 /*barriers*/ + (resid ? kResidSmemBytes : 0) + 1024 /*alignment slack*/;
+    return kStages * kStageBytes + (resid ? kResidBiasBytes + kResidSmemBytes : kBiasSmemBytes) + 256 /*barriers*/ + 1024 /*alignment slack*/;
   }
 };
 
-// KIND 1 (RESID): the instantiation launched for the residual epilogue.  It is a kernel of its own because that epilogue
-// needs ~90 more registers per thread; the others stay small enough for a bandwidth-bound kernel of another
+// KIND 1 / 3 (RESID): the instantiations launched for the residual epilogue of an fp32 / a bf16 stream.  They are kernels of their own because
+// that epilogue takes eight warps and more registers per thread; the others stay small enough for a bandwidth-bound kernel of another
 // stream (the restoration of the rows that were not kept) to share the SMs with them.
 template <int BN, int KIND>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(gemm_threads(KIND), 1)
 gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmDev p) {
   using Cfg = GemmCfg<BN>;
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;
-  constexpr bool RESID = KIND == 1;   // KIND 2: the QKV projection with cosine attention / rotary positions on Q and K
+  constexpr bool RESID = is_resid(KIND);   // KIND 2: the QKV projection with cosine attention / rotary positions on Q and K
+  constexpr bool XB = KIND == 3;
+  constexpr int kBiasBytes = RESID ? kResidBiasBytes : kBiasSmemBytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint4* bias_s = reinterpret_cast<uint4*>(smem + STAGES * Cfg::kStageBytes);   // per-warp bias slice of the tile
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + STAGES * Cfg::kStageBytes + kBiasSmemBytes);
-  float* resid_s = reinterpret_cast<float*>(smem + STAGES * Cfg::kStageBytes + kBiasSmemBytes + 256);   // RESID: one tile per warp
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + STAGES * Cfg::kStageBytes + kBiasBytes);
+  float* resid_s = reinterpret_cast<float*>(smem + STAGES * Cfg::kStageBytes + kBiasBytes + 256);   // RESID: one tile per warp
   uint64_t* empty_bar = full_bar + STAGES;
   uint64_t* acc_full = empty_bar + STAGES;   // [2]
   uint64_t* acc_empty = acc_full + 2;        // [2]
@@ -84,7 +85,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 128); }
+    for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], gemm_threads(KIND) - 64); }
     mbar_fence_init();
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
@@ -173,39 +174,42 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int m0 = (tile % tiles_m) * BM, n0 = (tile / tiles_m) * BN;
       const int row = m0 + quarter * 32 + lane;
       const bool row_ok = row < p.M;
-      uint4* bias_w = bias_s + quarter * 32;
+      uint4* bias_w = bias_s + (RESID ? warp - 2 : quarter) * 32;
       stage_bias(p, bias_w, lane, n0, BN);
-      // residual epilogue (images of fewer than 32 rows take the row-per-thread path below): the first chunk
-      // of `out` is on its way while the accumulator is computed
-      const bool resid = RESID && (p.rows_per_image >= 32 || p.epilogue == EPI_F32);
-      ResidRows rr;
-      float4 xa[8], xb[8];
-      if (resid) {
-        rr = resid_rows(p, lane, m0 + quarter * 32);
-        residual_load_x(p, rr, xa, lane, n0);
+      const uint32_t t0 = tmem_base + lane_off + buf * Cfg::kAccStride;
+      if constexpr (RESID) {
+        const int half = (warp - 2) >> 2;
+        const auto release = [&] { tc_fence_before(); mbar_arrive(&acc_empty[buf]); };
+        // the first chunk of `out` is on its way while the accumulator is computed
+        const bool turned = p.rows_per_image >= 32 || p.epilogue == EPI_F32;   // (images of fewer than 32 rows take the row-per-thread path)
+        ResidRows rr;
+        typename ResidX<XB>::Raw x[8];
+        if (turned) {
+          rr = resid_rows(p, lane, m0 + quarter * 32);
+          residual_load_x<XB>(p, rr, x, lane, n0 + 32 * half);
+        }
+        if (!mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); break; }
+        tc_fence_after();
+        if (turned) {
+          residual_tile<XB, BN>(p, rr, x, t0, half, lane, n0, bias_w, resid_s + (warp - 2) * kResidTileFloats, release);
+        } else {
+          const int img = row_ok ? row / p.rows_per_image : 0, jrow = row_ok ? row - img * p.rows_per_image : 0;
+#pragma unroll 1
+          for (int c0 = 32 * half; c0 < BN; c0 += 64) {
+            uint32_t r[32];
+            tmem_ld32(t0 + c0, r);
+            tmem_wait_ld();
+            if (c0 + 64 >= BN) release();
+            if (row_ok && n0 + c0 < p.N) epilogue_chunk(p, r, row, img, jrow, n0 + c0, bias_w + c0 / 8);
+          }
+        }
+        continue;
       }
       if (!mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); break; }
       tc_fence_after();
       const int img = row_ok ? row / p.rows_per_image : 0;
       const int jrow = row_ok ? row - img * p.rows_per_image : 0;
-      const uint32_t t0 = tmem_base + lane_off + buf * Cfg::kAccStride;
-      if (resid) {   // whole warp: rows are re-distributed over the lanes
-        float* tile_s = resid_s + quarter * (32 * kResidTilePitch);
-#pragma unroll 1
-        for (int ch = 0; ch < BN / 32; ++ch) {   // rolled: the code of one chunk is fetched once and then reused
-          uint32_t r0[32];
-          tmem_ld32(t0 + 32 * ch, r0);
-          if (ch + 1 < BN / 32) residual_load_x(p, rr, xb, lane, n0 + 32 * (ch + 1));
-          tmem_wait_ld();
-          if (ch == BN / 32 - 1) {  // accumulator fully in registers: hand the buffer back to the MMA warp
-            tc_fence_before();
-            mbar_arrive(&acc_empty[buf]);
-          }
-          if (n0 + 32 * ch < p.N) residual_chunk(p, rr, r0, xa, tile_s, lane, n0 + 32 * ch, bias_w + 4 * ch);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) xa[i] = xb[i];
-        }
-      } else if (KIND == 2) {
+      if (KIND == 2) {
         qkv_extras_tile<BN>(p, t0, row, row_ok, img, jrow, n0, bias_w);
         tc_fence_before();
         mbar_arrive(&acc_empty[buf]);
@@ -252,7 +256,7 @@ void load_encode() {
 }
 
 template <int BN, int KIND> cudaError_t set_attr() {
-  return cudaFuncSetAttribute(gemm_bf16_kernel<BN, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<BN>::smem_bytes(KIND == 1));
+  return cudaFuncSetAttribute(gemm_bf16_kernel<BN, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<BN>::smem_bytes(is_resid(KIND)));
 }
 
 }  // namespace
@@ -279,6 +283,10 @@ cudaError_t gemm_init() {
   if (e == cudaSuccess) e = set_attr<256, 1>();
   if (e == cudaSuccess) e = set_attr<64, 0>();
   if (e == cudaSuccess) e = set_attr<64, 1>();
+  if (e == cudaSuccess) e = set_attr<64, 3>();
+  if (e == cudaSuccess) e = set_attr<128, 3>();
+  if (e == cudaSuccess) e = set_attr<192, 3>();
+  if (e == cudaSuccess) e = set_attr<256, 3>();
   if (e == cudaSuccess) e = set_attr<128, 2>();
   if (e == cudaSuccess) e = set_attr<192, 2>();
   if (e == cudaSuccess) e = set_attr<256, 2>();
@@ -303,13 +311,15 @@ static cudaError_t launch_bn(const GemmArgs& g, const GemmDev& p, int tiles_m, c
   const long tiles = (long)tiles_m * ((g.N + BN - 1) / BN);
   const int grid = (int)(tiles < g_num_sms ? tiles : g_num_sms);
   if (p.epilogue == EPI_RESIDUAL || p.epilogue == EPI_F32)
-    return launch_pdl(gemm_bf16_kernel<BN, 1>, dim3(grid), dim3(kGemmThreads), GemmCfg<BN>::smem_bytes(true), st, tmA, tmB, p);
+    return launch_pdl(gemm_bf16_kernel<BN, 1>, dim3(grid), dim3(gemm_threads(1)), GemmCfg<BN>::smem_bytes(true), st, tmA, tmB, p);
+  if (p.epilogue == EPI_RESIDUAL_XBF16)
+    return launch_pdl(gemm_bf16_kernel<BN, 3>, dim3(grid), dim3(gemm_threads(3)), GemmCfg<BN>::smem_bytes(true), st, tmA, tmB, p);
   if constexpr (BN < 128)
     if (p.epilogue == EPI_QKV_SPLIT && (p.qk_scale || p.rope_table)) return cudaErrorInvalidValue;   // never chosen for them
   if constexpr (BN >= 128)
     if (p.epilogue == EPI_QKV_SPLIT && (p.qk_scale || p.rope_table))
-      return launch_pdl(gemm_bf16_kernel<BN, 2>, dim3(grid), dim3(kGemmThreads), GemmCfg<BN>::smem_bytes(false), st, tmA, tmB, p);
-  return launch_pdl(gemm_bf16_kernel<BN, 0>, dim3(grid), dim3(kGemmThreads), GemmCfg<BN>::smem_bytes(false), st, tmA, tmB, p);
+      return launch_pdl(gemm_bf16_kernel<BN, 2>, dim3(grid), dim3(gemm_threads(2)), GemmCfg<BN>::smem_bytes(false), st, tmA, tmB, p);
+  return launch_pdl(gemm_bf16_kernel<BN, 0>, dim3(grid), dim3(gemm_threads(0)), GemmCfg<BN>::smem_bytes(false), st, tmA, tmB, p);
 }
 
 static int g_force_path = 0;

@@ -78,23 +78,47 @@ __device__ __forceinline__ void chunk_values(const GemmDev& p, const uint32_t (&
   }
 }
 
-// ---- residual epilogue: out[row, :] += gamma[image of row] * (acc + bias), fp32 in place (+ bf16 copy);
+// ---- residual epilogue: out[row, :] += gamma[image of row] * (acc + bias) in place, a stream of fp32 or (XB) bf16 (+ bf16 copy);
 // also the plain fp32 result (EPI_F32: out = acc + bias, gamma and aux unused) ----
-// The accumulator comes out of TMEM one row per thread; read-modify-writing the fp32 stream that way would
+// The accumulator comes out of TMEM one row per thread; read-modify-writing the stream that way would
 // touch 32 different rows per instruction.  Each 32 x 32 chunk is therefore turned through the warp's
-// shared-memory tile (row pitch 36 floats: conflict-free both ways) so that lane l works on columns
-// 4 * (l & 7) .. +3 of rows (l >> 3) + 4 * i, i = 0..7: 8 lanes cover the 128 contiguous bytes of one row, and
-// a lane's column group is the same for all its rows, so the gate is one float4 per chunk.  One warp issues
-// the whole epilogue of its 32 rows with nothing to hide its instruction latencies behind, so the number
-// of instructions per chunk is what bounds it (measured: taking the loads and stores out changed nothing):
-// everything that does not depend on the chunk (row validity, the image boundary, the row pointers) is
-// set up once per tile.
+// shared-memory tile, 16 rows at a time (row pitch 36 floats: conflict-free both ways), so that lane l works on columns
+// 4 * (l & 7) .. +3 of rows (l >> 3) + 4 * i, i = 0..7: 8 lanes cover the contiguous 32 columns of one row, and
+// a lane's column group is the same for all its rows, so the gate is one float4 per chunk.  A launch of one round ends with this epilogue
+// and nothing to run it under, and a warp alone on its scheduler waits out every latency of the chain TMEM -> turn -> stream -> store: eight
+// warps take turns with the 32-column chunks, two per accumulator row (us with four / eight warps, fp32 stream: N 2048 K 2048 M 576 11.9 / 10.5,
+// M 800 12.0 / 10.7, M 2304 20.8 / 19.7; K 8192 M 800 30.8 / 29.2; fp32 result 8192 x 4096 x 2048 163 / 117; a bf16 stream, which went row by
+// row before: K 2048 M 800 15.6 / 10.6, M 2304 28.0 / 18.2, K 8192 M 800 33.4 / 28.8).  Everything that does not depend on the chunk (row
+// validity, the image boundary, the row pointers) is set up once per tile.
+constexpr int kResidWarps = 8;
+__host__ __device__ constexpr bool is_resid(int kind) { return kind == 1 || kind == 3; }   // kernel instantiations for an fp32 / a bf16 stream
+__host__ __device__ constexpr int gemm_threads(int kind) { return 64 + 32 * (is_resid(kind) ? kResidWarps : 4); }   // producer, issuer, epilogue
 constexpr int kResidTilePitch = 36;
-constexpr int kResidSmemBytes = 4 * 32 * kResidTilePitch * 4;   // one tile per epilogue warp
+constexpr int kResidTileRows = 16;
+constexpr int kResidTileFloats = kResidTileRows * kResidTilePitch;
+constexpr int kResidSmemBytes = kResidWarps * kResidTileFloats * 4;   // one tile per epilogue warp
+constexpr int kResidBiasBytes = kResidWarps * 512;                    // one bias slice per epilogue warp
+
+template <bool XB> struct ResidX;      // four values of the stream
+template <> struct ResidX<false> {
+  using Raw = float4;
+  static __device__ __forceinline__ Raw load(const void* out, size_t at) { return *reinterpret_cast<const float4*>(static_cast<const float*>(out) + at); }
+  static __device__ __forceinline__ float4 value(const Raw& r) { return r; }
+  static __device__ __forceinline__ void store(void* out, size_t at, const float4& v) { *reinterpret_cast<float4*>(static_cast<float*>(out) + at) = v; }
+};
+template <> struct ResidX<true> {
+  using Raw = uint2;
+  static __device__ __forceinline__ Raw load(const void* out, size_t at) { return *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(out) + at); }
+  static __device__ __forceinline__ float4 value(const Raw& r) {
+    return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xFFFF0000u));
+  }
+  static __device__ __forceinline__ void store(void* out, size_t at, const float4& v) {   // rounded to nearest even once
+    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + at) = make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
+  }
+};
 
 struct ResidRows {
-  float* out0;             // &out[first row of the lane, 4 * (lane & 7)] (column offset of the chunk not included)
-  __nv_bfloat16* aux0;     // same position in the bf16 copy, or nullptr
+  size_t at0;              // element offset of &out[first row of the lane, 4 * (lane & 7)] (column offset of the chunk not included)
   const float* gam0;       // gate vector of the image of the warp's first row (+ the lane's column offset), or nullptr
   const float* gam1;       // gate vector of the next image
   int n_rows;              // the lane's rows i < n_rows exist
@@ -108,8 +132,7 @@ __device__ __forceinline__ ResidRows resid_rows(const GemmDev& p, int lane, int 
   ResidRows rr;
   const int r = row0 + (lane >> 3);
   const int cl = 4 * (lane & 7);
-  rr.out0 = static_cast<float*>(p.out) + (size_t)r * p.N + cl;
-  rr.aux0 = p.aux ? static_cast<__nv_bfloat16*>(p.aux) + (size_t)r * p.N + cl : nullptr;
+  rr.at0 = (size_t)r * p.N + cl;
   rr.n_rows = max(0, min(8, (p.M - r + 3) >> 2));
   rr.n_load = p.epilogue == EPI_F32 ? 0 : rr.n_rows;
   const int img0 = min(row0, p.M - 1) / p.rows_per_image;
@@ -119,46 +142,73 @@ __device__ __forceinline__ ResidRows resid_rows(const GemmDev& p, int lane, int 
   return rr;
 }
 
-// The lane's 8 float4 of `out` for the chunk at column `col`; fetched one chunk ahead of its use.
-__device__ __forceinline__ void residual_load_x(const GemmDev& p, const ResidRows& rr, float4 (&x)[8], int lane, int col) {
+// The lane's 8 x 4 values of `out` for the chunk at column `col`; fetched one chunk ahead of their use.
+template <bool XB>
+__device__ __forceinline__ void residual_load_x(const GemmDev& p, const ResidRows& rr, typename ResidX<XB>::Raw (&x)[8], int lane, int col) {
   const bool col_ok = col + 4 * (lane & 7) < p.N;
 #pragma unroll
   for (int i = 0; i < 8; ++i)
-    if (col_ok && i < rr.n_load) x[i] = *reinterpret_cast<const float4*>(rr.out0 + (size_t)(4 * i) * p.N + col);
+    if (col_ok && i < rr.n_load) x[i] = ResidX<XB>::load(p.out, rr.at0 + (size_t)(4 * i) * p.N + col);
 }
 
-__device__ __forceinline__ void residual_chunk(const GemmDev& p, const ResidRows& rr, const uint32_t (&r)[32], const float4 (&x)[8],
+template <bool XB>
+__device__ __forceinline__ void residual_chunk(const GemmDev& p, const ResidRows& rr, const uint32_t (&r)[32], const typename ResidX<XB>::Raw (&x)[8],
                                                float* tile, int lane, int col, const uint4* bias4) {
   float v[32];
   chunk_values(p, r, col, v, bias4);
+  const bool col_ok = col + 4 * (lane & 7) < p.N;
+  float4 g0 = make_float4(1.f, 1.f, 1.f, 1.f), g1 = g0;
+  if (col_ok && rr.gam0) {
+    g0 = dep_load4(rr.gam0 + col);
+    if (rr.n_first < rr.n_rows) g1 = dep_load4(rr.gam1 + col);
+  }
+  __nv_bfloat16* aux = static_cast<__nv_bfloat16*>(p.aux);
 #pragma unroll
-  for (int g = 0; g < 8; ++g)
-    *reinterpret_cast<float4*>(tile + lane * kResidTilePitch + 4 * g) = make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
-  __syncwarp();
-  if (col + 4 * (lane & 7) < p.N) {
-    float4 g0 = make_float4(1.f, 1.f, 1.f, 1.f), g1 = g0;
-    if (rr.gam0) {
-      g0 = dep_load4(rr.gam0 + col);
-      if (rr.n_first < rr.n_rows) g1 = dep_load4(rr.gam1 + col);
+  for (int pass = 0; pass < 2; ++pass) {     // rows 0..15, rows 16..31 of the warp's 32
+    if ((lane >> 4) == pass) {
+#pragma unroll
+      for (int g = 0; g < 8; ++g)
+        *reinterpret_cast<float4*>(tile + (lane & 15) * kResidTilePitch + 4 * g) = make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
     }
-    const float* trow = tile + (lane >> 3) * kResidTilePitch + 4 * (lane & 7);
+    __syncwarp();
+    if (col_ok) {
+      const float* trow = tile + (lane >> 3) * kResidTilePitch + 4 * (lane & 7);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (i < rr.n_rows) {
-        const float4 a = *reinterpret_cast<const float4*>(trow + 4 * i * kResidTilePitch);
-        const float4 gg = i < rr.n_first ? g0 : g1;
-        float4 xv = i < rr.n_load ? x[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        xv.x = fmaf(gg.x, a.x, xv.x); xv.y = fmaf(gg.y, a.y, xv.y); xv.z = fmaf(gg.z, a.z, xv.z); xv.w = fmaf(gg.w, a.w, xv.w);
-        *reinterpret_cast<float4*>(rr.out0 + (size_t)(4 * i) * p.N + col) = xv;
-        if (rr.aux0) {
-          uint2 o;
-          o.x = pack_bf16x2(a.x, a.y); o.y = pack_bf16x2(a.z, a.w);
-          *reinterpret_cast<uint2*>(rr.aux0 + (size_t)(4 * i) * p.N + col) = o;
+      for (int u = 0; u < 4; ++u) {
+        const int i = 4 * pass + u;
+        if (i < rr.n_rows) {
+          const float4 a = *reinterpret_cast<const float4*>(trow + 4 * u * kResidTilePitch);
+          const float4 gg = i < rr.n_first ? g0 : g1;
+          float4 xv = i < rr.n_load ? ResidX<XB>::value(x[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
+          xv.x = fmaf(gg.x, a.x, xv.x); xv.y = fmaf(gg.y, a.y, xv.y); xv.z = fmaf(gg.z, a.z, xv.z); xv.w = fmaf(gg.w, a.w, xv.w);
+          const size_t at = rr.at0 + (size_t)(4 * i) * p.N + col;
+          ResidX<XB>::store(p.out, at, xv);
+          if (aux) *reinterpret_cast<uint2*>(aux + at) = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
         }
       }
     }
+    __syncwarp();
   }
-  __syncwarp();
+}
+
+// A warp's share of the residual tile whose accumulator starts at TMEM address t0 (the warp's quarter of the lanes): the chunks
+// `half`, `half` + 2, ... of its 32 rows.  x: the first of them, already requested.  release(): the warp's last accumulator read is done.
+template <bool XB, int BN, typename Release>
+__device__ __forceinline__ void residual_tile(const GemmDev& p, const ResidRows& rr, typename ResidX<XB>::Raw (&x)[8], uint32_t t0, int half, int lane, int n0,
+                                              const uint4* bias_w, float* tile, Release release) {
+  constexpr int kChunks = BN / 32;
+#pragma unroll 1
+  for (int ch = half; ch < kChunks; ch += 2) {   // rolled: the code of one chunk is fetched once and then reused
+    uint32_t r[32];
+    typename ResidX<XB>::Raw nx[8];
+    tmem_ld32(t0 + 32 * ch, r);
+    if (ch + 2 < kChunks) residual_load_x<XB>(p, rr, nx, lane, n0 + 32 * (ch + 2));
+    tmem_wait_ld();
+    if (ch + 2 >= kChunks) release();            // accumulator fully in registers: hand the buffer back to the MMA warp
+    if (n0 + 32 * ch < p.N) residual_chunk<XB>(p, rr, r, x, tile, lane, n0 + 32 * ch, bias_w + 4 * ch);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = nx[i];
+  }
 }
 
 // One 32-column chunk of one accumulator row: bias, optional GELU, then the epilogue's store.

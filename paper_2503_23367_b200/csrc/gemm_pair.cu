@@ -28,7 +28,6 @@ namespace {
 
 constexpr int BM = 128;   // rows of A per CTA (256 per pair)
 constexpr int BK = 64;
-constexpr int kThreads = 192;
 constexpr int kATileBytes = BM * BK * 2;  // 16 KB
 
 template <int BN> struct PairCfg {
@@ -41,25 +40,27 @@ template <int BN> struct PairCfg {
   static constexpr int kAccStride = 256;
   // operand stages | per-warp bias slices | barriers | (residual-epilogue kernels only) one turning tile per warp
   static constexpr int smem_bytes(bool resid) {
-    return kStages * kStageBytes + kBiasSmemBytes + 256 /*barriers*/ + (resid ? kResidSmemBytes : 0) + 1024 /*alignment slack*/;
+    return kStages * kStageBytes + (resid ? kResidBiasBytes + kResidSmemBytes : kBiasSmemBytes) + 256 /*barriers*/ + 1024 /*alignment slack*/;
   }
 };
 
-// RESID: the instantiation launched for the residual epilogue (a kernel of its own: it needs far more registers).
-template <int BN, bool RESID>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+// KIND 1 / 3 (RESID): the instantiations launched for the residual epilogue of an fp32 / a bf16 stream (eight epilogue warps); 0: the others.
+template <int BN, int KIND>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads(KIND), 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmDev p) {
   using Cfg = PairCfg<BN>;
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;
+  constexpr bool RESID = is_resid(KIND), XB = KIND == 3;
+  constexpr int kBiasBytes = RESID ? kResidBiasBytes : kBiasSmemBytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint4* bias_s = reinterpret_cast<uint4*>(smem + STAGES * Cfg::kStageBytes);   // per-warp bias slice of the tile
-  float* resid_s = reinterpret_cast<float*>(smem + STAGES * Cfg::kStageBytes + kBiasSmemBytes + 256);   // RESID: one tile per warp
-  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + STAGES * Cfg::kStageBytes + kBiasSmemBytes);  // used in the leader
+  float* resid_s = reinterpret_cast<float*>(smem + STAGES * Cfg::kStageBytes + kBiasBytes + 256);   // RESID: one tile per warp
+  uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + STAGES * Cfg::kStageBytes + kBiasBytes);  // used in the leader
   uint64_t* empty_bar = full_bar + STAGES;   // one per CTA, completed by the leader's commits
   uint64_t* acc_full = empty_bar + STAGES;   // [2] one per CTA
-  uint64_t* acc_empty = acc_full + 2;        // [2] used in the leader: 256 arrivals
+  uint64_t* acc_empty = acc_full + 2;        // [2] used in the leader: an arrival of every epilogue thread of the pair
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
   pdl_trigger();
@@ -73,7 +74,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 256); }
+    for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 2 * (gemm_threads(KIND) - 64)); }
     mbar_fence_init();
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
@@ -164,39 +165,40 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       const int m0 = (tile % tiles_m) * (2 * BM) + (int)rank * BM, n0 = (tile / tiles_m) * BN;
       const int row = m0 + quarter * 32 + lane;
       const bool row_ok = row < p.M;
-      uint4* bias_w = bias_s + quarter * 32;
+      uint4* bias_w = bias_s + (RESID ? warp - 2 : quarter) * 32;
       stage_bias(p, bias_w, lane, n0, BN);
-      // residual epilogue (images of fewer than 32 rows take the row-per-thread path below): the first chunk
-      // of `out` is on its way while the accumulator is computed
-      const bool resid = RESID && (p.rows_per_image >= 32 || p.epilogue == EPI_F32);
-      ResidRows rr;
-      float4 xa[8], xb[8];
-      if (resid) {
-        rr = resid_rows(p, lane, m0 + quarter * 32);
-        residual_load_x(p, rr, xa, lane, n0);
-      }
-      if (!mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); break; }
-      tc_fence_after();
-      const int img = row_ok ? row / p.rows_per_image : 0;
-      const int jrow = row_ok ? row - img * p.rows_per_image : 0;
       const uint32_t t0 = tmem_base + lane_off + buf * Cfg::kAccStride;
-      if (resid) {   // whole warp: rows are re-distributed over the lanes
-        float* tile_s = resid_s + quarter * (32 * kResidTilePitch);
+      if constexpr (RESID) {
+        const int half = (warp - 2) >> 2;
+        const auto release = [&] { tc_fence_before(); mbar_arrive_cluster(&acc_empty[buf], 0); };
+        // the first chunk of `out` is on its way while the accumulator is computed
+        const bool turned = p.rows_per_image >= 32 || p.epilogue == EPI_F32;   // (images of fewer than 32 rows take the row-per-thread path)
+        ResidRows rr;
+        typename ResidX<XB>::Raw x[8];
+        if (turned) {
+          rr = resid_rows(p, lane, m0 + quarter * 32);
+          residual_load_x<XB>(p, rr, x, lane, n0 + 32 * half);
+        }
+        if (!mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); break; }
+        tc_fence_after();
+        if (turned) {
+          residual_tile<XB, BN>(p, rr, x, t0, half, lane, n0, bias_w, resid_s + (warp - 2) * kResidTileFloats, release);
+        } else {
+          const int img = row_ok ? row / p.rows_per_image : 0, jrow = row_ok ? row - img * p.rows_per_image : 0;
 #pragma unroll 1
-        for (int ch = 0; ch < BN / 32; ++ch) {   // rolled: the code of one chunk is fetched once and then reused
-          uint32_t r0[32];
-          tmem_ld32(t0 + 32 * ch, r0);
-          if (ch + 1 < BN / 32) residual_load_x(p, rr, xb, lane, n0 + 32 * (ch + 1));
-          tmem_wait_ld();
-          if (ch == BN / 32 - 1) {  // accumulator fully in registers: hand the buffer back to the MMA warp
-            tc_fence_before();
-            mbar_arrive_cluster(&acc_empty[buf], 0);
+          for (int c0 = 32 * half; c0 < BN; c0 += 64) {
+            uint32_t r[32];
+            tmem_ld32(t0 + c0, r);
+            tmem_wait_ld();
+            if (c0 + 64 >= BN) release();
+            if (row_ok && n0 + c0 < p.N) epilogue_chunk(p, r, row, img, jrow, n0 + c0, bias_w + c0 / 8);
           }
-          if (n0 + 32 * ch < p.N) residual_chunk(p, rr, r0, xa, tile_s, lane, n0 + 32 * ch, bias_w + 4 * ch);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) xa[i] = xb[i];
         }
       } else {
+        if (!mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); break; }
+        tc_fence_after();
+        const int img = row_ok ? row / p.rows_per_image : 0;
+        const int jrow = row_ok ? row - img * p.rows_per_image : 0;
 #pragma unroll 1
         for (int c0 = 0; c0 < BN; c0 += 64) {
           uint32_t r0[32], r1[32];
@@ -227,20 +229,26 @@ int g_pair_sms = 148;
 
 }  // namespace
 
-template <int BN, bool RESID> static cudaError_t set_pair_attr() {
-  return cudaFuncSetAttribute(gemm_pair_kernel<BN, RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<BN>::smem_bytes(RESID));
+template <int BN, int KIND> static cudaError_t set_pair_attr() {
+  return cudaFuncSetAttribute(gemm_pair_kernel<BN, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, PairCfg<BN>::smem_bytes(is_resid(KIND)));
 }
 
 cudaError_t gemm_pair_init() {
-  cudaError_t e = set_pair_attr<256, false>();
-  if (e == cudaSuccess) e = set_pair_attr<128, false>();
-  if (e == cudaSuccess) e = set_pair_attr<256, true>();
-  if (e == cudaSuccess) e = set_pair_attr<128, true>();
+  cudaError_t e = set_pair_attr<256, 0>();
+  if (e == cudaSuccess) e = set_pair_attr<128, 0>();
+  if (e == cudaSuccess) e = set_pair_attr<256, 1>();
+  if (e == cudaSuccess) e = set_pair_attr<128, 1>();
+  if (e == cudaSuccess) e = set_pair_attr<256, 3>();
+  if (e == cudaSuccess) e = set_pair_attr<128, 3>();
   if (e != cudaSuccess) return e;
   int dev = 0;
   e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   return cudaDeviceGetAttribute(&g_pair_sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
+template <int BN, int KIND> static cudaError_t launch_kind(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmDev& p, int pairs, cudaStream_t st) {
+  return launch_pdl(gemm_pair_kernel<BN, KIND>, dim3(2 * pairs), dim3(gemm_threads(KIND)), PairCfg<BN>::smem_bytes(is_resid(KIND)), st, tmA, tmB, p);
 }
 
 cudaError_t launch_gemm_pair(const GemmArgs& g, const GemmDev& p, int bn, cudaStream_t st) {
@@ -250,11 +258,9 @@ cudaError_t launch_gemm_pair(const GemmArgs& g, const GemmDev& p, int bn, cudaSt
   const long tiles = (long)((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + bn - 1) / bn);
   const int max_pairs = g_pair_sms / 2;
   const int pairs = (int)(tiles < max_pairs ? tiles : max_pairs);
-  const bool resid = p.epilogue == EPI_RESIDUAL || p.epilogue == EPI_F32;
-  if (bn == 256 && resid) return launch_pdl(gemm_pair_kernel<256, true>, dim3(2 * pairs), dim3(kThreads), PairCfg<256>::smem_bytes(true), st, tmA, tmB, p);
-  if (bn == 128 && resid) return launch_pdl(gemm_pair_kernel<128, true>, dim3(2 * pairs), dim3(kThreads), PairCfg<128>::smem_bytes(true), st, tmA, tmB, p);
-  if (bn == 256) return launch_pdl(gemm_pair_kernel<256, false>, dim3(2 * pairs), dim3(kThreads), PairCfg<256>::smem_bytes(false), st, tmA, tmB, p);
-  if (bn == 128) return launch_pdl(gemm_pair_kernel<128, false>, dim3(2 * pairs), dim3(kThreads), PairCfg<128>::smem_bytes(false), st, tmA, tmB, p);
+  const int kind = p.epilogue == EPI_RESIDUAL || p.epilogue == EPI_F32 ? 1 : (p.epilogue == EPI_RESIDUAL_XBF16 ? 3 : 0);
+  if (bn == 256) return kind == 1 ? launch_kind<256, 1>(tmA, tmB, p, pairs, st) : (kind == 3 ? launch_kind<256, 3>(tmA, tmB, p, pairs, st) : launch_kind<256, 0>(tmA, tmB, p, pairs, st));
+  if (bn == 128) return kind == 1 ? launch_kind<128, 1>(tmA, tmB, p, pairs, st) : (kind == 3 ? launch_kind<128, 3>(tmA, tmB, p, pairs, st) : launch_kind<128, 0>(tmA, tmB, p, pairs, st));
   return cudaErrorInvalidValue;
 }
 

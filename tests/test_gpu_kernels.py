@@ -640,6 +640,40 @@ def test_gemm_residual_epilogue_at_step_shapes(rows, N, K):
     assert np.abs(xd.cpu().numpy() - ref).max() <= 2e-3
 
 
+@pytest.mark.parametrize("path", [0, 2, 3, 4, 5, 6, 7])
+@pytest.mark.parametrize("B,rows,N,K", [(3, 33, 136, 72), (2, 127, 320, 264), (5, 20, 264, 128), (2, 301, 1032, 256)])
+@pytest.mark.parametrize("epilogue", [2, 5])
+def test_gemm_residual_epilogue_of_either_stream(B, rows, N, K, path, epilogue):
+    """Gate + residual into an fp32 (2) and a bf16 (5) stream on every tile: the image boundary inside a warp's 32 rows, images of
+    fewer than 32 rows (row per thread), rows and columns past the last tile's end, an odd number of 32-column chunks."""
+    M = B * rows
+    a = I.normal_bf16(93, (M, K)); w = I.normal_bf16(94, (N, K), 0.05); b = I.normal_bf16(95, (N,), 0.02)
+    gamma = I.normal(96, (B, N), 0.3)
+    xd = dev(I.normal(97, (M, N)))
+    if epilogue == 5:
+        xd = xd.bfloat16()
+    x = xd.double().cpu().numpy()
+    aux = torch.zeros((M, N), dtype=torch.bfloat16, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    assert fv.lib().fv_gemm_force_path(path) == 0
+    try:
+        fv.fv_gemm_bf16(bf16_dev(a), bf16_dev(w), bf16_dev(b), epilogue=epilogue, out=xd, aux=aux, gamma=dev(gamma), mod_stride=N, rows_per_image=rows, status=status)
+        torch.cuda.synchronize()
+    finally:
+        fv.lib().fv_gemm_force_path(0)
+    assert int(status.item()) == 0
+    af, wf = I.bf16_bits_to_f32(a).astype(np.float64), I.bf16_bits_to_f32(w).astype(np.float64)
+    y = O.linear(af, wf, I.bf16_bits_to_f32(b))
+    sums = 2 * K * 2.0 ** -24 * (np.abs(af) @ np.abs(wf).T + 1)        # fp32 accumulation of K products and the bias, any order
+    g = np.repeat(gamma.astype(np.float64), rows, axis=0)
+    ref = x + g * y
+    bound = np.abs(g) * sums + 2.0 ** -23 * np.abs(ref)
+    if epilogue == 5:
+        bound = bound + 2.0 ** -8 * (np.abs(ref) + bound)               # one rounding of the stream to bf16
+    assert (np.abs(xd.double().cpu().numpy() - ref) <= bound).all()
+    assert (np.abs(bf16_host(aux) - y) <= sums + 2.0 ** -8 * (np.abs(y) + sums)).all()
+
+
 # ------------------------------------------------------------------ attention over the KV cache
 ATTN_CASES = [  # B, rows, H, C, kv_len, cap
     (2, 85, 4, 256, 340, 344), (1, 300, 2, 256, 1000, 1024), (2, 128, 16, 1024, 485, 488), (1, 1, 4, 256, 1, 8),
