@@ -587,7 +587,16 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
   // restores its own.
   const bool fused = selecting && g_step_fused && !xb && select_fused_supported(B, n, C);
   // Small maps: one launch between two branches (select_small.cu); the last sublayer's restoration is a launch of its own.
-  const bool small = selecting && !fused && c.interp_mode == 0 && select_small_supported(B, n, C, xb);
+  const bool small_map = c.interp_mode == 0 && select_small_supported(B, n, C, xb);
+  const bool small = selecting && !fused && small_map;
+  // On the others the kept rows of a sublayer are restored by its last GEMM, straight from the accumulators: row j of the compact tensor is added to its
+  // token's row of x, and the column sums of the updated rows fall out of the same registers.  As a launch of their own (forwarded rows stored in bf16, read
+  // again, sums folded behind them) they took 13 us (64 x 64 tokens, C 2048), 19 (80 x 80) and 26 (128 x 128) between the GEMM and the selection that waits
+  // for them; the epilogue is 1 ... 5 us longer (us per block of a pruned step: 64 x 64 311 -> 282, two images 434 -> 393, 80 x 80 418 -> 387, 128 x 128 951 -> 919,
+  // four of 32 x 32 at C 1920 270 -> 262).  Images of fewer kept rows than a
+  // tile take that launch, and so do small maps whose kept set is given, which then come out as the one-launch form leaves them, bit for bit.
+  const bool gemm_restores = sub_pruned && !fused && !small_map && k >= kMinMapRows;
+  float* kept_partial = nullptr;        // the column sums that the last such GEMM left (in y_buf, which then holds no forwarded rows)
   if (selecting && !small && cudaMemsetAsync(ctx->sel_ws, 0, select_ticket_bytes(B), st) != cudaSuccess) return FV_ERR_CUDA;
   bool pending = false;                 // a restoration waits for the next selection's launch (fused: of the kept rows)
   const float* pending_gamma = nullptr;
@@ -617,7 +626,7 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
           e = launch_inv_from_idx(idx, B, k, n, ctx->inv, st);
         } else if (!fused && !small) {
           idx = ctx->idx;
-          e = launch_select(x, B, n, C, k, ctx->idx, ctx->inv, nullptr, nullptr, ctx->sel_ws, have_partials, st, xb);
+          e = launch_select(x, B, n, C, k, ctx->idx, ctx->inv, nullptr, nullptr, ctx->sel_ws, have_partials, st, xb, kept_partial, k);
         }
         if (e != cudaSuccess) { s = FV_ERR_CUDA; break; }
         if (!fused && !small && idx_trace_dev && cudaMemcpyAsync(idx_trace_dev + trace_off, idx, (size_t)B * k * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
@@ -674,7 +683,8 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
         // touch disjoint rows of x).
         if (cudaEventRecord(ctx->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) != cudaSuccess) { s = FV_ERR_CUDA; break; }
         e = launch_restore_residual(x, ctx->y_buf, cache_sub, inv_cur, gamma, mod_stride, B, k, h, w, hc, wc, C,
-                                    more ? ctx->sel_ws : nullptr, (fused && more) ? 3 : 1, c.interp_mode, ctx->side, xb);
+                                    more ? ctx->sel_ws : nullptr, more && fused ? 3 : 1, c.interp_mode, ctx->side, xb);
+        if (e == cudaSuccess && more && gemm_restores) e = launch_colsum_total(B, n, C, ctx->sel_ws, ctx->side);
         const cudaError_t e_join = cudaEventRecord(ctx->ev_join, ctx->side);   // recorded even if the launch failed
         forked = e_join == cudaSuccess;
         if (e != cudaSuccess || e_join != cudaSuccess) { s = FV_ERR_CUDA; break; }
@@ -725,7 +735,17 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
       GemmArgs o{};
       o.status = ctx->status; o.rows_per_image = k; o.mod_stride = mod_stride;
       o.a = last_in; o.w = last_w; o.bias = last_b; o.M = M; o.N = C; o.K = last_K;
-      if (sub_pruned) {
+      if (gemm_restores) {
+        o.epilogue = xb ? EPI_RESIDUAL_XBF16 : EPI_RESIDUAL; o.out = x; o.gamma = gamma;
+        o.row_idx = idx; o.row_inv = inv_cur; o.map_tokens = n;
+        kept_partial = more ? reinterpret_cast<float*>(ctx->y_buf) : nullptr;
+        o.colsum = kept_partial;
+        s = launch_gemm(o, st);
+        if (s != FV_OK) break;
+        if (cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess) { s = FV_ERR_CUDA; break; }
+        forked = false;
+        have_partials = more;
+      } else if (sub_pruned) {
         o.epilogue = EPI_BF16; o.out = ctx->y_buf;
         s = launch_gemm(o, st);
         if (s != FV_OK) break;

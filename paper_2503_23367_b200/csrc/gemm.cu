@@ -54,7 +54,7 @@ template <int BN> struct GemmCfg {
   }
 };
 
-// KIND 1 / 3 (RESID): the instantiations launched for the residual epilogue of an fp32 / a bf16 stream.  They are kernels of their own because
+// KIND 1 / 3 (RESID): the instantiations launched for the residual epilogue of an fp32 / a bf16 stream, 5 / 7 for rows of a map.  They are kernels of their own because
 // that epilogue takes eight warps and more registers per thread; the others stay small enough for a bandwidth-bound kernel of another
 // stream (the restoration of the rows that were not kept) to share the SMs with them.
 template <int BN, int KIND>
@@ -64,7 +64,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;
   constexpr bool RESID = is_resid(KIND);   // KIND 2: the QKV projection with cosine attention / rotary positions on Q and K
-  constexpr bool XB = KIND == 3;
+  constexpr bool XB = is_resid_bf16(KIND), MAP = is_resid_map(KIND);
   constexpr int kBiasBytes = RESID ? kResidBiasBytes : kBiasSmemBytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -169,6 +169,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int quarter = warp & 3;
     const uint32_t lane_off = uint32_t(quarter * 32) << 16;
     uint32_t lt = 0;
+    [[maybe_unused]] bool ok = true;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x, ++lt) {
       const uint32_t buf = lt & 1;
       const int m0 = (tile % tiles_m) * BM, n0 = (tile / tiles_m) * BN;
@@ -182,16 +183,21 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const auto release = [&] { tc_fence_before(); mbar_arrive(&acc_empty[buf]); };
         // the first chunk of `out` is on its way while the accumulator is computed
         const bool turned = p.rows_per_image >= 32 || p.epilogue == EPI_F32;   // (images of fewer than 32 rows take the row-per-thread path)
-        ResidRows rr;
+        ResidRows<MAP> rr;
         typename ResidX<XB>::Raw x[8];
         if (turned) {
-          rr = resid_rows(p, lane, m0 + quarter * 32);
-          residual_load_x<XB>(p, rr, x, lane, n0 + 32 * half);
+          rr = resid_rows<MAP>(p, lane, m0 + quarter * 32);
+          residual_load_x<XB, MAP>(p, rr, x, lane, n0 + 32 * half);
         }
-        if (!mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); break; }
+        if (ok && !mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); ok = false; }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!MAP && !ok) break;
         tc_fence_after();
-        if (turned) {
-          residual_tile<XB, BN>(p, rr, x, t0, half, lane, n0, bias_w, resid_s + (warp - 2) * kResidTileFloats, release);
+        if constexpr (MAP) {        // (images of at least 128 rows)
+          if (ok) residual_tile<XB, true, BN>(p, rr, x, t0, half, lane, n0, bias_w, resid_s + (warp - 2) * kResidTileFloats, release);
+          residual_tile_sums<BN>(p, resid_s, (int)threadIdx.x - 64, m0, n0, ok);
+        } else if (turned) {
+          residual_tile<XB, false, BN>(p, rr, x, t0, half, lane, n0, bias_w, resid_s + (warp - 2) * kResidTileFloats, release);
         } else {
           const int img = row_ok ? row / p.rows_per_image : 0, jrow = row_ok ? row - img * p.rows_per_image : 0;
 #pragma unroll 1
@@ -283,6 +289,14 @@ cudaError_t gemm_init() {
   if (e == cudaSuccess) e = set_attr<256, 1>();
   if (e == cudaSuccess) e = set_attr<64, 0>();
   if (e == cudaSuccess) e = set_attr<64, 1>();
+  if (e == cudaSuccess) e = set_attr<64, 5>();
+  if (e == cudaSuccess) e = set_attr<128, 5>();
+  if (e == cudaSuccess) e = set_attr<192, 5>();
+  if (e == cudaSuccess) e = set_attr<256, 5>();
+  if (e == cudaSuccess) e = set_attr<64, 7>();
+  if (e == cudaSuccess) e = set_attr<128, 7>();
+  if (e == cudaSuccess) e = set_attr<192, 7>();
+  if (e == cudaSuccess) e = set_attr<256, 7>();
   if (e == cudaSuccess) e = set_attr<64, 3>();
   if (e == cudaSuccess) e = set_attr<128, 3>();
   if (e == cudaSuccess) e = set_attr<192, 3>();
@@ -310,6 +324,10 @@ static cudaError_t launch_bn(const GemmArgs& g, const GemmDev& p, int tiles_m, c
   if (!make_tmap_bf16_2d(&tmB, g.w, g.N, g.K, BN)) return cudaErrorInvalidValue;
   const long tiles = (long)tiles_m * ((g.N + BN - 1) / BN);
   const int grid = (int)(tiles < g_num_sms ? tiles : g_num_sms);
+  if (p.row_idx && p.epilogue == EPI_RESIDUAL)
+    return launch_pdl(gemm_bf16_kernel<BN, 5>, dim3(grid), dim3(gemm_threads(5)), GemmCfg<BN>::smem_bytes(true), st, tmA, tmB, p);
+  if (p.row_idx)
+    return launch_pdl(gemm_bf16_kernel<BN, 7>, dim3(grid), dim3(gemm_threads(7)), GemmCfg<BN>::smem_bytes(true), st, tmA, tmB, p);
   if (p.epilogue == EPI_RESIDUAL || p.epilogue == EPI_F32)
     return launch_pdl(gemm_bf16_kernel<BN, 1>, dim3(grid), dim3(gemm_threads(1)), GemmCfg<BN>::smem_bytes(true), st, tmA, tmB, p);
   if (p.epilogue == EPI_RESIDUAL_XBF16)
@@ -333,7 +351,11 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
   // Q / K extras (cosine attention, rotary positions): one-CTA tiles that hold whole heads, no K split
   const bool qk_extras = g.epilogue == EPI_QKV_SPLIT && (g.qk_scale || g.rope_table);
   if (qk_extras && g.head_dim != 64 && g.head_dim != 128) return FV_ERR_UNSUPPORTED;
-  TileChoice tc = pick_tile(g.M, g.N, g.K, g_num_sms, qk_extras ? g.head_dim : 0);
+  // rows of a map: a tile's 128 rows hold at most two images, and the tile is one CTA's or a pair's
+  const bool map = g.row_idx != nullptr;
+  if (map && ((g.epilogue != EPI_RESIDUAL && g.epilogue != EPI_RESIDUAL_XBF16) || !g.row_inv || g.map_tokens <= 0 || g.rows_per_image < kMinMapRows || g.aux))
+    return FV_ERR_UNSUPPORTED;
+  TileChoice tc = pick_tile(g.M, g.N, g.K, g_num_sms, qk_extras ? g.head_dim : 0, !map);
   const TileChoice picked = tc;
   if (g_force_path == 1 && tc.pair) tc = TileChoice{256, false, 1};
   if (g_force_path == 2) tc = TileChoice{256, true, 1};
@@ -358,21 +380,22 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
   p.rope_table = qk_extras ? reinterpret_cast<const float2*>(g.rope_table) : nullptr;
   p.rope_idx = qk_extras ? g.rope_idx : nullptr;
   p.head_dim = g.head_dim;
+  p.row_idx = g.row_idx; p.row_inv = g.row_inv; p.map_tokens = g.map_tokens; p.colsum = g.colsum; p.colsum_slots = map_colsum_slots(g.rows_per_image);
   // K split over the CTAs of a cluster, the partials reduced through distributed shared memory.  Up to 48 rows two CTAs
   // share an SM (gemm_cluster.cu): 8 slices while the CTAs stay within one per SM, else 4 within two, else 2 (us at M 8, weights from HBM,
   // 8 / 4 / 2 slices: N 2048 K 2048 3.9 / 4.6 / 6.4; N 6144 9.1 / 6.7 / 8.0; N 8192 10.1 / 7.6 / 8.9; N 2048 K 8192 9.0 / 11.9 / 20;
   // 1024-wide models N 3072 3.7 / 3.6 / 4.2; N 1024 K 4096 4.6 / 6.4 / 10.3).  From 64 rows on the other tiles are as fast or faster.
   int cluster_slices = 0, cluster_bn = 0;
-  if (g_force_path == 0 && !qk_extras) {
+  if (g_force_path == 0 && !qk_extras && !map) {
     const long t128 = (g.N + 127) / 128;
     if (g.M <= 48 && g.K > 7 * BK && t128 <= g_num_sms) { cluster_bn = 128; cluster_slices = t128 * 8 <= g_num_sms ? 8 : (t128 * 4 <= 2 * g_num_sms ? 4 : 2); }
     else if (picked.slices > 1) { cluster_bn = picked.bn; cluster_slices = picked.slices; }
   }
-  if (g_force_path >= 8 && g_force_path <= 11 && !qk_extras) {   // 8: 128 wide x 4 slices, 9: 128 x 2, 10: 64 x 4, 11: 64 x 2
+  if (g_force_path >= 8 && g_force_path <= 11 && !qk_extras && !map) {   // 8: 128 wide x 4 slices, 9: 128 x 2, 10: 64 x 4, 11: 64 x 2
     cluster_bn = g_force_path <= 9 ? 128 : 64;
     cluster_slices = (g_force_path & 1) ? 2 : 4;
   }
-  if (g_force_path == 12 && !qk_extras && g.M <= 48) { cluster_bn = 128; cluster_slices = 8; }   // (few rows only)
+  if (g_force_path == 12 && !qk_extras && !map && g.M <= 48) { cluster_bn = 128; cluster_slices = 8; }   // (few rows only)
   if (cluster_slices) {
     const int num_kb = (g.K + BK - 1) / BK;
     p.kb_per_split = (num_kb + cluster_slices - 1) / cluster_slices;

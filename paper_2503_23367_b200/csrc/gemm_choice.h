@@ -14,7 +14,8 @@ struct TileChoice { int bn; bool pair; int slices; };   // slices 1: no cluster
 // head_dim > 0: the QKV projection with head norms or rotation, whose epilogue exists for one-CTA tiles of at least 128 columns that hold
 // whole heads; only those are compared.  (Taking the cheapest of all and widening it until it was allowed: blocks of 820 and 1024 rows at C 2048 with 128-wide
 // heads 133 and 139 us, now 129 and 135; 3249 rows at C 1024 193 -> 187.)
-inline TileChoice pick_tile(int M, int N, int K, int sms, int head_dim = 0) {
+// clusters false: the residual epilogue that writes rows of a map, which clusters do not have.
+inline TileChoice pick_tile(int M, int N, int K, int sms, int head_dim = 0, bool clusters = true) {
   const int num_kb = (K + 63) / 64;
   struct Cand { int bn; bool pair; int slices; double fixed_us, round_us, kb_us; };
   // Least-squares fits over M 36 ... 3277 x the four projection shapes of 1024-, 1920- and 2048-wide blocks, every candidate forced.  On
@@ -29,6 +30,7 @@ inline TileChoice pick_tile(int M, int N, int K, int sms, int head_dim = 0) {
   double best_cost = 1e30;
   for (const Cand& c : cand) {
     if (c.pair && M <= 256) continue;
+    if (!clusters && c.slices > 1) continue;
     if (head_dim > 0 && (c.pair || c.slices > 1 || c.bn < 128 || c.bn % head_dim)) continue;
     const int rows = c.pair ? 256 : 128;
     const int slots = c.pair ? sms / 2 : sms;

@@ -28,6 +28,12 @@ struct GemmDev {
   const float2* rope_table;   // [tokens of the scale][head_dim / 2] (cos, sin), or null
   const int32_t* rope_idx;    // [B, rows_per_image] original token index of every row, or null (row j = token j)
   int head_dim;
+  // residual epilogue of a pruned step (MAP instantiations): compact row r of A belongs to token row_idx[r] of its image's map
+  const int32_t* row_idx;     // [M]
+  const int32_t* row_inv;     // [images, map_tokens] the row of A that a token takes, -1 none: a row whose token does not name it is left out
+  int map_tokens;
+  float* colsum;              // [images, colsum_slots, N]: column sums of the updated rows, a slot per 128 rows of A that hold rows of the image; or null
+  int colsum_slots;
 };
 
 __device__ __forceinline__ float gelu_tanh_fast(float v) {
@@ -91,7 +97,10 @@ __device__ __forceinline__ void chunk_values(const GemmDev& p, const uint32_t (&
 // row before: K 2048 M 800 15.6 / 10.6, M 2304 28.0 / 18.2, K 8192 M 800 33.4 / 28.8).  Everything that does not depend on the chunk (row
 // validity, the image boundary, the row pointers) is set up once per tile.
 constexpr int kResidWarps = 8;
-__host__ __device__ constexpr bool is_resid(int kind) { return kind == 1 || kind == 3; }   // kernel instantiations for an fp32 / a bf16 stream
+// Kernel instantiations: 1 an fp32 stream, 3 a bf16 stream, + 4 with rows of a map (KIND 0 and 2 are not residual).
+__host__ __device__ constexpr bool is_resid(int kind) { return kind & 1; }
+__host__ __device__ constexpr bool is_resid_bf16(int kind) { return (kind & 3) == 3; }
+__host__ __device__ constexpr bool is_resid_map(int kind) { return (kind & 5) == 5; }
 __host__ __device__ constexpr int gemm_threads(int kind) { return 64 + 32 * (is_resid(kind) ? kResidWarps : 4); }   // producer, issuer, epilogue
 constexpr int kResidTilePitch = 36;
 constexpr int kResidTileRows = 16;
@@ -104,7 +113,7 @@ template <> struct ResidX<false> {
   using Raw = float4;
   static __device__ __forceinline__ Raw load(const void* out, size_t at) { return *reinterpret_cast<const float4*>(static_cast<const float*>(out) + at); }
   static __device__ __forceinline__ float4 value(const Raw& r) { return r; }
-  static __device__ __forceinline__ void store(void* out, size_t at, const float4& v) { *reinterpret_cast<float4*>(static_cast<float*>(out) + at) = v; }
+  static __device__ __forceinline__ float4 store(void* out, size_t at, const float4& v) { return *reinterpret_cast<float4*>(static_cast<float*>(out) + at) = v; }
 };
 template <> struct ResidX<true> {
   using Raw = uint2;
@@ -112,13 +121,16 @@ template <> struct ResidX<true> {
   static __device__ __forceinline__ float4 value(const Raw& r) {
     return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xFFFF0000u));
   }
-  static __device__ __forceinline__ void store(void* out, size_t at, const float4& v) {   // rounded to nearest even once
-    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + at) = make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
+  static __device__ __forceinline__ float4 store(void* out, size_t at, const float4& v) {   // rounded to nearest even once; returns what is stored
+    const uint2 r = make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
+    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(out) + at) = r;
+    return value(r);
   }
 };
 
-struct ResidRows {
-  size_t at0;              // element offset of &out[first row of the lane, 4 * (lane & 7)] (column offset of the chunk not included)
+template <bool MAP> struct ResidRows {
+  size_t at0;              // element offset of &out[first row of the lane, 4 * (lane & 7)] (column offset of the chunk not included); MAP: of row 0
+  int row[MAP ? 8 : 1];    // MAP: row of `out` of the lane's row i, or -1
   const float* gam0;       // gate vector of the image of the warp's first row (+ the lane's column offset), or nullptr
   const float* gam1;       // gate vector of the next image
   int n_rows;              // the lane's rows i < n_rows exist
@@ -128,11 +140,22 @@ struct ResidRows {
 };
 
 // Valid when an image has at least 32 rows (a warp's 32 rows then span at most two images).
-__device__ __forceinline__ ResidRows resid_rows(const GemmDev& p, int lane, int row0) {
-  ResidRows rr;
+template <bool MAP>
+__device__ __forceinline__ ResidRows<MAP> resid_rows(const GemmDev& p, int lane, int row0) {
+  ResidRows<MAP> rr;
   const int r = row0 + (lane >> 3);
   const int cl = 4 * (lane & 7);
-  rr.at0 = (size_t)r * p.N + cl;
+  rr.at0 = MAP ? (size_t)cl : (size_t)r * p.N + cl;
+  if constexpr (MAP) {
+    const int mine = row0 + lane;
+    int at = -1;
+    if (mine < p.M) {
+      const int img = mine / p.rows_per_image, t = dep_load(p.row_idx + mine);
+      if (t >= 0 && t < p.map_tokens && dep_load(p.row_inv + (size_t)img * p.map_tokens + t) == mine - img * p.rows_per_image) at = img * p.map_tokens + t;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) rr.row[i] = __shfl_sync(0xffffffffu, at, (lane >> 3) + 4 * i);
+  }
   rr.n_rows = max(0, min(8, (p.M - r + 3) >> 2));
   rr.n_load = p.epilogue == EPI_F32 ? 0 : rr.n_rows;
   const int img0 = min(row0, p.M - 1) / p.rows_per_image;
@@ -143,17 +166,20 @@ __device__ __forceinline__ ResidRows resid_rows(const GemmDev& p, int lane, int 
 }
 
 // The lane's 8 x 4 values of `out` for the chunk at column `col`; fetched one chunk ahead of their use.
-template <bool XB>
-__device__ __forceinline__ void residual_load_x(const GemmDev& p, const ResidRows& rr, typename ResidX<XB>::Raw (&x)[8], int lane, int col) {
+template <bool XB, bool MAP>
+__device__ __forceinline__ void residual_load_x(const GemmDev& p, const ResidRows<MAP>& rr, typename ResidX<XB>::Raw (&x)[8], int lane, int col) {
   const bool col_ok = col + 4 * (lane & 7) < p.N;
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-    if (col_ok && i < rr.n_load) x[i] = ResidX<XB>::load(p.out, rr.at0 + (size_t)(4 * i) * p.N + col);
+  for (int i = 0; i < 8; ++i) {
+    if (MAP ? (col_ok && rr.row[MAP ? i : 0] >= 0) : (col_ok && i < rr.n_load))
+      x[i] = ResidX<XB>::load(p.out, rr.at0 + (MAP ? (size_t)rr.row[MAP ? i : 0] : (size_t)(4 * i)) * p.N + col);
+  }
 }
 
-template <bool XB>
-__device__ __forceinline__ void residual_chunk(const GemmDev& p, const ResidRows& rr, const uint32_t (&r)[32], const typename ResidX<XB>::Raw (&x)[8],
-                                               float* tile, int lane, int col, const uint4* bias4) {
+// sum0 / sum1 (MAP): the lane's sums of the updated rows of the first / the next image, over its eight rows.
+template <bool XB, bool MAP>
+__device__ __forceinline__ void residual_chunk(const GemmDev& p, const ResidRows<MAP>& rr, const uint32_t (&r)[32], const typename ResidX<XB>::Raw (&x)[8],
+                                               float* tile, int lane, int col, const uint4* bias4, float4& sum0, float4& sum1) {
   float v[32];
   chunk_values(p, r, col, v, bias4);
   const bool col_ok = col + 4 * (lane & 7) < p.N;
@@ -176,14 +202,18 @@ __device__ __forceinline__ void residual_chunk(const GemmDev& p, const ResidRows
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int i = 4 * pass + u;
-        if (i < rr.n_rows) {
+        if (MAP ? rr.row[MAP ? i : 0] >= 0 : i < rr.n_rows) {
           const float4 a = *reinterpret_cast<const float4*>(trow + 4 * u * kResidTilePitch);
           const float4 gg = i < rr.n_first ? g0 : g1;
-          float4 xv = i < rr.n_load ? ResidX<XB>::value(x[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
+          float4 xv = MAP || i < rr.n_load ? ResidX<XB>::value(x[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
           xv.x = fmaf(gg.x, a.x, xv.x); xv.y = fmaf(gg.y, a.y, xv.y); xv.z = fmaf(gg.z, a.z, xv.z); xv.w = fmaf(gg.w, a.w, xv.w);
-          const size_t at = rr.at0 + (size_t)(4 * i) * p.N + col;
-          ResidX<XB>::store(p.out, at, xv);
-          if (aux) *reinterpret_cast<uint2*>(aux + at) = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+          const size_t at = rr.at0 + (MAP ? (size_t)rr.row[MAP ? i : 0] : (size_t)(4 * i)) * p.N + col;
+          xv = ResidX<XB>::store(p.out, at, xv);
+          if constexpr (MAP) {
+            float4& s = i < rr.n_first ? sum0 : sum1;
+            s.x += xv.x; s.y += xv.y; s.z += xv.z; s.w += xv.w;
+          }
+          if (!MAP && aux) *reinterpret_cast<uint2*>(aux + at) = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
         }
       }
     }
@@ -193,22 +223,62 @@ __device__ __forceinline__ void residual_chunk(const GemmDev& p, const ResidRows
 
 // A warp's share of the residual tile whose accumulator starts at TMEM address t0 (the warp's quarter of the lanes): the chunks
 // `half`, `half` + 2, ... of its 32 rows.  x: the first of them, already requested.  release(): the warp's last accumulator read is done.
-template <bool XB, int BN, typename Release>
-__device__ __forceinline__ void residual_tile(const GemmDev& p, const ResidRows& rr, typename ResidX<XB>::Raw (&x)[8], uint32_t t0, int half, int lane, int n0,
+// MAP with column sums: the warp leaves its own for the chunks it has had in its tile, [chunk][32], the next image's 128 floats behind.
+template <bool XB, bool MAP, int BN, typename Release>
+__device__ __forceinline__ void residual_tile(const GemmDev& p, const ResidRows<MAP>& rr, typename ResidX<XB>::Raw (&x)[8], uint32_t t0, int half, int lane, int n0,
                                               const uint4* bias_w, float* tile, Release release) {
   constexpr int kChunks = BN / 32;
+  float4 keep0 = make_float4(0.f, 0.f, 0.f, 0.f), keep1 = keep0;   // sums of chunk (lane >> 3) of the warp's up to four
 #pragma unroll 1
   for (int ch = half; ch < kChunks; ch += 2) {   // rolled: the code of one chunk is fetched once and then reused
     uint32_t r[32];
     typename ResidX<XB>::Raw nx[8];
     tmem_ld32(t0 + 32 * ch, r);
-    if (ch + 2 < kChunks) residual_load_x<XB>(p, rr, nx, lane, n0 + 32 * (ch + 2));
+    if (ch + 2 < kChunks) residual_load_x<XB, MAP>(p, rr, nx, lane, n0 + 32 * (ch + 2));
     tmem_wait_ld();
     if (ch + 2 >= kChunks) release();            // accumulator fully in registers: hand the buffer back to the MMA warp
-    if (n0 + 32 * ch < p.N) residual_chunk<XB>(p, rr, r, x, tile, lane, n0 + 32 * ch, bias_w + 4 * ch);
+    float4 sum0 = make_float4(0.f, 0.f, 0.f, 0.f), sum1 = sum0;
+    if (n0 + 32 * ch < p.N) residual_chunk<XB, MAP>(p, rr, r, x, tile, lane, n0 + 32 * ch, bias_w + 4 * ch, sum0, sum1);
+    if constexpr (MAP) {
+#pragma unroll
+      for (int o = 8; o <= 16; o <<= 1) {        // over the lanes that share the columns: all 32 rows
+        sum0.x += __shfl_xor_sync(0xffffffffu, sum0.x, o); sum0.y += __shfl_xor_sync(0xffffffffu, sum0.y, o);
+        sum0.z += __shfl_xor_sync(0xffffffffu, sum0.z, o); sum0.w += __shfl_xor_sync(0xffffffffu, sum0.w, o);
+        sum1.x += __shfl_xor_sync(0xffffffffu, sum1.x, o); sum1.y += __shfl_xor_sync(0xffffffffu, sum1.y, o);
+        sum1.z += __shfl_xor_sync(0xffffffffu, sum1.z, o); sum1.w += __shfl_xor_sync(0xffffffffu, sum1.w, o);
+      }
+      if ((lane >> 3) == (ch >> 1)) { keep0 = sum0; keep1 = sum1; }
+    }
 #pragma unroll
     for (int i = 0; i < 8; ++i) x[i] = nx[i];
   }
+  if constexpr (MAP) {
+    *reinterpret_cast<float4*>(tile + 4 * lane) = keep0;
+    *reinterpret_cast<float4*>(tile + 128 + 4 * lane) = keep1;
+  }
+}
+
+// Column sums of a tile's 128 rows, from what the eight epilogue warps have left in their tiles: one value per column and image, the
+// four quarters of the rows added in order.  All 256 epilogue threads, whether or not their waits came through: the barriers count them.
+template <int BN>
+__device__ __forceinline__ void residual_tile_sums(const GemmDev& p, const float* tiles, int et, int m0, int n0, bool ok) {
+  asm volatile("bar.sync 1, 256;" ::: "memory");
+  if (ok && p.colsum && et < BN && n0 + et < p.N && m0 < p.M) {
+    const int img0 = m0 / p.rows_per_image, last = min(m0 + 127, p.M - 1) / p.rows_per_image;   // (an image has at least 128 rows)
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {     // quarter q of the rows belongs to warps 2 + (q + 2) % 4 and four further on
+      const bool next = m0 + 32 * q < p.M && (m0 + 32 * q) / p.rows_per_image > img0;   // the quarter begins in the next image
+      const float* t = tiles + (((et >> 5) & 1) * 4 + ((q + 2) & 3)) * kResidTileFloats + (et >> 6) * 32 + (et & 31);
+      s0 += next ? 0.f : t[0];
+      s1 += next ? t[0] : t[128];
+    }
+    for (int i = img0; i <= last; ++i) {
+      const int slot = m0 / 128 - i * p.rows_per_image / 128;
+      p.colsum[((size_t)i * p.colsum_slots + slot) * p.N + n0 + et] = i == img0 ? s0 : s1;
+    }
+  }
+  asm volatile("bar.sync 1, 256;" ::: "memory");   // read before the next tile's chunks are turned
 }
 
 // One 32-column chunk of one accumulator row: bias, optional GELU, then the epilogue's store.

@@ -16,6 +16,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "gemm_epilogue.cuh"
 #include "internal.h"
 #include "sm100.cuh"
@@ -44,14 +46,14 @@ template <int BN> struct PairCfg {
   }
 };
 
-// KIND 1 / 3 (RESID): the instantiations launched for the residual epilogue of an fp32 / a bf16 stream (eight epilogue warps); 0: the others.
+// KIND 1 / 3 (RESID): the instantiations launched for the residual epilogue of an fp32 / a bf16 stream (eight epilogue warps), 5 / 7 for rows of a map; 0: the others.
 template <int BN, int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads(KIND), 1)
 gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmDev p) {
   using Cfg = PairCfg<BN>;
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;
-  constexpr bool RESID = is_resid(KIND), XB = KIND == 3;
+  constexpr bool RESID = is_resid(KIND), XB = is_resid_bf16(KIND), MAP = is_resid_map(KIND);
   constexpr int kBiasBytes = RESID ? kResidBiasBytes : kBiasSmemBytes;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -160,6 +162,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const int quarter = warp & 3;
     const uint32_t lane_off = uint32_t(quarter * 32) << 16;
     uint32_t lt = 0;
+    [[maybe_unused]] bool ok = true;
     for (int tile = pair; tile < total_tiles; tile += npairs, ++lt) {
       const uint32_t buf = lt & 1;
       const int m0 = (tile % tiles_m) * (2 * BM) + (int)rank * BM, n0 = (tile / tiles_m) * BN;
@@ -173,16 +176,21 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const auto release = [&] { tc_fence_before(); mbar_arrive_cluster(&acc_empty[buf], 0); };
         // the first chunk of `out` is on its way while the accumulator is computed
         const bool turned = p.rows_per_image >= 32 || p.epilogue == EPI_F32;   // (images of fewer than 32 rows take the row-per-thread path)
-        ResidRows rr;
+        ResidRows<MAP> rr;
         typename ResidX<XB>::Raw x[8];
         if (turned) {
-          rr = resid_rows(p, lane, m0 + quarter * 32);
-          residual_load_x<XB>(p, rr, x, lane, n0 + 32 * half);
+          rr = resid_rows<MAP>(p, lane, m0 + quarter * 32);
+          residual_load_x<XB, MAP>(p, rr, x, lane, n0 + 32 * half);
         }
-        if (!mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); break; }
+        if (ok && !mbar_wait(&acc_full[buf], (lt >> 1) & 1)) { report(p.status, DEV_TIMEOUT_EPI); ok = false; }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!MAP && !ok) break;
         tc_fence_after();
-        if (turned) {
-          residual_tile<XB, BN>(p, rr, x, t0, half, lane, n0, bias_w, resid_s + (warp - 2) * kResidTileFloats, release);
+        if constexpr (MAP) {        // (images of at least 128 rows)
+          if (ok) residual_tile<XB, true, BN>(p, rr, x, t0, half, lane, n0, bias_w, resid_s + (warp - 2) * kResidTileFloats, release);
+          residual_tile_sums<BN>(p, resid_s, (int)threadIdx.x - 64, m0, n0, ok);
+        } else if (turned) {
+          residual_tile<XB, false, BN>(p, rr, x, t0, half, lane, n0, bias_w, resid_s + (warp - 2) * kResidTileFloats, release);
         } else {
           const int img = row_ok ? row / p.rows_per_image : 0, jrow = row_ok ? row - img * p.rows_per_image : 0;
 #pragma unroll 1
@@ -238,6 +246,10 @@ cudaError_t gemm_pair_init() {
   if (e == cudaSuccess) e = set_pair_attr<128, 0>();
   if (e == cudaSuccess) e = set_pair_attr<256, 1>();
   if (e == cudaSuccess) e = set_pair_attr<128, 1>();
+  if (e == cudaSuccess) e = set_pair_attr<256, 5>();
+  if (e == cudaSuccess) e = set_pair_attr<128, 5>();
+  if (e == cudaSuccess) e = set_pair_attr<256, 7>();
+  if (e == cudaSuccess) e = set_pair_attr<128, 7>();
   if (e == cudaSuccess) e = set_pair_attr<256, 3>();
   if (e == cudaSuccess) e = set_pair_attr<128, 3>();
   if (e != cudaSuccess) return e;
@@ -258,9 +270,15 @@ cudaError_t launch_gemm_pair(const GemmArgs& g, const GemmDev& p, int bn, cudaSt
   const long tiles = (long)((g.M + 2 * BM - 1) / (2 * BM)) * ((g.N + bn - 1) / bn);
   const int max_pairs = g_pair_sms / 2;
   const int pairs = (int)(tiles < max_pairs ? tiles : max_pairs);
-  const int kind = p.epilogue == EPI_RESIDUAL || p.epilogue == EPI_F32 ? 1 : (p.epilogue == EPI_RESIDUAL_XBF16 ? 3 : 0);
-  if (bn == 256) return kind == 1 ? launch_kind<256, 1>(tmA, tmB, p, pairs, st) : (kind == 3 ? launch_kind<256, 3>(tmA, tmB, p, pairs, st) : launch_kind<256, 0>(tmA, tmB, p, pairs, st));
-  if (bn == 128) return kind == 1 ? launch_kind<128, 1>(tmA, tmB, p, pairs, st) : (kind == 3 ? launch_kind<128, 3>(tmA, tmB, p, pairs, st) : launch_kind<128, 0>(tmA, tmB, p, pairs, st));
+  auto go = [&](auto width) {
+    constexpr int W = decltype(width)::value;
+    const bool xb = p.epilogue == EPI_RESIDUAL_XBF16;
+    if (p.row_idx) return xb ? launch_kind<W, 7>(tmA, tmB, p, pairs, st) : launch_kind<W, 5>(tmA, tmB, p, pairs, st);
+    if (xb) return launch_kind<W, 3>(tmA, tmB, p, pairs, st);
+    return p.epilogue == EPI_RESIDUAL || p.epilogue == EPI_F32 ? launch_kind<W, 1>(tmA, tmB, p, pairs, st) : launch_kind<W, 0>(tmA, tmB, p, pairs, st);
+  };
+  if (bn == 256) return go(std::integral_constant<int, 256>());
+  if (bn == 128) return go(std::integral_constant<int, 128>());
   return cudaErrorInvalidValue;
 }
 

@@ -127,9 +127,11 @@ SelectWs select_ws_carve(void* workspace, int B, int n, int C);
 // Scores [B,n] (fp32), then exact per-image top-k -> idx [B,k] ascending, inv [B,n].  have_partials:
 // the group partials in the workspace already hold the column sums of x (left there by
 // launch_restore_residual), so the column-sum pass is skipped.
+// kept_partial (with have_partials): the sums are in two places instead, those of the rows that were not kept in one partial per image
+// (launch_colsum_total), those of kept_rows rows per image where the last GEMM of the sublayer left them (GemmArgs::colsum).
 // x_bf16 (select, gather, restore launchers): the residual stream is bf16 instead of fp32 (fv_config.resid_dtype).
 cudaError_t launch_select(const void* x, int B, int n, int C, int k, int32_t* idx, int32_t* inv, float* score,
-                          int32_t* near_tie, void* workspace, bool have_partials, cudaStream_t st, bool x_bf16 = false);
+                          int32_t* near_tie, void* workspace, bool have_partials, cudaStream_t st, bool x_bf16 = false, const float* kept_partial = nullptr, int kept_rows = 0);
 // The selection of a wrapped sublayer inside a scale step, in one launch with what surrounds it on the kept rows:
 // the previous sublayer's kept-row restoration before it (y != null) and the gather + LayerNorm + modulation of the
 // newly kept rows after it.  sel_ws holds the column sums of the rows the kernel does not update itself (left there
@@ -147,6 +149,8 @@ size_t select_fused_ws_bytes(int B, int C);
 size_t select_fused_sync_bytes(int B);            // leading bytes of fused_ws that must be zero before first use
 bool select_fused_supported(int B, int n, int C);
 cudaError_t launch_select_fused(const FusedSelect& f, cudaStream_t st);
+// The chunk partials that a restoration of the rows that were not kept has left (part 1) -> one partial per image, the image's first group partial.
+cudaError_t launch_colsum_total(int B, int n, int C, void* workspace, cudaStream_t st);
 cudaError_t launch_colsum(const float* x, int B, int n, int C, void* workspace, cudaStream_t st);   // column sums of a map -> sel_ws
 cudaError_t launch_inv_from_idx(const int32_t* idx, int B, int k, int n, int32_t* inv, cudaStream_t st);
 cudaError_t launch_inv_fill(int B, int n, int32_t* inv, cudaStream_t st);  // every token unkept (-1)
@@ -214,7 +218,16 @@ struct GemmArgs {
   const float* rope_table;    // [tokens of the scale][head_dim/2][2] fp32 (cos, sin) of the rotary angles
   const int32_t* rope_idx;    // [B, rows_per_image] original token of every row, or null (row j is token j)
   int head_dim;               // 64 or 128 (needed with either extra)
+  // EPI_RESIDUAL / EPI_RESIDUAL_XBF16 on the kept rows of a map (all null = out's rows are A's): row r of A is token row_idx[r] of its image, out is
+  // [images, map_tokens, N].  Images of at least kMinMapRows rows.
+  const int32_t* row_idx;     // [M]
+  const int32_t* row_inv;     // [images, map_tokens] row of A of a token, or -1 (rows whose token does not name them are left out)
+  int map_tokens;
+  float* colsum;              // [images, map_colsum_slots(rows_per_image), N] column sums of the updated rows, map_colsum_count() slots written; or null
 };
+constexpr int kMinMapRows = 128;
+__host__ __device__ inline int map_colsum_slots(int rows) { return rows / 128 + 2; }   // most 128-row blocks of A that hold rows of one image
+__host__ __device__ inline int map_colsum_count(int img, int rows) { return ((img + 1) * rows - 1) / 128 - img * rows / 128 + 1; }
 // (cos, sin) of the 2-D rotary angles of every token of an (h, w) map placed in the (h_last, w_last) frame:
 // first head_dim/4 pairs turn with the row coordinate y * h_last / h, the rest with x * w_last / w, pair j of
 // either group at frequency base^(-j / (head_dim/4)).  table: [h*w][head_dim/2][2] fp32.

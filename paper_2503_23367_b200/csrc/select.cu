@@ -104,6 +104,36 @@ __global__ void __launch_bounds__(64) colsum_fold_kernel(const float4* chunk_par
   group_partial[((size_t)b * ngroups + g) * C4 + c4] = acc;
 }
 
+// All chunk partials of an image -> one: grid (ceil(C4 / 16), B), 16 threads per four channels, each adds a sixteenth of the chunks (16 loads in
+// flight), then their sums are added in order.  It runs behind the restoration of the rows that were not kept, beside the sublayer's branch.  (The same by the
+// last CTAs of that kernel to arrive, group by group: 128 x 128 tokens, C 2048 40 -> 56 us, and the GEMM beside it 9 us longer.)
+__global__ void __launch_bounds__(256) colsum_total_kernel(const float4* chunk_partial, int C4, int nchunks, int ngroups, float4* __restrict__ group_partial) {
+  __shared__ float4 s_sum[16][16];
+  pdl_trigger();
+  pdl_wait();
+  const int b = blockIdx.y, q = threadIdx.x & 15, part = threadIdx.x >> 4, c4 = blockIdx.x * 16 + q;
+  const int per = (nchunks + 15) / 16, first = part * per, last = min(nchunks, first + per);
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (c4 < C4) {
+    const float4* src = chunk_partial + (size_t)b * nchunks * C4 + c4;
+    for (int c = first; c < last; c += 16) {
+      float4 v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (c + i < last) v[i] = src[(size_t)(c + i) * C4];
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (c + i < last) { acc.x += v[i].x; acc.y += v[i].y; acc.z += v[i].z; acc.w += v[i].w; }
+    }
+  }
+  s_sum[part][q] = acc;
+  __syncthreads();
+  if (threadIdx.x < 16 && c4 < C4) {
+    for (int p = 1; p < 16; ++p) { const float4 v = s_sum[p][q]; acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w; }
+    group_partial[(size_t)b * ngroups * C4 + c4] = acc;
+  }
+}
+
 // Exclusive prefix sum of one value per thread over the whole CTA (T threads, the template argument); returns the
 // exclusive prefix and, through `total`, the CTA-wide sum.  s_warp is 32 words of scratch.
 template <int T>
@@ -194,6 +224,38 @@ __device__ __forceinline__ void mean_from_partials_halves(float4* s_mean, float4
   }
 }
 static_assert(kMaxGroups == 16, "mean_from_partials_halves splits the groups 8 + 8");
+
+// The sums in two places: one partial of the rows that were not kept, and one per 128 of the compact rows (up to 27 at 128 x 128 tokens).  The
+// halves of the CTA take half of them each, eight loads in flight; stage: C4 float4 words.
+template <int T>
+__device__ __forceinline__ void mean_from_kept_partials(float4* s_mean, float4* stage, const float4* total, const float4* part, int np, int C4, int n) {
+  constexpr int H = T / 2;
+  const int half = (int)threadIdx.x / H, t = (int)threadIdx.x - half * H;
+  const int lo = half ? np / 2 : 0, hi = half ? np : np / 2;
+  const float fn = (float)n;
+  for (int c0 = 0; c0 < C4; c0 += H) {
+    const int c4 = c0 + t;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c4 < C4) {
+      if (half == 0) acc = __ldcg(total + c4);
+      for (int g0 = lo; g0 < hi; g0 += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+          if (g0 + g < hi) v[g] = __ldcg(part + (size_t)(g0 + g) * C4 + c4);
+#pragma unroll
+        for (int g = 0; g < 8; ++g)
+          if (g0 + g < hi) { acc.x += v[g].x; acc.y += v[g].y; acc.z += v[g].z; acc.w += v[g].w; }
+      }
+      if (half == 1) stage[c4] = acc;
+    }
+    __syncthreads();
+    if (half == 0 && c4 < C4) {
+      const float4 u = stage[c4];
+      s_mean[c4] = make_float4((acc.x + u.x) / fn, (acc.y + u.y) / fn, (acc.z + u.z) / fn, (acc.w + u.w) / fn);
+    }
+  }
+}
 
 // ---- Eq. 5 / Algorithm 1: squared deviation from the mean, one warp per token row; the warps of an image stride
 // over its rows.
@@ -499,7 +561,7 @@ __device__ __forceinline__ void topk_image(const float* __restrict__ sc, int n, 
 // max(9 C, n) * 4 bytes (mean token and staged partial sums, then keys).
 template <typename XT>
 __global__ void __launch_bounds__(kSelectThreads, 1) score_topk_kernel(const XT* x,
-                                                                  const float4* group_partial, int ngroups, int n,
+                                                                  const float4* group_partial, int ngroups, const float4* kept_partial, int kept_rows, int n,
                                                                   int C4, int k, int staged, float* __restrict__ score,
                                                                   unsigned int* img_tickets, unsigned int* img_range, int32_t* __restrict__ idx,
                                                                   int32_t* __restrict__ inv, int32_t* __restrict__ near_tie) {
@@ -511,7 +573,10 @@ __global__ void __launch_bounds__(kSelectThreads, 1) score_topk_kernel(const XT*
   const int b = blockIdx.y, tid = threadIdx.x;
   pdl_trigger();
   pdl_wait();
-  if (staged) mean_from_partials_halves<kSelectThreads>(s_mean, s_mean + C4, group_partial + (size_t)b * ngroups * C4, ngroups, C4, n);
+  if (kept_partial)      // (the image's first group partial is the sum of all its rows that were not kept)
+    mean_from_kept_partials<kSelectThreads>(s_mean, s_mean + C4, group_partial + (size_t)b * ngroups * C4, kept_partial + (size_t)b * map_colsum_slots(kept_rows) * C4,
+                                            map_colsum_count(b, kept_rows), C4, n);
+  else if (staged) mean_from_partials_halves<kSelectThreads>(s_mean, s_mean + C4, group_partial + (size_t)b * ngroups * C4, ngroups, C4, n);
   else mean_from_partials<kSelectThreads>(s_mean, group_partial + (size_t)b * ngroups * C4, ngroups, nullptr, 0, C4, n);   // very wide maps
   __syncthreads();
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;
@@ -878,7 +943,7 @@ static cudaError_t launch_colsum_t(const XT* x, int B, int n, int C, const Selec
 
 template <typename XT>
 static cudaError_t launch_select_t(const XT* x, int B, int n, int C, int k, int32_t* idx, int32_t* inv, float* sc, int32_t* near_tie,
-                                   const SelectWs& w, bool have_partials, cudaStream_t st) {
+                                   const SelectWs& w, bool have_partials, cudaStream_t st, const float* kept_partial, int kept_rows) {
   const int C4 = C / 4;
   if (!have_partials)
     launch_colsum_t(x, B, n, C, w, st);
@@ -894,13 +959,13 @@ static cudaError_t launch_select_t(const XT* x, int B, int n, int C, int k, int3
   unsigned int* img_tickets = w.tickets + (size_t)B * kMaxGroups;
   unsigned int* img_range = w.tickets + (size_t)B * (kMaxGroups + 1);
   const float4* gp = reinterpret_cast<const float4*>(w.group_partial);
-  launch_pdl(score_topk_kernel<XT>, dim3(per_image, B), dim3(kSelectThreads), smem, st, x, gp, w.ngroups, n, C4, k, staged, sc, img_tickets,
+  launch_pdl(score_topk_kernel<XT>, dim3(per_image, B), dim3(kSelectThreads), smem, st, x, gp, w.ngroups, reinterpret_cast<const float4*>(kept_partial), kept_rows, n, C4, k, staged, sc, img_tickets,
              img_range, idx, inv, near_tie);
   return cudaGetLastError();
 }
 
 cudaError_t launch_select(const void* x, int B, int n, int C, int k, int32_t* idx, int32_t* inv, float* score,
-                          int32_t* near_tie, void* workspace, bool have_partials, cudaStream_t st, bool x_bf16) {
+                          int32_t* near_tie, void* workspace, bool have_partials, cudaStream_t st, bool x_bf16, const float* kept_partial, int kept_rows) {
   if (!have_partials && select_small_supported(B, n, C, x_bf16)) {   // one launch, no scratch
     SmallSelect f{};
     f.x = const_cast<void*>(x); f.x_bf16 = x_bf16; f.B = B; f.n = n; f.C = C; f.k = k; f.h = 1; f.w = n; f.hc = 1; f.wc = 1;
@@ -913,8 +978,8 @@ cudaError_t launch_select(const void* x, int B, int n, int C, int k, int32_t* id
   const double sel_bytes = (double)B * n * C * es + 4.0 * B * n + 4.0 * B * ((double)k + n);
   // the stand-alone column-sum pass reads the map a second time
   LaunchScope scope(KC_SELECT, have_partials ? 1 : 3, sel_bytes, sel_bytes + (have_partials ? 0.0 : (double)B * n * C * es), st);
-  if (x_bf16) return launch_select_t(static_cast<const __nv_bfloat16*>(x), B, n, C, k, idx, inv, sc, near_tie, w, have_partials, st);
-  return launch_select_t(static_cast<const float*>(x), B, n, C, k, idx, inv, sc, near_tie, w, have_partials, st);
+  if (x_bf16) return launch_select_t(static_cast<const __nv_bfloat16*>(x), B, n, C, k, idx, inv, sc, near_tie, w, have_partials, st, kept_partial, kept_rows);
+  return launch_select_t(static_cast<const float*>(x), B, n, C, k, idx, inv, sc, near_tie, w, have_partials, st, kept_partial, kept_rows);
 }
 
 // ---- the fused selection of a scale step
@@ -988,6 +1053,14 @@ cudaError_t launch_colsum(const float* x, int B, int n, int C, void* workspace, 
   const SelectWs w = select_ws_carve(workspace, B, n, C);
   LaunchScope scope(KC_SELECT, 2, (double)B * n * C * 4.0, (double)B * n * C * 4.0, st);
   return launch_colsum_t(x, B, n, C, w, st);
+}
+
+cudaError_t launch_colsum_total(int B, int n, int C, void* workspace, cudaStream_t st) {
+  const SelectWs w = select_ws_carve(workspace, B, n, C);
+  const int C4 = C / 4;
+  LaunchScope scope(KC_RESTORE, 1, 0.0, 0.0, st);
+  return launch_pdl(colsum_total_kernel, dim3((C4 + 15) / 16, B), dim3(256), 0, st, reinterpret_cast<const float4*>(w.chunk_partial), C4, w.nchunks, w.ngroups,
+                    reinterpret_cast<float4*>(w.group_partial));
 }
 
 cudaError_t launch_inv_fill(int B, int n, int32_t* inv, cudaStream_t st) {

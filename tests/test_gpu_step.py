@@ -4,6 +4,8 @@ Forced-index mode (the oracle's kept indices are fed to the GPU) isolates floati
 every token must be within max-abs 3e-2 and cosine >= 0.999 of the fp64 oracle.  Free-running mode
 checks the integer side: the first pruned sublayer sees identical inputs on both sides, so its kept
 set must match the oracle's (up to near-ties at the threshold)."""
+import copy
+
 import numpy as np
 import pytest
 import torch
@@ -294,6 +296,64 @@ def test_small_map_step_equals_the_separate_kernels(h, w, hc, wc, C, H, B, B_max
     assert ctx.device_status() == 0
     assert torch.equal(outs[0], outs[1])
     assert torch.equal(outs[0], outs[2])
+    ctx.close()
+
+
+@pytest.mark.parametrize("resid_dtype", [0, 1])
+@pytest.mark.parametrize("h,w,hc,wc,C,H,B,keep", [(26, 31, 10, 10, 256, 2, 3, 0.16), (48, 41, 13, 9, 1920, 30, 1, 0.33), (32, 32, 16, 16, 1024, 8, 3, 0.5),
+                                                  (29, 29, 12, 12, 1152, 9, 2, 0.9985)])
+def test_kept_rows_restored_by_the_last_gemm(h, w, hc, wc, C, H, B, keep, resid_dtype):
+    """Kept rows added to the map by the GEMM that produces them: against the same step on one image at a time (tiles without an image
+    boundary, other tile widths), as few kept rows as the route takes, a last tile of three rows, one token that is not kept.  Every selection behind the
+    first takes its column sums from these GEMMs: with zero branches x never changes, so all of them must keep the first one's set."""
+    wl = I.Workload("kept rows", L=2, C=C, H=H, B=B, sides=(hc, h), keep=(1.0, keep), cross_len=64, mlp_ratio=2, seed=815)
+    k = O.kept_count(keep, h, w)
+    assert k >= 128
+    x = torch.from_numpy(I.token_map(831, B, h, w, C, "structured")).to(DEV)
+    mt = I.model_tensors(wl)
+
+    def ctx_of(tensors, images):
+        ctx = fv.FvContext(wl.L, C, H, [(hc, wc), (h, w)], 0, images, k, tensors, cross_len=64, mlp_ratio=2, device=DEV, resid_dtype=resid_dtype)
+        for l in range(wl.L):
+            for si in range(3):
+                c = ctx.cache_view(l, si)
+                c.copy_(_bf16_t(I.normal_bf16(821 + 3 * l + si, (B,) + tuple(c.shape[1:])))[:images])
+        ctx.prepare_text(images)
+        ctx.set_state(1, 0)
+        return ctx
+
+    ctx = ctx_of(mt, B)
+    x = x.to(ctx.x_dtype)
+    trace = torch.full((wl.L, 3, B, k), -1, dtype=torch.int32, device=DEV)
+    got = ctx.var_step(x, 1, keep, idx_trace=trace)
+    ctx.set_state(1, 0)
+    assert torch.equal(got, ctx.var_step(x, 1, keep, forced_idx=trace))        # the kept sets given: the same arithmetic
+    assert ctx.device_status() == 0
+    ctx.close()
+    first_image = copy.copy(mt)
+    first_image.mod, first_image.text = mt.mod[:, :1].copy(), mt.text[:1].copy()
+    one = ctx_of(first_image, 1)
+    alone = one.var_step(x[:1], 1, keep, forced_idx=trace[:, :, :1].contiguous())
+    # other tiles: fp32 sums in another order, at most one bf16 rounding apart in any activation on the way
+    err, cos = per_token_errors(got[:1].float().cpu().numpy(), alone.double().cpu().numpy())
+    assert err <= MAX_ABS * (4 if resid_dtype else 1) and cos >= MIN_COS
+    assert one.device_status() == 0
+    one.close()
+    zero = _zero_branch_tensors(wl)
+    ctx = ctx_of(zero, B)
+    for l in range(wl.L):
+        for si in range(3):
+            ctx.cache_view(l, si).zero_()
+    assert torch.equal(ctx.var_step(x, 1, keep, idx_trace=trace), x)
+    sets = trace.cpu().numpy()
+    score = O.pts_score(x.double().cpu().numpy())
+    tau = np.sort(score, axis=1)[:, ::-1][:, k - 1]
+    first = O.pts_topk(score, k)
+    for l in range(wl.L):
+        for si in range(3):
+            for b in range(B):
+                diff = np.setxor1d(sets[l, si, b], first[b])
+                assert np.all(np.abs(score[b, diff] - tau[b]) <= 1e-5 * tau[b])
     ctx.close()
 
 
