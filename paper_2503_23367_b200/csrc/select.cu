@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(256) colsum_chunk_kernel(const XT* x, int n, i
 // chunks in turn would change the order of the additions, so one thread adds them all, 16 loads in flight.  A launch of its own
 // behind the streaming kernel: folding by the last CTA of a group to arrive needs zeroed counters (a memset before
 // every stand-alone selection) and puts a fence, an atomic and a reload at the end of every CTA.  It also zeroes the counters
-// and range words of the scoring kernel behind it.
+// of the scoring kernel behind it.
 __global__ void __launch_bounds__(64) colsum_fold_kernel(const float4* chunk_partial, int C4, int nchunks, int group, int ngroups, float4* __restrict__ group_partial,
                                                          unsigned int* tickets, int ticket_words) {
   pdl_trigger();
@@ -132,32 +132,6 @@ __global__ void __launch_bounds__(256) colsum_total_kernel(const float4* chunk_p
     for (int p = 1; p < 16; ++p) { const float4 v = s_sum[p][q]; acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w; }
     group_partial[(size_t)b * ngroups * C4 + c4] = acc;
   }
-}
-
-// Exclusive prefix sum of one value per thread over the whole CTA (T threads, the template argument); returns the
-// exclusive prefix and, through `total`, the CTA-wide sum.  s_warp is 32 words of scratch.
-template <int T>
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s_warp, uint32_t* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  __syncthreads();  // s_warp may still be read from a previous scan
-  if (lane == 31) s_warp[warp] = inc;
-  __syncthreads();
-  uint32_t wv = lane < (T / 32) ? s_warp[lane] : 0u;
-  uint32_t winc = wv;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t t = __shfl_up_sync(0xffffffffu, winc, o);
-    if (lane >= o) winc += t;
-  }
-  uint32_t warp_excl = __shfl_sync(0xffffffffu, winc - wv, warp);
-  *total = __shfl_sync(0xffffffffu, winc, 31);
-  return warp_excl + inc - v;
 }
 
 // ---- Eq. 4: the mean token of image b from up to two sets of at most kMaxGroups partial column sums, added in a
@@ -260,12 +234,8 @@ __device__ __forceinline__ void mean_from_kept_partials(float4* s_mean, float4* 
 // ---- Eq. 5 / Algorithm 1: squared deviation from the mean, one warp per token row; the warps of an image stride
 // over its rows.
 // BATCH: 16-byte loads a lane requests together (8 with 64 registers per thread, 16 with 128).
-// lo / hi: running smallest / largest score key (the bit pattern without its sign) of the rows this warp has scored.
-// inv (may be null): the inverse map of the image is set to "not kept" for every row scored here, so that the CTA
-// that ranks the image only has to write the entries of the kept rows (one SM stores slowly).
 template <int T, int BATCH, typename XT>
-__device__ __forceinline__ void score_rows(const XT* x, const float4* s_mean, int b, int n, int C4, float* __restrict__ score,
-                                           int32_t* __restrict__ inv, uint32_t& lo, uint32_t& hi) {
+__device__ __forceinline__ void score_rows(const XT* x, const float4* s_mean, int b, int n, int C4, float* __restrict__ score) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // from the last row to the first: the kernel before has walked the map upwards, its end is what L2 still holds
   for (int r = n - 1 - ((int)blockIdx.x * (T / 32) + warp); r >= 0; r -= gridDim.x * (T / 32)) {
@@ -291,12 +261,7 @@ __device__ __forceinline__ void score_rows(const XT* x, const float4* s_mean, in
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
-      score[(size_t)b * n + r] = acc;
-      if (inv) inv[(size_t)b * n + r] = -1;
-    }
-    const uint32_t key = __float_as_uint(acc) & 0x7FFFFFFFu;
-    lo = min(lo, key); hi = max(hi, key);
+    if (lane == 0) score[(size_t)b * n + r] = acc;
   }
 }
 
@@ -305,55 +270,58 @@ constexpr int kFirstDigitBits = 11;                 // the first radix digit: up
 constexpr int kHistBins = 1 << kFirstDigitBits;
 constexpr int kCandMax = 1024;                      // longest candidate list kept beside the keys
 constexpr int kCountMax = 128;                      // a list this short is finished by counting
-struct TopkShared {
-  uint32_t hist[kHistBins];      // radix histogram; afterwards the kept / equal counts per 128 tokens of the compaction
+struct __align__(16) TopkShared {
+  uint32_t hist[kHistBins];      // radix histogram
   uint32_t cand[2][kCandMax];    // keys that still share the threshold's leading digits
   uint32_t warp[32];
   uint32_t range[64];
-  uint32_t prefix, remaining, nbin, near, ncand[2];
+  uint32_t prefix, remaining, nbin, near, ncand[2], tau, need_eq;
 };
-static_assert(kTopkMaxTokens / 128 <= 512 && kTopkMaxTokens % 4 == 0, "one count per 128 tokens and thread; keys in 16-byte words");
-
-// Smallest and largest score key of the image, gathered while the scores are computed: every CTA folds the keys of
-// its rows and adds them to two words per image with integer atomics (order-independent); the words hold ~min and
-// max so that zero means "nothing yet", and the CTA that ranks the image zeroes them again.
-template <int T>
-__device__ __forceinline__ void publish_range(uint32_t lo, uint32_t hi, TopkShared& sh, unsigned int* range_b) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) { sh.range[warp] = lo; sh.range[32 + warp] = hi; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (T / 32); ++w) { lo = min(lo, sh.range[w]); hi = max(hi, sh.range[32 + w]); }
-    if (lo <= hi) { atomicMax(range_b, ~lo); atomicMax(range_b + 1, hi); }
-  }
-}
+static_assert(kTopkMaxTokens < 65536 && kTopkMaxTokens % 128 == 0, "two counts in a word; keys in whole chunks");
 
 // The bin, counted from the top, in which the running count reaches sh.remaining: its index is added to sh.prefix at
-// `shift`, sh.remaining becomes the rank inside the bin and sh.nbin the bin's count.  All threads; ends with a barrier.
+// `shift`, sh.remaining becomes the rank inside the bin and sh.nbin the bin's count.  All threads; ends with a barrier.  Half of the warps of a
+// CTA of 1024 do it: every warp more only takes issue slots from those that have bins.
 template <int T>
 __device__ __forceinline__ void threshold_bin(TopkShared& sh, int nbins, int shift) {
-  const int tid = threadIdx.x;
-  uint32_t local[4], sum = 0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int W = kHistBins / 128;       // warps with bins, four per lane
+  static_assert(W <= T / 32, "four bins per lane cover the histogram");
+  const uint32_t rem = sh.remaining;       // read before the barrier, rewritten after it
+  uint32_t local[4] = {0u, 0u, 0u, 0u}, sum = 0, inc = 0;
+  if (warp < W) {
+    if (nbins >= 4) {
+      const int q = nbins / 4 - 1 - tid;
+      if (q >= 0) { const uint4 v = reinterpret_cast<const uint4*>(sh.hist)[q]; local[0] = v.w; local[1] = v.z; local[2] = v.y; local[3] = v.x; }
+    } else if (tid == 0) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int bin = nbins - 1 - 4 * tid - j;
-    local[j] = bin >= 0 ? sh.hist[bin] : 0u;
-    sum += local[j];
+      for (int j = 0; j < 4; ++j)
+        if (j < nbins) local[j] = sh.hist[nbins - 1 - j];
+    }
+    sum = local[0] + local[1] + local[2] + local[3];
+    inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (lane == 31) sh.warp[warp] = inc;
   }
-  const uint32_t rem = sh.remaining;   // read before the barriers of the scan, rewritten after them
-  uint32_t tot;
-  const uint32_t excl = block_exclusive_scan<T>(sum, sh.warp, &tot);
-  if (excl < rem && excl + sum >= rem) {   // exactly one thread
-    uint32_t cum = excl;
+  __syncthreads();
+  if (warp < W) {
+    const uint32_t excl = __reduce_add_sync(0xffffffffu, lane < warp ? sh.warp[lane] : 0u) + inc - sum;
+    if (excl < rem && excl + sum >= rem) {   // exactly one thread
+      uint32_t cum = excl;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (cum + local[j] >= rem) {
-        sh.prefix |= (uint32_t)(nbins - 1 - 4 * tid - j) << shift;
-        sh.remaining = rem - cum;
-        sh.nbin = local[j];
-        break;
+      for (int j = 0; j < 4; ++j) {
+        if (cum + local[j] >= rem) {
+          sh.prefix |= (uint32_t)(nbins - 1 - 4 * tid - j) << shift;
+          sh.remaining = rem - cum;
+          sh.nbin = local[j];
+          break;
+        }
+        cum += local[j];
       }
-      cum += local[j];
     }
   }
   __syncthreads();
@@ -361,69 +329,80 @@ __device__ __forceinline__ void threshold_bin(TopkShared& sh, int nbins, int shi
 
 // ---- exact top-k of one image by one CTA (all T threads): radix select on the fp32 bit patterns of the
 // scores (s >= 0, so they order like the values), ties to the lowest index, ascending output, inverse map.
-// range_b: the image's two range words (see publish_range), complete when this is called.
-//   1. one sweep brings the scores from L2 into shared memory as keys relative to the smallest, and counts the first
-//      digit -- the top 11 bits of the range the keys really span, so that the counts spread over the bins;
+//   1. one sweep brings the scores from L2 into shared memory and finds the range they span, the next counts the first digit of the
+//      keys relative to the smallest -- the top 11 bits of that range, so that the counts spread over the bins;
 //   2. the keys inside the threshold's bin (a few dozen on a map of distinct scores) are copied to a list, which
 //      is finished by counting when it is short and by 8-bit digits otherwise; a bin too full for the list (many
 //      equal scores) is refined with 8-bit digits over all keys until it fits;
-//   3. ordered compaction: counts per 128 tokens, one scan over them, then every lane knows the output slots of its
-//      four tokens.
-// One SM does all of this while the others idle, and its instruction issue is what the sweeps wait for: they take
-// four keys per lane and 16-byte shared-memory accesses.
+//   3. ordered compaction: every warp owns a run of tokens; the warps' counts, added up, give each its first output slot.
+// One SM does all of this while the others idle, in a chain of short phases with a barrier between them, and its instruction issue is what the
+// sweeps wait for: four keys per lane and 16-byte accesses, few phases, no warps without work in them.  Us from the last score to the kept set,
+// 4096 / 16384 tokens (device timestamps): with the range gathered by all CTAs through atomics, counts of 128 tokens scanned by the whole CTA and only
+// kept tokens written to the inverse map 7.2 / 13.5; now 5.4 / 9.6.
 template <int T>
 __device__ __forceinline__ void topk_image(const float* __restrict__ sc, int n, int k, uint32_t* s_keys, TopkShared& sh,
-                                           int32_t* __restrict__ idx_b, int32_t* __restrict__ inv_b, int32_t* near_tie_b,
-                                           unsigned int* range_b) {
+                                           int32_t* __restrict__ idx_b, int32_t* __restrict__ inv_b, int32_t* near_tie_b) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t kmin = ~__ldcg(range_b), kmax = __ldcg(range_b + 1);
-  const uint32_t range = kmax >= kmin ? kmax - kmin : 0u;
-  const int bits = range ? 32 - __clz(range) : 0;
-  int width = min(bits, kFirstDigitBits);
-  int shift = bits - width;
 #pragma unroll
   for (int j = 0; j < kHistBins / T; ++j) sh.hist[tid + j * T] = 0u;
   if (tid == 0) { sh.prefix = 0u; sh.remaining = (uint32_t)k; sh.near = 0u; sh.ncand[0] = 0u; sh.ncand[1] = 0u; }
-  __syncthreads();
-  if (tid == 0) { range_b[0] = 0u; range_b[1] = 0u; }   // every thread has read them
 
-  // ---- 1. scores -> keys, first digit counted on the way.  Up to eight 16-byte loads per thread are requested
-  // before the first is used (one CTA fetching them one dependent load at a time took longer than the ranking).
+  // ---- 1. scores -> keys (bit patterns; the mask drops the sign of -0).  Up to four 16-byte loads per thread are requested before the first is
+  // used (one CTA fetching them one dependent load at a time took longer than the ranking).
   const int n4 = (n % 4 == 0 && (reinterpret_cast<uintptr_t>(sc) & 15u) == 0) ? n / 4 : 0;
-  const uint32_t top = (1u << width) - 1u;
-  for (int i0 = tid; i0 < n4; i0 += T * 8) {
-    float4 v[8];
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+  for (int i0 = tid; i0 < n4; i0 += T * 4) {
+    float4 v[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
+    for (int u = 0; u < 4; ++u)
       if (i0 + u * T < n4) v[u] = __ldcg(reinterpret_cast<const float4*>(sc) + i0 + u * T);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i4 = i0 + u * T;
-      if (i4 < n4) {
+    for (int u = 0; u < 4; ++u) {
+      if (i0 + u * T < n4) {
         uint4 key;
-        key.x = (__float_as_uint(v[u].x) & 0x7FFFFFFFu) - kmin;   // the mask drops the sign of -0
-        key.y = (__float_as_uint(v[u].y) & 0x7FFFFFFFu) - kmin;
-        key.z = (__float_as_uint(v[u].z) & 0x7FFFFFFFu) - kmin;
-        key.w = (__float_as_uint(v[u].w) & 0x7FFFFFFFu) - kmin;
-        reinterpret_cast<uint4*>(s_keys)[i4] = key;
-        // (the clamp only matters if the range words were damaged, e.g. by two launches sharing one workspace)
-        atomicAdd(&sh.hist[min(key.x >> shift, top)], 1u); atomicAdd(&sh.hist[min(key.y >> shift, top)], 1u);
-        atomicAdd(&sh.hist[min(key.z >> shift, top)], 1u); atomicAdd(&sh.hist[min(key.w >> shift, top)], 1u);
+        key.x = __float_as_uint(v[u].x) & 0x7FFFFFFFu; key.y = __float_as_uint(v[u].y) & 0x7FFFFFFFu;
+        key.z = __float_as_uint(v[u].z) & 0x7FFFFFFFu; key.w = __float_as_uint(v[u].w) & 0x7FFFFFFFu;
+        reinterpret_cast<uint4*>(s_keys)[i0 + u * T] = key;
+        lo = min(min(lo, min(key.x, key.y)), min(key.z, key.w));
+        hi = max(max(hi, max(key.x, key.y)), max(key.z, key.w));
       }
     }
   }
   for (int i = 4 * n4 + tid; i < n; i += T) {
-    const uint32_t key = (__float_as_uint(__ldcg(sc + i)) & 0x7FFFFFFFu) - kmin;
+    const uint32_t key = __float_as_uint(__ldcg(sc + i)) & 0x7FFFFFFFu;
     s_keys[i] = key;
-    atomicAdd(&sh.hist[min(key >> shift, top)], 1u);
+    lo = min(lo, key); hi = max(hi, key);
+  }
+  if (tid < (128 - n % 128) % 128) s_keys[n + tid] = 0u;   // (read by the compaction)
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) { sh.range[warp] = lo; sh.range[32 + warp] = hi; }
+  __syncthreads();
+  const uint32_t kmin = __reduce_min_sync(0xffffffffu, lane < T / 32 ? sh.range[lane] : 0xFFFFFFFFu);
+  const uint32_t kmax = __reduce_max_sync(0xffffffffu, lane < T / 32 ? sh.range[32 + lane] : 0u);
+  const uint32_t range = kmax - kmin;
+  const int bits = range ? 32 - __clz(range) : 0;
+  int width = min(bits, kFirstDigitBits);
+  int shift = bits - width;
+  for (int i = tid; i < n4; i += T) {     // (every thread meets the keys it has written)
+    uint4 key = reinterpret_cast<const uint4*>(s_keys)[i];
+    key.x -= kmin; key.y -= kmin; key.z -= kmin; key.w -= kmin;
+    reinterpret_cast<uint4*>(s_keys)[i] = key;
+    atomicAdd(&sh.hist[key.x >> shift], 1u); atomicAdd(&sh.hist[key.y >> shift], 1u);
+    atomicAdd(&sh.hist[key.z >> shift], 1u); atomicAdd(&sh.hist[key.w >> shift], 1u);
+  }
+  for (int i = 4 * n4 + tid; i < n; i += T) {
+    const uint32_t key = s_keys[i] - kmin;
+    s_keys[i] = key;
+    atomicAdd(&sh.hist[key >> shift], 1u);
   }
   __syncthreads();
 
-  // ---- 2. the k-th largest key: after this sh.prefix is that key (relative to kmin) and sh.remaining how many of
-  // the keys equal to it belong to the kept set.
+  // ---- 2. the k-th largest key, tau (relative to kmin), and how many of the keys equal to it belong to the kept set, need_eq.
   bool listed = false;
   int cur = 0;
   uint32_t nlist = 0;
+  bool counted = false;
   for (;;) {
     threshold_bin<T>(sh, 1 << width, shift);
     if (shift == 0) break;                        // every bit of the range is decided
@@ -448,14 +427,16 @@ __device__ __forceinline__ void topk_image(const float* __restrict__ sc, int n, 
       __syncthreads();
       if (nlist <= (uint32_t)kCountMax) {         // finish by counting: the key with fewer than `remaining` keys above
         const uint32_t rem = sh.remaining;        // it and at least `remaining` keys not below it
-        __syncthreads();
-        if ((uint32_t)tid < nlist) {
-          const uint32_t key = sh.cand[cur][tid];
-          uint32_t gt = 0, eq = 0;
-          for (uint32_t j = 0; j < nlist; ++j) { const uint32_t c = sh.cand[cur][j]; gt += c > key; eq += c == key; }
-          if (gt < rem && rem <= gt + eq) { sh.prefix = key; sh.remaining = rem - gt; }   // equal keys write the same
+        for (uint32_t i = warp; i < nlist; i += T / 32) {    // a warp per candidate, its lanes along the list
+          const uint32_t key = sh.cand[cur][i];
+          uint32_t p = 0;                           // above it | equal to it
+          for (uint32_t j = lane; j < nlist; j += 32) { const uint32_t c = sh.cand[cur][j]; p += (uint32_t)(c > key) + ((uint32_t)(c == key) << 16); }
+          p = __reduce_add_sync(0xffffffffu, p);
+          const uint32_t gt = p & 0xFFFFu, eq = p >> 16;
+          if (lane == 0 && gt < rem && rem <= gt + eq) { sh.tau = key; sh.need_eq = rem - gt; }   // equal keys write the same
         }
         __syncthreads();
+        counted = true;
         break;
       }
     }
@@ -480,71 +461,75 @@ __device__ __forceinline__ void topk_image(const float* __restrict__ sc, int n, 
     }
     __syncthreads();
   }
-  const uint32_t tau = sh.prefix;  // relative to kmin
-  const uint32_t need_eq = sh.remaining;
-  __syncthreads();                 // the histogram is reused below
+  const uint32_t tau = counted ? sh.tau : sh.prefix;  // relative to kmin
+  const uint32_t need_eq = counted ? sh.need_eq : sh.remaining;
 
-  // ---- 3. ordered compaction, 128 consecutive tokens per warp step (four per lane).  Counts per 128 tokens of the
-  // keys above the threshold (low half) and equal to it (high half; n <= 49152 keeps either total below 2^16), one
-  // scan over them, then every lane knows the output slots of its tokens.
-  uint32_t* seg = sh.hist;
-  const int nchunk = (n + 127) / 128;      // <= 384: one per thread in the scan
-  const uint4* s_keys4 = reinterpret_cast<const uint4*>(s_keys);   // the allocation is padded to whole 16-byte words
-  for (int c = warp; c < nchunk; c += (T / 32)) {
-    const int i0 = c * 128 + lane * 4;
-    uint32_t p = 0;
-    if (i0 < n) {
-      const uint4 v = s_keys4[i0 >> 2];
-      const uint32_t key[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (i0 + e < n) p += (uint32_t)(key[e] > tau) + ((uint32_t)(key[e] == tau) << 16);
-    }
-    p = __reduce_add_sync(0xffffffffu, p);
-    if (lane == 0) seg[c] = p;
-  }
+  // ---- 3. ordered compaction.  A warp owns a run of 128-token chunks, four tokens per lane.  Counts: keys above the threshold in the low half, equal
+  // to it in the high half (n <= 49152 keeps either total below 2^16).  The words behind the last key are zero: should that equal the
+  // threshold, they still come behind all the real ones, of which there are enough.  (A vote per 32 tokens costs four population counts, which take
+  // eight cycles each.)
+  const int nchunk = (n + 127) / 128, per_warp = (nchunk + T / 32 - 1) / (T / 32);
+  const int c_lo = warp * per_warp, c_hi = min(nchunk, c_lo + per_warp);
+  const uint4* mine = reinterpret_cast<const uint4*>(s_keys) + lane;
+  const auto counts = [&](const uint4& v) {
+    return (uint32_t)(v.x > tau) + (uint32_t)(v.y > tau) + (uint32_t)(v.z > tau) + (uint32_t)(v.w > tau) +
+           (((uint32_t)(v.x == tau) + (uint32_t)(v.y == tau) + (uint32_t)(v.z == tau) + (uint32_t)(v.w == tau)) << 16);
+  };
+  uint32_t count = 0;
+  for (int c = c_lo; c < c_hi; ++c) count += counts(mine[c * 32]);
+  count = __reduce_add_sync(0xffffffffu, count);
+  if (lane == 0) sh.warp[warp] = count;
   __syncthreads();
-  {
-    const uint32_t mine = tid < nchunk ? seg[tid] : 0u;
-    uint32_t tot;
-    const uint32_t before = block_exclusive_scan<T>(mine, sh.warp, &tot);
-    if (tid < nchunk) seg[tid] = before;
-  }
-  __syncthreads();
+  uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? sh.warp[lane] : 0u);   // (at most 32 warps)
   const float tau_f = __uint_as_float(tau + kmin);
   const float band = 1e-5f * tau_f;
   uint32_t near = 0;
-  for (int c = warp; c < nchunk; c += (T / 32)) {
+  const bool inv16 = inv_b && n % 4 == 0 && (reinterpret_cast<uintptr_t>(inv_b) & 15u) == 0;
+#pragma unroll 1
+  for (int c = c_lo; c < c_hi; ++c) {
     const int i0 = c * 128 + lane * 4;
-    uint32_t key[4] = {0u, 0u, 0u, 0u};
-    uint32_t p = 0;
-    if (i0 < n) {
-      const uint4 v = s_keys4[i0 >> 2];
-      key[0] = v.x; key[1] = v.y; key[2] = v.z; key[3] = v.w;
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (i0 + e < n) p += (uint32_t)(key[e] > tau) + ((uint32_t)(key[e] == tau) << 16);
-    }
+    const uint4 v = mine[c * 32];
+    const uint32_t key[4] = {v.x, v.y, v.z, v.w};
+    const uint32_t p = counts(v);
     uint32_t inc = p;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
       if (lane >= o) inc += t;
     }
-    const uint32_t base = seg[c] + inc - p;
-    uint32_t gt_before = base & 0xFFFFu, eq_before = base >> 16;
+    const uint32_t mine_before = before + inc - p;
+    before += __shfl_sync(0xffffffffu, inc, 31);
+    int32_t slot[4];
+    if (!__any_sync(0xffffffffu, p >> 16)) {
+      int pos = (int)((mine_before & 0xFFFFu) + min(mine_before >> 16, need_eq));   // kept tokens before this lane's
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (i0 + e < n) {
+      for (int e = 0; e < 4; ++e) {
+        slot[e] = -1;
+        if (key[e] > tau) { slot[e] = pos; idx_b[pos] = i0 + e; ++pos; }
+      }
+    } else {
+      uint32_t gt_before = mine_before & 0xFFFFu, eq_before = mine_before >> 16;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
         const bool is_gt = key[e] > tau, is_eq = key[e] == tau;
+        slot[e] = -1;
         if (is_gt || (is_eq && eq_before < need_eq)) {          // equal keys: the lowest indices
-          const uint32_t pos = gt_before + min(eq_before, need_eq);   // kept tokens before this one
-          idx_b[pos] = i0 + e;
-          if (inv_b) inv_b[i0 + e] = (int32_t)pos;   // the other entries were set to -1 when the rows were scored
+          slot[e] = (int32_t)(gt_before + min(eq_before, need_eq));
+          idx_b[slot[e]] = i0 + e;
         }
         gt_before += is_gt; eq_before += is_eq;
-        if (near_tie_b) near += (fabsf(__uint_as_float(key[e] + kmin) - tau_f) <= band);
       }
+    }
+    if (inv16) {
+      if (i0 < n) *reinterpret_cast<int4*>(inv_b + i0) = make_int4(slot[0], slot[1], slot[2], slot[3]);
+    } else if (inv_b) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (i0 + e < n) inv_b[i0 + e] = slot[e];
+    }
+    if (near_tie_b) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) near += i0 + e < n && fabsf(__uint_as_float(key[e] + kmin) - tau_f) <= band;
     }
   }
   if (near_tie_b) {
@@ -563,7 +548,7 @@ template <typename XT>
 __global__ void __launch_bounds__(kSelectThreads, 1) score_topk_kernel(const XT* x,
                                                                   const float4* group_partial, int ngroups, const float4* kept_partial, int kept_rows, int n,
                                                                   int C4, int k, int staged, float* __restrict__ score,
-                                                                  unsigned int* img_tickets, unsigned int* img_range, int32_t* __restrict__ idx,
+                                                                  unsigned int* img_tickets, int32_t* __restrict__ idx,
                                                                   int32_t* __restrict__ inv, int32_t* __restrict__ near_tie) {
   extern __shared__ float4 s_dyn[];
   float4* s_mean = s_dyn;
@@ -579,10 +564,8 @@ __global__ void __launch_bounds__(kSelectThreads, 1) score_topk_kernel(const XT*
   else if (staged) mean_from_partials_halves<kSelectThreads>(s_mean, s_mean + C4, group_partial + (size_t)b * ngroups * C4, ngroups, C4, n);
   else mean_from_partials<kSelectThreads>(s_mean, group_partial + (size_t)b * ngroups * C4, ngroups, nullptr, 0, C4, n);   // very wide maps
   __syncthreads();
-  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-  score_rows<kSelectThreads, 8, XT>(x, s_mean, b, n, C4, score, inv, lo, hi);
-  publish_range<kSelectThreads>(lo, hi, sh, img_range + 2 * b);
-  __threadfence();  // this thread's scores (and range) are visible device-wide before the CTA takes its ticket
+  score_rows<kSelectThreads, 8, XT>(x, s_mean, b, n, C4, score);
+  __threadfence();  // this thread's scores are visible device-wide before the CTA takes its ticket
 
   // ---- the last CTA of this image to get here ranks the image
   __syncthreads();
@@ -594,8 +577,7 @@ __global__ void __launch_bounds__(kSelectThreads, 1) score_topk_kernel(const XT*
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  topk_image<kSelectThreads>(score + (size_t)b * n, n, k, s_keys, sh, idx + (size_t)b * k, inv ? inv + (size_t)b * n : nullptr, near_tie ? near_tie + b : nullptr,
-             img_range + 2 * b);
+  topk_image<kSelectThreads>(score + (size_t)b * n, n, k, s_keys, sh, idx + (size_t)b * k, inv ? inv + (size_t)b * n : nullptr, near_tie ? near_tie + b : nullptr);
 }
 
 // ------------------------------------------------------------------------------------------------------------
@@ -620,7 +602,7 @@ struct FusedSelectArgs {
   unsigned int* done; unsigned int done_target;
   // phase 1
   const float4* group_partial; int ngroups;
-  float* score; unsigned int* img_tickets; unsigned int* img_range; int32_t* idx; int32_t* inv;
+  float* score; unsigned int* img_tickets; int32_t* idx; int32_t* inv;
   unsigned int* ready; unsigned int epoch;
   // phase 2
   const float* sigma; const float* beta; uint2* a_out;
@@ -812,9 +794,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) select_fused_kernel(const Fus
   mean_from_partials<kTopkThreads>(s_dyn, a.group_partial + (size_t)b * a.ngroups * C4, a.ngroups,
                      a.y ? a.kept_group + (size_t)b * a.ngk * C4 : nullptr, a.y ? a.ngk : 0, C4, n);
   __syncthreads();
-  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-  score_rows<kTopkThreads, 16, float>(reinterpret_cast<const float*>(a.x), s_dyn, b, n, C4, a.score, a.inv, lo, hi);
-  publish_range<kTopkThreads>(lo, hi, sh, a.img_range + 2 * b);
+  score_rows<kTopkThreads, 16, float>(reinterpret_cast<const float*>(a.x), s_dyn, b, n, C4, a.score);
   __threadfence();
   __syncthreads();
   if (tid == 0) {
@@ -829,8 +809,7 @@ __global__ void __launch_bounds__(kTopkThreads, 1) select_fused_kernel(const Fus
   float4* s_beta = nullptr;
   if (last) {
     __threadfence();
-    topk_image<kTopkThreads>(a.score + (size_t)b * n, n, a.k, reinterpret_cast<uint32_t*>(s_dyn), sh, a.idx + (size_t)b * a.k, a.inv + (size_t)b * n, nullptr,
-               a.img_range + 2 * b);
+    topk_image<kTopkThreads>(a.score + (size_t)b * n, n, a.k, reinterpret_cast<uint32_t*>(s_dyn), sh, a.idx + (size_t)b * a.k, a.inv + (size_t)b * n, nullptr);
     __threadfence();
     __syncthreads();
     if (tid == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.ready + b), "r"(a.epoch) : "memory");
@@ -882,7 +861,7 @@ __global__ void inv_scatter_kernel(const int32_t* idx, int B, int k, int n, int3
 
 }  // namespace
 
-// group arrival counters [B, kMaxGroups], image arrival counters [B], score range words [B, 2]
+// group arrival counters [B, kMaxGroups], image arrival counters [B], two spare words per image
 size_t select_ticket_bytes(int B) { return align_up((size_t)B * (kMaxGroups + 3) * sizeof(unsigned int), 256); }
 
 static void chunking(int n, int* nchunks, int* group, int* ngroups) {
@@ -947,7 +926,7 @@ static cudaError_t launch_select_t(const XT* x, int B, int n, int C, int k, int3
   const int C4 = C / 4;
   if (!have_partials)
     launch_colsum_t(x, B, n, C, w, st);
-  const size_t keys_smem = ((size_t)n + 3) / 4 * 16;   // whole 16-byte words
+  const size_t keys_smem = ((size_t)n + 127) / 128 * 512;   // whole chunks of the compaction
   const int staged = (size_t)C * 4 * 9 <= kTopkMaxSmem;  // room for the mean token and eight staged partial sums
   const size_t mean_smem = (size_t)C * 4 * (staged ? 9 : 1);
   const size_t smem = keys_smem > mean_smem ? keys_smem : mean_smem;
@@ -957,10 +936,8 @@ static cudaError_t launch_select_t(const XT* x, int B, int n, int C, int k, int3
   if (per_image > need) per_image = need;
   if (per_image < 1) per_image = 1;
   unsigned int* img_tickets = w.tickets + (size_t)B * kMaxGroups;
-  unsigned int* img_range = w.tickets + (size_t)B * (kMaxGroups + 1);
   const float4* gp = reinterpret_cast<const float4*>(w.group_partial);
-  launch_pdl(score_topk_kernel<XT>, dim3(per_image, B), dim3(kSelectThreads), smem, st, x, gp, w.ngroups, reinterpret_cast<const float4*>(kept_partial), kept_rows, n, C4, k, staged, sc, img_tickets,
-             img_range, idx, inv, near_tie);
+  launch_pdl(score_topk_kernel<XT>, dim3(per_image, B), dim3(kSelectThreads), smem, st, x, gp, w.ngroups, reinterpret_cast<const float4*>(kept_partial), kept_rows, n, C4, k, staged, sc, img_tickets, idx, inv, near_tie);
   return cudaGetLastError();
 }
 
@@ -991,7 +968,7 @@ size_t select_fused_ws_bytes(int B, int C) {
 }
 
 static size_t fused_smem_bytes(int n, int C) {
-  const size_t keys = ((size_t)n + 3) / 4 * 16;
+  const size_t keys = ((size_t)n + 127) / 128 * 512;
   const size_t vec = (size_t)C * 4;                       // the mean token
   const int rows_par = kTopkThreads / (C / 8);
   const size_t comb = (size_t)(rows_par > 1 ? rows_par - 1 : 0) * C * 4;
@@ -1036,7 +1013,7 @@ cudaError_t launch_select_fused(const FusedSelect& f, cudaStream_t st) {
   a.epoch = ++*f.epoch;
   a.group_partial = reinterpret_cast<const float4*>(w.group_partial); a.ngroups = w.ngroups;
   a.score = w.score; a.img_tickets = w.tickets + (size_t)f.B * kMaxGroups;
-  a.img_range = w.tickets + (size_t)f.B * (kMaxGroups + 1); a.idx = f.idx; a.inv = f.inv;
+  a.idx = f.idx; a.inv = f.inv;
   a.sigma = f.sigma; a.beta = f.beta; a.a_out = reinterpret_cast<uint2*>(f.a_out);
   a.status = f.status;
   // algorithmic bytes: the selection (x once, scores, indices), the gather (kept rows in, bf16 out) and, when it
