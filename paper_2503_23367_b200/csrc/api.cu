@@ -587,7 +587,7 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
   // restores its own.
   const bool fused = selecting && g_step_fused && !xb && select_fused_supported(B, n, C);
   // Small maps: one launch between two branches (select_small.cu); the last sublayer's restoration is a launch of its own.
-  const bool small_map = c.interp_mode == 0 && select_small_supported(B, n, C, xb);
+  const bool small_map = c.interp_mode == 0 && select_small_in_step(B, n, C, xb, k >= kMinMapRows);
   const bool small = selecting && !fused && small_map;
   // On the others the kept rows of a sublayer are restored by its last GEMM, straight from the accumulators: row j of the compact tensor is added to its
   // token's row of x, and the column sums of the updated rows fall out of the same registers.  As a launch of their own (forwarded rows stored in bf16, read

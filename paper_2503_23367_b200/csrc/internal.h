@@ -166,6 +166,7 @@ struct SmallSelect {
 };
 cudaError_t select_small_init();
 bool select_small_supported(int B, int n, int C, bool x_bf16);
+bool select_small_in_step(int B, int n, int C, bool x_bf16, bool gemm_could_restore);   // between two sublayers of a step
 cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st);
 
 // ---- rows.cu : gather + LayerNorm + modulate, restore (+ gate and residual) ----------------------

@@ -420,7 +420,8 @@ cudaError_t select_small_init() {
 // through its rows alone, so the gain over the separate kernels (some 9 ... 12 us per sublayer on the smallest maps) is used up
 // at about 50 rows, or 200 KB of them.  Measured, us per block of 2 sublayers (3 at C 2048), separate kernels -> this one: 16 rows C 1024
 // 91 -> 69, C 2048 161 -> 137; 32 rows (clusters of 8) C 1024 107 -> 94; 21 rows C 1920 179 -> 170; 25 rows C 2048 183 -> 190; 36 rows
-// C 256 74 -> 63, C 512 84 -> 80, C 1024 bf16 stream 119 -> 107; 64 rows C 256 76 -> 78, C 512 90 -> 98, C 1024 bf16 148 -> 155.
+// C 256 74 -> 63, C 512 84 -> 80, C 1024 bf16 stream 119 -> 107; 64 rows C 256 76 -> 78, C 512 90 -> 98, C 1024 bf16 148 -> 155.  (Against separate
+// kernels with a launch for the kept rows, which images of fewer than 128 of them still take.)
 static int small_cluster(int B, int n, int C, bool x_bf16) {
   if (C % 128 || C > 2048) return 0;
   const int cl = g_clusters[1] >= B ? 16 : (g_clusters[0] >= B ? 8 : 0);
@@ -430,6 +431,16 @@ static int small_cluster(int B, int n, int C, bool x_bf16) {
   return cl;
 }
 bool select_small_supported(int B, int n, int C, bool x_bf16) { return small_cluster(B, n, C, x_bf16) > 0; }
+
+// Inside a step, between two sublayers whose last GEMM could restore the kept rows itself (128 of them per image): that route's selection has no
+// restoration in front of it and beats the one launch unless a CTA has very little to work through.  Us per block of 2 sublayers (3 at C 2048), this kernel ->
+// that route: 16 rows C 1024 68 -> 75 (two images 68 -> 74, four 78 -> 78), C 256 49 -> 55, C 2048 152 -> 147 (two images 164 -> 152), C 1920 bf16 stream 114 -> 108;
+// 21 rows C 1920 117 -> 103 (four images 169 -> 151); 25 rows C 512 74 -> 68, C 1024 78 -> 74; 32 rows C 1024, eight images, 94 -> 92; 36 rows
+// C 256 62 -> 60, C 512 74 -> 67, C 1024 bf16 98 -> 80.
+bool select_small_in_step(int B, int n, int C, bool x_bf16, bool gemm_could_restore) {
+  const int cl = small_cluster(B, n, C, x_bf16);
+  return cl > 0 && (!gemm_could_restore || ((n + cl - 1) / cl <= 16 && C <= 1024));
+}
 
 cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st) {
   const int cl = small_cluster(f.B, f.n, f.C, f.x_bf16);
