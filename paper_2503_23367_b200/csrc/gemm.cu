@@ -340,6 +340,17 @@ static cudaError_t launch_bn(const GemmArgs& g, const GemmDev& p, int tiles_m, c
   return launch_pdl(gemm_bf16_kernel<BN, 0>, dim3(grid), dim3(gemm_threads(0)), GemmCfg<BN>::smem_bytes(false), st, tmA, tmB, p);
 }
 
+// Bytes of the operands and results of a GEMM: A, W, and what its epilogue reads and writes (a residual epilogue the stream both ways, a copy of the branch
+// output beside it, the column sums of the rows of a map).
+static double operand_bytes(const GemmArgs& g) {
+  const double mn = (double)g.M * g.N;
+  double out = mn * (g.epilogue == EPI_RESIDUAL ? 8.0 : (g.epilogue == EPI_RESIDUAL_XBF16 || g.epilogue == EPI_F32 ? 4.0 : 2.0));
+  if (g.aux && (g.epilogue == EPI_RESIDUAL || g.epilogue == EPI_RESIDUAL_XBF16)) out += 2.0 * mn;
+  if (g.colsum)
+    for (int img = 0; img < g.M / g.rows_per_image; ++img) out += 4.0 * g.N * map_colsum_count(img, g.rows_per_image);
+  return 2.0 * ((double)g.M * g.K + (double)g.N * g.K) + out;
+}
+
 static int g_force_path = 0;
 void gemm_force_path(int path) { g_force_path = path; }
 
@@ -401,7 +412,7 @@ fv_status launch_gemm(const GemmArgs& g, cudaStream_t st) {
     p.kb_per_split = (num_kb + cluster_slices - 1) / cluster_slices;
     p.kb_per_split += p.kb_per_split & 1;   // even: a pipeline stage of the cluster kernel may hold two k-blocks of ONE slice
   }
-  LaunchScope scope(KC_GEMM, 1, 2.0 * g.M * (double)g.N * g.K, 2.0 * ((double)g.M * g.K + (double)g.N * g.K + (double)g.M * g.N), st);
+  LaunchScope scope(KC_GEMM, 1, 2.0 * g.M * (double)g.N * g.K, operand_bytes(g), st);
   if (cluster_slices) return launch_gemm_cluster(g, p, cluster_bn, cluster_slices, st) == cudaSuccess ? FV_OK : FV_ERR_CUDA;
   if (tc.pair) {
     cudaError_t e2 = launch_gemm_pair(g, p, bn, st);

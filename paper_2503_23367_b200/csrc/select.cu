@@ -1035,7 +1035,8 @@ cudaError_t launch_colsum(const float* x, int B, int n, int C, void* workspace, 
 cudaError_t launch_colsum_total(int B, int n, int C, void* workspace, cudaStream_t st) {
   const SelectWs w = select_ws_carve(workspace, B, n, C);
   const int C4 = C / 4;
-  LaunchScope scope(KC_RESTORE, 1, 0.0, 0.0, st);
+  const double bytes = 4.0 * B * C * (w.nchunks + 1.0);   // the chunk partials and their sum
+  LaunchScope scope(KC_RESTORE, 1, bytes, bytes, st);
   return launch_pdl(colsum_total_kernel, dim3((C4 + 15) / 16, B), dim3(256), 0, st, reinterpret_cast<const float4*>(w.chunk_partial), C4, w.nchunks, w.ngroups,
                     reinterpret_cast<float4*>(w.group_partial));
 }

@@ -357,6 +357,36 @@ def test_kept_rows_restored_by_the_last_gemm(h, w, hc, wc, C, H, B, keep, resid_
     ctx.close()
 
 
+@pytest.mark.parametrize("resid_dtype", [0, 1])
+def test_bytes_counted_for_the_gemms_and_the_restoration_of_a_step(resid_dtype):
+    """fv_profile_read's dram_bytes of both classes is the sum over their launches of operands and results: for a residual GEMM the stream read
+    and written (with the copy for the cache, or the column sums of the kept rows), for a pruned step's side stream the restoration
+    of the other rows and the sum of its partials."""
+    h, w, hc, wc, C, B, keep, L, ratio = 26, 31, 10, 10, 256, 3, 0.16, 2, 2
+    wl = I.Workload("bytes", L=L, C=C, H=2, B=B, sides=(hc, h), keep=(1.0, keep), mlp_ratio=ratio, seed=816)
+    n, nc, k, F, s = h * w, hc * wc, O.kept_count(keep, h, w), ratio * C, 4 if resid_dtype else 8
+    ctx = fv.FvContext(L, C, 2, [(hc, wc), (h, w)], 0, B, nc + k, I.model_tensors(wl), mlp_ratio=ratio, device=DEV, resid_dtype=resid_dtype)
+    xs = [torch.from_numpy(I.token_map(832, B, a, b, C, "structured")).to(DEV).to(ctx.x_dtype) for a, b in ((hc, wc), (h, w))]
+
+    def gemms(M, out):          # QKV, out-projection and both MLP GEMMs of every block; out: bytes the two residual epilogues move, all blocks
+        return L * 2 * (M * C + 3 * C * C + 3 * M * C + M * C + C * C + M * C + F * C + M * F + M * F + F * C) + out
+
+    fv.fv_profile_read()
+    ctx.var_step(xs[0], 0, 1.0)
+    got = fv.fv_profile_read()
+    assert got["gemm"]["dram_bytes"] == gemms(B * nc, 2 * L * (s + 2) * B * nc * C)
+    assert got["restore"]["dram_bytes"] == 0
+    ctx.var_step(xs[1], 1, keep)
+    got = fv.fv_profile_read()
+    blocks = sum((b * k + k - 1) // 128 - b * k // 128 + 1 for b in range(B))       # 128-row blocks of the compact rows, once per image they hold
+    selections = 2 * L                                                               # the last one has no selection behind it
+    assert got["gemm"]["dram_bytes"] == gemms(B * k, selections * s * B * k * C + (selections - 1) * 4 * C * blocks)
+    assert got["restore"]["launches"] == 2 * selections - 1
+    assert got["restore"]["dram_bytes"] == selections * B * C * (s * (n - k) + 2 * nc) + (selections - 1) * 4 * B * C * (-(-n // 32) + 1)
+    assert ctx.device_status() == 0
+    ctx.close()
+
+
 def test_free_running_selection_matches_oracle_on_identical_input():
     wl = I.WORKLOADS["tiny"]
     mt = I.model_tensors(wl)
