@@ -58,8 +58,7 @@ template <int BN> struct GemmCfg {
 // that epilogue takes eight warps and more registers per thread; the others stay small enough for a bandwidth-bound kernel of another
 // stream (the restoration of the rows that were not kept) to share the SMs with them.
 template <int BN, int KIND>
-__global__ void __launch_bounds__(gemm_threads(KIND), 1)
-gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmDev p) {
+__device__ __forceinline__ void gemm_body(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmDev& p) {
   using Cfg = GemmCfg<BN>;
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;
@@ -246,6 +245,18 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   }
 }
 
+template <int BN, int KIND>
+__global__ void __launch_bounds__(gemm_threads(KIND), 1)
+gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmDev p) { gemm_body<BN, KIND>(tmA, tmB, p); }
+
+// The kept rows of a large map on 64-wide tiles (gemm_leaves_room): this kernel's CTAs come early, before all CTAs of the restoration of the other rows
+// are placed, and wait.  Ten warps put three on a scheduler, so 3 x R registers a lane and two warps of the restoration (80) fit the scheduler's 512 up
+// to R = 117; with 158 the restoration had to crowd on the SMs left (56 ... 60 us instead of 38 ... 44 behind two images of 64 x 64 tokens, C 2048, 143 kept
+// rows; us per block there 285 -> 250; one image, C 1920, 400 rows 191 -> 170; 80 x 80, C 1920, 300 rows 191 -> 171; 96 x 96, C 2048, 300 rows 314 -> 284).
+template <int KIND>
+__global__ void __maxnreg__(112)
+gemm_beside_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmDev p) { gemm_body<64, KIND>(tmA, tmB, p); }
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -289,6 +300,8 @@ cudaError_t gemm_init() {
   if (e == cudaSuccess) e = set_attr<256, 1>();
   if (e == cudaSuccess) e = set_attr<64, 0>();
   if (e == cudaSuccess) e = set_attr<64, 1>();
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_beside_kernel<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::smem_bytes(true));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_beside_kernel<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::smem_bytes(true));
   if (e == cudaSuccess) e = set_attr<64, 5>();
   if (e == cudaSuccess) e = set_attr<128, 5>();
   if (e == cudaSuccess) e = set_attr<192, 5>();
@@ -324,6 +337,9 @@ static cudaError_t launch_bn(const GemmArgs& g, const GemmDev& p, int tiles_m, c
   if (!make_tmap_bf16_2d(&tmB, g.w, g.N, g.K, BN)) return cudaErrorInvalidValue;
   const long tiles = (long)tiles_m * ((g.N + BN - 1) / BN);
   const int grid = (int)(tiles < g_num_sms ? tiles : g_num_sms);
+  if constexpr (BN == 64)
+    if (p.row_idx && gemm_leaves_room(g.M, g.rows_per_image, g.map_tokens, g.N))
+      return launch_pdl(p.epilogue == EPI_RESIDUAL ? gemm_beside_kernel<5> : gemm_beside_kernel<7>, dim3(grid), dim3(gemm_threads(5)), GemmCfg<BN>::smem_bytes(true), st, tmA, tmB, p);
   if (p.row_idx && p.epilogue == EPI_RESIDUAL)
     return launch_pdl(gemm_bf16_kernel<BN, 5>, dim3(grid), dim3(gemm_threads(5)), GemmCfg<BN>::smem_bytes(true), st, tmA, tmB, p);
   if (p.row_idx)

@@ -358,6 +358,69 @@ def test_kept_rows_restored_by_the_last_gemm(h, w, hc, wc, C, H, B, keep, resid_
 
 
 @pytest.mark.parametrize("resid_dtype", [0, 1])
+@pytest.mark.parametrize("sub", [0, 1])
+@pytest.mark.parametrize("h,w,hc,wc,C,H,B,keep", [(26, 31, 10, 10, 256, 2, 3, 0.16), (48, 41, 13, 9, 1920, 30, 5, 0.3), (64, 64, 13, 9, 1024, 16, 2, 0.035)])
+def test_kept_rows_restored_by_every_tile_of_the_last_gemm(h, w, hc, wc, C, H, B, keep, sub, resid_dtype):
+    """Every tile that can restore the kept rows (one CTA of 64 ... 256 columns, that of 64 in both its builds, pairs of 128 and 256) against the oracle, with image boundaries inside
+    its rows, a ragged last tile, and at the second shape more tiles than the GPU has SMs, so that accumulators and the tiles that turn rows are used again.
+    One sublayer alone has a nonzero branch, so the map that the selections behind it see is the step's output: each must keep that map's set, for which it
+    has only the column sums that the GEMM left.  The map is far from zero mean and its scores are dense: without one 32 x 32
+    block of the sums the kept set of the first shape changes in 22 places, without that of the second in 14."""
+    wl = I.Workload("every tile", L=2, C=C, H=H, B=B, sides=(hc, h), keep=(1.0, keep), mlp_ratio=1, seed=817)
+    mt = _zero_branch_tensors(wl)
+    if sub == 0:
+        mt.w_o[0], mt.b_o[0] = I.normal_bf16(833, (C, C), 0.3), I.normal_bf16(834, (C,), 0.3)
+    else:
+        mt.w_fc2[0], mt.b_fc2[0] = I.normal_bf16(833, (C, C), 0.04), I.normal_bf16(834, (C,), 0.3)
+    n, k = h * w, O.kept_count(keep, h, w)
+    x = I.token_map(835, B, h, w, C, "iid") + np.float32(6.0)
+    if resid_dtype:
+        x = _bf16_round(x)
+    ctx = fv.FvContext(wl.L, C, H, [(hc, wc), (h, w)], 0, B, k, mt, mlp_ratio=1, device=DEV, resid_dtype=resid_dtype)
+    for l in range(wl.L):
+        for si in range(2):
+            ctx.cache_view(l, si).zero_()
+    xd = torch.from_numpy(x).to(DEV).to(ctx.x_dtype)
+    first = O.pts_topk(O.pts_score(x), k)
+    forced = {(0, name): first for name in SUB_NAMES[2]}
+    orc = O.VarOracle(1, C, H, [(hc, wc), (h, w)], cache_step=0, weights=helpers_oracle_weights(mt), B=B)
+    orc.step = 1
+    orc.cache[0] = {name: np.zeros((B, hc * wc, C)) for name in SUB_NAMES[2]}
+    ref = orc.var_step(x, 1, keep, forced_idx=forced)
+    kept = np.zeros((B, n), dtype=bool)
+    np.put_along_axis(kept, first, True, axis=1)
+    bound = MAX_ABS + (2.0 ** -8 * np.abs(ref).max() if resid_dtype else 0.0)            # (bf16 stream: one rounding)
+    for path in (2, 3, 4, 5, 6, 7):
+        trace = torch.full((wl.L, 2, B, k), -1, dtype=torch.int32, device=DEV)
+        ctx.set_state(1, 0)
+        assert fv.lib().fv_gemm_force_path(path) == 0
+        try:
+            got = ctx.var_step(xd, 1, keep, idx_trace=trace).double().cpu().numpy()
+        finally:
+            fv.lib().fv_gemm_force_path(0)
+        assert ctx.device_status() == 0
+        sets = trace.cpu().numpy()
+        mine = np.zeros((B, n), dtype=bool)
+        np.put_along_axis(mine, sets[0, sub].astype(np.int64), True, axis=1)
+        assert np.array_equal(got[~mine], x[~mine].astype(np.float64)), path             # nothing but the kept rows is touched
+        both = mine & kept
+        assert both.sum() >= B * k - 4, path                                              # (the sets differ at near-ties alone: below)
+        err, cos = per_token_errors(got[both], ref[both])
+        assert err <= bound and cos >= MIN_COS, (path, err, cos)
+        if not resid_dtype:
+            assert per_token_errors(got[both] - x[both], ref[both] - x[both])[1] >= MIN_COS, path
+        for l in range(wl.L):
+            for si in range(2):
+                score = O.pts_score(x if (l, si) <= (0, sub) else got)
+                tau = np.sort(score, axis=1)[:, ::-1][:, k - 1]
+                want = O.pts_topk(score, k)
+                for b in range(B):
+                    diff = np.setxor1d(sets[l, si, b], want[b])
+                    assert np.all(np.abs(score[b, diff] - tau[b]) <= 1e-5 * tau[b]), (path, l, si, b, len(diff))
+    ctx.close()
+
+
+@pytest.mark.parametrize("resid_dtype", [0, 1])
 def test_bytes_counted_for_the_gemms_and_the_restoration_of_a_step(resid_dtype):
     """fv_profile_read's dram_bytes of both classes is the sum over their launches of operands and results: for a residual GEMM the stream read
     and written (with the copy for the cache, or the column sums of the kept rows), for a pruned step's side stream the restoration
