@@ -434,12 +434,14 @@ bool select_small_supported(int B, int n, int C, bool x_bf16) { return small_clu
 
 // Inside a step, between two sublayers whose last GEMM could restore the kept rows itself (128 of them per image): that route's selection has no
 // restoration in front of it and beats the one launch unless a CTA has very little to work through.  Us per block of 2 sublayers (3 at C 2048), this kernel ->
-// that route: 16 rows C 1024 68 -> 75 (two images 68 -> 74, four 78 -> 78), C 256 49 -> 55, C 2048 152 -> 147 (two images 164 -> 152), C 1920 bf16 stream 114 -> 108;
-// 21 rows C 1920 117 -> 103 (four images 169 -> 151); 25 rows C 512 74 -> 68, C 1024 78 -> 74; 32 rows C 1024, eight images, 94 -> 92; 36 rows
-// C 256 62 -> 60, C 512 74 -> 67, C 1024 bf16 98 -> 80.
+// that route, one / two / four images.  16 rows: C 256 50 -> 55 / 50 -> 56 / 54 -> 58, C 512 59 -> 63 / 59 -> 64 / 66 -> 65, C 768 63 -> 70 / 71 -> 69 / 71 -> 74, C 1024 67 -> 74 / 75 -> 76 /
+// 80 -> 82, C 1152 82 -> 78 / 82 -> 82 / 87 -> 88, C 1536 92 -> 89 / 98 -> 92 / 108 -> 102, C 2048 153 -> 146 / 164 -> 152 / 193 -> 185.  From 17 rows on a thread has a second
+// chunk of them: 18 rows C 512 64 -> 62 / 63 -> 64 / 67 -> 66, C 1024 73 -> 73 / 80 -> 77 / 85 -> 86, C 1536 102 -> 90 / 108 -> 94 / 120 -> 105.  Narrow models have so
+// little to move that it stays ahead: 23 rows C 128 52 -> 55 / 52 -> 55 / 55 -> 57, C 256 54 -> 57 / 57 -> 58 / 57 -> 58, C 384 57 -> 60 / 59 -> 61 / 65 -> 64; 28 rows C 128 54 -> 55 / 55 -> 55 /
+// 58 -> 58, C 256 57 -> 58 / 59 -> 60 / 63 -> 60, C 384 61 -> 62 / 62 -> 63 / 70 -> 66; 33 rows C 256 62 -> 60 / 63 -> 60 / 67 -> 63.  A bf16 stream has its lines in the same places.
 bool select_small_in_step(int B, int n, int C, bool x_bf16, bool gemm_could_restore) {
   const int cl = small_cluster(B, n, C, x_bf16);
-  return cl > 0 && (!gemm_could_restore || ((n + cl - 1) / cl <= 16 && C <= 1024));
+  return cl > 0 && (!gemm_could_restore || (C <= 1024 && (n + cl - 1) / cl <= (C <= 384 ? 24 : 16)));
 }
 
 cudaError_t launch_select_small(const SmallSelect& f, cudaStream_t st) {

@@ -299,6 +299,25 @@ def test_small_map_step_equals_the_separate_kernels(h, w, hc, wc, C, H, B, B_max
     ctx.close()
 
 
+# How many restoration launches a step of 2 blocks x 2 sublayers makes: 1 with one launch between two sublayers (only the last one restores by itself);
+# 7 where the last GEMM restores the kept rows (the other rows of every sublayer, and the sums of all but the last); 8 where a launch does.
+@pytest.mark.parametrize("resid_dtype", [0, 1])
+@pytest.mark.parametrize("h,w,C,H,B,keep,launches", [
+    (16, 16, 1024, 16, 1, 0.6, 1), (16, 17, 1024, 16, 1, 0.6, 7), (16, 16, 1152, 18, 1, 0.6, 7), (16, 24, 384, 6, 1, 0.6, 1), (16, 25, 256, 4, 1, 0.6, 7), (16, 17, 512, 8, 1, 0.6, 7), (18, 18, 1920, 30, 2, 0.75, 7), (18, 18, 1920, 30, 2, 0.35, 1),
+    (20, 28, 384, 6, 1, 0.9, 7), (20, 28, 384, 6, 1, 0.2, 1), (26, 31, 256, 2, 3, 0.16, 7), (26, 31, 256, 2, 3, 0.15, 8), (64, 64, 2048, 16, 1, 0.03, 8), (64, 64, 2048, 16, 1, 0.032, 7)])
+def test_route_of_a_pruned_step(h, w, C, H, B, keep, launches, resid_dtype):
+    wl = I.Workload("route", L=2, C=C, H=H, B=B, sides=(8, h), keep=(1.0, keep), mlp_ratio=1, seed=818)
+    ctx = fv.FvContext(wl.L, C, H, [(8, 8), (h, w)], 0, B, O.kept_count(keep, h, w), I.model_tensors(wl), mlp_ratio=1, device=DEV, resid_dtype=resid_dtype)
+    for l in range(wl.L):
+        for si in range(2):
+            ctx.cache_view(l, si).zero_()
+    ctx.set_state(1, 0)
+    fv.fv_profile_read()
+    ctx.var_step(torch.zeros((B, h * w, C), dtype=ctx.x_dtype, device=DEV), 1, keep)
+    assert fv.fv_profile_read()["restore"]["launches"] == launches and ctx.device_status() == 0
+    ctx.close()
+
+
 @pytest.mark.parametrize("resid_dtype", [0, 1])
 @pytest.mark.parametrize("h,w,hc,wc,C,H,B,keep", [(26, 31, 10, 10, 256, 2, 3, 0.16), (48, 41, 13, 9, 1920, 30, 1, 0.33), (32, 32, 16, 16, 1024, 8, 3, 0.5),
                                                   (29, 29, 12, 12, 1152, 9, 2, 0.9985)])
