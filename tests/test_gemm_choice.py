@@ -9,9 +9,9 @@ PROGRAM = r"""
 #include <cstdio>
 #include "paper_2503_23367_b200/csrc/gemm_choice.h"
 int main() {
-  int M, N, K, hd;
-  while (scanf("%d %d %d %d", &M, &N, &K, &hd) == 4) {
-    const fv::TileChoice t = fv::pick_tile(M, N, K, 148, hd);
+  int M, N, K, hd, clusters;
+  while (scanf("%d %d %d %d %d", &M, &N, &K, &hd, &clusters) == 5) {
+    const fv::TileChoice t = fv::pick_tile(M, N, K, 148, hd, clusters);
     printf("%d %d %d\n", t.bn, (int)t.pair, t.slices);
   }
 }
@@ -26,8 +26,8 @@ def pick(tmp_path_factory):
         f.write(PROGRAM)
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", ROOT, src, "-o", exe], check=True)
 
-    def run(shapes):
-        text = "\n".join(" ".join(map(str, s)) for s in shapes)
+    def run(shapes, clusters=1):
+        text = "\n".join(" ".join(map(str, (*s, clusters))) for s in shapes)
         out = subprocess.run([exe], input=text, check=True, capture_output=True, text=True).stdout
         return [tuple(map(int, line.split())) for line in out.splitlines()]
 
@@ -38,6 +38,27 @@ def _one_cta_cost(bn, M, N, K):
     fixed, per_round, per_kb = {128: (3.63, 0.81, 0.214), 192: (3.53, 1.79, 0.251), 256: (2.87, 2.28, 0.343)}[bn]
     ctas = -(-M // 128) * -(-N // bn)
     return fixed + -(-ctas // 148) * (per_round + -(-K // 64) * per_kb)
+
+
+def _cost(bn, pair, M, N, K):
+    fixed, per_round, per_kb = {(64, 0): (3.17, 0.42, 0.151), (128, 0): (3.63, 0.81, 0.214), (192, 0): (3.53, 1.79, 0.251), (256, 0): (2.87, 2.28, 0.343),
+                                (128, 1): (5.09, 1.11, 0.168), (256, 1): (6.47, 1.55, 0.292)}[bn, pair]
+    ctas = -(-M // (256 if pair else 128)) * -(-N // bn)
+    return fixed + -(-ctas // (74 if pair else 148)) * (per_round + -(-K // 64) * per_kb)
+
+
+@pytest.mark.parametrize("C", [256, 1024, 1920, 2048])
+def test_rows_of_a_map_take_the_cheapest_tile_that_is_no_cluster(pick, C):
+    seen = set()
+    for K in (C, 4 * C):
+        shapes = [(M, C, K, 0) for M in range(128, 6600, 37)]
+        for (M, _, _, _), (bn, pair, slices) in zip(shapes, pick(shapes, clusters=0)):
+            assert slices == 1
+            every = [(b, 0) for b in (64, 128, 192, 256)] + ([(128, 1), (256, 1)] if M > 256 else [])
+            assert _cost(bn, pair, M, C, K) <= min(_cost(*t, M, C, K) for t in every) + 1e-6, (M, K, bn, pair)
+            seen.add((bn, pair))
+    if C == 2048:
+        assert seen == {(64, 0), (128, 0), (192, 0), (256, 0), (128, 1), (256, 1)}         # every build of that epilogue is in use
 
 
 @pytest.mark.parametrize("C,head_dim", [(256, 64), (512, 64), (1024, 64), (1024, 128), (1536, 128), (1920, 64), (2048, 128)])

@@ -187,14 +187,24 @@ def _zero_branch_tensors(wl):
 
 
 ZERO_BRANCH_CASES = [  # h, w, hc, wc, C, H, B, B_max, keep, kind, oracle_runs_the_step
-    (40, 40, 32, 32, 2048, 16, 2, 2, 0.6, "structured", False),      # chunks fold in clusters of 4
-    (48, 48, 32, 32, 2048, 16, 2, 2, 0.4, "structured", False),      # clusters of 5
-    (64, 64, 32, 32, 2048, 16, 2, 2, 0.2, "structured", False),      # clusters of 8
+    (40, 40, 32, 32, 2048, 16, 2, 2, 0.6, "structured", False),      # 128 kept rows or more: the last GEMM leaves their sums, the side stream one
+    (48, 48, 32, 32, 2048, 16, 2, 2, 0.4, "structured", False),      # partial of all the others (fused: groups of chunks, folded through global memory)
+    (64, 64, 32, 32, 2048, 16, 2, 2, 0.2, "structured", False),
     (64, 64, 32, 32, 2048, 16, 2, 2, 0.2, "iid", False),
-    (33, 31, 10, 10, 256, 4, 3, 4, 0.5, "iid", True),                # ragged last chunk, partial batch, groups of 2
-    (50, 50, 13, 13, 1920, 30, 1, 1, 0.25, "structured", True),      # ragged last group (79 chunks in groups of 5)
-    (96, 96, 48, 48, 2048, 16, 1, 1, 0.2, "structured", False),      # groups of 18: fold through global memory
-    (128, 128, 48, 48, 2048, 16, 1, 1, 0.2, "structured", False),    # groups of 32, the 2K zero-shot step
+    (33, 31, 10, 10, 256, 4, 3, 4, 0.5, "iid", True),                # ragged last chunk, partial batch
+    (50, 50, 13, 13, 1920, 30, 1, 1, 0.25, "structured", True),
+    (96, 96, 48, 48, 2048, 16, 1, 1, 0.2, "structured", False),
+    (128, 128, 48, 48, 2048, 16, 1, 1, 0.2, "structured", False),    # the 2K zero-shot step
+]
+# Fewer than 128 kept rows: a launch of its own restores them and folds the chunks of all rows, group by group.
+ZERO_BRANCH_FEW_ROWS = [
+    (33, 31, 10, 10, 256, 4, 3, 4, 0.12, "iid", True),               # groups of 2, ragged last chunk, partial batch
+    (40, 40, 32, 32, 2048, 16, 2, 2, 0.07, "structured", False),     # groups of 4, each folded by a cluster
+    (48, 48, 32, 32, 2048, 16, 2, 2, 0.05, "structured", False),     # 5
+    (64, 64, 32, 32, 2048, 16, 2, 2, 0.03, "structured", False),     # 8
+    (50, 50, 13, 13, 1920, 30, 1, 1, 0.05, "structured", False),     # ragged last group (79 chunks in groups of 5)
+    (96, 96, 48, 48, 2048, 16, 1, 1, 0.0135, "structured", False),   # 18: through global memory
+    (128, 128, 48, 48, 2048, 16, 1, 1, 0.0077, "structured", False), # 32
 ]
 
 
@@ -202,7 +212,7 @@ ZERO_BRANCH_CASES = [  # h, w, hc, wc, C, H, B, B_max, keep, kind, oracle_runs_t
 @pytest.mark.parametrize("h,w,hc,wc,C,H,B,B_max,keep,kind,full_oracle", ZERO_BRANCH_CASES)
 def test_every_selection_of_a_step_on_bit_identical_input(h, w, hc, wc, C, H, B, B_max, keep, kind, full_oracle, fused):
     """Inside fv_var_step only the first selection sums the token map itself; every later one takes Eq. 4's column
-    sums from the restoration before it (rows that were not kept on a side stream, kept rows + fold after the last
+    sums from the restoration before it (rows that were not kept on a side stream, kept rows by the last
     GEMM).  With every branch ending in a zero projection and zero sublayer caches, each restoration adds exactly 0,
     so x entering EVERY sublayer is bit-identical on both sides and each of the 2 blocks x 3 selections must keep
     the oracle's set (any difference on a near-tie at the threshold, within 1e-5 relative).  Runs at the bench
@@ -261,11 +271,19 @@ def test_every_selection_of_a_step_on_bit_identical_input(h, w, hc, wc, C, H, B,
     ctx.close()
 
 
+@pytest.mark.parametrize("h,w,hc,wc,C,H,B,B_max,keep,kind,full_oracle", ZERO_BRANCH_FEW_ROWS)
+def test_every_selection_of_a_step_that_keeps_few_rows(h, w, hc, wc, C, H, B, B_max, keep, kind, full_oracle):
+    assert O.kept_count(keep, h, w) < 128
+    test_every_selection_of_a_step_on_bit_identical_input(h, w, hc, wc, C, H, B, B_max, keep, kind, full_oracle, 0)
+
+
 # Maps small enough for the one-launch form (a cluster of CTAs per image): one row per CTA, CTAs without a row, ragged last CTA, clusters
-# of 16 and (eight images) of 8, one and two chunks of rows per thread, channel groups that are not whole warps.
+# of 16 and (eight images) of 8, one and two chunks of rows per thread, channel groups that are not whole warps.  Those that keep 128 rows or more on more
+# than a few rows per CTA go with the last GEMM instead (18 x 18 at 0.75, 20 x 28 at 0.9: test_route_of_a_pruned_step has both).
 SMALL_MAPS = [(1, 3, 1, 1, 128, 2, 2, 2, 0.5, "iid"), (5, 7, 3, 3, 256, 4, 3, 4, 0.3, "iid"), (16, 16, 10, 10, 1024, 16, 1, 1, 0.5, "structured"),
               (13, 13, 10, 10, 1024, 16, 8, 8, 0.6, "structured"), (18, 18, 13, 13, 1920, 30, 2, 3, 0.75, "structured"), (24, 24, 9, 13, 256, 4, 2, 2, 0.15, "iid"),
-              (12, 12, 8, 8, 2048, 16, 2, 2, 0.6, "structured"), (20, 28, 13, 13, 384, 6, 1, 1, 0.9, "iid")]
+              (12, 12, 8, 8, 2048, 16, 2, 2, 0.6, "structured"), (20, 28, 13, 13, 384, 6, 1, 1, 0.9, "iid"),
+              (18, 18, 13, 13, 1920, 30, 2, 3, 0.35, "structured"), (20, 28, 13, 13, 384, 6, 1, 1, 0.2, "iid")]
 
 
 @pytest.mark.parametrize("h,w,hc,wc,C,H,B,B_max,keep,kind", SMALL_MAPS)
@@ -595,7 +613,8 @@ def test_bf16_residual_stream_schedule_against_the_oracle():
 
 
 @pytest.mark.parametrize("h,w,hc,wc,C,H,B,B_max,keep", [(64, 64, 32, 32, 2048, 16, 2, 2, 0.2), (33, 31, 10, 10, 256, 4, 3, 4, 0.5),
-                                                      (128, 128, 48, 48, 2048, 16, 1, 1, 0.2)])
+                                                      (128, 128, 48, 48, 2048, 16, 1, 1, 0.2), (33, 31, 10, 10, 256, 4, 3, 4, 0.12),
+                                                      (64, 64, 32, 32, 2048, 16, 2, 2, 0.03), (128, 128, 48, 48, 2048, 16, 1, 1, 0.0077)])
 def test_bf16_residual_stream_every_selection_on_bit_identical_input(h, w, hc, wc, C, H, B, B_max, keep):
     """The zero-branch step (see test_every_selection_of_a_step_on_bit_identical_input) with a bf16 stream: x + 0 is
     exact in bf16 too, so every one of the six selections -- five of them from the column sums the bf16 restoration
