@@ -593,7 +593,8 @@ fv_status fv_var_step(fv_ctx* ctx, const void* tokens_dev, int32_t B, int32_t sc
   // token's row of x, and the column sums of the updated rows fall out of the same registers.  As a launch of their own (forwarded rows stored in bf16, read
   // again, sums folded behind them) they took 13 us (64 x 64 tokens, C 2048), 19 (80 x 80) and 26 (128 x 128) between the GEMM and the selection that waits
   // for them; the epilogue is 1 ... 5 us longer (us per block of a pruned step: 64 x 64 311 -> 282, two images 434 -> 393, 80 x 80 418 -> 387, 128 x 128 951 -> 919,
-  // four of 32 x 32 at C 1920 270 -> 262).  Images of fewer kept rows than a
+  // four of 32 x 32 at C 1920 270 -> 262), also where the clusters that this epilogue lacks would have had the shorter GEMM (one image, 130 kept rows: 24 x 24, C 1024 96 -> 76, 32 x 32,
+  // C 2048 200 -> 165, 64 x 64, C 2048 276 -> 210; 300 rows of 48 x 48, C 1920 139 -> 122).  Images of fewer kept rows than a
   // tile take that launch, and so do small maps whose kept set is given, which then come out as the one-launch form leaves them, bit for bit.
   const bool gemm_restores = sub_pruned && !fused && !small_map && k >= kMinMapRows;
   float* kept_partial = nullptr;        // the column sums that the last such GEMM left (in y_buf, which then holds no forwarded rows)

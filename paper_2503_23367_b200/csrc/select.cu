@@ -199,8 +199,10 @@ __device__ __forceinline__ void mean_from_partials_halves(float4* s_mean, float4
 }
 static_assert(kMaxGroups == 16, "mean_from_partials_halves splits the groups 8 + 8");
 
-// The sums in two places: one partial of the rows that were not kept, and one per 128 of the compact rows (up to 27 at 128 x 128 tokens).  The
-// halves of the CTA take half of them each, eight loads in flight; stage: C4 float4 words.
+// The sums in two places: one partial of the rows that were not kept, and one per 128 of the compact rows (kept_rows / 128, two more where the
+// image begins and ends inside a block).  The halves of the CTA take half of them each, eight loads in flight; stage: C4 float4 words.  They are not folded to a fixed number
+// first: at keep 0.8 of 128 x 128 tokens they are 104, and the step is still ahead of the one that folds (us per block, that / this: C 2048 3890 / 3844, C 1024 2066 / 2055,
+// C 256 588 / 573; keep 0.5 2263 / 2201, 1106 / 1093, 359 / 342; 64 x 64 at 0.8 645 / 608, 281 / 267, 129 / 117).
 template <int T>
 __device__ __forceinline__ void mean_from_kept_partials(float4* s_mean, float4* stage, const float4* total, const float4* part, int np, int C4, int n) {
   constexpr int H = T / 2;
@@ -861,7 +863,7 @@ __global__ void inv_scatter_kernel(const int32_t* idx, int B, int k, int n, int3
 
 }  // namespace
 
-// group arrival counters [B, kMaxGroups], image arrival counters [B], two spare words per image
+// Group arrival counters [B, kMaxGroups], image arrival counters [B]; two words per image more that nothing reads: callers size their workspaces by this, so it stays.
 size_t select_ticket_bytes(int B) { return align_up((size_t)B * (kMaxGroups + 3) * sizeof(unsigned int), 256); }
 
 static void chunking(int n, int* nchunks, int* group, int* ngroups) {
