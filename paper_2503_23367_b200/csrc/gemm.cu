@@ -58,7 +58,7 @@ template <int BN> struct GemmCfg {
 // that epilogue takes eight warps and more registers per thread; the others stay small enough for a bandwidth-bound kernel of another
 // stream (the restoration of the rows that were not kept) to share the SMs with them.
 template <int BN, int KIND>
-__device__ __forceinline__ void gemm_body(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmDev& p) {
+__device__ __forceinline__ void gemm_body(const CUtensorMap& tmA, const CUtensorMap& tmB, const GemmDev p) {
   using Cfg = GemmCfg<BN>;
   constexpr int STAGES = Cfg::kStages;
   constexpr int KPS = Cfg::kKps;

@@ -228,16 +228,16 @@ template <bool XB, bool MAP, int BN, typename Release>
 __device__ __forceinline__ void residual_tile(const GemmDev& p, const ResidRows<MAP>& rr, typename ResidX<XB>::Raw (&x)[8], uint32_t t0, int half, int lane, int n0,
                                               const uint4* bias_w, float* tile, Release release) {
   constexpr int kChunks = BN / 32;
+  constexpr bool kOne = MAP && kChunks == 2;   // one chunk per warp: no loop, and no registers for a next one
   float4 keep0 = make_float4(0.f, 0.f, 0.f, 0.f), keep1 = keep0;   // sums of chunk (lane >> 3) of the warp's up to four
 #pragma unroll 1
-  for (int i = 0; i < kChunks / 2; ++i) {        // rolled: the code of one chunk is fetched once and then reused
-    const int ch = half + 2 * i;
+  for (int ch = half; ch < (kOne ? half + 1 : kChunks); ch += 2) {   // rolled: the code of one chunk is fetched once and then reused
     uint32_t r[32];
     typename ResidX<XB>::Raw nx[8];
     tmem_ld32(t0 + 32 * ch, r);
-    if (i + 1 < kChunks / 2) residual_load_x<XB, MAP>(p, rr, nx, lane, n0 + 32 * (ch + 2));
+    if (!kOne && ch + 2 < kChunks) residual_load_x<XB, MAP>(p, rr, nx, lane, n0 + 32 * (ch + 2));
     tmem_wait_ld();
-    if (i + 1 == kChunks / 2) release();           // accumulator fully in registers: hand the buffer back to the MMA warp
+    if (kOne || ch + 2 >= kChunks) release();            // accumulator fully in registers: hand the buffer back to the MMA warp
     float4 sum0 = make_float4(0.f, 0.f, 0.f, 0.f), sum1 = sum0;
     if (n0 + 32 * ch < p.N) residual_chunk<XB, MAP>(p, rr, r, x, tile, lane, n0 + 32 * ch, bias_w + 4 * ch, sum0, sum1);
     if constexpr (MAP) {
@@ -251,7 +251,7 @@ __device__ __forceinline__ void residual_tile(const GemmDev& p, const ResidRows<
       if ((lane >> 3) == (ch >> 1)) { keep0 = sum0; keep1 = sum1; }
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) x[j] = nx[j];
+    for (int i = 0; i < 8; ++i) x[i] = nx[i];
   }
   if constexpr (MAP) {
     *reinterpret_cast<float4*>(tile + 4 * lane) = keep0;
