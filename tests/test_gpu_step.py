@@ -283,7 +283,8 @@ def test_every_selection_of_a_step_that_keeps_few_rows(h, w, hc, wc, C, H, B, B_
 SMALL_MAPS = [(1, 3, 1, 1, 128, 2, 2, 2, 0.5, "iid"), (5, 7, 3, 3, 256, 4, 3, 4, 0.3, "iid"), (16, 16, 10, 10, 1024, 16, 1, 1, 0.5, "structured"),
               (13, 13, 10, 10, 1024, 16, 8, 8, 0.6, "structured"), (18, 18, 13, 13, 1920, 30, 2, 3, 0.75, "structured"), (24, 24, 9, 13, 256, 4, 2, 2, 0.15, "iid"),
               (12, 12, 8, 8, 2048, 16, 2, 2, 0.6, "structured"), (20, 28, 13, 13, 384, 6, 1, 1, 0.9, "iid"),
-              (18, 18, 13, 13, 1920, 30, 2, 3, 0.35, "structured"), (20, 28, 13, 13, 384, 6, 1, 1, 0.2, "iid")]
+              (18, 18, 13, 13, 1920, 30, 2, 3, 0.35, "structured"), (20, 28, 13, 13, 384, 6, 1, 1, 0.2, "iid"),
+              (16, 23, 10, 10, 384, 6, 2, 2, 0.6, "structured")]
 
 
 @pytest.mark.parametrize("h,w,hc,wc,C,H,B,B_max,keep,kind", SMALL_MAPS)
